@@ -612,8 +612,10 @@ constexpr int64_t kMaxSolveRank = 32768;      // the solve's r x r core and its 
 // Per-column-group products U_in^T V and U W.  FP32 factors run both on the tensor cores
 // (tcgen05, 3xTF32 with FP32 sums per row chunk) whenever the factor allows it (not disabled
 // by HDF_FLAG_CUDA_CORES, 16-byte aligned rows, at least 256 rows and 64 columns); below that
-// and for FP64 factors the CUDA-core tile kernels run.  One GroupWork serves every group of up
-// to cmax columns of one call; its buffers come from the stream-ordered pool.
+// and for FP64 factors the CUDA-core tile kernels run, and for FP64 groups of at most four
+// columns the streaming kernels of few_cols.cu (at four columns the product takes 1.84 ms
+// instead of 7.3 at 5,000 x 22,568 and 14.0 instead of 16.3 at 100,000 x 10,680).  One GroupWork serves every group of up to cmax columns of one call; its buffers come
+// from the stream-ordered pool.
 struct GroupWork {
     bool tc = false;         // tensor cores: the partial sums in `part` are FP32
     int nchunk = 0, tch = 0;
@@ -627,6 +629,7 @@ static bool tc_usable(const hdf_factor* f, int64_t n, int64_t r) {
            reinterpret_cast<uintptr_t>(f->U.p) % 16 == 0 && f->info.ldu % 4 == 0;
 }
 
+template <typename T>
 static hdf_status group_setup(const hdf_factor* fin, const hdf_factor* fout, int64_t r, int cmax, GroupWork& g,
                               cudaStream_t st) {
     const int64_t nin = fin->info.n, nout = fout->info.n;
@@ -638,7 +641,17 @@ static hdf_status group_setup(const hdf_factor* fin, const hdf_factor* fout, int
     } else {
         g.nchunk = utv_chunks(nin, r, cmax);
         g.chunk = (nin + g.nchunk - 1) / g.nchunk;
-        HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)g.nchunk * cmax * r, st));
+        int64_t slices = (int64_t)g.nchunk * cmax;
+        if (sizeof(T) == 8) {
+            // every group width up to kFewCols that a call of cmax columns can end with
+            for (int c = 1; c <= std::min(cmax, kFewCols); ++c) {
+                int64_t chunk;
+                int k;
+                few_utv_split(nin, r, c, &chunk, &k);
+                slices = std::max(slices, (int64_t)k * c);
+            }
+        }
+        HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)slices * r, st));
     }
     return HDF_OK;
 }
@@ -656,6 +669,13 @@ static hdf_status group_utv(const hdf_factor* fin, int64_t r, const T* V, int64_
                           g.twork.as<float>(), fin->dev_err.as<int>(), st, true);
         }
     }
+    if constexpr (sizeof(T) == 8) {
+        if (cg <= kFewCols) {
+            int64_t chunk;
+            few_utv_split(nin, r, cg, &chunk, np);
+            return few_utv(fin->U.as<double>(), fin->info.ldu, nin, r, V, ldv, cg, chunk, *np, g.part.as<double>(), st);
+        }
+    }
     *np = g.nchunk;
     launch_utv<T>(ct_for(cg), fin->U.as<T>(), fin->info.ldu, nin, r, V, ldv, cg, g.nchunk, g.chunk,
                   g.part.as<double>(), st);
@@ -670,11 +690,9 @@ static hdf_status group_reduce(const GroupWork& g, int np, int64_t r, int cg, co
                                cudaStream_t st) {
     HDF_COUNT_LAUNCH();
     if (g.tc)
-        dev::k_reduce_scale<T, float><<<grid_for(r * cg, 256, 1 << 30), 256, 0, st>>>(
-            reinterpret_cast<const float*>(g.part.p), np, r, cg, S, W, Wd);
+        dev::launch_reduce_scale<T>(reinterpret_cast<const float*>(g.part.p), np, r, cg, S, W, Wd, st);
     else
-        dev::k_reduce_scale<T><<<grid_for(r * cg, 256, 1 << 30), 256, 0, st>>>(g.part.as<double>(), np, r, cg, S, W,
-                                                                               Wd);
+        dev::launch_reduce_scale<T>(g.part.as<double>(), np, r, cg, S, W, Wd, st);
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
@@ -690,6 +708,10 @@ static hdf_status group_uw(const hdf_factor* fout, int64_t r, const T* W, int cg
                          reinterpret_cast<const float*>(W), cg, (float)alpha, reinterpret_cast<const float*>(B), ldb,
                          (float)beta, reinterpret_cast<float*>(Y), ldy, g.twork.as<float>(), fout->dev_err.as<int>(),
                          st);
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (cg <= kFewCols)
+            return few_uw(fout->U.as<double>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy, st);
     }
     launch_uw<T>(ct_for(cg), fout->U.as<T>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy, st);
     HDF_CUDA(cudaGetLastError());
@@ -716,8 +738,7 @@ static hdf_status matvec_free(const hdf_factor* f, const T* V, int64_t ldv, int 
         if (hdf_status e = mf_utv<T>(f, V + j0 * ldv, ldv, cg, part, &np, st); e != HDF_OK) return e;
         if (rec && j0 == 0) HDF_CUDA(cudaEventRecord(fm->mv_ev[1], st));
         HDF_COUNT_LAUNCH();
-        dev::k_reduce_scale<T><<<grid_for(r * cg, 256, 1 << 30), 256, 0, st>>>(part.as<double>(), np, r, cg, S_scale,
-                                                                               W.as<T>(), nullptr);
+        dev::launch_reduce_scale<T>(part.as<double>(), np, r, cg, S_scale, W.as<T>(), nullptr, st);
         HDF_CUDA(cudaGetLastError());
         if (rec && j0 == 0) HDF_CUDA(cudaEventRecord(fm->mv_ev[2], st));
         if (hdf_status e = mf_uw<T>(f, W.as<T>(), cg, Y + j0 * ldy, ldy, st); e != HDF_OK) return e;
@@ -751,7 +772,7 @@ static hdf_status matvec_t(const hdf_factor* f, const hdf_factor* fin, const T* 
     const int cmax = std::min(ncols, kMaxGroup);
     if (f->mf.on) return matvec_free<T>(f, V, ldv, ncols, Y, ldy, S_scale, alpha, B, beta, st);
     GroupWork g;
-    if (hdf_status e = group_setup(fin, f, r, cmax, g, st); e != HDF_OK) return e;
+    if (hdf_status e = group_setup<T>(fin, f, r, cmax, g, st); e != HDF_OK) return e;
     DevBuf W;
     HDF_CUDA(W.alloc_on(sizeof(T) * (size_t)r * cmax, st));
     hdf_factor* fm = const_cast<hdf_factor*>(f);
@@ -785,13 +806,12 @@ hdf_status utv_reduce(const hdf_factor* f, const T* V, int64_t ldv, int c, const
         int np = 0;
         if (hdf_status e = mf_utv<T>(f, V, ldv, c, part, &np, st); e != HDF_OK) return e;
         HDF_COUNT_LAUNCH();
-        dev::k_reduce_scale<T><<<grid_for(r * c, 256, 1 << 30), 256, 0, st>>>(part.as<double>(), np, r, c, S_scale,
-                                                                              W, Wd);
+        dev::launch_reduce_scale<T>(part.as<double>(), np, r, c, S_scale, W, Wd, st);
         HDF_CUDA(cudaGetLastError());
         return HDF_OK;
     }
     GroupWork g;
-    if (hdf_status e = group_setup(f, f, r, c, g, st); e != HDF_OK) return e;
+    if (hdf_status e = group_setup<T>(f, f, r, c, g, st); e != HDF_OK) return e;
     int np = 0;
     if (hdf_status e = group_utv<T>(f, r, V, ldv, c, g, &np, st); e != HDF_OK) return e;
     if (hdf_status e = group_reduce<T>(g, np, r, c, S_scale, W, Wd, st); e != HDF_OK) return e;
@@ -864,7 +884,7 @@ static hdf_status woodbury_apply(hdf_factor* f, double lambda, const T* Bin, int
     }
     const int cmax = std::min(ncols, kMaxGroup);
     GroupWork g;
-    if (hdf_status e = group_setup(f, f, r, cmax, g, st); e != HDF_OK) return e;
+    if (hdf_status e = group_setup<T>(f, f, r, cmax, g, st); e != HDF_OK) return e;
     DevBuf Wd, Zd, Wt;
     HDF_CUDA(Wd.alloc_on(sizeof(double) * (size_t)r * cmax, st));
     HDF_CUDA(Zd.alloc_on(sizeof(double) * (size_t)r * cmax, st));

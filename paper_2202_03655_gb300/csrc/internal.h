@@ -73,6 +73,15 @@ hdf_status mf_uw(const hdf_factor* f, const T* W, int c, T* Y, int64_t ldy, cuda
 hdf_status tc_uw(const float* U, int64_t ldU, int64_t n, int64_t r, const float* W, int c, float alpha, const float* B,
                  int64_t ldb, float beta, float* Y, int64_t ldy, float* work, int* err, cudaStream_t st);
 
+// FP64 products of one to four columns (few_cols.cu).  few_utv writes nchunk partial slices of
+// c x r (few_utv_split); r even, U and W 16-byte aligned with even leading dimension.
+constexpr int kFewCols = 4;
+void few_utv_split(int64_t n, int64_t r, int c, int64_t* chunk, int* nchunk);
+hdf_status few_utv(const double* U, int64_t ldU, int64_t n, int64_t r, const double* V, int64_t ldv, int c,
+                   int64_t chunk, int nchunk, double* part, cudaStream_t st);
+hdf_status few_uw(const double* U, int64_t ldU, int64_t n, int64_t r, const double* W, int c, double alpha,
+                  const double* B, int64_t ldb, double beta, double* Y, int64_t ldy, cudaStream_t st);
+
 // W = S_scale .* (U^T V) for one group of c <= 64 columns: W (r x c row-major, bulk) and/or
 // Wd (r x c, FP64).  S_scale may be null (no scaling).  Allocates its partial sums.
 template <typename T>

@@ -110,10 +110,8 @@ hdf_status run(const hdf_factor* f, const T* V, int64_t ldv, int ncols, T* Y, in
         // by k_reduce_scale, so nothing left from an earlier call is read
         utv<T>(ct, U, f->info.ldu, n, r, V + j0 * ldv, ldv, cg, nchunk, chunk, part, st);
         HDF_CUDA(cudaGetLastError());
-        const int64_t work = r * cg;
         HDF_COUNT_LAUNCH();
-        hdf::dev::k_reduce_scale<T><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(part, nchunk, r, cg, S, W,
-                                                                                    nullptr);
+        hdf::dev::launch_reduce_scale<T>(part, nchunk, r, cg, S, W, nullptr, st);
         HDF_CUDA(cudaGetLastError());
         uw<T>(ct, U, f->info.ldu, n, r, W, cg, Y + j0 * ldy, ldy, st);
         HDF_CUDA(cudaGetLastError());
