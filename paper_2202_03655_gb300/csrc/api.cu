@@ -609,15 +609,17 @@ static int utv_chunks(int64_t n, int64_t r, int cg) {
 constexpr int kMaxGroup = 64;
 constexpr int64_t kMaxSolveRank = 32768;      // the solve's r x r core and its factors on the device
 
-// Per-column-group products U_in^T V and U W.  FP32 factors run both on the tensor cores
-// (tcgen05, 3xTF32 with FP32 sums per row chunk) whenever the factor allows it (not disabled
-// by HDF_FLAG_CUDA_CORES, 16-byte aligned rows, at least 256 rows and 64 columns); below that
-// and for FP64 factors the CUDA-core tile kernels run, and for FP64 groups of at most four
-// columns the streaming kernels of few_cols.cu (at four columns the product takes 1.84 ms
-// instead of 7.3 at 5,000 x 22,568 and 14.0 instead of 16.3 at 100,000 x 10,680).  One GroupWork serves every group of up to cmax columns of one call; its buffers come
-// from the stream-ordered pool.
+// Per-column-group products U_in^T V and U W.  The tensor cores take them whenever the factor
+// allows it (not disabled by HDF_FLAG_CUDA_CORES, 16-byte aligned rows, at least 256 rows and 64
+// columns): FP32 factors as 3xTF32 with FP32 sums per row chunk, FP64 factors by exact integer
+// slices (tc_f64.cuh) unless the group is so narrow or small that the streaming kernels of
+// few_cols.cu are faster (f64_tensor below).  What is left -- FP64 groups of up to four columns on
+// those kernels, everything else on the register-tiled CUDA-core kernels.  One GroupWork serves
+// every group of up to cmax columns of one call; its buffers come from the stream-ordered pool.
 struct GroupWork {
-    bool tc = false;         // tensor cores: the partial sums in `part` are FP32
+    bool tc = false;         // FP32 on the tensor cores: the partial sums in `part` are FP32
+    bool f64 = false;        // FP64 on the tensor cores for the groups that f64_tensor names
+    DevBuf uwpart;           // its column splits of U W
     int nchunk = 0, tch = 0;
     int64_t chunk = 0, tchunk = 0;
     DevBuf part;             // partial sums: nchunk (or tch) x cmax x r, FP64
@@ -625,15 +627,27 @@ struct GroupWork {
 };
 
 static bool tc_usable(const hdf_factor* f, int64_t n, int64_t r) {
-    return f->prec == HDF_FP32 && f->use_tc && n >= 256 && r >= 64 &&
+    return f->use_tc && n >= 256 && r >= 64 &&
            reinterpret_cast<uintptr_t>(f->U.p) % 16 == 0 && f->info.ldu % 4 == 0;
+}
+
+// Whether a group of c columns of an FP64 product with n x r entries of U goes to the tensor cores
+// (where usable).  One column streams at the FP64 pipe's rate, about as fast as the slices are formed
+// (100,000 x 10,680: 3.71 ms; two to four columns by slices 3.50 ms).  Two to four columns: from
+// about 4 million entries on (20,001 x 424: 0.081 ms against 0.109 at two columns; 100,000 x 10,680:
+// 3.5 against 7.3 ms; below, at 2,000 x 440, 0.045 against 0.034 to 0.043 ms).  More: always (2,000 x
+// 440, 5 columns: 0.045 against 0.78 ms on the register-tiled kernels).
+static bool f64_tensor(int64_t n, int64_t r, int c) {
+    return c > kFewCols || (c >= 2 && n * r >= (4 << 20));
 }
 
 template <typename T>
 static hdf_status group_setup(const hdf_factor* fin, const hdf_factor* fout, int64_t r, int cmax, GroupWork& g,
                               cudaStream_t st) {
     const int64_t nin = fin->info.n, nout = fout->info.n;
-    g.tc = tc_usable(fin, nin, r) && tc_usable(fout, nout, r);
+    const bool tensor = tc_usable(fin, nin, r) && tc_usable(fout, nout, r);
+    g.tc = tensor && sizeof(T) == 4;
+    g.f64 = tensor && sizeof(T) == 8 && (f64_tensor(nin, r, cmax) || f64_tensor(nout, r, cmax));
     if (g.tc) {
         tc_utv_split(nin, r, &g.tchunk, &g.tch);
         HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)g.tch * cmax * r, st));
@@ -649,6 +663,22 @@ static hdf_status group_setup(const hdf_factor* fin, const hdf_factor* fout, int
                 int k;
                 few_utv_split(nin, r, c, &chunk, &k);
                 slices = std::max(slices, (int64_t)k * c);
+            }
+        }
+        if (g.f64) {
+            // the slices of V are 14 bytes per entry of up to 32 columns; where so much is not left
+            // beside a large factor, the CUDA-core kernels need none
+            const size_t wb = tc_f64_work_bytes(std::max(nin, r), cmax);
+            const cudaError_t e = g.twork.alloc_on(wb, st);
+            if (e == cudaErrorMemoryAllocation && wb > ((size_t)256 << 20)) {
+                cudaGetLastError();
+                g.f64 = false;
+            } else {
+                HDF_CUDA(e);
+                int kper;
+                slices = std::max(slices, (int64_t)tc_f64_utv_splits(nin, r, &kper) * cmax);
+                if (const int ns = tc_f64_uw_splits(nout, r, &kper); ns > 1)
+                    HDF_CUDA(g.uwpart.alloc_on(sizeof(double) * (size_t)ns * std::min(cmax, 32) * nout, st));
             }
         }
         HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)slices * r, st));
@@ -670,6 +700,12 @@ static hdf_status group_utv(const hdf_factor* fin, int64_t r, const T* V, int64_
         }
     }
     if constexpr (sizeof(T) == 8) {
+        if (g.f64 && f64_tensor(nin, r, cg)) {
+            int kper;
+            *np = tc_f64_utv_splits(nin, r, &kper);
+            return tc_f64_utv(fin->U.as<double>(), fin->info.ldu, nin, r, V, ldv, cg, g.part.as<double>(), g.twork.p,
+                              fin->dev_err.as<int>(), st);
+        }
         if (cg <= kFewCols) {
             int64_t chunk;
             few_utv_split(nin, r, cg, &chunk, np);
@@ -710,6 +746,9 @@ static hdf_status group_uw(const hdf_factor* fout, int64_t r, const T* W, int cg
                          st);
     }
     if constexpr (sizeof(T) == 8) {
+        if (g.f64 && f64_tensor(nout, r, cg))
+            return tc_f64_uw(fout->U.as<double>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy,
+                             g.uwpart.as<double>(), g.twork.p, fout->dev_err.as<int>(), st);
         if (cg <= kFewCols)
             return few_uw(fout->U.as<double>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy, st);
     }

@@ -73,6 +73,19 @@ hdf_status mf_uw(const hdf_factor* f, const T* W, int c, T* Y, int64_t ldy, cuda
 hdf_status tc_uw(const float* U, int64_t ldU, int64_t n, int64_t r, const float* W, int c, float alpha, const float* B,
                  int64_t ldb, float beta, float* Y, int64_t ldy, float* work, int* err, cudaStream_t st);
 
+// FP64 products on the tensor cores (tc_f64.cuh) for c <= 64 columns: U 16-byte aligned rows, V
+// n x c column-major, W r x c row-major.  tc_f64_utv writes tc_f64_utv_splits slices of c x r into
+// part; tc_f64_uw takes a part of tc_f64_uw_splits x min(c, 32) x n when that is above 1.
+// work: tc_f64_work_bytes of the contraction length.
+size_t tc_f64_work_bytes(int64_t k, int c);
+int tc_f64_utv_splits(int64_t n, int64_t r, int* kper);
+int tc_f64_uw_splits(int64_t n, int64_t r, int* kper);
+hdf_status tc_f64_utv(const double* U, int64_t ldU, int64_t n, int64_t r, const double* V, int64_t ldv, int c,
+                      double* part, void* work, int* err, cudaStream_t st);
+hdf_status tc_f64_uw(const double* U, int64_t ldU, int64_t n, int64_t r, const double* W, int c, double alpha,
+                     const double* B, int64_t ldb, double beta, double* Y, int64_t ldy, double* part, void* work,
+                     int* err, cudaStream_t st);
+
 // FP64 products of one to four columns (few_cols.cu).  few_utv writes nchunk partial slices of
 // c x r (few_utv_split); r even, U and W 16-byte aligned with even leading dimension.
 constexpr int kFewCols = 4;

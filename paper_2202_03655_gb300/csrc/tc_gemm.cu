@@ -35,6 +35,7 @@
 // lanes once.  Every wait on an mbarrier is bounded by a clock limit; on expiry the kernel
 // records an error, drains its own copies and MMAs, frees its TMEM and returns.
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -736,6 +737,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     cta_teardown<BN>(tmem, warp);
 }
 
+#include "tc_f64.cuh"
+
 // ------------------------------------------------ matrix-free products on the tensor cores
 // The products of a matrix-free factor (mfree.cu): the stored Z rows are the A operand, brought
 // by TMA exactly like the U tiles of k_tc_utv / k_tc_uw; only the small second operand changes.
@@ -1355,17 +1358,18 @@ static EncodeFn encode_fn() {
     return fn;
 }
 
-// 2-D FP32 tensor map: inner dimension `inner` (contiguous), outer `outer` with row stride
+// 2-D tensor map (FP32 unless `type` says otherwise): inner dimension `inner` (contiguous), outer `outer` with row stride
 // `stride_bytes`; box {box_inner, box_outer}; zero fill out of bounds.
 static bool make_map(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
-                     uint32_t box_inner, uint32_t box_outer, bool swizzle128) {
+                     uint32_t box_inner, uint32_t box_outer, bool swizzle128,
+                     CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_FLOAT32) {
     EncodeFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {inner, outer};
     const cuuint64_t strides[1] = {stride_bytes};
     const cuuint32_t box[2] = {box_inner, box_outer};
     const cuuint32_t es[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, es,
+    return fn(m, type, 2, const_cast<void*>(ptr), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -1434,7 +1438,118 @@ static hdf_status utv_bn(const float* U, int64_t ldU, int64_t n, int64_t r, cons
     return HDF_OK;
 }
 
+// Slices of one group of at most CP columns and the product with U.
+template <int CP, bool TRANS>
+static hdf_status f64_launch(const double* U, int64_t ldU, int64_t n, const __half* slices, int64_t kpad,
+                             const f64::Args& a, cudaStream_t st) {
+    CUtensorMap mU, mB;
+    const bool enc = TRANS ? make_map(&mU, U, (uint64_t)ldU, (uint64_t)n, (uint64_t)ldU * 8, BM, f64::KB, false,
+                                      CU_TENSOR_MAP_DATA_TYPE_FLOAT64)
+                           : make_map(&mU, U, (uint64_t)ldU, (uint64_t)n, (uint64_t)ldU * 8, 16, BM, true,
+                                      CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
+    if (!enc || !make_map(&mB, slices, (uint64_t)kpad, f64::NS * CP, (uint64_t)kpad * 2, f64::KB, f64::NS * CP, true,
+                          CU_TENSOR_MAP_DATA_TYPE_FLOAT16))
+        return fail(HDF_ECUDA, "FP64 tensor-core product: cannot encode a tensor map");
+    const size_t sm = f64::Sm<CP>::bytes();
+    auto kern = f64::k_tc_f64<CP, TRANS>;
+    HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HDF_COUNT_LAUNCH();
+    kern<<<std::min(a.nitems, num_sms()), f64::THREADS, sm, st>>>(mU, mB, a);
+    HDF_CUDA(cudaGetLastError());
+    return HDF_OK;
+}
+
 }  // namespace tc
+
+// ------------------------------------------------------------------ FP64 products (tc_f64.cuh)
+static int f64_cp(int c) { return c <= 16 ? 16 : 32; }
+static int64_t f64_kpad(int64_t k) { return (k + tc::f64::KB - 1) / tc::f64::KB * tc::f64::KB; }
+
+// Bytes of the slices and exponents of one sub-group of at most 32 columns over a contraction of k.
+size_t tc_f64_work_bytes(int64_t k, int c) {
+    const int cp = f64_cp(std::min(c, 32));
+    const int64_t kp = f64_kpad(k);
+    return (size_t)tc::f64::NS * cp * kp * 2 + (size_t)(kp / tc::f64::KB) * cp * sizeof(int) + 256;
+}
+
+// Row splits of U^T V (slices of the partial sums) and column splits of U W (1: written directly).
+int tc_f64_utv_splits(int64_t n, int64_t r, int* kper) {
+    int ns = 1;
+    tc::f64::choose_split((r + tc::BM - 1) / tc::BM, f64_kpad(n) / tc::f64::KB, 152, 152, kper, &ns);
+    return ns;
+}
+int tc_f64_uw_splits(int64_t n, int64_t r, int* kper) {
+    int ns = 1;
+    tc::f64::choose_split((n + tc::BM - 1) / tc::BM, f64_kpad(r) / tc::f64::KB, 152,
+                          std::max<int64_t>(1, std::min<int64_t>(16, (4 << 20) / n)), kper, &ns);
+    return ns;
+}
+
+hdf_status tc_f64_utv(const double* U, int64_t ldU, int64_t n, int64_t r, const double* V, int64_t ldv, int c,
+                      double* part, void* work, int* err, cudaStream_t st) {
+    int kper = 0;
+    const int ns = tc_f64_utv_splits(n, r, &kper);
+    const int64_t kpad = f64_kpad(n);
+    for (int j0 = 0; j0 < c; j0 += 32) {
+        const int cg = std::min(32, c - j0), cp = f64_cp(cg);
+        __half* sl = static_cast<__half*>(work);
+        int* eb = reinterpret_cast<int*>(sl + (size_t)tc::f64::NS * cp * kpad);
+        const unsigned g = (unsigned)((kpad / tc::f64::KB * cp + 7) / 8);
+        HDF_COUNT_LAUNCH();
+        if (cp == 16) tc::f64::k_f64_prep_v<16><<<g, 256, 0, st>>>(V + j0 * ldv, ldv, n, cg, kpad, sl, eb);
+        else tc::f64::k_f64_prep_v<32><<<g, 256, 0, st>>>(V + j0 * ldv, ldv, n, cg, kpad, sl, eb);
+        HDF_CUDA(cudaGetLastError());
+        tc::f64::Args a{};
+        a.n = n; a.r = r; a.nkb = (int)(kpad / tc::f64::KB); a.kper = kper;
+        a.mblocks = (int)((r + tc::BM - 1) / tc::BM);
+        a.nitems = a.mblocks * ns;
+        a.c = cg; a.eb = eb; a.err = err;
+        a.part = part; a.ctot = c; a.j0 = j0;
+        if (hdf_status e = cp == 16 ? tc::f64_launch<16, true>(U, ldU, n, sl, kpad, a, st)
+                                    : tc::f64_launch<32, true>(U, ldU, n, sl, kpad, a, st);
+            e != HDF_OK)
+            return e;
+    }
+    return HDF_OK;
+}
+
+hdf_status tc_f64_uw(const double* U, int64_t ldU, int64_t n, int64_t r, const double* W, int c, double alpha,
+                     const double* B, int64_t ldb, double beta, double* Y, int64_t ldy, double* part, void* work,
+                     int* err, cudaStream_t st) {
+    int kper = 0;
+    const int ns = tc_f64_uw_splits(n, r, &kper);
+    const int64_t kpad = f64_kpad(r);
+    for (int j0 = 0; j0 < c; j0 += 32) {
+        const int cg = std::min(32, c - j0), cp = f64_cp(cg);
+        __half* sl = static_cast<__half*>(work);
+        int* eb = reinterpret_cast<int*>(sl + (size_t)tc::f64::NS * cp * kpad);
+        const unsigned g = (unsigned)((kpad / tc::f64::KB * cp + 7) / 8);
+        HDF_COUNT_LAUNCH();
+        if (cp == 16) tc::f64::k_f64_prep_w<16><<<g, 256, 0, st>>>(W + j0, r, c, cg, kpad, sl, eb);
+        else tc::f64::k_f64_prep_w<32><<<g, 256, 0, st>>>(W + j0, r, c, cg, kpad, sl, eb);
+        HDF_CUDA(cudaGetLastError());
+        tc::f64::Args a{};
+        a.n = n; a.r = r; a.nkb = (int)(kpad / tc::f64::KB); a.kper = kper;
+        a.mblocks = (int)((n + tc::BM - 1) / tc::BM);
+        a.nitems = a.mblocks * ns;
+        a.c = cg; a.eb = eb; a.err = err;
+        a.alpha = alpha; a.beta = beta;
+        a.B = B ? B + j0 * ldb : nullptr; a.ldb = ldb;
+        a.Y = Y + j0 * ldy; a.ldy = ldy;
+        a.part = ns > 1 ? part : nullptr;
+        if (hdf_status e = cp == 16 ? tc::f64_launch<16, false>(U, ldU, n, sl, kpad, a, st)
+                                    : tc::f64_launch<32, false>(U, ldU, n, sl, kpad, a, st);
+            e != HDF_OK)
+            return e;
+        if (ns > 1) {
+            HDF_COUNT_LAUNCH();
+            tc::f64::k_f64_uw_finish<<<dim3((unsigned)((n + 255) / 256), (unsigned)cg), 256, 0, st>>>(
+                part, ns, n, cg, alpha, a.B, ldb, beta, a.Y, ldy);
+            HDF_CUDA(cudaGetLastError());
+        }
+    }
+    return HDF_OK;
+}
 
 bool encode_map_f32(CUtensorMap_st* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
                     uint32_t box_inner, uint32_t box_outer, bool swizzle128) {
