@@ -35,6 +35,7 @@
 #include <sys/stat.h>
 #include <vector>
 
+#include "few_cols.cuh"
 #include "hdf_kernels.cuh"
 #include "internal.h"
 #include "planner.h"
@@ -415,6 +416,33 @@ __global__ void __launch_bounds__(256) k_batch_uw(const MvSet* __restrict__ sets
                                  (T)1, nullptr, 0, (T)0, Y + S.off, ldy, w.blk * dev::UwShape<CT>::RB, Us, Ws);
         __syncthreads();
     }
+}
+
+// FP64 sets with one to four columns: the streaming bodies of few_cols.cuh, one block per item.
+// U^T V: (set, row chunk, 128 columns), four threads down the rows of a column pair; U W: 64 (one
+// or two columns) or 32 rows of a set.  Chunks are short (few_chunk), since sets of a few hundred
+// rows are otherwise one chunk each and leave most of the chip idle: 30 sets of about 460 rows and
+// 134 columns took 0.565 + 0.109 ms for U^T V and U W of one column on the register-tiled kernels,
+// 0.012 + 0.013 ms here.
+constexpr int kFewTx = 6;                // log2 of the threads across the columns
+inline int64_t few_chunk(int64_t n) { return std::min<int64_t>(4096, std::max<int64_t>(64, (n / 32 + 63) / 64 * 64)); }
+template <int C>
+__global__ void __launch_bounds__(256) k_batch_few_utv(const MvSet* __restrict__ sets, const MvItem* __restrict__ items,
+                                                       const double* __restrict__ V, int64_t ldv) {
+    const MvItem w = items[blockIdx.x];
+    const MvSet& S = sets[w.set];
+    const int64_t i0 = (int64_t)w.chunk * S.chunk;
+    few::few_utv_block<C>(reinterpret_cast<const double*>(S.U), S.ldU, S.r, V + S.off, ldv, i0, min(S.n, i0 + S.chunk),
+                          w.blk, kFewTx, S.part + (int64_t)w.chunk * C * S.r);
+}
+template <int C>
+__global__ void __launch_bounds__(256) k_batch_few_uw(const MvSet* __restrict__ sets, const MvItem* __restrict__ items,
+                                                      double* __restrict__ Y, int64_t ldy) {
+    const MvItem w = items[blockIdx.x];
+    const MvSet& S = sets[w.set];
+    few::few_uw_block<C, (C <= 2 ? 8 : 4)>(reinterpret_cast<const double*>(S.U), S.ldU, S.n, S.r,
+                                           reinterpret_cast<const double*>(S.W), 1.0, nullptr, 0, 0.0, Y + S.off, ldy,
+                                           0, w.blk);
 }
 
 // ------------------------------------------------ skinny FP32 matvec (c <= 16)
@@ -1501,8 +1529,9 @@ static hdf_status batch_matvec_t(hdf_batch* b, const T* V, int64_t ldv, int c, T
         std::vector<MvSet> ms(ns);
         std::vector<MvItem> iu, ir, iw;
         const int ct = ct_for(c);
-        const bool skinny = sizeof(T) == 4 && ct <= 16;
+        const bool skinny = sizeof(T) == 4 && ct <= 16, few = sizeof(T) == 8 && c <= kFewCols;
         int AB = (ct == 1) ? 256 : 128, RB = (ct == 1) ? 256 : 128;
+        if (few) { AB = 2 << kFewTx; RB = c <= 2 ? 64 : 32; }
         if (skinny) {                     // the streaming kernels' columns / rows per item
             AB = (ct <= 8) ? kPipeCols : SkinnyShape<16>::AB;
             RB = 32;                      // k_batch_uw_b: one 32-row tile per item (from the set table)
@@ -1512,7 +1541,7 @@ static hdf_status batch_matvec_t(hdf_batch* b, const T* V, int64_t ldv, int c, T
         for (int s = 0; s < ns; ++s) {
             const int64_t n = b->info[s].n, r = (b->info[s].rank > 0) ? b->info[s].ldu : 0;   // padded width
             ms[s].n = n; ms[s].r = r; ms[s].ldU = b->info[s].ldu; ms[s].off = b->off[s];
-            ms[s].chunk = 4096;
+            ms[s].chunk = few ? few_chunk(n) : 4096;
             ms[s].nchunk = (int)std::max<int64_t>(1, (n + ms[s].chunk - 1) / ms[s].chunk);
             poff[s] = ptot;
             ptot += (int64_t)ms[s].nchunk * c * std::max<int64_t>(1, r);
@@ -1634,6 +1663,20 @@ static hdf_status batch_matvec_t(hdf_batch* b, const T* V, int64_t ldv, int c, T
                 HDF_B_SK(8, k_batch_utv_p<8>, k_batch_uw_b<8>, utv_pipe_smem<8>(), bw_smem<8>())
                 HDF_B_SK(16, k_batch_utv_s<16>, k_batch_uw_b<16>, 0, bw_smem<16>())
 #undef HDF_B_SK
+            }
+        } else
+        if (sizeof(T) == 8 && c <= kFewCols) {
+            const double* Vd = reinterpret_cast<const double*>(V);
+            double* Yd = reinterpret_cast<double*>(Y);
+            switch (c) {
+#define HDF_B_FEW(C)                                                                                              \
+    case C:                                                                                                       \
+        if (b->n_utv) k_batch_few_utv<C><<<b->n_utv, 256, 0, b->cap>>>(S, b->mvitems_utv.as<MvItem>(), Vd, ldv);   \
+        if (b->n_red) k_batch_reduce<T><<<b->n_red, 256, 0, b->cap>>>(S, b->mvitems_red.as<MvItem>(), c);          \
+        if (b->n_uw) k_batch_few_uw<C><<<b->n_uw, 256, 0, b->cap>>>(S, b->mvitems_uw.as<MvItem>(), Yd, ldy);       \
+        break;
+                HDF_B_FEW(1) HDF_B_FEW(2) HDF_B_FEW(3) HDF_B_FEW(4)
+#undef HDF_B_FEW
             }
         } else
         switch (ct) {

@@ -44,3 +44,21 @@ def test_few_columns_cross_and_infinities():
     b = np.ones(333)
     b[17] = np.nan
     assert np.isnan(f.matvec(to_dev(b)).cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("c", [1, 2, 3, 4, 5])
+def test_batched_sets_match_single_builds(c):
+    """FP64 batches of few columns: ragged sets (below, at and above one chunk and one row block)
+    against the same sets built alone, whose products are checked above."""
+    from paper_2202_03655_gb300 import hdf
+    g = np.random.default_rng(77)
+    sizes = [1, 7, 63, 64, 65, 300, 2049, 5000]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    x = g.uniform(-1, 1, (off[-1], 3))
+    ells = g.uniform(0.5, 1.0, len(sizes))
+    V = g.standard_normal((off[-1], c))
+    Y = hdf.build_batched(to_dev(x), off, "gaussian", ells, 1e-6, precision="fp64").matvec(to_dev(V)).cpu().numpy()
+    for s in range(len(sizes)):
+        sl = slice(off[s], off[s + 1])
+        y = hdf.build(to_dev(x[sl]), "gaussian", ells[s], 1e-6).matvec(to_dev(V[sl])).cpu().numpy()
+        assert np.linalg.norm(Y[sl] - y) <= 10e-6 * np.linalg.norm(y)      # two factors of the same tolerance
