@@ -54,38 +54,64 @@ __global__ void k_km_assign(const double* __restrict__ x, int64_t n, int d, int 
 }
 
 // Update step, first stage: block b sums the coordinates (and counts) of its chunk's points per
-// cluster with fixed-order tree sums: part[(b k + c) (d + 1) + j], j = d the count.
+// cluster: part[(b k + c) (d + 1) + j], j = d the count.  The chunk (kKmChunk points) is staged in
+// shared memory with its labels; warp w takes the clusters w, w + 8, ... and adds their points with
+// fixed-order sums.  Bound by the passes over the staged labels (k chunk / 8 per warp) and the FP64
+// adds of the shuffles; 128 points per block, so that a few thousand points fill the chip.  With
+// 2,048 points per block and a block-wide tree per cluster and coordinate it took 0.49 ms at 13,760
+// points, d = 8, 30 clusters (7 blocks); now 0.010 ms.
+constexpr int kKmChunk = 128;
 __global__ void __launch_bounds__(256) k_km_partial(const double* __restrict__ x, int64_t n, int d, int k,
-                                                    const int* __restrict__ labels, int64_t chunk,
-                                                    double* __restrict__ part) {
-    __shared__ double sh[256];
-    const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-    for (int c = 0; c < k; ++c) {
-        double acc[dev::kMaxD + 1];
-        for (int j = 0; j <= d; ++j) acc[j] = 0.0;
-        for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x)
-            if (labels[i] == c) {
-                for (int j = 0; j < d; ++j) acc[j] += x[i * d + j];
-                acc[d] += 1.0;
+                                                    const int* __restrict__ labels, double* __restrict__ part) {
+    __shared__ double xs[kKmChunk * dev::kMaxD];
+    __shared__ int ls[kKmChunk];
+    const int64_t i0 = blockIdx.x * (int64_t)kKmChunk;
+    const int cnt = (int)min((int64_t)kKmChunk, n - i0);
+    for (int e = threadIdx.x; e < cnt * d; e += blockDim.x) xs[e] = x[i0 * d + e];
+    for (int e = threadIdx.x; e < kKmChunk; e += blockDim.x) ls[e] = e < cnt ? labels[i0 + e] : -1;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int c = warp; c < k; c += 8) {
+        double* out = part + ((int64_t)blockIdx.x * k + c) * (d + 1);
+        // lane j <= d adds coordinate j (or 1) of the cluster's points in order
+        double acc = 0.0;
+#pragma unroll
+        for (int q = 0; q < kKmChunk; q += 32) {
+            unsigned m = __ballot_sync(0xffffffffu, ls[q + lane] == c);
+            while (m) {
+                const int e = q + __ffs(m) - 1;
+                m &= m - 1;
+                if (lane < d) acc += xs[e * d + lane];
+                else if (lane == d) acc += 1.0;
             }
-        for (int j = 0; j <= d; ++j) {
-            const double t = dev::block_sum_256(acc[j], sh);
-            if (threadIdx.x == 0) part[((int64_t)blockIdx.x * k + c) * (d + 1) + j] = t;
         }
+        if (lane <= d) out[lane] = acc;
     }
 }
 
-// Update step, second stage: centre c = mean of its points (partials added in block order); a
-// centre without points stays where it is.
+// Update step, second stage: centre c = mean of its points (one warp per cluster; lanes take the
+// blocks in turn, then a fixed butterfly); a centre without points stays where it is.
 __global__ void k_km_finish(const double* __restrict__ part, int G, int k, int d, double* __restrict__ C) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (c >= k) return;
     double s[dev::kMaxD + 1];
-    for (int j = 0; j <= d; ++j) s[j] = 0.0;
-    for (int b = 0; b < G; ++b)
-        for (int j = 0; j <= d; ++j) s[j] += part[((int64_t)b * k + c) * (d + 1) + j];
-    if (s[d] > 0.0)
-        for (int j = 0; j < d; ++j) C[c * d + j] = s[j] / s[d];
+#pragma unroll
+    for (int j = 0; j <= dev::kMaxD; ++j) s[j] = 0.0;
+    for (int b = lane; b < G; b += 32)
+#pragma unroll
+        for (int j = 0; j <= dev::kMaxD; ++j)
+            if (j <= d) s[j] += part[((int64_t)b * k + c) * (d + 1) + j];
+#pragma unroll
+    for (int j = 0; j <= dev::kMaxD; ++j)
+        for (int o = 16; o > 0; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
+    double count = 0.0;
+#pragma unroll
+    for (int j = 0; j <= dev::kMaxD; ++j)
+        if (j == d) count = s[j];
+    if (lane == 0 && count > 0.0)
+#pragma unroll
+        for (int j = 0; j < dev::kMaxD; ++j)
+            if (j < d) C[c * d + j] = s[j] / count;
 }
 
 __global__ void k_gather_rows(const double* __restrict__ x, int d, const int64_t* __restrict__ idx, int64_t m,
@@ -175,6 +201,110 @@ void launch_direct(int d, dim3 g, cudaStream_t st, const float* a, int64_t m, co
 #undef HDF_DK
 }
 
+// The off-diagonal blocks of K^ stored once: M[j ldk + i] = the FP32 value that k_direct_kernel
+// forms for the pair (i, j), zero within a cluster and in the padding columns.  A conjugate-gradient
+// solve applies the same matrix hundreds of times, and forming a value (d differences, a square
+// root, an exponential) costs several times the 4 bytes of reading it: 13,760 points, d = 8, one
+// product 0.43 ms evaluated, 0.12 ms stored (6.3 TB/s), 0.29 ms to store.
+constexpr int kOffTile = 64;         // columns j per block of k_off_store
+constexpr int kOffRows = 1024;       // rows i per block (four per thread)
+template <int DD>
+__global__ void __launch_bounds__(256) k_off_store(const float* __restrict__ a, int64_t n, int64_t ldk, int kernel,
+                                                   float inv_ell, const int* __restrict__ cl, float* __restrict__ M) {
+    __shared__ float bs[kOffTile][DD];
+    __shared__ int cs[kOffTile];
+    const int64_t j0 = blockIdx.y * (int64_t)kOffTile;
+    const int nt = (int)min((int64_t)kOffTile, n - j0);
+    for (int e = threadIdx.x; e < nt * DD; e += 256) bs[e / DD][e % DD] = a[j0 * DD + e];
+    for (int e = threadIdx.x; e < nt; e += 256) cs[e] = cl[j0 + e];
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)kOffRows + 4 * threadIdx.x;
+    if (i >= ldk) return;
+    float ai[4][DD];
+    int ci[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int64_t q = min(i + u, n - 1);
+#pragma unroll
+        for (int e = 0; e < DD; ++e) ai[u][e] = a[q * DD + e];
+        ci[u] = i + u < n ? cl[q] : -1;
+    }
+    for (int r = 0; r < nt; ++r) {
+        float kv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float s = 0.f;
+#pragma unroll
+            for (int q = 0; q < DD; ++q) { const float t = ai[u][q] - bs[r][q]; s = fmaf(t, t, s); }
+            kv[u] = dev::kernel_value_f(kernel, sqrtf(s), inv_ell);
+            if (ci[u] == cs[r] || ci[u] < 0) kv[u] = 0.f;
+        }
+        *reinterpret_cast<float4*>(M + (j0 + r) * ldk + i) = make_float4(kv[0], kv[1], kv[2], kv[3]);
+    }
+}
+void launch_off_store(int d, cudaStream_t st, const float* a, int64_t n, int64_t ldk, int kernel, float inv_ell,
+                      const int* cl, float* M) {
+    const dim3 g((unsigned)((ldk + kOffRows - 1) / kOffRows), (unsigned)((n + kOffTile - 1) / kOffTile));
+#define HDF_OS(DD) case DD: k_off_store<DD><<<g, 256, 0, st>>>(a, n, ldk, kernel, inv_ell, cl, M); break;
+    switch (d) { HDF_OS(1) HDF_OS(2) HDF_OS(3) HDF_OS(4) HDF_OS(5) HDF_OS(6) HDF_OS(7) HDF_OS(8) }
+#undef HDF_OS
+}
+
+// part[s n + i] = sum over the columns j of split s of M[j ldk + i] w_j (M is symmetric, so its rows
+// are read along i, 16 bytes a thread).  The same exact products and FP32-pair sums as
+// k_direct_kernel per 128 columns, added in FP64.  Bound by the read of M.
+constexpr int kOffK = 128;
+__global__ void __launch_bounds__(256) k_off_apply(const float* __restrict__ M, int64_t n, int64_t ldk,
+                                                   const double* __restrict__ w, int64_t split,
+                                                   double* __restrict__ part) {
+    __shared__ float2 ws[kOffK];                 // w_j = hi + lo
+    const int64_t i = blockIdx.x * (int64_t)kOffRows + 4 * threadIdx.x;
+    const bool act = i < ldk;
+    const int64_t j0 = blockIdx.y * split, j1 = min(n, j0 + split);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t t0 = j0; t0 < j1; t0 += kOffK) {
+        const int nt = (int)min((int64_t)kOffK, j1 - t0);
+        __syncthreads();
+        if (threadIdx.x < nt) {
+            const double wv = w[t0 + threadIdx.x];
+            const float hi = (float)wv;
+            ws[threadIdx.x] = make_float2(hi, (float)(wv - (double)hi));
+        }
+        __syncthreads();
+        if (!act) continue;
+        float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* Mt = M + t0 * ldk + i;
+#pragma unroll 8
+        for (int r = 0; r < nt; ++r) {
+            const float4 kv = __ldcs(reinterpret_cast<const float4*>(Mt + (int64_t)r * ldk));
+            const float2 wr = ws[r];
+            const float k4[4] = {kv.x, kv.y, kv.z, kv.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float p = k4[u] * wr.x;
+                const float e = fmaf(k4[u], wr.y, fmaf(k4[u], wr.x, -p));    // exact error of p, plus k w_lo
+                float s, t;
+                dev::two_sum(sh[u], p, s, t);
+                sh[u] = s;
+                sl[u] += t + e;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] += (double)sh[u] + (double)sl[u];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (i + u < n) part[blockIdx.y * n + i + u] = acc[u];
+}
+// Column splits of k_off_apply: about eight blocks per SM, whole tiles of kOffK columns.
+int64_t off_split(int64_t n, int64_t ldk, int* S) {
+    const int64_t rb = (ldk + kOffRows - 1) / kOffRows, tiles = (n + kOffK - 1) / kOffK;
+    const int64_t s = std::max<int64_t>(1, std::min<int64_t>(8 * 152 / rb, tiles));
+    const int64_t split = (tiles + s - 1) / s * kOffK;
+    *S = (int)((n + split - 1) / split);
+    return split;
+}
+
 // out[i] = alpha v[i] + (add ? add[i] : 0) + sum_s part[s m + i]
 __global__ void k_direct_finish(const double* __restrict__ part, int S, int64_t m, double alpha,
                                 const double* __restrict__ v, const double* __restrict__ add, double* __restrict__ out) {
@@ -227,35 +357,92 @@ __global__ void k_to_f64(const float* __restrict__ v, int64_t n, double* __restr
     if (i < n) out[i] = (double)v[i];
 }
 
-// part[b] = sum over the block's chunk of a_i b_i (fixed-order tree sums), two pairs at once.
-__global__ void __launch_bounds__(256) k_dot2(const double* __restrict__ a, const double* __restrict__ b,
-                                              const double* __restrict__ c, const double* __restrict__ e, int64_t n,
-                                              int64_t chunk, double* __restrict__ part) {
-    __shared__ double sh[256];
-    const int64_t i0 = blockIdx.x * chunk, i1 = min(n, i0 + chunk);
-    double s1 = 0.0, s2 = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        s1 += a[i] * b[i];
-        if (c) s2 += c[i] * e[i];
-    }
-    const double t1 = dev::block_sum_256(s1, sh);
-    const double t2 = dev::block_sum_256(s2, sh);
-    if (threadIdx.x == 0) { part[2 * blockIdx.x] = t1; part[2 * blockIdx.x + 1] = t2; }
+// ----------------------------------------------- conjugate gradients on the device
+// One iteration is a fixed chain of kernels; its scalars live in CgState, so that the host reads
+// the state only every few iterations.  At 13,760 points an iteration went from 0.85 ms (0.43 the
+// off-diagonal blocks, 0.57 + 0.11 the HDF blocks partly hidden, two host round trips) to 0.21 ms.  Iteration it reads rz[it & 1] and writes rz[(it + 1) & 1].  After
+// `done` every kernel returns at once, so iterations enqueued past the end change nothing.  Every
+// block adds the partial sums of a dot product itself, in the same fixed order.
+struct CgState {
+    double rz[2];
+    double nb, rtol;             // norm of the right-hand side
+    double res;                  // relative residual after iteration `it`
+    int it, done, bad;           // bad: p . q <= 0
+};
+
+// Sum of m values v[stride e + off] by a 256-thread block, the same on every block and thread.
+__device__ __forceinline__ double block_total(const double* __restrict__ v, int m, int stride, int off, double* sh) {
+    double s = 0.0;
+    for (int e = threadIdx.x; e < m; e += 256) s += v[(int64_t)stride * e + off];
+    return dev::block_sum_256(s, sh);
 }
 
-// x += alpha p; r -= alpha q
-__global__ void k_cg_step(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
-                          const double* __restrict__ q, double alpha, int64_t n) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// nb = |r|, rz[0] = r . z from the partial sums (2 per block) of k_block_gemv.
+__global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ part, int m, double rtol, CgState* S) {
+    __shared__ double sh[256];
+    const double rz = block_total(part, m, 2, 0, sh), bb = block_total(part, m, 2, 1, sh);
+    if (threadIdx.x == 0) {
+        S->rz[0] = rz; S->rz[1] = 0.0;
+        S->nb = sqrt(bb); S->rtol = rtol;
+        S->res = bb > 0.0 ? 1.0 : 0.0;
+        S->it = 0; S->bad = 0;
+        S->done = !(bb > 0.0);
+    }
+}
+
+// q = lambda p + add + sum_s part[s n + .] and the block's part of p . q.
+__global__ void __launch_bounds__(256) k_cg_finish(const double* __restrict__ part, int nsplit, int64_t n, double lam,
+                                                   const double* __restrict__ p, const double* __restrict__ add,
+                                                   double* __restrict__ q, double* __restrict__ dot,
+                                                   const CgState* __restrict__ S) {
+    __shared__ double sh[256];
+    if (S->done) return;
+    const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+    double d = 0.0;
+    if (i < n) {
+        double s = lam * p[i] + add[i];
+        for (int t = 0; t < nsplit; ++t) s += part[t * n + i];
+        q[i] = s;
+        d = p[i] * s;
+    }
+    const double tot = dev::block_sum_256(d, sh);
+    if (threadIdx.x == 0) dot[blockIdx.x] = tot;
+}
+
+// alpha = rz / (p . q); x += alpha p; r -= alpha q.
+__global__ void __launch_bounds__(256) k_cg_step(double* __restrict__ x, double* __restrict__ r,
+                                                 const double* __restrict__ p, const double* __restrict__ q, int64_t n,
+                                                 const double* __restrict__ dot, int m, int it, CgState* S) {
+    __shared__ double sh[256];
+    if (S->done) return;
+    const double pq = block_total(dot, m, 1, 0, sh);
+    if (!(pq > 0.0)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) { S->bad = 1; S->it = it; S->done = 1; }
+        return;
+    }
+    const double alpha = S->rz[(it - 1) & 1] / pq;
+    const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
     if (i >= n) return;
     x[i] += alpha * p[i];
     r[i] -= alpha * q[i];
 }
 
-// p = z + beta p
-__global__ void k_cg_dir(double* __restrict__ p, const double* __restrict__ z, double beta, int64_t n) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) p[i] = z[i] + beta * p[i];
+// Residual check; beta = rz_new / rz; p = z + beta p.  dot: (r . z, r . r) of every gemv block.
+__global__ void __launch_bounds__(256) k_cg_dir(double* __restrict__ p, const double* __restrict__ z, int64_t n,
+                                                const double* __restrict__ dot, int m, int it, CgState* S) {
+    __shared__ double sh[256];
+    if (S->done) return;
+    const double rz = block_total(dot, m, 2, 0, sh), rr = block_total(dot, m, 2, 1, sh);
+    const double res = sqrt(rr) / S->nb;
+    const bool end = res <= S->rtol;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        S->res = res;
+        S->it = it;
+        S->rz[it & 1] = rz;
+        if (end) S->done = 1;
+    }
+    const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+    if (!end && i < n) p[i] = z[i] + rz / S->rz[(it - 1) & 1] * p[i];
 }
 
 // ------------------------------------------------------------------- preconditioner
@@ -274,20 +461,36 @@ __global__ void k_block_matrices(const double* __restrict__ xp, int d, const int
     }
 }
 
-// z = M r: one warp per row of the block-diagonal inverse (packed as above).
-__global__ void k_block_gemv(const double* __restrict__ inv, const int64_t* __restrict__ offs,
-                             const int64_t* __restrict__ ioff, const int* __restrict__ cl, int64_t n,
-                             const double* __restrict__ r, double* __restrict__ z) {
-    const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const int c = cl[row];
-    const int64_t a0 = offs[c], nc = offs[c + 1] - a0, i = row - a0;
-    const double* M = inv + ioff[c] + i * nc;
-    double s = 0.0;
-    for (int64_t j = lane; j < nc; j += 32) s += M[j] * r[a0 + j];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) z[row] = s;
+// z = M r: one warp per row of the block-diagonal inverse (packed as above), four loads in flight
+// per lane.  With dot (and a state that is not done): (r . z, r . r) of the block's rows as well.
+__global__ void __launch_bounds__(256) k_block_gemv(const double* __restrict__ inv, const int64_t* __restrict__ offs,
+                                                    const int64_t* __restrict__ ioff, const int* __restrict__ cl,
+                                                    int64_t n, const double* __restrict__ r, double* __restrict__ z,
+                                                    double* __restrict__ dot, const CgState* __restrict__ S) {
+    __shared__ double sh[2][8];
+    if (S && S->done) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t row = blockIdx.x * (int64_t)8 + warp;
+    double s = 0.0, rv = 0.0;
+    if (row < n) {
+        const int c = cl[row];
+        const int64_t a0 = offs[c], nc = offs[c + 1] - a0, i = row - a0;
+        const double* M = inv + ioff[c] + i * nc;
+        const double* rc = r + a0;
+        rv = r[row];
+#pragma unroll 4
+        for (int64_t j = lane; j < nc; j += 32) s = fma(__ldcs(M + j), rc[j], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) z[row] = s;
+    }
+    if (!dot) return;
+    if (lane == 0) { sh[0][warp] = row < n ? rv * s : 0.0; sh[1][warp] = rv * rv; }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int q = 0; q < 8; ++q) t += sh[threadIdx.x][q];
+        dot[2 * (int64_t)blockIdx.x + threadIdx.x] = t;
+    }
 }
 
 // --------------------------------------- block preconditioner: batched SPD inverse (FP64)
@@ -553,16 +756,26 @@ struct hdf_krr {
     DevBuf perm, xp, xp32, cl, doffs, dioff, inv;
     hdf_batch* batch = nullptr;
     DevBuf vb, yb, hd, part, dotp;       // work: bulk-typed vectors, HDF result, direct-kernel partials
+    DevBuf koff;                         // the stored off-diagonal blocks (none: evaluated per product)
+    int64_t ldk = 0;
+    DevBuf cgst;                         // CgState of the running solve
+    CgState* cgh = nullptr;              // two pinned copies for the host
+    cudaEvent_t cgev[2] = {nullptr, nullptr};
     int S = 1;
     int64_t split = 0;
     double t_build = 0.0, t_precond = 0.0;
-    ~hdf_krr() { if (batch) hdf_batch_free(batch); }
+    ~hdf_krr() {
+        if (batch) hdf_batch_free(batch);
+        if (cgh) cudaFreeHost(cgh);
+        for (cudaEvent_t e : cgev) if (e) cudaEventDestroy(e);
+    }
 };
 
 namespace {
 
-// tp = lambda vp + K^ vp in cluster order (vp, tp length n, FP64, device)
-hdf_status apply_perm(hdf_krr* K, const double* vp, double* tp, cudaStream_t st) {
+// The parts of K^ vp in cluster order (vp FP64, length n): the HDF blocks into K->hd, the splits of
+// the off-diagonal blocks into K->part.
+hdf_status apply_parts(hdf_krr* K, const double* vp, cudaStream_t st) {
     const int64_t n = K->n;
     const int gb = blocks_for(n, 256, 1 << 30);
     hdf_status s;
@@ -577,41 +790,36 @@ hdf_status apply_perm(hdf_krr* K, const double* vp, double* tp, cudaStream_t st)
         s = hdf_batch_matvec(K->batch, vp, n, 1, K->hd.p, n, reinterpret_cast<hdf_stream>(st));
         if (s != HDF_OK) return s;
     }
-    dim3 g((unsigned)((n + kDkRows - 1) / kDkRows), (unsigned)K->S);
     HDF_COUNT_LAUNCH();
-    launch_direct(K->d, g, st, K->xp32.as<float>(), n, K->xp32.as<float>(), n, K->kernel, (float)(1.0 / K->ell), vp,
-                  K->cl.as<int>(), K->cl.as<int>(), K->split, K->part.as<double>());
-    HDF_COUNT_LAUNCH();
-    k_direct_finish<<<gb, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, vp, K->hd.as<double>(), tp);
+    if (K->koff.p) {
+        const dim3 g((unsigned)((K->ldk + kOffRows - 1) / kOffRows), (unsigned)K->S);
+        k_off_apply<<<g, 256, 0, st>>>(K->koff.as<float>(), n, K->ldk, vp, K->split, K->part.as<double>());
+    } else {
+        dim3 g((unsigned)((n + kDkRows - 1) / kDkRows), (unsigned)K->S);
+        launch_direct(K->d, g, st, K->xp32.as<float>(), n, K->xp32.as<float>(), n, K->kernel, (float)(1.0 / K->ell),
+                      vp, K->cl.as<int>(), K->cl.as<int>(), K->split, K->part.as<double>());
+    }
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
 
-hdf_status precond_perm(hdf_krr* K, const double* rp, double* zp, cudaStream_t st) {
+// tp = lambda vp + K^ vp in cluster order (vp, tp length n, FP64, device)
+hdf_status apply_perm(hdf_krr* K, const double* vp, double* tp, cudaStream_t st) {
+    if (hdf_status s = apply_parts(K, vp, st); s != HDF_OK) return s;
     HDF_COUNT_LAUNCH();
-    k_block_gemv<<<blocks_for(K->n * 32, 256, 1 << 30), 256, 0, st>>>(K->inv.as<double>(), K->doffs.as<int64_t>(),
-                                                                     K->dioff.as<int64_t>(), K->cl.as<int>(), K->n,
-                                                                     rp, zp);
+    k_direct_finish<<<blocks_for(K->n, 256, 1 << 30), 256, 0, st>>>(K->part.as<double>(), K->S, K->n, K->lam, vp,
+                                                                    K->hd.as<double>(), tp);
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
 
-// (a . b, c . e) with deterministic partial sums (c may be null)
-hdf_status dot2(hdf_krr* K, const double* a, const double* b, const double* c, const double* e, double* r1,
-                double* r2, cudaStream_t st) {
-    const int64_t n = K->n;
-    const int G = blocks_for(n, 4096, 256);
-    const int64_t chunk = (n + G - 1) / G;
+hdf_status precond_perm(hdf_krr* K, const double* rp, double* zp, cudaStream_t st, double* dot = nullptr,
+                        const CgState* S = nullptr) {
     HDF_COUNT_LAUNCH();
-    k_dot2<<<G, 256, 0, st>>>(a, b, c, e, n, chunk, K->dotp.as<double>());
+    k_block_gemv<<<(unsigned)((K->n + 7) / 8), 256, 0, st>>>(K->inv.as<double>(), K->doffs.as<int64_t>(),
+                                                             K->dioff.as<int64_t>(), K->cl.as<int>(), K->n, rp, zp, dot,
+                                                             S);
     HDF_CUDA(cudaGetLastError());
-    double h[512];
-    HDF_CUDA(cudaMemcpyAsync(h, K->dotp.p, sizeof(double) * 2 * G, cudaMemcpyDeviceToHost, st));
-    HDF_CUDA(cudaStreamSynchronize(st));
-    double s1 = 0.0, s2 = 0.0;
-    for (int g = 0; g < G; ++g) { s1 += h[2 * g]; s2 += h[2 * g + 1]; }
-    *r1 = s1;
-    if (r2) *r2 = s2;
     return HDF_OK;
 }
 
@@ -635,8 +843,7 @@ hdf_status hdf_kmeans(const double* x_dev, int64_t n, int d, int k, const int64_
     k_gather_rows<<<blocks_for((int64_t)k * d, 256, 1 << 30), 256, 0, st>>>(x_dev, d, idx.as<int64_t>(), k,
                                                                            C.as<double>());
     HDF_CUDA(cudaMemsetAsync(labels_dev, 0xff, sizeof(int) * n, st));      // -1: every label changes first
-    const int G = blocks_for(n, 2048, 512);
-    const int64_t chunk = (n + G - 1) / G;
+    const int G = (int)((n + kKmChunk - 1) / kKmChunk);
     HDF_CUDA(part.alloc_on(sizeof(double) * (size_t)G * k * (d + 1), st));
     HDF_CUDA(chg.alloc_on(sizeof(int), st));
     int it = 0;
@@ -651,9 +858,9 @@ hdf_status hdf_kmeans(const double* x_dev, int64_t n, int d, int k, const int64_
         HDF_CUDA(cudaStreamSynchronize(st));
         if (changes == 0 && it > 1) break;
         HDF_COUNT_LAUNCH();
-        k_km_partial<<<G, 256, 0, st>>>(x_dev, n, d, k, labels_dev, chunk, part.as<double>());
+        k_km_partial<<<G, 256, 0, st>>>(x_dev, n, d, k, labels_dev, part.as<double>());
         HDF_COUNT_LAUNCH();
-        k_km_finish<<<blocks_for(k, 128, 1 << 20), 128, 0, st>>>(part.as<double>(), G, k, d, C.as<double>());
+        k_km_finish<<<(k + 3) / 4, 128, 0, st>>>(part.as<double>(), G, k, d, C.as<double>());
         HDF_CUDA(cudaGetLastError());
     }
     if (it > max_iter) it = max_iter;
@@ -825,10 +1032,26 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         if (hbad) return bail(fail(HDF_ESINGULAR, "hdf_krr_build: a block lambda I + K_cc is not positive definite"));
     }
     // work space
-    K->split = direct_split(n, n, &K->S);
+    // the off-diagonal blocks are stored while they take at most 8 GiB (46,000 points) and the
+    // device has room; else every product evaluates them
+    K->ldk = (n + 3) / 4 * 4;
+    const size_t kbytes = sizeof(float) * (size_t)n * K->ldk;
+    if (kbytes <= ((size_t)8 << 30) && K->koff.alloc_on(kbytes, st) == cudaSuccess) {
+        HDF_COUNT_LAUNCH();
+        launch_off_store(d, st, K->xp32.as<float>(), n, K->ldk, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
+                         K->koff.as<float>());
+        KRR_CUDA(cudaGetLastError());
+        K->split = off_split(n, K->ldk, &K->S);
+    } else {
+        cudaGetLastError();
+        K->split = direct_split(n, n, &K->S);
+    }
     KRR_CUDA(K->part.alloc(sizeof(double) * (size_t)K->S * n));
     KRR_CUDA(K->hd.alloc(sizeof(double) * n));
-    KRR_CUDA(K->dotp.alloc(sizeof(double) * 512));
+    KRR_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
+    KRR_CUDA(K->cgst.alloc(sizeof(CgState)));
+    KRR_CUDA(cudaMallocHost(reinterpret_cast<void**>(&K->cgh), 2 * sizeof(CgState)));
+    for (cudaEvent_t& e : K->cgev) KRR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if (prec == HDF_FP32) {
         KRR_CUDA(K->vb.alloc(sizeof(float) * n));
         KRR_CUDA(K->yb.alloc(sizeof(float) * n));
@@ -884,35 +1107,48 @@ hdf_status hdf_krr_solve(hdf_krr* K, const double* y_dev, double rtol, int max_i
     HDF_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * n, st));
     HDF_COUNT_LAUNCH();
     k_gather_vec<<<gb, 256, 0, st>>>(y_dev, K->perm.as<int64_t>(), n, r);
-    if (hdf_status s = precond_perm(K, r, z, st); s != HDF_OK) return s;
+    CgState* S = K->cgst.as<CgState>();
+    double* dot = K->dotp.as<double>();
+    const int mgemv = (int)((n + 7) / 8);
+    if (hdf_status s = precond_perm(K, r, z, st, dot); s != HDF_OK) return s;
     HDF_CUDA(cudaMemcpyAsync(p, z, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-    double rz = 0.0, bb = 0.0;
-    if (hdf_status s = dot2(K, r, z, r, r, &rz, &bb, st); s != HDF_OK) return s;
-    const double nb = std::sqrt(bb);
-    int it = 0;
-    double res = (nb > 0.0) ? 1.0 : 0.0;
-    if (nb > 0.0) {
-        for (it = 1; it <= max_iter; ++it) {
-            if (hdf_status s = apply_perm(K, p, q, st); s != HDF_OK) return s;
-            double pq = 0.0;
-            if (hdf_status s = dot2(K, p, q, nullptr, nullptr, &pq, nullptr, st); s != HDF_OK) return s;
-            if (!(pq > 0.0)) return fail(HDF_ESINGULAR, "hdf_krr_solve: the operator is not positive definite");
-            const double alpha = rz / pq;
-            HDF_COUNT_LAUNCH();
-            k_cg_step<<<gb, 256, 0, st>>>(x, r, p, q, alpha, n);
-            HDF_CUDA(cudaGetLastError());
-            if (hdf_status s = precond_perm(K, r, z, st); s != HDF_OK) return s;
-            double rz_new = 0.0, rr = 0.0;
-            if (hdf_status s = dot2(K, r, z, r, r, &rz_new, &rr, st); s != HDF_OK) return s;
-            res = std::sqrt(rr) / nb;
-            if (res <= rtol) break;
-            HDF_COUNT_LAUNCH();
-            k_cg_dir<<<gb, 256, 0, st>>>(p, z, rz_new / rz, n);
-            HDF_CUDA(cudaGetLastError());
-            rz = rz_new;
+    HDF_COUNT_LAUNCH();
+    k_cg_init<<<1, 256, 0, st>>>(dot, mgemv, rtol, S);
+    HDF_CUDA(cudaGetLastError());
+    // the host looks at the state of kPoll iterations ago while the next kPoll are enqueued
+    constexpr int kPoll = 4;
+    int polls = 0;
+    bool done = false;
+    auto poll = [&]() -> hdf_status {
+        HDF_CUDA(cudaMemcpyAsync(&K->cgh[polls & 1], S, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+        HDF_CUDA(cudaEventRecord(K->cgev[polls & 1], st));
+        if (polls > 0) {
+            HDF_CUDA(cudaEventSynchronize(K->cgev[(polls - 1) & 1]));
+            done = K->cgh[(polls - 1) & 1].done != 0;
         }
-        if (it > max_iter) it = max_iter;
+        ++polls;
+        return HDF_OK;
+    };
+    for (int it = 1; it <= max_iter && !done; ++it) {
+        if (it % kPoll == 1)
+            if (hdf_status s = poll(); s != HDF_OK) return s;
+        if (done) break;
+        if (hdf_status s = apply_parts(K, p, st); s != HDF_OK) return s;
+        HDF_COUNT_LAUNCH();
+        k_cg_finish<<<gb, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, p, K->hd.as<double>(), q, dot, S);
+        HDF_COUNT_LAUNCH();
+        k_cg_step<<<gb, 256, 0, st>>>(x, r, p, q, n, dot, gb, it, S);
+        HDF_CUDA(cudaGetLastError());
+        if (hdf_status s = precond_perm(K, r, z, st, dot, S); s != HDF_OK) return s;
+        HDF_COUNT_LAUNCH();
+        k_cg_dir<<<gb, 256, 0, st>>>(p, z, n, dot, mgemv, it, S);
+        HDF_CUDA(cudaGetLastError());
     }
+    HDF_CUDA(cudaMemcpyAsync(&K->cgh[0], S, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+    HDF_CUDA(cudaStreamSynchronize(st));
+    if (K->cgh[0].bad) return fail(HDF_ESINGULAR, "hdf_krr_solve: the operator is not positive definite");
+    const int it = K->cgh[0].it;
+    const double res = K->cgh[0].res;
     HDF_COUNT_LAUNCH();
     k_scatter_vec<<<gb, 256, 0, st>>>(x, K->perm.as<int64_t>(), n, w_dev);
     HDF_CUDA(cudaGetLastError());
@@ -941,6 +1177,7 @@ hdf_status hdf_krr_info(const hdf_krr* K, int* nclusters, int64_t* rank_total, d
 void hdf_krr_free(hdf_krr* K) {
     if (!K) return;
     cudaDeviceSynchronize();
+    K->koff.st = nullptr;            // nothing reads it any more: back to the pool on the legacy stream
     delete K;
 }
 
