@@ -891,10 +891,13 @@ extern "C" hdf_status hdf_matvec_transpose(const hdf_factor* f, const void* V_de
 // --------------------------------------------------------------------------- solve
 
 namespace hdf {
-// The device LU of the Woodbury core (lu.cu).
-hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, cudaStream_t st);
-hdf_status lu_solve_device(int64_t r, const double* LU, const int* dperm, const double* zi, double* z, int nc,
-                           cudaStream_t st);
+// The Woodbury core: without pivoting (ldl.cu), with (lu.cu), and the substitutions of both.
+hdf_status ldl_factor_device(int64_t r, const double* G, const std::vector<double>& Spad, const double* dS, double lambda,
+                             double* C, DevBuf& dperm, DevBuf& dinv, int* err, cudaStream_t st);
+hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, int* err, cudaStream_t st);
+hdf_status lu_dinv_device(int64_t r, const double* LU, DevBuf& dinv, cudaStream_t st);
+hdf_status tri_solve_device(int64_t r, const double* M, const DevBuf& dinv, const int* dperm, bool symmetric,
+                            const double* zi, double* z, int nc, int* err, cudaStream_t st);
 hdf_status core_init_device(const double* G, const double* Spad, double lambda, int64_t r, double* C, cudaStream_t st);
 }  // namespace hdf
 
@@ -908,7 +911,7 @@ __global__ void k_cast_from_double(const double* __restrict__ z, T* __restrict__
 }  // namespace
 
 // Xout = (lambda I + U S U^T)^{-1} Bin = (Bin - U C^{-1} U^T Bin) / lambda, C = lambda S^{-1} + U^T U,
-// with C's LU factors on the device (f->core): per group of <= 64 columns, U^T Bin (FP64 sums),
+// with C's factors on the device (f->core_lu): per group of <= 64 columns, U^T Bin (FP64 sums),
 // the two triangular solves on the device, then U times the result.
 template <typename T>
 static hdf_status woodbury_apply(hdf_factor* f, double lambda, const T* Bin, int64_t ldb, int ncols, T* Xout,
@@ -935,8 +938,8 @@ static hdf_status woodbury_apply(hdf_factor* f, double lambda, const T* Bin, int
         if (hdf_status e = group_reduce<T>(g, np, r, cg, (const T*)nullptr, (T*)nullptr, Wd.as<double>(), st);
             e != HDF_OK)
             return e;
-        if (hdf_status e = lu_solve_device(r, f->core_lu.as<double>(), f->core_perm.as<int>(), Wd.as<double>(),
-                                           Zd.as<double>(), cg, st);
+        if (hdf_status e = tri_solve_device(r, f->core_lu.as<double>(), f->core_dinv, f->core_perm.as<int>(),
+                                            f->core_sym, Wd.as<double>(), Zd.as<double>(), cg, f->dev_err.as<int>(), st);
             e != HDF_OK)
             return e;
         HDF_COUNT_LAUNCH();
@@ -1001,11 +1004,19 @@ static hdf_status solve_t(hdf_factor* f, double lambda, const T* B, int64_t ldb,
         }
         if (!f->core_lu.p) HDF_CUDA(f->core_lu.alloc(sizeof(double) * (size_t)r * r));
         f->core_lambda = -1.0;
-        if (hdf_status e = core_init_device(f->core_G.as<double>(), f->core_S.as<double>(), lambda, r,
-                                            f->core_lu.as<double>(), st);
-            e != HDF_OK)
-            return e;
-        if (hdf_status e = lu_factor_device(r, f->core_lu.as<double>(), f->core_perm, st); e != HDF_OK) return e;
+        hdf_status e = ldl_factor_device(r, f->core_G.as<double>(), f->plan.Spad, f->core_S.as<double>(), lambda,
+                                         f->core_lu.as<double>(), f->core_perm, f->core_dinv, f->dev_err.as<int>(), st);
+        f->core_sym = e == HDF_OK;
+        // factors from a kernel that gave up a wait are not kept
+        if (e == HDF_OK || e == HDF_ESINGULAR)
+            if (hdf_status de = take_device_error(f); de != HDF_OK) return de;
+        if (e == HDF_ESINGULAR) {        // lambda I + K~ is not positive definite: pivoted LU
+            e = core_init_device(f->core_G.as<double>(), f->core_S.as<double>(), lambda, r, f->core_lu.as<double>(), st);
+            if (e == HDF_OK) e = lu_factor_device(r, f->core_lu.as<double>(), f->core_perm, f->dev_err.as<int>(), st);
+            if (e == HDF_OK) e = lu_dinv_device(r, f->core_lu.as<double>(), f->core_dinv, st);
+            if (e == HDF_OK) e = take_device_error(f);
+        }
+        if (e != HDF_OK) return e;
         f->core_lambda = lambda;
         f->info.lu_ms = now_ms() - t0;
     }

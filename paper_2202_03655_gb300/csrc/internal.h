@@ -86,6 +86,11 @@ hdf_status tc_f64_uw(const double* U, int64_t ldU, int64_t n, int64_t r, const d
                      const double* B, int64_t ldb, double beta, double* Y, int64_t ldy, double* part, void* work,
                      int* err, cudaStream_t st);
 
+// Trailing updates of the core factorizations by the same slices (tc_gemm.cu).
+size_t tc_f64_update_bytes(int64_t c);
+hdf_status tc_f64_update(const double* P, int64_t ldp, int64_t m, int w, const double* sg, const double* Q, int64_t ldq,
+                         int64_t c, double* C, int64_t ldc, void* work, int* err, cudaStream_t st);
+
 // FP64 products of one to four columns (few_cols.cu).  few_utv writes nchunk partial slices of
 // c x r (few_utv_split); r even, U and W 16-byte aligned with even leading dimension.
 constexpr int kFewCols = 4;
@@ -220,10 +225,11 @@ struct hdf_factor {
     size_t esz = 8;                 // bytes per bulk element
     DevBuf U, S;                    // U n x ldu, S rank (bulk type)
     std::vector<double> S_host;
-    // solve core: U^T U (FP64, r x r, kept after the first solve), the LU factors of
-    // lambda S^-1 + U^T U for core_lambda (row-major, in place) and their row permutation, S on
-    // the padded columns (FP64), all on the device
-    DevBuf core_G, core_lu, core_perm, core_S;
+    // solve core: U^T U (FP64, r x r, kept after the first solve), the factors of
+    // lambda S^-1 + U^T U for core_lambda (row-major, in place), their order and the inverses of
+    // their diagonal tiles, S on the padded columns (FP64), all on the device
+    DevBuf core_G, core_lu, core_perm, core_S, core_dinv;
+    bool core_sym = false;          // core_lu holds L J L^T without pivoting (ldl.cu), else the pivoted LU
     double core_lambda = -1.0;
     // tensor-core matvec (FP32 factors): enabled unless HDF_FLAG_CUDA_CORES; dev_err is set by
     // a kernel whose bounded wait expired

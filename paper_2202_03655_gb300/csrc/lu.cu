@@ -1,15 +1,16 @@
 // The core of the Woodbury solve (Sec. 1, Sherman-Morrison-Woodbury, with the system of
 // Eq. opt): C = lambda S^-1 + U^T U (r x r, FP64, row-major) is factored P C = L U by a blocked
 // right-looking LU with partial pivoting.  S holds eigenvalues of both signs (the truncated
-// expansion is not positive definite), so C is indefinite and needs pivoting.
+// expansion is not positive definite), so C is indefinite and in general needs pivoting.
 //
 // Work split.  Each panel of NB columns is factored with partial pivoting on the host (its
 // rows split over the host threads, three barriers per column); the row interchanges of the
 // panel are applied to the rest of the matrix on the device; U12 = L11^-1 A12 is one small GEMM
 // with the host-inverted unit lower L11; the trailing update A22 -= L21 U12 -- nearly all of
-// the 2/3 r^3 flops -- is an FP64 register-tiled GEMM on the device.  The factors stay on the
-// device, and the solves L y = P z, U x = y run there as blocked substitutions (diagonal blocks
-// in one CTA, the off-diagonal updates by the same GEMM).
+// the 2/3 r^3 flops -- runs on the tensor cores by the exact integer slices of tc_f64.cuh (0.83 to
+// 0.49 s at r = 10,000, with the attempt of ldl.cu before it).  The factors stay on the device for
+// the substitutions of ldl.cu.  ldl.cu's factorization without pivoting comes first;
+// this one serves the systems that it finds indefinite.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,7 +24,7 @@
 namespace hdf {
 namespace lu {
 
-constexpr int NB = 64;        // panel width (and block size of the substitutions)
+constexpr int NB = 64;        // panel width
 
 // C = G + diag(lambda / S_a), with 1 on the diagonal of padding columns (S_a = 0: zero columns of U).
 __global__ void k_core(const double* __restrict__ G, const double* __restrict__ Spad, double lambda, int64_t r,
@@ -98,46 +99,6 @@ __global__ void __launch_bounds__(256) k_dgemm(int64_t m, int64_t n, int64_t k, 
             C[i * ldc + j] = beta * old + alpha * acc[u][v];
         }
     }
-}
-
-// z (rows of a w x nc block, row stride ldz) <- T^-1 z for the diagonal block T of the factors
-// (rows and columns b0..b0+w of the r x r LU): lower with unit diagonal (lower = true) or upper.
-// One CTA, thread j = column j of z.
-__global__ void k_trsv_block(const double* __restrict__ LU, int64_t r, int64_t b0, int w, bool lower, double* z,
-                             int64_t ldz, int nc) {
-    __shared__ double T[NB][NB + 1];
-    __shared__ double Z[NB][65];
-    for (int e = threadIdx.x; e < w * w; e += blockDim.x) T[e / w][e % w] = LU[(b0 + e / w) * r + b0 + e % w];
-    for (int e = threadIdx.x; e < w * nc; e += blockDim.x) Z[e / nc][e % nc] = z[(e / nc) * ldz + e % nc];
-    __syncthreads();
-    const int j = threadIdx.x;
-    if (j < nc) {
-        if (lower) {
-            for (int i = 0; i < w; ++i) {
-                double s = Z[i][j];
-                for (int l = 0; l < i; ++l) s -= T[i][l] * Z[l][j];
-                Z[i][j] = s;
-            }
-        } else {
-            for (int i = w - 1; i >= 0; --i) {
-                double s = Z[i][j];
-                for (int l = i + 1; l < w; ++l) s -= T[i][l] * Z[l][j];
-                Z[i][j] = s / T[i][i];
-            }
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < w * nc; e += blockDim.x) z[(e / nc) * ldz + e % nc] = Z[e / nc][e % nc];
-}
-
-// zo[a] = zi[perm[a]] (r x nc row-major): the row interchanges of the factorization, folded
-// into one permutation on the host.
-__global__ void k_gather_rows(const double* __restrict__ zi, double* __restrict__ zo, int64_t r, int nc,
-                              const int* __restrict__ perm) {
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= r * nc) return;
-    const int64_t a = idx / nc;
-    zo[idx] = zi[(int64_t)perm[a] * nc + idx % nc];
 }
 
 // ------------------------------------------------------------------ host panel
@@ -220,7 +181,7 @@ hdf_status core_init_device(const double* G, const double* Spad, double lambda, 
 
 // P C = L U in place on the device (row-major r x r); dperm receives the row permutation
 // (row a of P C is row perm[a] of C).  HDF_ESINGULAR if a pivot is zero.  Synchronises.
-hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, cudaStream_t st) {
+hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, int* err, cudaStream_t st) {
     using namespace lu;
     std::vector<int> piv_host(r, 0);
     DevBuf dpiv;
@@ -228,6 +189,8 @@ hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, cudaStream_t st
     std::vector<double> panel, linv;
     DevBuf dlinv;
     HDF_CUDA(dlinv.alloc(sizeof(double) * NB * NB));
+    DevBuf work;
+    HDF_CUDA(work.alloc_on(tc_f64_update_bytes(r), st));
     for (int64_t kb = 0; kb < r; kb += NB) {
         const int64_t ke = std::min<int64_t>(r, kb + NB);
         const int w = (int)(ke - kb);
@@ -262,11 +225,12 @@ hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, cudaStream_t st
         HDF_COUNT_LAUNCH();
         k_dgemm<<<dim3((unsigned)((nt + GT - 1) / GT), 1), 256, 0, st>>>(w, nt, w, 1.0, dlinv.as<double>(), w,
                                                                        C + kb * r + ke, r, 0.0, C + kb * r + ke, r);
-        // A22 -= L21 U12
-        HDF_COUNT_LAUNCH();
-        k_dgemm<<<dim3((unsigned)((nt + GT - 1) / GT), (unsigned)((nt + GT - 1) / GT)), 256, 0, st>>>(
-            nt, nt, w, -1.0, C + ke * r + kb, r, C + kb * r + ke, r, 1.0, C + ke * r + ke, r);
         HDF_CUDA(cudaGetLastError());
+        // A22 -= L21 U12
+        if (hdf_status e = tc_f64_update(C + ke * r + kb, r, nt, w, nullptr, C + kb * r + ke, r, nt, C + ke * r + ke, r,
+                                         work.p, err, st);
+            e != HDF_OK)
+            return e;
         HDF_CUDA(cudaStreamSynchronize(st));     // panel and linv are reused
     }
     HDF_CUDA(cudaStreamSynchronize(st));
@@ -275,40 +239,6 @@ hdf_status lu_factor_device(int64_t r, double* C, DevBuf& dperm, cudaStream_t st
     for (int64_t a = 0; a < r; ++a) std::swap(perm[a], perm[piv_host[a]]);
     HDF_CUDA(dperm.alloc(sizeof(int) * std::max<int64_t>(1, r)));
     HDF_CUDA(cudaMemcpy(dperm.p, perm.data(), sizeof(int) * r, cudaMemcpyHostToDevice));
-    return HDF_OK;
-}
-
-// z (r x nc row-major, device, nc <= 64) = C^-1 zi with the factors of lu_factor_device; zi is
-// left unchanged.
-hdf_status lu_solve_device(int64_t r, const double* LU, const int* dperm, const double* zi, double* z, int nc,
-                           cudaStream_t st) {
-    using namespace lu;
-    HDF_COUNT_LAUNCH();
-    k_gather_rows<<<(unsigned)((r * nc + 255) / 256), 256, 0, st>>>(zi, z, r, nc, dperm);
-    for (int64_t b0 = 0; b0 < r; b0 += NB) {                 // L y = P z
-        const int w = (int)std::min<int64_t>(NB, r - b0);
-        HDF_COUNT_LAUNCH();
-        k_trsv_block<<<1, 64, 0, st>>>(LU, r, b0, w, true, z + b0 * nc, nc, nc);
-        const int64_t rest = r - b0 - w;
-        if (rest > 0) {
-            HDF_COUNT_LAUNCH();
-            k_dgemm<<<dim3((unsigned)((nc + GT - 1) / GT), (unsigned)((rest + GT - 1) / GT)), 256, 0, st>>>(
-                rest, nc, w, -1.0, LU + (b0 + w) * r + b0, r, z + b0 * nc, nc, 1.0, z + (b0 + w) * nc, nc);
-        }
-    }
-    const int64_t nblk = (r + NB - 1) / NB;
-    for (int64_t b = nblk - 1; b >= 0; --b) {                // U x = y
-        const int64_t b0 = b * NB;
-        const int w = (int)std::min<int64_t>(NB, r - b0);
-        HDF_COUNT_LAUNCH();
-        k_trsv_block<<<1, 64, 0, st>>>(LU, r, b0, w, false, z + b0 * nc, nc, nc);
-        if (b0 > 0) {
-            HDF_COUNT_LAUNCH();
-            k_dgemm<<<dim3((unsigned)((nc + GT - 1) / GT), (unsigned)((b0 + GT - 1) / GT)), 256, 0, st>>>(
-                b0, nc, w, -1.0, LU + b0, r, z + b0 * nc, nc, 1.0, z, nc);
-        }
-    }
-    HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
 

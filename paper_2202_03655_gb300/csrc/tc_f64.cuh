@@ -102,24 +102,33 @@ struct Args {
     int nitems, nkb;         // work items; 64-value blocks along K of the whole contraction
     int kper;                // blocks per item (the last item of a row of items may have fewer)
     int mblocks;             // U^T V: 128-column blocks; U W: 128-row tiles
-    int c;                   // columns of this call (<= CP)
-    const int* eb;           // exponents of the small operand: [block][CP]
+    int c;                   // columns of this call (<= ncg CP)
+    const int* eb;           // exponents of the small operand: [block][ncg CP]
     double alpha, beta;
     const double* B; int64_t ldb;
     double* Y; int64_t ldy;  // U W: the result (null: write slices to part)
     double* part;            // slices: U^T V [(split ctot + j0 + j) r + a], U W [(split c + j) n + i]
     int ctot, j0;            // U^T V: columns of the whole group, first column of this call
+    int ncg;                 // groups of CP columns of the small operand (items run over them too)
+    double* C; int64_t ldc;  // U W of a trailing update: C[i ldc + col] -= the product
+    int tri;                 // only for the tiles that meet the lower triangle (col <= i)
     int* err;
 };
 
-// Blocks of item `it`: [k0, k1) of the contraction, M block mb, split index.
-struct Item { int k0, k1, mb, split; };
+// Blocks of item `it`: [k0, k1) of the contraction (none for a tile above the diagonal of a
+// trailing update), M block mb, column group cg with c columns, split index.
+struct Item { int k0, k1, mb, cg, c, split; };
+template <int CP>
 __device__ __forceinline__ Item item_of(const Args& p, int it) {
     Item w;
     w.mb = it % p.mblocks;
-    w.split = it / p.mblocks;
+    const int rest = it / p.mblocks;
+    w.cg = rest % p.ncg;
+    w.split = rest / p.ncg;
+    w.c = min(CP, p.c - w.cg * CP);
     w.k0 = w.split * p.kper;
     w.k1 = min(p.nkb, w.k0 + p.kper);
+    if (p.tri && w.mb * BM + BM <= w.cg * CP) w.k1 = w.k0;
     return w;
 }
 
@@ -204,14 +213,14 @@ __device__ __forceinline__ uint32_t block_exponent(uint32_t hmax) {
 }
 
 // Slices of the small operand: value(k, col) for K index k and column col < c, zero beyond kn and
-// c.  One warp per (64-deep block, column of CP): lane l takes k = 2 l and 2 l + 1.
-// out[((col / 16 * 7 + slice) 16 + col mod 16) kpad + k], eb[block CP + col].
-template <int CP, typename F>
-__device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int64_t kpad, __half* out, int* eb) {
+// c, for cp columns (whole groups).  One warp per (64-deep block, column): lane l takes k = 2 l and
+// 2 l + 1.  out[((col / 16 * 7 + slice) 16 + col mod 16) kpad + k], eb[block cp + col].
+template <typename F>
+__device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int cp, int64_t kpad, __half* out, int* eb) {
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t blk = wid / CP;
-    const int col = (int)(wid % CP);
+    const int64_t blk = wid / cp;
+    const int col = (int)(wid % cp);
     if (blk >= kpad / KB) return;
     const int64_t k = blk * KB + 2 * lane;
     const double x0 = (col < c && k < kn) ? value(k, col) : 0.0;
@@ -220,7 +229,7 @@ __device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int64_t k
     uint32_t hm = max(h0 & 0x7fffffffu, h1 & 0x7fffffffu);
     hm = __reduce_max_sync(0xffffffffu, hm);
     const uint32_t ex = block_exponent(hm);
-    if (lane == 0) eb[blk * CP + col] = (int)ex;
+    if (lane == 0) eb[blk * cp + col] = (int)ex;
     const uint64_t a = biased_int(h0, (uint32_t)__double2loint(x0), ex);
     const uint64_t b = biased_int(h1, (uint32_t)__double2loint(x1), ex);
     uint32_t* o = reinterpret_cast<uint32_t*>(out + (int64_t)(col / GC * NS * GC + col % GC) * kpad + k);
@@ -234,16 +243,20 @@ __device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int64_t k
     o[5 * sl] = z ? 0u : digit_pair<5>(a, b);
     o[6 * sl] = z ? 0u : digit_pair<6>(a, b);
 }
-template <int CP>
-__global__ void __launch_bounds__(256) k_f64_prep_v(const double* __restrict__ V, int64_t ldv, int64_t n, int c,
+__global__ void __launch_bounds__(256) k_f64_prep_v(const double* __restrict__ V, int64_t ldv, int64_t n, int c, int cp,
                                                     int64_t kpad, __half* __restrict__ out, int* __restrict__ eb) {
-    prep_block<CP>([&](int64_t k, int col) { return V[k + (int64_t)col * ldv]; }, n, c, kpad, out, eb);
+    prep_block([&](int64_t k, int col) { return V[k + (int64_t)col * ldv]; }, n, c, cp, kpad, out, eb);
 }
-// W is r x ldw row-major, columns j0 .. j0 + c.
-template <int CP>
-__global__ void __launch_bounds__(256) k_f64_prep_w(const double* __restrict__ W, int64_t r, int ldw, int c,
+// W is r x ldw row-major.
+__global__ void __launch_bounds__(256) k_f64_prep_w(const double* __restrict__ W, int64_t r, int64_t ldw, int c, int cp,
                                                     int64_t kpad, __half* __restrict__ out, int* __restrict__ eb) {
-    prep_block<CP>([&](int64_t k, int col) { return W[k * ldw + col]; }, r, c, kpad, out, eb);
+    prep_block([&](int64_t k, int col) { return W[k * ldw + col]; }, r, c, cp, kpad, out, eb);
+}
+// Column col is row col of the panel P (ldp), its entries times the signs sg.
+__global__ void __launch_bounds__(256) k_f64_prep_panel(const double* __restrict__ P, int64_t ldp, int kn, int c, int cp,
+                                                        const double* __restrict__ sg, __half* __restrict__ out,
+                                                        int* __restrict__ eb) {
+    prep_block([&](int64_t k, int col) { return sg[k] * P[(int64_t)col * ldp + k]; }, kn, c, cp, KB, out, eb);
 }
 
 // The rare results of level_sums: a 64-bit integer below 2^32 in magnitude, an exponent outside
@@ -343,7 +356,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {                                 // raw U tiles
             uint32_t g = 0;
             for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
-                const Item w = item_of(p, it);
+                const Item w = item_of<CP>(p, it);
                 for (int kb = w.k0; kb < w.k1; ++kb, ++g) {
                     const uint32_t s = g % S_UD;
                     if (!mbar_wait(&sm.uempty[s], ((g / S_UD) & 1) ^ 1)) { ok = false; break; }
@@ -365,12 +378,12 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) {                                 // stacked slices of the small operand
             uint32_t g = 0;
             for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
-                const Item w = item_of(p, it);
+                const Item w = item_of<CP>(p, it);
                 for (int kb = w.k0; kb < w.k1; ++kb, ++g) {
                     const uint32_t s = g % SB_;
                     if (!mbar_wait(&sm.bempty[s], ((g / SB_) & 1) ^ 1)) { ok = false; break; }
                     mbar_expect_tx(&sm.bfull[s], bbytes<CP>());
-                    tma_load_2d(sm.B + s * bbytes<CP>(), &mB, kb * KB, 0, &sm.bfull[s]);
+                    tma_load_2d(sm.B + s * bbytes<CP>(), &mB, kb * KB, w.cg * (NS * CP), &sm.bfull[s]);
                 }
             }
             if (!producer_drain(sm.bfull, SB_, g)) ok = false;
@@ -379,7 +392,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     } else if (warp == 1) {                              // MMA issue (converged warp)
         uint32_t g = 0, u = 0;                           // blocks, (block, group) pairs
         for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
-            const Item w = item_of(p, it);
+            const Item w = item_of<CP>(p, it);
             for (int kb = w.k0; kb < w.k1 && ok; ++kb, ++g) {
                 const uint32_t s = g % SB_;
 #pragma unroll
@@ -434,7 +447,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + kAcolD + 128 * h;
         uint32_t g = 0;
         for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
-            const Item w = item_of(p, it);
+            const Item w = item_of<CP>(p, it);
             for (int kb = w.k0; kb < w.k1; ++kb, ++g) {
                 const uint32_t s = g % S_UD;
                 if (!warp_wait(&sm.ufull[s], (g / S_UD) & 1)) { ok = false; break; }
@@ -508,12 +521,12 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16) + colg;
         uint32_t g = 0;
         for (int it = blockIdx.x; it < p.nitems && ok; it += gridDim.x) {
-            const Item w = item_of(p, it);
+            const Item w = item_of<CP>(p, it);
             double acc[PC];
 #pragma unroll
             for (int j = 0; j < PC; ++j) acc[j] = 0.0;
             for (int kb = w.k0; kb < w.k1; ++kb, ++g) {
-                const int eb = special_exponent(lane < PC ? p.eb[(int64_t)kb * CP + col0 + lane] : 0);
+                const int eb = special_exponent(lane < PC ? p.eb[((int64_t)kb * p.ncg + w.cg) * CP + col0 + lane] : 0);
                 if (!warp_wait(&sm.efull[g % EX], (g / EX) & 1)) { ok = false; break; }
                 const int ea = special_exponent((int)sm.expo[(g % EX) * BM + m]);
                 const uint32_t u = NG == 1 ? g : NG * g + set, b = u % NACC_;
@@ -530,13 +543,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                     tmem_ld_wait();
                     level_sums(L, eab, acc + c0);
                 };
-                if (col0 + PC <= p.c) {                  // straight-line: the four-column chains overlap
+                if (col0 + PC <= w.c) {                  // straight-line: the four-column chains overlap
 #pragma unroll
                     for (int c0 = 0; c0 < PC; c0 += 4) four(c0);
                 } else {                                 // without the padding columns
 #pragma unroll
                     for (int c0 = 0; c0 < PC; c0 += 4)
-                        if (col0 + c0 < p.c) four(c0);
+                        if (col0 + c0 < w.c) four(c0);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -548,17 +561,19 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (a < p.r) {
 #pragma unroll
                     for (int j = 0; j < PC; ++j)
-                        if (col0 + j < p.c)
+                        if (col0 + j < w.c)
                             p.part[((int64_t)w.split * p.ctot + p.j0 + col0 + j) * p.r + a] = acc[j];
                 }
             } else {
                 const int64_t i = (int64_t)w.mb * BM + m;
-                if (i < p.n) {
+                if (i < p.n && w.k0 < w.k1) {
 #pragma unroll
                     for (int j = 0; j < PC; ++j) {
                         const int64_t col = col0 + j;
-                        if (col < p.c) {
-                            if (p.part) {
+                        if (col < w.c) {
+                            if (p.C) {
+                                p.C[i * p.ldc + w.cg * CP + col] -= acc[j];
+                            } else if (p.part) {
                                 p.part[((int64_t)w.split * p.c + col) * p.n + i] = acc[j];
                             } else {
                                 double out = p.alpha * acc[j];
