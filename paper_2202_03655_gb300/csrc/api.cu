@@ -16,6 +16,7 @@
 #include "hdf_kernels.cuh"
 #include "internal.h"
 #include "planner.h"
+#include "rows_lane.h"
 
 using namespace hdf;
 
@@ -1153,7 +1154,11 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     HDF_CUDA(dA.alloc(sizeof(T) * cA.size() + 16));
     HDF_CUDA(dB.alloc(sizeof(T) * cB.size() + 16));
     const int64_t ldF = ((int64_t)nF + 31) / 32 * 32;       // 128-byte rows (FP32): whole-sector stores
-    if (dF.alloc_on(sizeof(T) * (size_t)n * ldF, st) != cudaSuccess) {
+    const int mtp = ((m0 + m1 + 7) / 8) * 8;
+    // FP32 factors with few columns: rows straight from the points, without the F buffer
+    RowsLanePlan lanes;
+    const bool by_lane = sizeof(T) == 4 && !mfree && rows_lane_plan(d, L, fc, tb, lanes);
+    if (!by_lane && dF.alloc_on(sizeof(T) * (size_t)n * ldF, st) != cudaSuccess) {
         cudaGetLastError();
         return fail(HDF_ENOMEM, "hdf_build: cannot allocate the radial factor buffer");
     }
@@ -1161,7 +1166,6 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     if (!Qmat[1].empty()) HDF_CUDA(cudaMemcpyAsync(dQ1.p, Qmat[1].data(), sizeof(double) * Qmat[1].size(), cudaMemcpyHostToDevice, st));
     // FP32 factors: [Qmat0 | Qmat1] as (hi, lo) float pairs for the compensated radial basis,
     // (L+1) x mtp with the odd columns zero in row L and mtp a multiple of 8
-    const int mtp = ((m0 + m1 + 7) / 8) * 8;
     if (sizeof(T) == 4) {
         std::vector<float> qc((size_t)2 * (L + 1) * mtp, 0.f);
         auto put = [&](int l, int o, double v) {
@@ -1194,7 +1198,7 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     struct EvGuard { cudaEvent_t* e; ~EvGuard() { for (int q = 0; q < 3; ++q) cudaEventDestroy(e[q]); } } evg{ev};
     HDF_CUDA(cudaEventRecord(ev[0], st));
     // A5a: radial factors F
-    {
+    if (!by_lane) {
         dev::RFParams R{};
         R.x = x; R.n = n; R.d = d; R.c = cen; R.inv2R = inv2R; R.L = L;
         R.Qm0 = dQ0.as<double>(); R.nb0 = nb0; R.m0 = m0;
@@ -1229,7 +1233,12 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         HDF_CUDA(cudaGetLastError());
     }
     HDF_CUDA(cudaEventRecord(ev[1], st));
-    if (mfree) {
+    if (by_lane) {
+        if (hdf_status e = rows_lane(lanes, x, n, d, cen, inv2R, L, tb, dA.as<float>(), dB.as<float>(),
+                                     f->U.as<float>(), st);
+            e != HDF_OK)
+            return e;
+    } else if (mfree) {
         // A5b, matrix-free: the Z and P_0 F rows instead of U
         if (hdf_status e = mf_write<T>(f, x, n, d, cen, inv2R, fc, tb, dF.p, ldF, dA.p, dB.p, st); e != HDF_OK)
             return e;
