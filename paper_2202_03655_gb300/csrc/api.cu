@@ -1150,7 +1150,10 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     HDF_CUDA(dchains.alloc(sizeof(int16_t) * std::max<size_t>(1, tb.chains.size())));
     HDF_CUDA(PL.dqdesc.alloc(sizeof(uint32_t) * tb.qdesc.size()));
     HDF_CUDA(PL.dychain.alloc(sizeof(int32_t) * tb.ychain.size()));
-    HDF_CUDA(PL.dgslot.alloc(sizeof(int32_t) * tb.gslot.size()));
+    // harmonic slots: gbase (d = 3) or ydesc
+    const void* gy = d == 3 ? (const void*)tb.gbase.data() : (const void*)tb.ydesc.data();
+    const size_t gy_bytes = sizeof(int32_t) * (d == 3 ? tb.gbase.size() : tb.ydesc.size());
+    HDF_CUDA(PL.dslots.alloc(std::max<size_t>(16, gy_bytes)));
     HDF_CUDA(dA.alloc(sizeof(T) * cA.size() + 16));
     HDF_CUDA(dB.alloc(sizeof(T) * cB.size() + 16));
     const int64_t ldF = ((int64_t)nF + 31) / 32 * 32;       // 128-byte rows (FP32): whole-sector stores
@@ -1187,7 +1190,7 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         HDF_CUDA(cudaMemcpyAsync(dchains.p, tb.chains.data(), sizeof(int16_t) * tb.chains.size(), cudaMemcpyHostToDevice, st));
     HDF_CUDA(cudaMemcpyAsync(PL.dqdesc.p, tb.qdesc.data(), sizeof(uint32_t) * tb.qdesc.size(), cudaMemcpyHostToDevice, st));
     HDF_CUDA(cudaMemcpyAsync(PL.dychain.p, tb.ychain.data(), sizeof(int32_t) * tb.ychain.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(PL.dgslot.p, tb.gslot.data(), sizeof(int32_t) * tb.gslot.size(), cudaMemcpyHostToDevice, st));
+    if (gy_bytes) HDF_CUDA(cudaMemcpyAsync(PL.dslots.p, gy, gy_bytes, cudaMemcpyHostToDevice, st));
     if (!cA.empty()) {
         HDF_CUDA(cudaMemcpyAsync(dA.p, cA.data(), sizeof(T) * cA.size(), cudaMemcpyHostToDevice, st));
         HDF_CUDA(cudaMemcpyAsync(dB.p, cB.data(), sizeof(T) * cB.size(), cudaMemcpyHostToDevice, st));
@@ -1250,7 +1253,8 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         P.x = x; P.n = n; P.d = d; P.c = cen; P.inv2R = inv2R;
         P.L = L_used; P.tri = ht.tri;
         P.chains = dchains.as<int16_t>(); P.nH = (int)nH; P.cstride = chain_stride(d);
-        P.ychain = PL.dychain.as<int32_t>(); P.nYp = tb.nYp; P.gslot = PL.dgslot.as<int32_t>();
+        P.ychain = PL.dychain.as<int32_t>(); P.nYp = tb.nYp;
+        P.gbase = PL.dslots.as<int32_t>(); P.ydesc = PL.dslots.as<uint32_t>(); P.yw = tb.yw;
         P.qdesc = PL.dqdesc.as<uint32_t>(); P.nF = nF;
         P.F = dF.p; P.ldF = ldF;
         P.U = f->U.p; P.ldU = I.ldu;
@@ -1268,7 +1272,8 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         for (int attempt = 0; attempt < 4 && pick.warps == 0; ++attempt) {
             const bool pre = (attempt % 2) == 0, staged = attempt < 2;
             const size_t pw = sizeof(T) * (size_t)dev::uwriter_per_warp(levels, ht.tri, L_used, tb.nYp, nF, pre);
-            const size_t tabs = staged ? dev::uwriter_tab_bytes(nq, (int)nH, chain_stride(d), tb.nYp, pre) : 0;
+            const size_t tabs = staged ? dev::uwriter_tab_bytes(nq, (int)nH, chain_stride(d), tb.nYp, levels, L_used, tb.yw, pre)
+                                       : 0;
             if (coef + tabs >= budget) continue;
             const int w = (int)std::min<size_t>(32, (budget - coef - tabs) / pw);
             if (w >= (attempt < 3 ? 8 : 1)) pick = Cfg{pre, staged, w, pw, tabs};

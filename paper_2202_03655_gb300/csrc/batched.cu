@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(1024) k_batch_urows(const BuildSet* __restrict
         __syncthreads();
         dev::uwriter_zero_slots<T>(S.uw, S.pre != 0, base, lane);
         const int64_t i0 = (int64_t)w.y * pts_per_item, i1 = min(i0 + pts_per_item, S.uw.n);
-        const dev::UWTabs X{S.uw.qdesc, S.uw.chains, S.uw.gslot, S.uw.ychain};
+        const dev::UWTabs X{S.uw.qdesc, S.uw.chains, S.uw.ychain, S.uw.gbase, S.uw.ydesc};
         for (int64_t i = i0 + warp; i < i1; i += nwarps) dev::uwriter_point<T>(S.uw, X, S.pre != 0, i, cA, cB, base, lane);
         __syncthreads();
     }
@@ -1237,7 +1237,8 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         offs[s].ch = put(tb.chains.data(), sizeof(int16_t) * tb.chains.size());
         offs[s].qd = put(tb.qdesc.data(), sizeof(uint32_t) * tb.qdesc.size());
         offs[s].yc = put(tb.ychain.data(), sizeof(int32_t) * tb.ychain.size());
-        offs[s].gs = put(tb.gslot.data(), sizeof(int32_t) * tb.gslot.size());
+        offs[s].gs = d == 3 ? put(tb.gbase.data(), sizeof(int32_t) * tb.gbase.size())
+                            : put(tb.ydesc.data(), sizeof(uint32_t) * tb.ydesc.size());
         offs[s].ca = put(cA.data(), sizeof(T) * cA.size());
         offs[s].cb = put(cB.data(), sizeof(T) * cB.size());
         for (int64_t a = 0; a < tb.ldU; ++a) Sd[b->soff[s] + a] = (T)tb.Spad[a];
@@ -1297,7 +1298,8 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         P.L = tb.L_used; P.tri = tb.tri;
         P.chains = reinterpret_cast<const int16_t*>(A + offs[s].ch); P.nH = tb.nH; P.cstride = chain_stride(d);
         P.ychain = reinterpret_cast<const int32_t*>(A + offs[s].yc); P.nYp = tb.nYp;
-        P.gslot = reinterpret_cast<const int32_t*>(A + offs[s].gs);
+        P.gbase = reinterpret_cast<const int32_t*>(A + offs[s].gs);
+        P.ydesc = reinterpret_cast<const uint32_t*>(A + offs[s].gs); P.yw = tb.yw;
         P.qdesc = reinterpret_cast<const uint32_t*>(A + offs[s].qd); P.nF = tb.nF;
         P.F = R.F; P.ldF = R.ldF;
         P.U = b->U.as<T>() + b->uoff[s]; P.ldU = tb.ldU;

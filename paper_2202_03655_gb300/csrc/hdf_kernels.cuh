@@ -643,8 +643,9 @@ struct UWParams {
     const int16_t* chains;     // nH x cstride: level offsets, trig index, zero padding
     int nH, cstride;
     const int32_t* ychain;     // nYp padded harmonic slots -> chain (-1: padding)
-    const int32_t* gslot;      // nH: padded slot of each harmonic
     int nYp;
+    const int32_t* gbase;      // d = 3: slot of (k, m = 0)
+    const uint32_t* ydesc; int yw;   // d >= 4: per slot, factors of the harmonic (see make_tables)
     const uint32_t* qdesc;     // ldU / VW chunks, two words each (see make_tables)
     int nF;
     const void* F; int64_t ldF;
@@ -657,40 +658,40 @@ struct UWParams {
 // The index tables the U writer reads for every point (global, or staged in shared memory).
 struct UWTabs {
     const uint32_t* qdesc;     // two words per chunk (see make_tables)
-    const int16_t* chains;
-    const int32_t* gslot;
+    const int16_t* chains;     // harmonics formed per chunk only
     const int32_t* ychain;
+    const int32_t* gbase;      // harmonics precomputed
+    const uint32_t* ydesc;
 };
 
-// Bytes of the staged index tables: qdesc, chains, gslot, and ychain when harmonics are not
-// precomputed; the kernel lays them out in this order, each 16-byte aligned.
-__host__ __device__ inline size_t uwriter_tab_bytes(int64_t nq, int nH, int cstride, int nYp, bool pre) {
-    return align16(sizeof(uint32_t) * 2 * nq) + align16(sizeof(int16_t) * (size_t)nH * cstride) +
-           align16(sizeof(int32_t) * (size_t)nH) + (pre ? 0 : align16(sizeof(int32_t) * (size_t)nYp));
+// Bytes of the staged index tables: qdesc, then gbase (d = 3) or ydesc when harmonics are
+// precomputed, chains and ychain when they are not; the kernel lays them out in this order, each
+// 16-byte aligned.
+__host__ __device__ inline size_t uwriter_tab_bytes(int64_t nq, int nH, int cstride, int nYp, int levels, int L, int yw,
+                                                    bool pre) {
+    const size_t q = align16(sizeof(uint32_t) * 2 * nq);
+    if (pre) return q + (levels == 1 ? align16(sizeof(int32_t) * (size_t)(L + 1)) : align16(sizeof(uint32_t) * (size_t)yw * nYp));
+    return q + align16(sizeof(int16_t) * (size_t)nH * cstride) + align16(sizeof(int32_t) * (size_t)nYp);
 }
+
+// Elements of a warp's G table (d >= 4: (L + 1)^2 and a zero; d = 3 writes the slots directly).
+__host__ __device__ inline int uwriter_g_size(int levels, int L) { return levels == 1 ? 0 : (L + 1) * (L + 1) + 1; }
 
 // Shared elements (type T) per warp of the U writer (a multiple of 16 bytes).
 __host__ __device__ inline int uwriter_per_warp(int levels, int tri, int L, int nYp, int nF, bool pre) {
-    return ((levels * tri + 2 * L + 1 + (pre ? nYp : 0) + nF + 1) + 3) & ~3;
+    return ((pre ? nYp + (levels - 1) * tri + uwriter_g_size(levels, L) : levels * tri + 2 * L + 1) + nF + 1 + 3) & ~3;
 }
 
-// Direction x_hat of point i (differences in FP64, normalisation in the bulk precision T; the
-// zero vector gets e_0), then the level tables of the normalised three-term recurrences
-// (levels x tri, lanes over mu') and the trigonometric powers (x0 + i x1)^mu times the
-// normalisers (2L+1, index L + mu), written by one warp into its shared tbl and trig.
+// Direction x_hat of point i: differences in FP64, normalisation in the bulk precision T; the
+// zero vector gets e_0.  xh is indexed with compile-time indices only (loops over kMaxD with the
+// dimension as a predicate), so that it stays in registers.
 template <typename T>
-__device__ __forceinline__ void point_harmonic_tables(const double* __restrict__ x, int d, const Center& cen,
-                                                      double inv2R, int L, int tri, const T* cA, const T* cB,
-                                                      T* tbl, T* trig, int64_t i, int lane, bool have_x = false,
-                                                      double x_lane = 0.0) {
-    const int levels = d - 2;
-    // FP32 factors: lane j forms coordinate j once and the warp shares it by shuffles (FP64
-    // issues at a small fraction of the FP32 rate here).
-    // xh is indexed with compile-time indices only (loops over kMaxD with the dimension as a
-    // predicate), so that it stays in registers
-    T xh[kMaxD];
+__device__ __forceinline__ void point_direction(const double* __restrict__ x, int d, const Center& cen, double inv2R,
+                                                int64_t i, int lane, bool have_x, double x_lane, T* xh) {
     T s = (T)0;
     if constexpr (sizeof(T) == 4) {
+        // FP32 factors: lane j forms coordinate j once and the warp shares it by shuffles (FP64
+        // issues at a small fraction of the FP32 rate here).
         double cj = cen.c[0];                    // this lane's centre coordinate (register selects)
 #pragma unroll
         for (int j = 1; j < kMaxD; ++j) cj = (lane == j) ? cen.c[j] : cj;
@@ -718,45 +719,69 @@ __device__ __forceinline__ void point_harmonic_tables(const double* __restrict__
 #pragma unroll
         for (int j = 0; j < kMaxD; ++j) xh[j] = (j == 0) ? (T)1 : (T)0;
     }
-    // level tables: lanes over mu'
-    for (int j = 0; j < levels; ++j) {
-        const int D = d - 1 - j;
-        T q = (T)0, z = (T)0;
+}
+
+// Level table j (j < levels) of the normalised three-term recurrences, lanes over mu'.
+template <typename T>
+__device__ __forceinline__ void level_table(const T* xh, int d, int j, int L, int tri, const T* cA, const T* cB, T* tb,
+                                            int lane) {
+    const int D = d - 1 - j;
+    T q = (T)0, z = (T)0;
 #pragma unroll
-        for (int m = 0; m < kMaxD; ++m) {
-            if (m <= D) q += xh[m] * xh[m];
-            if (m == D) z = xh[m];
-        }
-        const T qq = q;
-        const T* A = cA + j * tri;
-        const T* B = cB + j * tri;
-        T* tb = tbl + j * tri;
-        for (int mu = lane; mu <= L; mu += 32) {
-            const int o = mu * (L + 1) - mu * (mu - 1) / 2;
-            const int nmax = L - mu;
-            T pm2 = A[o];
-            tb[o] = pm2;
-            if (nmax >= 1) {
-                T pm1 = A[o + 1] * z;
-                tb[o + 1] = pm1;
-                for (int nn = 2; nn <= nmax; ++nn) {
-                    const T pn = A[o + nn] * z * pm1 - B[o + nn] * qq * pm2;
-                    tb[o + nn] = pn;
-                    pm2 = pm1;
-                    pm1 = pn;
-                }
+    for (int m = 0; m < kMaxD; ++m) {
+        if (m <= D) q += xh[m] * xh[m];
+        if (m == D) z = xh[m];
+    }
+    const T qq = q;
+    const T* A = cA + j * tri;
+    const T* B = cB + j * tri;
+    for (int mu = lane; mu <= L; mu += 32) {
+        const int o = mu * (L + 1) - mu * (mu - 1) / 2;
+        const int nmax = L - mu;
+        T pm2 = A[o];
+        tb[o] = pm2;
+        if (nmax >= 1) {
+            T pm1 = A[o + 1] * z;
+            tb[o + 1] = pm1;
+            for (int nn = 2; nn <= nmax; ++nn) {
+                const T pn = A[o + nn] * z * pm1 - B[o + nn] * qq * pm2;
+                tb[o + nn] = pn;
+                pm2 = pm1;
+                pm1 = pn;
             }
         }
     }
-    // trig powers (x0 + i x1)^mu by binary powering in the bulk precision, lanes over mu
+}
+
+// (x0 + i x1)^mu by binary powering in the bulk precision.
+template <typename T>
+__device__ __forceinline__ void trig_power(T x0, T x1, int mu, T& re, T& im) {
+    T br = x0, bi = x1, rr = (T)1, ri = (T)0;
+    int e = mu;
+    while (e) {
+        if (e & 1) { const T t = rr * br - ri * bi; ri = rr * bi + ri * br; rr = t; }
+        const T t = br * br - bi * bi; bi = (T)2 * br * bi; br = t;
+        e >>= 1;
+    }
+    re = rr;
+    im = ri;
+}
+
+// The direction of point i, then the level tables (levels x tri, lanes over mu') and the
+// trigonometric powers (x0 + i x1)^mu times the normalisers (2L+1, index L + mu), written by one
+// warp into its shared tbl and trig.
+template <typename T>
+__device__ __forceinline__ void point_harmonic_tables(const double* __restrict__ x, int d, const Center& cen,
+                                                      double inv2R, int L, int tri, const T* cA, const T* cB,
+                                                      T* tbl, T* trig, int64_t i, int lane, bool have_x = false,
+                                                      double x_lane = 0.0) {
+    const int levels = d - 2;
+    T xh[kMaxD];
+    point_direction<T>(x, d, cen, inv2R, i, lane, have_x, x_lane, xh);
+    for (int j = 0; j < levels; ++j) level_table<T>(xh, d, j, L, tri, cA, cB, tbl + j * tri, lane);
     for (int mu = lane; mu <= L; mu += 32) {
-        T br = (T)xh[0], bi = (T)xh[1], rr = (T)1, ri = (T)0;
-        int e = mu;
-        while (e) {
-            if (e & 1) { const T t = rr * br - ri * bi; ri = rr * bi + ri * br; rr = t; }
-            const T t = br * br - bi * bi; bi = (T)2 * br * bi; br = t;
-            e >>= 1;
-        }
+        T rr, ri;
+        trig_power<T>(xh[0], xh[1], mu, rr, ri);
         if (mu == 0) {
             trig[L] = (T)0.3989422804014327;             // 1/sqrt(2 pi)
         } else {
@@ -766,17 +791,81 @@ __device__ __forceinline__ void point_harmonic_tables(const double* __restrict__
     }
 }
 
+// All harmonics of point i into the warp's slots Ys.  Lane m runs the last level's recurrence and
+// multiplies each value by the trigonometric factors +-m at once: in d = 3 these are the harmonics
+// and go to their slots, for d >= 4 they form G, and slot y is G[g] times its prefix (the tables Pl of the
+// levels before the last).  With a table of every level, one of the trigonometric factors and a
+// pass over the chains (two or more index words and as many factors per harmonic), the harmonics
+// took more than half of the instructions of a row at some hundred columns.
+template <typename T>
+__device__ __forceinline__ void point_harmonics(const double* __restrict__ x, int d, const Center& cen, double inv2R,
+                                                int L, int tri, const T* cA, const T* cB, const int32_t* gbase,
+                                                const uint32_t* ydesc, int nYp, T* Ys, T* Pl, T* G, int64_t i, int lane,
+                                                bool have_x, double x_lane) {
+    const int levels = d - 2;
+    T xh[kMaxD];
+    point_direction<T>(x, d, cen, inv2R, i, lane, have_x, x_lane, xh);
+    for (int j = 0; j < levels - 1; ++j) level_table<T>(xh, d, j, L, tri, cA, cB, Pl + j * tri, lane);
+    const T z = xh[2], qq = xh[0] * xh[0] + xh[1] * xh[1] + xh[2] * xh[2];
+    const T* A = cA + (levels - 1) * tri;
+    const T* B = cB + (levels - 1) * tri;
+    for (int m = lane; m <= L; m += 32) {
+        T rr, ri;
+        trig_power<T>(xh[0], xh[1], m, rr, ri);
+        rr *= m == 0 ? (T)0.3989422804014327 : (T)0.5641895835477563;    // 1/sqrt(2 pi), 1/sqrt(pi)
+        ri *= (T)0.5641895835477563;
+        const T* a = A + m * (L + 1) - m * (m - 1) / 2 - m;              // indexed by mu = m + n
+        const T* b = B + (a - A);
+        T p1 = (T)0, p2 = (T)0;
+        for (int mu = m; mu <= L; ++mu) {
+            const T v = mu == m ? a[mu] : mu == m + 1 ? a[mu] * z : a[mu] * z * p1 - b[mu] * qq * p2;
+            p2 = p1;
+            p1 = v;
+            if (levels == 1) {
+                const int g = gbase[mu];
+                if (g >= 0) {
+                    Ys[g + m] = v * rr;
+                    if (m > 0) Ys[g - m] = v * ri;
+                }
+            } else {
+                T* g = G + mu * (mu + 1);
+                g[m] = v * rr;
+                if (m > 0) g[-m] = v * ri;
+            }
+        }
+    }
+    if (levels == 1) return;
+    __syncwarp();
+    if (levels <= 4) {
+        for (int y = lane; y < nYp; y += 32) {
+            const uint2 w = *reinterpret_cast<const uint2*>(ydesc + 2 * y);
+            T v = G[w.x & 0xffffu] * Pl[w.x >> 16];
+            if (levels >= 3) v *= Pl[w.y & 0xffffu];
+            if (levels >= 4) v *= Pl[w.y >> 16];
+            Ys[y] = v;
+        }
+    } else {
+        for (int y = lane; y < nYp; y += 32) {
+            const uint4 w = *reinterpret_cast<const uint4*>(ydesc + 4 * y);
+            T v = G[w.x & 0xffffu] * Pl[w.x >> 16] * Pl[w.y & 0xffffu] * Pl[w.y >> 16] * Pl[w.z & 0xffffu];
+            if (levels >= 6) v *= Pl[w.z >> 16];
+            Ys[y] = v;
+        }
+    }
+}
+
 // One point's U row, executed by one warp.  cA/cB: level recurrences in shared memory;
-// base: this warp's shared area (P.per_warp elements, 16-byte aligned), laid out as
-// [harmonic slots (pre only)] [level tables] [trig powers] [radial factors].  pre: the
-// harmonics of the point are computed once into the slots; otherwise each chunk's harmonics
-// are multiplied out from the level tables as it is written.  A VW-wide chunk of the row meets
+// base: this warp's shared area (P.per_warp elements, 16-byte aligned), laid out as [harmonic
+// slots] [level tables but the last] [G] [radial factors] (pre) or [level tables] [trig powers]
+// [radial factors].  pre: the harmonics of the point are computed once into the slots; otherwise
+// each chunk's harmonics are multiplied out from the level tables as it is written.  A VW-wide chunk of the row meets
 // one or two (k, s) blocks; its two descriptor words give each block's radial factor and first
 // harmonic slot.
 // The radial-factor slots of a warp's shared area (nF + 1, the last one zero).
 template <typename T>
 __device__ __forceinline__ T* uwriter_fs(const UWParams& P, bool pre, T* base) {
-    return base + (pre ? P.nYp : 0) + (P.d - 2) * P.tri + 2 * P.L + 1;
+    const int levels = P.d - 2;
+    return base + (pre ? P.nYp + (levels - 1) * P.tri + uwriter_g_size(levels, P.L) : levels * P.tri + 2 * P.L + 1);
 }
 
 // Radial factors and coordinate of one point loaded into registers one point ahead of use (FP32
@@ -809,29 +898,25 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
                                               double x_lane = 0.0) {
     const int levels = P.d - 2;
     T* Ys = base;                                // nYp (pre only)
-    T* tbl = base + (pre ? P.nYp : 0);           // levels * tri
-    T* trig = tbl + levels * P.tri;              // 2L+1, index L + mu
-    T* Fs = trig + 2 * P.L + 1;                  // nF + 1
+    T* Pl = base + P.nYp;                        // (levels - 1) * tri (pre only)
+    T* G = Pl + (levels - 1) * P.tri;            // G (pre only)
+    T* tbl = base;                               // levels * tri, then 2L+1 trig, index L + mu (not pre)
+    T* trig = tbl + levels * P.tri;
+    T* Fs = uwriter_fs<T>(P, pre, base);         // nF + 1
     const T* Fg = reinterpret_cast<const T*>(P.F);
     T* Ug = reinterpret_cast<T*>(P.U);
     typedef typename Vec2<T>::type VT;
     constexpr int VW = Vec2<T>::w;
-    point_harmonic_tables<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane, staged, x_lane);
+    // padding slots are zeroed once per warp (d = 3) or written as zeros
+    if (pre)
+        point_harmonics<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, X.gbase, X.ydesc, P.nYp, Ys, Pl, G, i, lane,
+                           staged, x_lane);
+    else
+        point_harmonic_tables<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane, staged, x_lane);
     // this point's radial factors (staged: already in Fs, written by the caller)
     if (!staged) {
         for (int f = lane; f < P.nF; f += 32) Fs[f] = Fg[i * P.ldF + f];
         if (lane == 0) Fs[P.nF] = (T)0;
-    }
-    __syncwarp();
-    if (pre) {
-        // padding slots were zeroed once per warp and are never written
-        for (int g = lane; g < P.nH; g += 32) {
-            const int16_t* c = X.chains + (int64_t)g * P.cstride;
-            const int slot = X.gslot[g];
-            T v = trig[P.L + c[levels]];
-            for (int j = 0; j < levels; ++j) v *= tbl[j * P.tri + c[j]];
-            Ys[slot] = v;
-        }
     }
     __syncwarp();
     // row write: one VW-wide chunk per lane per step, four (FP64: two) steps in flight.  A chunk
@@ -896,11 +981,14 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
     __syncwarp();
 }
 
-// Zeroes a warp's harmonic slots once (the padding slots are never written afterwards).
+// Zeroes a warp's harmonic slots and G's last entry once (padding slots of d = 3 and that entry are
+// never written afterwards).
 template <typename T>
 __device__ __forceinline__ void uwriter_zero_slots(const UWParams& P, bool pre, T* base, int lane) {
-    if (pre)
+    if (pre) {
         for (int g = lane; g < P.nYp; g += 32) base[g] = (T)0;
+        if (P.d > 3 && lane == 0) base[P.nYp + (P.d - 3) * P.tri + uwriter_g_size(P.d - 2, P.L) - 1] = (T)0;
+    }
     __syncwarp();
 }
 
@@ -918,7 +1006,7 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
         cA[idx] = reinterpret_cast<const T*>(P.coefA)[idx];
         cB[idx] = reinterpret_cast<const T*>(P.coefB)[idx];
     }
-    UWTabs X{P.qdesc, P.chains, P.gslot, P.ychain};
+    UWTabs X{P.qdesc, P.chains, P.ychain, P.gbase, P.ydesc};
     if constexpr (STAGED) {
         // staged in shared memory (STAGED is a compile-time choice, so that the table reads
         // compile to shared-memory loads)
@@ -929,14 +1017,19 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
         for (int64_t k = threadIdx.x; k < 2 * nq; k += blockDim.x) q[k] = P.qdesc[k];
         X.qdesc = q;
         tp += align16(sizeof(uint32_t) * 2 * nq);
-        int16_t* ch = reinterpret_cast<int16_t*>(tp);
-        for (int64_t k = threadIdx.x; k < (int64_t)P.nH * P.cstride; k += blockDim.x) ch[k] = P.chains[k];
-        tp += align16(sizeof(int16_t) * (size_t)P.nH * P.cstride);
-        int32_t* gs = reinterpret_cast<int32_t*>(tp);
-        for (int k = threadIdx.x; k < P.nH; k += blockDim.x) gs[k] = P.gslot[k];
-        tp += align16(sizeof(int32_t) * (size_t)P.nH);
-        X.chains = ch; X.gslot = gs;
-        if (!PRE) {
+        if (PRE && levels == 1) {
+            int32_t* gb = reinterpret_cast<int32_t*>(tp);
+            for (int k = threadIdx.x; k <= P.L; k += blockDim.x) gb[k] = P.gbase[k];
+            X.gbase = gb;
+        } else if (PRE) {
+            uint32_t* yd = reinterpret_cast<uint32_t*>(tp);
+            for (int k = threadIdx.x; k < P.yw * P.nYp; k += blockDim.x) yd[k] = P.ydesc[k];
+            X.ydesc = yd;
+        } else {
+            int16_t* ch = reinterpret_cast<int16_t*>(tp);
+            for (int64_t k = threadIdx.x; k < (int64_t)P.nH * P.cstride; k += blockDim.x) ch[k] = P.chains[k];
+            tp += align16(sizeof(int16_t) * (size_t)P.nH * P.cstride);
+            X.chains = ch;
             int32_t* yc = reinterpret_cast<int32_t*>(tp);
             for (int k = threadIdx.x; k < P.nYp; k += blockDim.x) yc[k] = P.ychain[k];
             X.ychain = yc;

@@ -181,9 +181,9 @@ struct FactorPlan {
     std::vector<int> sk, fbase, cbase, hbase;  // per k: kept count, F column, U column, harmonic bases
     // device copies: Qmat0, Qmat1 (FP64), Wt (m_max x nF, bulk), colk (F column -> k),
     // chains (nH x (d-1) int16), hk (harmonic -> k), ktab (per k: fbase, s_k, cbase, |H_k|, hbase,
-    // padded |H_k|), qdesc (chunk descriptors), ychain (padded harmonic slots -> chain),
+    // padded |H_k|), qdesc (chunk descriptors), ychain (padded harmonic slots -> chain), slots (gbase or ydesc of make_tables),
     // coefA/coefB (level recurrences, bulk)
-    DevBuf dQ0, dQ1, dQC, dW, dcolk, dchains, dhk, dktab, dqdesc, dychain, dgslot, dA, dB;
+    DevBuf dQ0, dQ1, dQC, dW, dcolk, dchains, dhk, dktab, dqdesc, dychain, dslots, dA, dB;
     std::vector<int64_t> colmap;               // padded column of each true column of U
     std::vector<double> Spad;                  // S on the padded columns (0 on padding)
     // d S_k / d l (s_k x s_k), computed on first use by the adjoint

@@ -860,6 +860,16 @@ bool make_tables(const FactorChoice& fc, int d, int L, int vw, DeviceTables& t, 
     t.cbase.assign(L + 2, 0);
     t.ychain.assign(std::max(1, t.nYp), -1);
     t.gslot.assign(std::max(1, t.nH), 0);
+    const int levels = d - 2, stride = chain_stride(d), Lu = t.L_used;
+    if (levels == 1) {
+        t.gbase.assign(Lu + 1, -1);
+        for (int k = 0; k <= Lu; ++k)
+            if (sk[k] > 0) t.gbase[k] = yoff[k] + k;
+    } else {
+        t.yw = d <= 6 ? 2 : 4;
+        t.ydesc.assign((size_t)std::max(1, t.nYp) * t.yw, 0);
+        for (int y = 0; y < t.nYp; ++y) t.ydesc[(size_t)y * t.yw] = (uint32_t)((Lu + 1) * (Lu + 1));
+    }
     // U's column blocks (k, s) follow each other without padding, except that a block of fewer
     // than vw harmonics (degree 0, and degree 1 in d = 3) is padded to vw zero-extended columns, so
     // that every vw-wide chunk of a row meets at most two blocks
@@ -869,6 +879,13 @@ bool make_tables(const FactorChoice& fc, int d, int L, int vw, DeviceTables& t, 
             t.hk[g] = (uint8_t)k;
             t.ychain[yoff[k] + (g - t.hbase[k])] = g;
             t.gslot[g] = yoff[k] + (g - t.hbase[k]);
+            if (levels == 1) continue;
+            const int16_t* c = &t.chains[(size_t)g * stride];
+            const int m = c[levels], am = std::abs(m), mu = c[levels - 1] - (am * (Lu + 1) - am * (am - 1) / 2) + am;
+            uint32_t f[8] = {(uint32_t)(mu * mu + mu + m), 0, 0, 0, 0, 0, 0, 0};
+            for (int j = 0; j < levels - 1; ++j) f[1 + j] = (uint32_t)(j * t.tri + c[j]);
+            for (int w = 0; w < t.yw; ++w)
+                t.ydesc[(size_t)t.gslot[g] * t.yw + w] = f[2 * w] | (f[2 * w + 1] << 16);
         }
         const int hkc = (sk[k] > 0) ? (int)ht.count[k] : 0;
         ucols[k] = (hkc > 0 && hkc < vw) ? vw : hkc;

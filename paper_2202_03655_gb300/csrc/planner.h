@@ -133,6 +133,13 @@ struct DeviceTables {
     std::vector<int16_t> chains;             // nH x (d-1)
     std::vector<int32_t> ychain;             // nYp: chain of each padded Y slot, -1 for padding
     std::vector<int32_t> gslot;              // nH: padded Y slot of each harmonic
+    // Harmonic slots from G[mu, m] = (last level) x (trigonometric factor m), mu = mu_{d-3} (the degree in
+    // d = 3).  d = 3: gbase[k] + m is the slot of (k, m), -1 for a degree without columns.  d >= 4: slot
+    // y = G[g] prod_j P_j[p_j], 16-bit fields (p_j counted from the first level table) in yw words:
+    // g | p_0 << 16, p_1 | p_2 << 16 (, p_3 | p_4 << 16, 0); G's entry (L_used + 1)^2 is zero (padding).
+    std::vector<int32_t> gbase;
+    std::vector<uint32_t> ydesc;
+    int yw = 0;
     std::vector<uint32_t> qdesc;             // 2 ldU / vw: per chunk (F << 20 | split << 18 | slot, F << 20 | slot)
     std::vector<int64_t> colmap;             // rank: padded column of each true column
     std::vector<double> Spad;                // ldU: S on the padded columns (0 on padding)
