@@ -298,13 +298,14 @@ struct MomentJob {
 hdf_status radial_moments(const double* x, int64_t n, int d, const dev::Center& cen, double inv2R, int L, int prec,
                           MomentJob& job, cudaStream_t st) {
     const int nmom = 2 * L + 2;
-    const int gmom = grid_for(n, 8192, 2 * 152);
+    const size_t msm_df = sizeof(float2) * 256 * (size_t)(nmom + 1);
+    const bool df = prec == HDF_FP32 && msm_df <= 200 * 1024;
+    const int gmom = dev::moment_blocks(n, df ? dev::kMomTileDf : dev::kMomTile);
     const int64_t mchunk = (n + gmom - 1) / gmom;
     HDF_CUDA(job.mpart.alloc_on(sizeof(double) * (size_t)gmom * nmom, st));
     HDF_CUDA(job.msum.alloc_on(sizeof(double) * nmom, st));
     HDF_COUNT_LAUNCH();
-    const size_t msm_df = sizeof(float2) * 256 * (size_t)(nmom + 1);
-    if (prec == HDF_FP32 && msm_df <= 200 * 1024) {
+    if (df) {
         HDF_CUDA(cudaFuncSetAttribute(dev::k_radial_moments_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)msm_df));
         dev::k_radial_moments_df<<<gmom, 256, msm_df, st>>>(x, n, d, mchunk, cen, inv2R, nmom, job.mpart.as<double>());
@@ -314,8 +315,7 @@ hdf_status radial_moments(const double* x, int64_t n, int d, const dev::Center& 
     }
     HDF_CUDA(cudaGetLastError());
     HDF_COUNT_LAUNCH();
-    dev::k_reduce_cols<<<grid_for(nmom, 256, 1 << 20), 256, 0, st>>>(job.mpart.as<double>(), gmom, nmom,
-                                                                    job.msum.as<double>());
+    dev::k_reduce_cols<<<nmom, 256, 0, st>>>(job.mpart.as<double>(), gmom, nmom, job.msum.as<double>());
     HDF_CUDA(cudaGetLastError());
     job.mom.assign(nmom, 0.0);
     return HDF_OK;
