@@ -1210,13 +1210,20 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         R.F = dF.p; R.ldF = ldF;
         const int grid = grid_for((n + dev::kFTile - 1) / dev::kFTile, 1, 152 * 8);
         const size_t sm64 = dev::radialF_smem(L, m0, m1, sizeof(T));
-        size_t sm32 = dev::radialF_df_smem(L, m0, m1, mtp, nF, true);
-        R.stage_wt = 1;
-        if (sm32 > 200 * 1024) { sm32 = dev::radialF_df_smem(L, m0, m1, mtp, nF, false); R.stage_wt = 0; }
+        // as many tiles between barriers as shared memory takes (at most eight, but no fewer CTAs than
+        // SMs for it), Wt staged if one tile then fits
+        size_t sm32 = dev::radialF_df_smem(L, m0, m1, mtp, nF, true, 1);
+        R.stage_wt = sm32 <= 200 * 1024 ? 1 : 0;
+        R.tiles = 1;
+        for (int t = 8; t >= 1; t /= 2) {
+            sm32 = dev::radialF_df_smem(L, m0, m1, mtp, nF, R.stage_wt != 0, t);
+            R.tiles = t;
+            if (sm32 <= 200 * 1024 && (n + t * dev::kFTile - 1) / (t * dev::kFTile) >= 2 * 152) break;
+        }
         if (sizeof(T) == 4 && sm32 <= 200 * 1024) {
             R.QC = PL.dQC.as<float2>();
             R.mtp = mtp;
-            const int kopt = dev::radialF_df_kopt(m0 + m1, dev::kRfThreads / 32 - 1);
+            const int kopt = dev::radialF_df_kopt(m0 + m1, R.tiles, dev::kRfThreads / 32);
             auto rk = kopt == 2 ? dev::k_radial_F_df<2> : kopt == 4 ? dev::k_radial_F_df<4> : dev::k_radial_F_df<8>;
             HDF_CUDA(cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm32));
             int occ = 0, nsm = 0, dv = 0;
@@ -1224,7 +1231,8 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
             HDF_CUDA(cudaGetDevice(&dv));
             HDF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dv));
             const int g32 = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)nsm * std::max(occ, 1),
-                                                                          (n + dev::kFTile - 1) / dev::kFTile));
+                                                                          (n + R.tiles * dev::kFTile - 1) /
+                                                                              (R.tiles * dev::kFTile)));
             HDF_COUNT_LAUNCH();
             rk<<<g32, dev::kRfThreads, sm32, st>>>(R);
         } else {

@@ -255,9 +255,9 @@ struct BuildSet {
 };
 
 // Shared memory of the double-float radial phase of the batched build for `tiles` tiles per
-// item: one buffer of basis pairs and rho per tile, then Q.
+// item: basis pairs and rho, then Q, of each tile.
 inline size_t batch_df_tile_smem(int L, int mt, int tiles) {
-    return (size_t)tiles * dev::radialF_df_basis_bytes(L) + sizeof(float) * (size_t)mt * dev::kFTile;
+    return (size_t)tiles * (dev::radialF_df_basis_bytes(L) + sizeof(float) * (size_t)mt * dev::kFTile);
 }
 
 // A5 for every set in two persistent phases, each with its own register and shared-memory budget:
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256, 2) k_batch_radial(const BuildSet* __restr
                                                          const int2* __restrict__ items, int nitems, int* counter,
                                                          int tiles_per_item) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_item;
+    __shared__ int s_item, s_unit[2];
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
         __syncthreads();
@@ -281,12 +281,13 @@ __global__ void __launch_bounds__(256, 2) k_batch_radial(const BuildSet* __restr
         const BuildSet& S = sets[w.x];
         const int64_t t0 = (int64_t)w.y * tiles_per_item * dev::kFTile;
         if constexpr (sizeof(T) == 4) {
-            // FP32 sets always carry the double-float tables (QC).  First the basis values of all
-            // the item's tiles at once (thread = point), then per tile Q (S.rf.kopt outputs per
-            // thread) and F by all warps.
-            const int LP1 = S.rf.L + 1;
+            // FP32 sets always carry the double-float tables (QC).  The basis values of all the
+            // item's tiles (thread = point), their Q units (S.rf.kopt outputs each), their F units;
+            // the warps take units from a counter.
+            const int LP1 = S.rf.L + 1, mt = S.rf.m0 + S.rf.m1, lane = threadIdx.x & 31;
             const size_t bb = dev::radialF_df_basis_bytes(S.rf.L);
             const int ntile = (int)min((int64_t)tiles_per_item, (S.rf.n - t0 + dev::kFTile - 1) / dev::kFTile);
+            if (threadIdx.x < 2) s_unit[threadIdx.x] = 0;
             for (int pt = threadIdx.x; pt < ntile * dev::kFTile; pt += blockDim.x) {
                 const int q = pt / dev::kFTile;
                 float2* Tq = reinterpret_cast<float2*>(smem_raw + q * bb);
@@ -295,18 +296,25 @@ __global__ void __launch_bounds__(256, 2) k_batch_radial(const BuildSet* __restr
             }
             __syncthreads();
             float* Qs = reinterpret_cast<float*>(smem_raw + tiles_per_item * bb);
-            for (int q = 0; q < ntile; ++q) {
+            const int ko = S.rf.kopt, groups = (mt + ko - 1) / ko;
+            for (int u = dev::next_unit(&s_unit[0], lane); u < ntile * groups; u = dev::next_unit(&s_unit[0], lane)) {
+                const int q = u / groups, o0 = (u % groups) * ko;
                 const float2* Tq = reinterpret_cast<const float2*>(smem_raw + q * bb);
                 const float* rq = reinterpret_cast<const float*>(Tq + dev::kFTile * LP1);
-                if (S.rf.kopt == 2)
-                    dev::radialF_df_q<2>(S.rf, Tq, rq, S.rf.QC, Qs, threadIdx.x, blockDim.x);
+                float* Qq = Qs + (size_t)q * mt * dev::kFTile;
+                if (ko == 2)
+                    dev::radialF_df_q<2>(S.rf, Tq, rq, S.rf.QC, Qq, o0, lane);
                 else
-                    dev::radialF_df_q<4>(S.rf, Tq, rq, S.rf.QC, Qs, threadIdx.x, blockDim.x);
-                __syncthreads();
-                dev::radialF_df_f(S.rf, t0 + (int64_t)q * dev::kFTile, Qs, reinterpret_cast<const float*>(S.rf.Wt),
-                                  threadIdx.x, blockDim.x);
-                __syncthreads();
+                    dev::radialF_df_q<4>(S.rf, Tq, rq, S.rf.QC, Qq, o0, lane);
             }
+            __syncthreads();
+            const int fgroups = (int)((S.rf.ldF + 31) / 32);
+            for (int u = dev::next_unit(&s_unit[1], lane); u < ntile * fgroups; u = dev::next_unit(&s_unit[1], lane)) {
+                const int q = u / fgroups;
+                dev::radialF_df_f(S.rf, t0 + (int64_t)q * dev::kFTile, Qs + (size_t)q * mt * dev::kFTile,
+                                  reinterpret_cast<const float*>(S.rf.Wt), 32 * (u % fgroups), lane);
+            }
+            __syncthreads();
         } else {
             for (int q = 0; q < tiles_per_item; ++q) {
                 const int64_t tq = t0 + (int64_t)q * dev::kFTile;
@@ -1290,7 +1298,7 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         if (sizeof(T) == 4 && offs[s].mtp > 0) {
             R.QC = reinterpret_cast<const float2*>(A + offs[s].qc);
             R.mtp = offs[s].mtp;
-            R.kopt = std::min(4, dev::radialF_df_kopt(fc.m[0] + fc.m[1], 256 / 32));   // 2 or 4
+            R.kopt = std::min(4, dev::radialF_df_kopt(fc.m[0] + fc.m[1], 4, 256 / 32));   // 2 or 4
         }
         R.F = dF.as<T>() + foff[s]; R.ldF = tb.nF;
         dev::UWParams& P = bs[s].uw;

@@ -286,7 +286,8 @@ struct RFParams {
     const double* Qm0; int nb0, m0;
     const double* Qm1; int nb1, m1;
     const float2* QC; int mtp;   // FP32 factors: [Qm0 | Qm1] as (hi, lo) float pairs, (L+1) x mtp
-    int kopt;                    // FP32 factors in the batched build: outputs per thread of the Q part
+    int kopt;                    // FP32 factors in the batched build: outputs per Q unit
+    int tiles;                   // FP32 factors, single build: tiles between two barriers
     int stage_wt;                // FP32 factors: copy Wt into shared memory
     const void* Wt; const uint8_t* colpar; int nF;
     void* F; int64_t ldF;
@@ -436,75 +437,81 @@ __device__ __forceinline__ void radialF_df_basis(const RFParams& P, int64_t t0, 
     }
 }
 
-// Q part, by the nth compute threads (thread = point p and a group of kOpt outputs: each basis
-// value read from shared memory serves kOpt outputs, one 16-byte load brings two outputs).
-template <int kOpt = 8>
+// The Q and F parts as units of one warp, which the warps of a CTA take from a counter: the parts
+// of several tiles run between two barriers, so that no warp waits for the one with the most work.
+// Q unit: lane = point of the tile, kOpt outputs from o0 (each basis value read from shared memory
+// serves kOpt outputs, one 16-byte load brings two outputs).
+template <int kOpt>
 __device__ __forceinline__ void radialF_df_q(const RFParams& P, const float2* Ts, const float* rh, const float2* QC,
-                                             float* Qs, int tid, int nth) {
-    const int LP1 = P.L + 1;
-    const int mt = P.m0 + P.m1;
-    const int p = tid % kFTile;
-    const float2* Tp = Ts + p * LP1;
-    for (int o0 = (tid / kFTile) * kOpt; o0 < mt; o0 += (nth / kFTile) * kOpt) {
-        float sh[kOpt], c[kOpt];
+                                             float* Qs, int o0, int lane) {
+    const int LP1 = P.L + 1, mt = P.m0 + P.m1;
+    const float2* Tp = Ts + lane * LP1;
+    float sh[kOpt], c[kOpt];
 #pragma unroll
-        for (int j = 0; j < kOpt; ++j) { sh[j] = 0.f; c[j] = 0.f; }
-        for (int l = 0; l < LP1; ++l) {
-            const float2 a = Tp[l];
-            const float4* qr = reinterpret_cast<const float4*>(QC + (size_t)l * P.mtp + o0);
+    for (int j = 0; j < kOpt; ++j) { sh[j] = 0.f; c[j] = 0.f; }
+#pragma unroll 2
+    for (int l = 0; l < LP1; ++l) {
+        const float2 a = Tp[l];
+        const float4* qr = reinterpret_cast<const float4*>(QC + (size_t)l * P.mtp + o0);
 #pragma unroll
-            for (int j2 = 0; j2 < kOpt / 2; ++j2) {
-                const float4 b = qr[j2];
-                dot2_step(a, b.x, b.y, sh[2 * j2], c[2 * j2]);
-                dot2_step(a, b.z, b.w, sh[2 * j2 + 1], c[2 * j2 + 1]);
-            }
+        for (int j2 = 0; j2 < kOpt / 2; ++j2) {
+            const float4 b = qr[j2];
+            dot2_step(a, b.x, b.y, sh[2 * j2], c[2 * j2]);
+            dot2_step(a, b.z, b.w, sh[2 * j2 + 1], c[2 * j2 + 1]);
         }
+    }
 #pragma unroll
-        for (int j = 0; j < kOpt; ++j) {
-            const int o = o0 + j;
-            if (o < mt) {
-                float q = sh[j] + c[j];
-                if (o >= P.m0) q *= rh[p];
-                Qs[o * kFTile + p] = q;
-            }
+    for (int j = 0; j < kOpt; ++j) {
+        const int o = o0 + j;
+        if (o < mt) {
+            float q = sh[j] + c[j];
+            if (o >= P.m0) q *= rh[lane];
+            Qs[o * kFTile + lane] = q;
         }
     }
 }
 
-// F part: thread = column; Wt from shared memory (Ws, max(m0, m1) x nF) when staged.
-__device__ __forceinline__ void radialF_df_f(const RFParams& P, int64_t t0, const float* Qs, const float* Ws,
-                                             int tid, int nth) {
+// F unit: lane = column, 32 columns from col0; Wt from shared memory (Ws, max(m0, m1) x nF) when
+// staged.
+__device__ __forceinline__ void radialF_df_f(const RFParams& P, int64_t t0, const float* Qs, const float* Ws, int col0,
+                                             int lane) {
     const int cnt = (int)min((int64_t)kFTile, P.n - t0);
     float* F = reinterpret_cast<float*>(P.F);
-    for (int col = tid; col < P.ldF; col += nth) {
-        if (col >= P.nF) {                       // row padding: zeros, so that sectors are whole
-#pragma unroll
-            for (int p = 0; p < kFTile; ++p)
-                if (p < cnt) F[(t0 + p) * P.ldF + col] = 0.f;
-            continue;
-        }
-        const int par = P.colpar[col];
-        const int ob = par ? P.m0 : 0, mp = par ? P.m1 : P.m0;
-        float acc[kFTile];
-#pragma unroll
-        for (int p = 0; p < kFTile; ++p) acc[p] = 0.f;
-#pragma unroll 4
-        for (int l = 0; l < mp; ++l) {
-            const float w = Ws[(size_t)l * P.nF + col];
-            const float4* q = reinterpret_cast<const float4*>(Qs + (ob + l) * kFTile);
-#pragma unroll
-            for (int p4 = 0; p4 < kFTile / 4; ++p4) {
-                const float4 v = q[p4];
-                acc[4 * p4 + 0] += v.x * w;
-                acc[4 * p4 + 1] += v.y * w;
-                acc[4 * p4 + 2] += v.z * w;
-                acc[4 * p4 + 3] += v.w * w;
-            }
-        }
+    const int col = col0 + lane;
+    if (col >= P.ldF) return;
+    if (col >= P.nF) {                           // row padding: zeros, so that sectors are whole
 #pragma unroll
         for (int p = 0; p < kFTile; ++p)
-            if (p < cnt) F[(t0 + p) * P.ldF + col] = acc[p];
+            if (p < cnt) F[(t0 + p) * P.ldF + col] = 0.f;
+        return;
     }
+    const int par = P.colpar[col];
+    const int ob = par ? P.m0 : 0, mp = par ? P.m1 : P.m0;
+    float acc[kFTile];
+#pragma unroll
+    for (int p = 0; p < kFTile; ++p) acc[p] = 0.f;
+    for (int l = 0; l < mp; ++l) {
+        const float w = Ws[(int64_t)l * P.nF + col];
+        const float4* q4 = reinterpret_cast<const float4*>(Qs + (ob + l) * kFTile);
+#pragma unroll
+        for (int p4 = 0; p4 < kFTile / 4; ++p4) {
+            const float4 v = q4[p4];
+            acc[4 * p4 + 0] += v.x * w;
+            acc[4 * p4 + 1] += v.y * w;
+            acc[4 * p4 + 2] += v.z * w;
+            acc[4 * p4 + 3] += v.w * w;
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < kFTile; ++p)
+        if (p < cnt) F[(t0 + p) * P.ldF + col] = acc[p];
+}
+
+// The next unit of a warp from a shared counter.
+__device__ __forceinline__ int next_unit(int* counter, int lane) {
+    int u = 0;
+    if (lane == 0) u = atomicAdd(counter, 1);
+    return __shfl_sync(0xffffffffu, u, 0);
 }
 
 // Radial factors of the points [t0, t0 + kFTile): block-wide, ends with a barrier.
@@ -575,39 +582,44 @@ __global__ void __launch_bounds__(256) k_radial_F(RFParams P) {
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) radialF_tile<T>(P, tile * kFTile, smem_raw);
 }
 
-// Shared memory of k_radial_F_df: QC, Wt (when staged), two buffers of basis values, Q.
+// Shared memory of k_radial_F_df: QC, Wt (when staged), two buffers of basis values and one of Q for
+// each of `tiles` tiles.
 __host__ __device__ inline size_t radialF_df_basis_bytes(int L) {
     return align16(sizeof(float2) * kFTile * (L + 1) + sizeof(float) * kFTile);
 }
-__host__ __device__ inline size_t radialF_df_smem(int L, int m0, int m1, int mtp, int nF, bool stage_wt) {
+__host__ __device__ inline size_t radialF_df_smem(int L, int m0, int m1, int mtp, int nF, bool stage_wt, int tiles) {
     const int mmax = m0 > m1 ? m0 : m1;
     return align16(sizeof(float2) * (size_t)(L + 1) * mtp) +
-           (stage_wt ? align16(sizeof(float) * (size_t)mmax * nF) : 0) + 2 * radialF_df_basis_bytes(L) +
-           sizeof(float) * (size_t)(m0 + m1) * kFTile;
+           (stage_wt ? align16(sizeof(float) * (size_t)mmax * nF) : 0) +
+           tiles * (2 * radialF_df_basis_bytes(L) + sizeof(float) * (size_t)(m0 + m1) * kFTile);
 }
 
-// Outputs per thread of the Q part (2, 4 or 8) for mt outputs over qwarps warps: the fewest
-// outputs per thread after rounding (each warp takes whole groups of kOpt outputs for its 32
-// points), larger groups on ties (fewer shared loads per output).
-__host__ __device__ inline int radialF_df_kopt(int mt, int qwarps) {
+// Outputs per Q unit (2, 4 or 8) for mt outputs of `tiles` tiles over `warps` warps: the fewest
+// outputs per warp after rounding, larger groups on ties (fewer shared loads per output).
+__host__ __device__ inline int radialF_df_kopt(int mt, int tiles, int warps) {
     int best = 8, cost = 1 << 30;
     for (int k = 8; k >= 2; k /= 2) {
-        const int groups = (mt + k - 1) / k;
-        const int c = ((groups + qwarps - 1) / qwarps) * k;
+        const int units = tiles * ((mt + k - 1) / k);
+        const int c = ((units + warps - 1) / warps) * k;
         if (c < cost) { cost = c; best = k; }
     }
     return best;
 }
 
-// FP32 factors, one CTA of kRfThreads per SM.  Per tile of kFTile points: warps 1.. form Q while
-// warp 0 computes the basis values of the CTA's next tile into the other buffer, then all warps
-// form F.  QC (and Wt when P.stage_wt) are staged per CTA.
+// FP32 factors, one CTA of kRfThreads per SM, P.tiles tiles of kFTile points between two barriers:
+// the basis of the CTA's next tiles and the Q units of the current ones, then the F units, warps
+// taking units from a counter.  QC (and Wt when P.stage_wt) are staged per CTA.  Bound by the FP32
+// issue of the Dot2 products; with one tile between barriers (warp 0 forming the next basis, the
+// others a fixed share of Q) the warps waited for one another half of the time: 1,000,000 points,
+// L = 32: RADNUM.
 constexpr int kRfThreads = 512;
 template <int KOPT>
 static __global__ void __launch_bounds__(kRfThreads, 1) k_radial_F_df(RFParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int LP1 = P.L + 1;
+    __shared__ int counter[2];
+    const int LP1 = P.L + 1, mt = P.m0 + P.m1, NT = P.tiles;
     const int mmax = P.m0 > P.m1 ? P.m0 : P.m1;
+    const int lane = threadIdx.x & 31;
     unsigned char* sp = smem_raw;
     float2* QC = reinterpret_cast<float2*>(sp);
     sp += align16(sizeof(float2) * (size_t)LP1 * P.mtp);
@@ -618,30 +630,45 @@ static __global__ void __launch_bounds__(kRfThreads, 1) k_radial_F_df(RFParams P
         Ws = w;
         sp += align16(sizeof(float) * (size_t)mmax * P.nF);
     }
-    float2* Tb[2];
-    float* rb[2];
-    for (int b = 0; b < 2; ++b) {
-        Tb[b] = reinterpret_cast<float2*>(sp);
-        rb[b] = reinterpret_cast<float*>(Tb[b] + kFTile * LP1);
-        sp += radialF_df_basis_bytes(P.L);
-    }
-    float* Qs = reinterpret_cast<float*>(sp);
+    const size_t bb = radialF_df_basis_bytes(P.L);
+    unsigned char* basis = sp;                   // [2][NT]
+    float* Qs = reinterpret_cast<float*>(sp + 2 * NT * bb);
+    auto Tb = [&](int buf, int q) { return reinterpret_cast<float2*>(basis + (buf * NT + q) * bb); };
     for (int t = threadIdx.x; t < LP1 * P.mtp; t += blockDim.x) QC[t] = P.QC[t];
     const int64_t ntiles = (P.n + kFTile - 1) / kFTile;
-    if (threadIdx.x < kFTile && blockIdx.x < ntiles) radialF_df_basis(P, blockIdx.x * kFTile, threadIdx.x, Tb[0], rb[0]);
+    const int64_t nsup = (ntiles + NT - 1) / NT;
+    auto form_basis = [&](int64_t sup, int q, int buf) {
+        const int64_t t0 = (sup * NT + q) * kFTile;
+        float2* T = Tb(buf, q);
+        radialF_df_basis(P, t0, lane, T, reinterpret_cast<float*>(T + kFTile * LP1));
+    };
+    if (threadIdx.x < 2) counter[threadIdx.x] = 0;
+    if (blockIdx.x < nsup && (int)(threadIdx.x >> 5) < NT) form_basis(blockIdx.x, threadIdx.x >> 5, 0);
     __syncthreads();
+    const int groups = (mt + KOPT - 1) / KOPT, fgroups = (int)((P.ldF + 31) / 32);
     int cur = 0;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        if (threadIdx.x < 32) {
-            const int64_t nxt = tile + gridDim.x;
-            if (nxt < ntiles && threadIdx.x < kFTile) radialF_df_basis(P, nxt * kFTile, threadIdx.x, Tb[cur ^ 1], rb[cur ^ 1]);
-        } else {
-            radialF_df_q<KOPT>(P, Tb[cur], rb[cur], QC, Qs, threadIdx.x - 32, kRfThreads - 32);
+    for (int64_t sup = blockIdx.x; sup < nsup; sup += gridDim.x, cur ^= 1) {
+        const int64_t nxt = sup + gridDim.x;
+        const int nt = (int)min((int64_t)NT, ntiles - sup * NT);
+        const int nb = nxt < nsup ? (int)min((int64_t)NT, ntiles - nxt * NT) : 0;
+        for (int u = next_unit(&counter[0], lane); u < nb + nt * groups; u = next_unit(&counter[0], lane)) {
+            if (u < nb) {
+                form_basis(nxt, u, cur ^ 1);
+            } else {
+                const int q = (u - nb) / groups, g = (u - nb) % groups;
+                const float2* T = Tb(cur, q);
+                radialF_df_q<KOPT>(P, T, reinterpret_cast<const float*>(T + kFTile * LP1), QC,
+                                   Qs + (size_t)q * mt * kFTile, g * KOPT, lane);
+            }
         }
         __syncthreads();
-        radialF_df_f(P, tile * kFTile, Qs, Ws, threadIdx.x, kRfThreads);
+        if (threadIdx.x == 0) counter[0] = 0;    // every warp is past its last unit; read again after the barrier below
+        for (int u = next_unit(&counter[1], lane); u < nt * fgroups; u = next_unit(&counter[1], lane)) {
+            const int q = u / fgroups, g = u % fgroups;
+            radialF_df_f(P, (sup * NT + q) * kFTile, Qs + (size_t)q * mt * kFTile, Ws, 32 * g, lane);
+        }
         __syncthreads();
-        cur ^= 1;
+        if (threadIdx.x == 0) counter[1] = 0;    // likewise, before the next F units' barrier
     }
 }
 
