@@ -1269,36 +1269,45 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         P.coefA = dA.p; P.coefB = dB.p;
         const int levels = d - 2;
         // One CTA per SM with as many warps as shared memory holds (up to 32): the coefficient
-        // tables and, when they fit, the per-point index tables are shared by all its warps.
-        // Preference: harmonics precomputed per point (pre) with staged tables, then the
-        // on-the-fly variant with staged tables, then either with tables read from global.
+        // tables and, when they fit, the index tables are shared by all its warps.  The first form
+        // that leaves eight warps is taken: harmonics in slots; harmonics as products (d >= 4) with a
+        // descriptor per column, then per chunk; slots, then products, with the descriptors in
+        // global memory; tables of every level; the last takes what is left.
         const size_t coef = dev::align16(sizeof(T) * 2 * (size_t)levels * ht.tri);
         const size_t budget = 226 * 1024;
-        const int64_t nq = I.ldu / (int64_t)(sizeof(T) == 4 ? 4 : 2);
-        struct Cfg { bool pre, staged; int warps; size_t pw; size_t tabs; };
-        Cfg pick{false, false, 0, 0, 0};
-        for (int attempt = 0; attempt < 4 && pick.warps == 0; ++attempt) {
-            const bool pre = (attempt % 2) == 0, staged = attempt < 2;
-            const size_t pw = sizeof(T) * (size_t)dev::uwriter_per_warp(levels, ht.tri, L_used, tb.nYp, nF, pre);
-            const size_t tabs = staged ? dev::uwriter_tab_bytes(nq, (int)nH, chain_stride(d), tb.nYp, levels, L_used, tb.yw, pre)
-                                       : 0;
+        using UK = void (*)(dev::UWParams);
+        struct Cfg { int mode, desc; UK kern; };
+        const Cfg forms[] = {
+            {dev::kSlots, dev::kChunks, dev::k_uwriter<T, dev::kSlots, false, dev::kChunks>},
+            {dev::kProducts, dev::kColumns, dev::k_uwriter<T, dev::kProducts, false, dev::kColumns>},
+            {dev::kProducts, dev::kChunks, dev::k_uwriter<T, dev::kProducts, false, dev::kChunks>},
+            {dev::kSlots, dev::kGlobal, dev::k_uwriter<T, dev::kSlots, false, dev::kGlobal>},
+            {dev::kProducts, dev::kGlobal, dev::k_uwriter<T, dev::kProducts, false, dev::kGlobal>},
+            {dev::kChains, dev::kChunks, dev::k_uwriter<T, dev::kChains, false, dev::kChunks>},
+            {dev::kChains, dev::kGlobal, dev::k_uwriter<T, dev::kChains, false, dev::kGlobal>},
+        };
+        UK kern = nullptr;
+        int warps = 0;
+        size_t pw = 0, tabs = 0;
+        for (const Cfg& c : forms) {
+            if (c.mode == dev::kProducts && levels == 1) continue;
+            pw = sizeof(T) * (size_t)dev::uwriter_per_warp(levels, ht.tri, L_used, tb.nYp, nF, c.mode);
+            tabs = dev::uwriter_tab_bytes(I.ldu, vw, (int)nH, chain_stride(d), tb.nYp, levels, L_used, tb.yw, c.mode, c.desc);
             if (coef + tabs >= budget) continue;
-            const int w = (int)std::min<size_t>(32, (budget - coef - tabs) / pw);
-            if (w >= (attempt < 3 ? 8 : 1)) pick = Cfg{pre, staged, w, pw, tabs};
+            warps = (int)std::min<size_t>(32, (budget - coef - tabs) / pw);
+            if (warps < (c.kern == forms[6].kern ? 1 : 8)) { warps = 0; continue; }
+            kern = c.kern;
+            // FP32 factors, harmonics in slots, tables staged, nF <= 32 kPfF: the next point's
+            // radial factors and coordinate are prefetched into registers
+            if constexpr (sizeof(T) == 4)
+                if (c.mode == dev::kSlots && c.desc == dev::kChunks && nF <= 32 * dev::kPfF)
+                    kern = dev::k_uwriter<T, dev::kSlots, true, dev::kChunks>;
+            break;
         }
-        if (pick.warps == 0) return fail(HDF_ETOOBIG, "hdf_build: harmonic tables exceed shared memory");
-        const bool pre = pick.pre;
-        const int warps = pick.warps;
-        P.per_warp = (int)(pick.pw / sizeof(T));
-        P.tab_bytes = (int)pick.tabs;
-        const size_t sm = dev::align16((size_t)warps * pick.pw + sizeof(T) * 2 * (size_t)levels * ht.tri) + pick.tabs;
-        const bool stg = pick.staged;
-        auto kern = pre ? (stg ? dev::k_uwriter<T, true, false, true> : dev::k_uwriter<T, true, false, false>)
-                        : (stg ? dev::k_uwriter<T, false, false, true> : dev::k_uwriter<T, false, false, false>);
-        // FP32 factors, harmonics precomputed, tables staged, nF <= 32 kPfF: the next point's
-        // radial factors and coordinate are prefetched into registers
-        if constexpr (sizeof(T) == 4)
-            if (pre && stg && nF <= 32 * dev::kPfF) kern = dev::k_uwriter<T, true, true, true>;
+        if (warps == 0) return fail(HDF_ETOOBIG, "hdf_build: harmonic tables exceed shared memory");
+        P.per_warp = (int)(pw / sizeof(T));
+        P.tab_bytes = (int)tabs;
+        const size_t sm = dev::align16((size_t)warps * pw + sizeof(T) * 2 * (size_t)levels * ht.tri) + tabs;
         HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         int occ = 0;
         HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, sm));

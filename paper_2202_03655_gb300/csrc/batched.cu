@@ -33,6 +33,7 @@
 #include <sstream>
 #include <string>
 #include <sys/stat.h>
+#include <type_traits>
 #include <vector>
 
 #include "few_cols.cuh"
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(256) k_seg_gram(const double* __restrict__ x, 
 struct BuildSet {
     dev::RFParams rf;
     dev::UWParams uw;
-    int pre;
+    int mode;                        // dev::UWMode
 };
 
 // Shared memory of the double-float radial phase of the batched build for `tiles` tiles per
@@ -348,10 +349,20 @@ __global__ void __launch_bounds__(1024) k_batch_urows(const BuildSet* __restrict
             cB[idx] = reinterpret_cast<const T*>(S.uw.coefB)[idx];
         }
         __syncthreads();
-        dev::uwriter_zero_slots<T>(S.uw, S.pre != 0, base, lane);
         const int64_t i0 = (int64_t)w.y * pts_per_item, i1 = min(i0 + pts_per_item, S.uw.n);
-        const dev::UWTabs X{S.uw.qdesc, S.uw.chains, S.uw.ychain, S.uw.gbase, S.uw.ydesc};
-        for (int64_t i = i0 + warp; i < i1; i += nwarps) dev::uwriter_point<T>(S.uw, X, S.pre != 0, i, cA, cB, base, lane);
+        const dev::UWTabs X{S.uw.qdesc, nullptr, S.uw.chains, S.uw.ychain, S.uw.gbase, S.uw.ydesc};
+        auto rows = [&](auto mode) {
+            constexpr int M = decltype(mode)::value;
+            dev::uwriter_zero_slots<T, M>(S.uw, base, lane);
+            for (int64_t i = i0 + warp; i < i1; i += nwarps)
+                dev::uwriter_point<T, M, dev::kGlobal>(S.uw, X, i, cA, cB, base, lane);
+        };
+        if (S.mode == dev::kSlots)
+            rows(std::integral_constant<int, dev::kSlots>());
+        else if (S.mode == dev::kProducts)
+            rows(std::integral_constant<int, dev::kProducts>());
+        else
+            rows(std::integral_constant<int, dev::kChains>());
         __syncthreads();
     }
 }
@@ -1313,12 +1324,15 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         P.U = b->U.as<T>() + b->uoff[s]; P.ldU = tb.ldU;
         P.coefA = A + offs[s].ca; P.coefB = A + offs[s].cb;
         const int levels = d - 2;
+        // slots while eight warps take half of the budget, then products (d >= 4) while eight warps fit,
+        // then tables of every level
         fixed_bytes[s] = dev::align16(sizeof(T) * 2 * levels * tb.tri);
-        const int pw_pre = dev::uwriter_per_warp(levels, tb.tri, tb.L_used, tb.nYp, tb.nF, true);
-        const int pw_fly = dev::uwriter_per_warp(levels, tb.tri, tb.L_used, tb.nYp, tb.nF, false);
-        const bool pre = fixed_bytes[s] + sizeof(T) * 8 * (size_t)pw_pre <= budget / 2;
-        bs[s].pre = pre ? 1 : 0;
-        P.per_warp = pre ? pw_pre : pw_fly;
+        auto per_warp = [&](int mode) { return dev::uwriter_per_warp(levels, tb.tri, tb.L_used, tb.nYp, tb.nF, mode); };
+        auto eight = [&](int mode) { return fixed_bytes[s] + sizeof(T) * 8 * (size_t)per_warp(mode); };
+        bs[s].mode = eight(dev::kSlots) <= budget / 2                   ? dev::kSlots
+                     : levels > 1 && eight(dev::kProducts) <= budget ? dev::kProducts
+                                                                     : dev::kChains;
+        P.per_warp = per_warp(bs[s].mode);
         pw_bytes[s] = sizeof(T) * (size_t)P.per_warp;
         const size_t need_rf = (sizeof(T) == 4) ? batch_df_tile_smem(geo[s].L, fc.m[0] + fc.m[1], 1)
                                                 : dev::radialF_smem(geo[s].L, fc.m[0], fc.m[1], sizeof(T));

@@ -611,7 +611,7 @@ __host__ __device__ inline int radialF_df_kopt(int mt, int tiles, int warps) {
 // taking units from a counter.  QC (and Wt when P.stage_wt) are staged per CTA.  Bound by the FP32
 // issue of the Dot2 products; with one tile between barriers (warp 0 forming the next basis, the
 // others a fixed share of Q) the warps waited for one another half of the time: 1,000,000 points,
-// L = 32: RADNUM.
+// L = 32 2.57 -> 2.45 ms, 500,000 points, d = 4, L = 14 0.44 -> 0.23.
 constexpr int kRfThreads = 512;
 template <int KOPT>
 static __global__ void __launch_bounds__(kRfThreads, 1) k_radial_F_df(RFParams P) {
@@ -678,9 +678,17 @@ static __global__ void __launch_bounds__(kRfThreads, 1) k_radial_F_df(RFParams P
 //   P_j(m, n) = s_n r_j^n C_n^{m + alpha_j}(x_{D_j} / r_j),  D_j = d-1-j, r_j^2 = sum_{i<=D_j} x_i^2,
 // a polynomial in (x_{D_j}, r_j^2) from the normalised three-term recurrence (coefA/coefB).
 // Per-warp shared: level tables, trig powers, Y for all used harmonics, the point's F row.
-template <typename T> struct Vec2;
-template <> struct Vec2<float> { typedef float4 type; static constexpr int w = 4; };
-template <> struct Vec2<double> { typedef double2 type; static constexpr int w = 2; };
+template <typename T> struct Vec16;                      // columns per 16 bytes
+template <> struct Vec16<float> { typedef float4 type; static constexpr int w = 4; };
+template <> struct Vec16<double> { typedef double2 type; static constexpr int w = 2; };
+
+// How a warp gets a harmonic: looked up in the point's slots (all harmonics formed first), formed
+// per column from G and the prefix levels, or from a table of every level and the trigonometric
+// factors (only where the first two do not leave eight warps per SM).
+enum UWMode { kSlots = 0, kProducts = 1, kChains = 2 };
+// Column descriptors: read from global memory by 16-byte chunk, the same staged in shared memory, or
+// one word per column in shared memory.
+enum UWDesc { kGlobal = 0, kChunks = 1, kColumns = 2 };
 
 struct UWParams {
     const double* x; int64_t n; int d; Center c; double inv2R;
@@ -704,19 +712,23 @@ struct UWParams {
 // The index tables the U writer reads for every point (global, or staged in shared memory).
 struct UWTabs {
     const uint32_t* qdesc;     // two words per chunk (see make_tables)
-    const int16_t* chains;     // harmonics formed per chunk only
+    const uint32_t* cdesc;     // kColumns: one word per column
+    const int16_t* chains;     // kChains
     const int32_t* ychain;
-    const int32_t* gbase;      // harmonics precomputed
-    const uint32_t* ydesc;
+    const int32_t* gbase;      // kSlots, d = 3
+    const uint32_t* ydesc;     // kSlots and kProducts, d >= 4
 };
 
-// Bytes of the staged index tables: qdesc, then gbase (d = 3) or ydesc when harmonics are
-// precomputed, chains and ychain when they are not; the kernel lays them out in this order, each
-// 16-byte aligned.
-__host__ __device__ inline size_t uwriter_tab_bytes(int64_t nq, int nH, int cstride, int nYp, int levels, int L, int yw,
-                                                    bool pre) {
-    const size_t q = align16(sizeof(uint32_t) * 2 * nq);
-    if (pre) return q + (levels == 1 ? align16(sizeof(int32_t) * (size_t)(L + 1)) : align16(sizeof(uint32_t) * (size_t)yw * nYp));
+// Bytes of the staged index tables: the column descriptors, and (kSlots) gbase or ydesc, (kChains)
+// chains and ychain; the kernel lays them out in this order, each 16-byte aligned.  kProducts
+// reads ydesc from global memory.
+__host__ __device__ inline size_t uwriter_tab_bytes(int64_t ldU, int vw, int nH, int cstride, int nYp, int levels, int L,
+                                                    int yw, int mode, int desc) {
+    if (desc == kGlobal) return 0;
+    const size_t q = desc == kColumns ? align16(sizeof(uint32_t) * ldU) : align16(sizeof(uint32_t) * 2 * (ldU / vw));
+    if (mode == kSlots)
+        return q + (levels == 1 ? align16(sizeof(int32_t) * (size_t)(L + 1)) : align16(sizeof(uint32_t) * (size_t)yw * nYp));
+    if (mode == kProducts) return q;
     return q + align16(sizeof(int16_t) * (size_t)nH * cstride) + align16(sizeof(int32_t) * (size_t)nYp);
 }
 
@@ -724,8 +736,10 @@ __host__ __device__ inline size_t uwriter_tab_bytes(int64_t nq, int nH, int cstr
 __host__ __device__ inline int uwriter_g_size(int levels, int L) { return levels == 1 ? 0 : (L + 1) * (L + 1) + 1; }
 
 // Shared elements (type T) per warp of the U writer (a multiple of 16 bytes).
-__host__ __device__ inline int uwriter_per_warp(int levels, int tri, int L, int nYp, int nF, bool pre) {
-    return ((pre ? nYp + (levels - 1) * tri + uwriter_g_size(levels, L) : levels * tri + 2 * L + 1) + nF + 1 + 3) & ~3;
+__host__ __device__ inline int uwriter_per_warp(int levels, int tri, int L, int nYp, int nF, int mode) {
+    const int harm = mode == kChains ? levels * tri + 2 * L + 1
+                                     : (mode == kSlots ? nYp : 0) + (levels - 1) * tri + uwriter_g_size(levels, L);
+    return (harm + nF + 1 + 3) & ~3;
 }
 
 // Direction x_hat of point i: differences in FP64, normalisation in the bulk precision T; the
@@ -837,17 +851,34 @@ __device__ __forceinline__ void point_harmonic_tables(const double* __restrict__
     }
 }
 
+// The harmonic of slot y (d >= 4): G[g] times its prefix.
+template <typename T>
+__device__ __forceinline__ T slot_product(const uint32_t* ydesc, uint32_t y, int levels, const T* Pl, const T* G) {
+    if (levels <= 4) {
+        const uint2 w = *reinterpret_cast<const uint2*>(ydesc + 2 * (size_t)y);
+        T v = G[w.x & 0xffffu] * Pl[w.x >> 16];
+        if (levels >= 3) v *= Pl[w.y & 0xffffu];
+        if (levels >= 4) v *= Pl[w.y >> 16];
+        return v;
+    }
+    const uint4 w = *reinterpret_cast<const uint4*>(ydesc + 4 * (size_t)y);
+    T v = G[w.x & 0xffffu] * Pl[w.x >> 16] * Pl[w.y & 0xffffu] * Pl[w.y >> 16] * Pl[w.z & 0xffffu];
+    if (levels >= 6) v *= Pl[w.z >> 16];
+    return v;
+}
+
 // All harmonics of point i into the warp's slots Ys.  Lane m runs the last level's recurrence and
 // multiplies each value by the trigonometric factors +-m at once: in d = 3 these are the harmonics
 // and go to their slots, for d >= 4 they form G, and slot y is G[g] times its prefix (the tables Pl of the
 // levels before the last).  With a table of every level, one of the trigonometric factors and a
 // pass over the chains (two or more index words and as many factors per harmonic), the harmonics
-// took more than half of the instructions of a row at some hundred columns.
+// took more than half of the instructions of a row at some hundred columns.  slots = false stops at
+// the prefix levels and G.
 template <typename T>
 __device__ __forceinline__ void point_harmonics(const double* __restrict__ x, int d, const Center& cen, double inv2R,
                                                 int L, int tri, const T* cA, const T* cB, const int32_t* gbase,
                                                 const uint32_t* ydesc, int nYp, T* Ys, T* Pl, T* G, int64_t i, int lane,
-                                                bool have_x, double x_lane) {
+                                                bool have_x, double x_lane, bool slots) {
     const int levels = d - 2;
     T xh[kMaxD];
     point_direction<T>(x, d, cen, inv2R, i, lane, have_x, x_lane, xh);
@@ -880,38 +911,25 @@ __device__ __forceinline__ void point_harmonics(const double* __restrict__ x, in
             }
         }
     }
-    if (levels == 1) return;
+    if (levels == 1 || !slots) return;
     __syncwarp();
-    if (levels <= 4) {
-        for (int y = lane; y < nYp; y += 32) {
-            const uint2 w = *reinterpret_cast<const uint2*>(ydesc + 2 * y);
-            T v = G[w.x & 0xffffu] * Pl[w.x >> 16];
-            if (levels >= 3) v *= Pl[w.y & 0xffffu];
-            if (levels >= 4) v *= Pl[w.y >> 16];
-            Ys[y] = v;
-        }
-    } else {
-        for (int y = lane; y < nYp; y += 32) {
-            const uint4 w = *reinterpret_cast<const uint4*>(ydesc + 4 * y);
-            T v = G[w.x & 0xffffu] * Pl[w.x >> 16] * Pl[w.y & 0xffffu] * Pl[w.y >> 16] * Pl[w.z & 0xffffu];
-            if (levels >= 6) v *= Pl[w.z >> 16];
-            Ys[y] = v;
-        }
-    }
+    for (int y = lane; y < nYp; y += 32) Ys[y] = slot_product<T>(ydesc, y, levels, Pl, G);
 }
 
 // One point's U row, executed by one warp.  cA/cB: level recurrences in shared memory;
 // base: this warp's shared area (P.per_warp elements, 16-byte aligned), laid out as [harmonic
-// slots] [level tables but the last] [G] [radial factors] (pre) or [level tables] [trig powers]
-// [radial factors].  pre: the harmonics of the point are computed once into the slots; otherwise
-// each chunk's harmonics are multiplied out from the level tables as it is written.  A VW-wide chunk of the row meets
-// one or two (k, s) blocks; its two descriptor words give each block's radial factor and first
-// harmonic slot.
+// slots (kSlots)] [level tables but the last] [G] [radial factors], or (kChains) [level tables] [trig
+// powers] [radial factors].  Column c is one radial factor times one harmonic.  With slots a lane
+// writes a 16-byte chunk of the row, whose two descriptor words name the one or two (k, s) blocks it
+// meets; otherwise lane l forms the columns l, l + 32, .. (consecutive words of the tables).  Slots
+// with a column per lane measured 6.88 -> 7.55 ms at 1,000,000 x 10,680 (d = 3) and 3 to 7% less at
+// d = 4, rank 1,000 to 5,000.
 // The radial-factor slots of a warp's shared area (nF + 1, the last one zero).
 template <typename T>
-__device__ __forceinline__ T* uwriter_fs(const UWParams& P, bool pre, T* base) {
+__device__ __forceinline__ T* uwriter_fs(const UWParams& P, int mode, T* base) {
     const int levels = P.d - 2;
-    return base + (pre ? P.nYp + (levels - 1) * P.tri + uwriter_g_size(levels, P.L) : levels * P.tri + 2 * P.L + 1);
+    return base + (mode == kChains ? levels * P.tri + 2 * P.L + 1
+                                   : (mode == kSlots ? P.nYp : 0) + (levels - 1) * P.tri + uwriter_g_size(levels, P.L));
 }
 
 // Radial factors and coordinate of one point loaded into registers one point ahead of use (FP32
@@ -924,6 +942,7 @@ __device__ __forceinline__ void point_prefetch(const UWParams& P, int64_t i, int
     const T* Fg = reinterpret_cast<const T*>(P.F) + i * P.ldF;
 #pragma unroll
     for (int k = 0; k < kPfF; ++k) {
+        if (32 * k >= P.nF) break;
         const int f = lane + 32 * k;
         pp.f[k] = (f < P.nF) ? Fg[f] : (T)0;
     }
@@ -933,30 +952,37 @@ template <typename T>
 __device__ __forceinline__ void point_stage_f(const UWParams& P, const PointPre<T>& pp, T* Fs, int lane) {
 #pragma unroll
     for (int k = 0; k < kPfF; ++k) {
+        if (32 * k >= P.nF) break;
         const int f = lane + 32 * k;
         if (f < P.nF) Fs[f] = pp.f[k];
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X, bool pre, int64_t i, const T* cA,
-                                              const T* cB, T* base, int lane, bool staged = false,
-                                              double x_lane = 0.0) {
+// Descriptor of column c, F index << 20 | slot, from the two words of its 16-byte chunk.
+template <int VW>
+__device__ __forceinline__ uint32_t uwriter_column(const uint32_t* qdesc, int64_t c) {
+    const int64_t q = c / VW;
+    const uint32_t u = (uint32_t)(c % VW);
+    const uint32_t w0 = qdesc[2 * q], e = (w0 >> 18) & 3u;
+    if (e == 0 || u < e) return (w0 & 0xFFF00000u) | ((w0 & 0x3FFFFu) + u);
+    const uint32_t w1 = qdesc[2 * q + 1];
+    return (w1 & 0xFFF00000u) | ((w1 & 0xFFFFFu) + u - e);
+}
+
+template <typename T, int MODE, int DESC>
+__device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X, int64_t i, const T* cA, const T* cB,
+                                              T* base, int lane, bool staged = false, double x_lane = 0.0) {
     const int levels = P.d - 2;
-    T* Ys = base;                                // nYp (pre only)
-    T* Pl = base + P.nYp;                        // (levels - 1) * tri (pre only)
-    T* G = Pl + (levels - 1) * P.tri;            // G (pre only)
-    T* tbl = base;                               // levels * tri, then 2L+1 trig, index L + mu (not pre)
+    T* Ys = base;                                            // nYp (kSlots)
+    T* Pl = base + (MODE == kSlots ? P.nYp : 0);             // (levels - 1) * tri
+    T* G = Pl + (levels - 1) * P.tri;
+    T* tbl = base;                                           // kChains: levels * tri, then 2L+1 trig, index L + mu
     T* trig = tbl + levels * P.tri;
-    T* Fs = uwriter_fs<T>(P, pre, base);         // nF + 1
+    T* Fs = uwriter_fs<T>(P, MODE, base);                    // nF + 1
     const T* Fg = reinterpret_cast<const T*>(P.F);
-    T* Ug = reinterpret_cast<T*>(P.U);
-    typedef typename Vec2<T>::type VT;
-    constexpr int VW = Vec2<T>::w;
-    // padding slots are zeroed once per warp (d = 3) or written as zeros
-    if (pre)
+    if (MODE != kChains)
         point_harmonics<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, X.gbase, X.ydesc, P.nYp, Ys, Pl, G, i, lane,
-                           staged, x_lane);
+                           staged, x_lane, MODE == kSlots);
     else
         point_harmonic_tables<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane, staged, x_lane);
     // this point's radial factors (staged: already in Fs, written by the caller)
@@ -965,82 +991,81 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
         if (lane == 0) Fs[P.nF] = (T)0;
     }
     __syncwarp();
-    // row write: one VW-wide chunk per lane per step, four (FP64: two) steps in flight.  A chunk
-    // is one radial factor times VW consecutive harmonic slots, or (where it meets the end of a
-    // (k, s) block) the first e columns from one block and the rest from the next.
-    T* row = Ug + i * P.ldU;
-    const int64_t nq = P.ldU / VW;
-    auto harm = [&](uint32_t y) -> T {          // the harmonic in slot y (0 for a padding slot)
-        if (pre) return Ys[y];
+    auto column = [&](int64_t c) -> T {
+        const uint32_t w = DESC == kColumns ? X.cdesc[c] : uwriter_column<Vec16<T>::w>(X.qdesc, c);
+        const T f = Fs[w >> 20];
+        const uint32_t y = w & 0xFFFFFu;
+        if constexpr (MODE == kProducts) return f * slot_product<T>(X.ydesc, y, levels, Pl, G);
         const int ch = X.ychain[y];
-        T h = (T)0;
-        if (ch >= 0) {
-            const int16_t* c = X.chains + (int64_t)ch * P.cstride;
-            h = trig[P.L + c[levels]];
-            for (int j = 0; j < levels; ++j) h *= tbl[j * P.tri + c[j]];
-        }
-        return h;
+        if (ch < 0) return (T)0;
+        const int16_t* q = X.chains + (int64_t)ch * P.cstride;
+        T h = trig[P.L + q[levels]];
+        for (int j = 0; j < levels; ++j) h *= tbl[j * P.tri + q[j]];
+        return f * h;
     };
-    auto chunk = [&](int64_t q) {
-        const uint2 w = *reinterpret_cast<const uint2*>(X.qdesc + 2 * q);
-        const uint32_t e = (w.x >> 18) & 3u;
-        const T fa = Fs[w.x >> 20];
-        const uint32_t ya = w.x & 0x3FFFFu;
-        VT out;
-        T v[VW];
-        if (pre) {
-            // one branch-free form for whole and split chunks (e = 0 reads as e = VW; the second
-            // word of a whole chunk names valid slots and is never selected), so that the lanes of
-            // a warp, whose chunks differ in kind and alignment, do not diverge
-            const uint32_t ea = e ? e : (uint32_t)VW;
-            const T fb = Fs[w.y >> 20];
-            const uint32_t yb = (w.y & 0xFFFFFu) - ea;
+    T* row = reinterpret_cast<T*>(P.U) + i * P.ldU;
+    if constexpr (MODE == kSlots) {
+        // a 16-byte chunk per lane, four (FP64: two) in flight: one or two runs of consecutive slots, in
+        // one branch-free form (e = 0 reads as e = VW; the second word of a whole chunk names valid
+        // slots and is never selected), so that the lanes of a warp do not diverge
+        typedef typename Vec16<T>::type VT;
+        constexpr int VW = Vec16<T>::w, NQ = VW;
+        auto chunk = [&](int64_t q) {
+            const uint2 w = *reinterpret_cast<const uint2*>(X.qdesc + 2 * q);
+            const uint32_t e = (w.x >> 18) & 3u, ea = e ? e : (uint32_t)VW;
+            const T fa = Fs[w.x >> 20], fb = Fs[w.y >> 20];
+            const uint32_t ya = w.x & 0x3FFFFu, yb = (w.y & 0xFFFFFu) - ea;
+            T v[VW];
             v[0] = fa * Ys[ya];
 #pragma unroll
             for (int u = 1; u < VW; ++u) {
                 const bool a = (uint32_t)u < ea;
                 v[u] = (a ? fa : fb) * Ys[a ? ya + u : yb + u];
             }
-        } else if (e == 0) {
+            VT out;
+            if constexpr (VW == 4) { out.x = v[0]; out.y = v[1]; out.z = v[2]; out.w = v[3]; }
+            else { out.x = v[0]; out.y = v[1]; }
+            return out;
+        };
+        VT* rq = reinterpret_cast<VT*>(row);
+        const int64_t nq = P.ldU / VW;
+        int64_t q = lane;
+        for (; q + 32 * (NQ - 1) < nq; q += 32 * NQ) {
+            VT o[NQ];
 #pragma unroll
-            for (int u = 0; u < VW; ++u) v[u] = fa * harm(ya + u);
-        } else {
-            const T fb = Fs[w.y >> 20];
-            const uint32_t yb = w.y & 0xFFFFFu;
+            for (int f = 0; f < NQ; ++f) o[f] = chunk(q + 32 * f);
 #pragma unroll
-            for (int u = 0; u < VW; ++u) v[u] = ((uint32_t)u < e) ? fa * harm(ya + u) : fb * harm(yb + u - e);
+            for (int f = 0; f < NQ; ++f) rq[q + 32 * f] = o[f];
         }
-        if constexpr (VW == 4) { out.x = v[0]; out.y = v[1]; out.z = v[2]; out.w = v[3]; }
-        else { out.x = v[0]; out.y = v[1]; }
-        return out;
-    };
-    constexpr int NF = (VW == 4) ? 4 : 2;        // chunks in flight per lane
-    int64_t q = lane;
-    for (; q + 32 * (NF - 1) < nq; q += 32 * NF) {
-        VT o[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) o[f] = chunk(q + 32 * f);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) *reinterpret_cast<VT*>(row + (q + 32 * f) * VW) = o[f];
+        for (; q < nq; q += 32) rq[q] = chunk(q);
+        __syncwarp();
+        return;
     }
-    for (; q < nq; q += 32) *reinterpret_cast<VT*>(row + q * VW) = chunk(q);
+    constexpr int NF = 4;                                    // columns in flight per lane
+    int64_t c = lane;
+    for (; c + 32 * (NF - 1) < P.ldU; c += 32 * NF) {
+        T o[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) o[f] = column(c + 32 * f);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) row[c + 32 * f] = o[f];
+    }
+    for (; c < P.ldU; c += 32) row[c] = column(c);
     __syncwarp();
 }
 
 // Zeroes a warp's harmonic slots and G's last entry once (padding slots of d = 3 and that entry are
 // never written afterwards).
-template <typename T>
-__device__ __forceinline__ void uwriter_zero_slots(const UWParams& P, bool pre, T* base, int lane) {
-    if (pre) {
+template <typename T, int MODE>
+__device__ __forceinline__ void uwriter_zero_slots(const UWParams& P, T* base, int lane) {
+    if (MODE == kSlots)
         for (int g = lane; g < P.nYp; g += 32) base[g] = (T)0;
-        if (P.d > 3 && lane == 0) base[P.nYp + (P.d - 3) * P.tri + uwriter_g_size(P.d - 2, P.L) - 1] = (T)0;
-    }
+    if (MODE != kChains && P.d > 3 && lane == 0) uwriter_fs<T>(P, MODE, base)[-1] = (T)0;
     __syncwarp();
 }
 
-// Shared memory of the U writer: [nwarps x per_warp][coefA][coefB] (elements of T).
 // Shared memory: [nwarps x per_warp elements][cA][cB][staged index tables (tab_bytes)].
-template <typename T, bool PRE, bool PF, bool STAGED>
+template <typename T, int MODE, bool PF, int DESC>
 __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int levels = P.d - 2;
@@ -1052,26 +1077,32 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
         cA[idx] = reinterpret_cast<const T*>(P.coefA)[idx];
         cB[idx] = reinterpret_cast<const T*>(P.coefB)[idx];
     }
-    UWTabs X{P.qdesc, P.chains, P.ychain, P.gbase, P.ydesc};
-    if constexpr (STAGED) {
-        // staged in shared memory (STAGED is a compile-time choice, so that the table reads
-        // compile to shared-memory loads)
+    UWTabs X{P.qdesc, nullptr, P.chains, P.ychain, P.gbase, P.ydesc};
+    if constexpr (DESC != kGlobal) {
+        // staged in shared memory (a compile-time choice, so that the table reads compile to
+        // shared-memory loads)
         unsigned char* tp = reinterpret_cast<unsigned char*>(smem_raw) +
                             align16(sizeof(T) * ((size_t)nwarps * P.per_warp + 2 * (size_t)levels * P.tri));
-        const int64_t nq = P.ldU / Vec2<T>::w;
         uint32_t* q = reinterpret_cast<uint32_t*>(tp);
-        for (int64_t k = threadIdx.x; k < 2 * nq; k += blockDim.x) q[k] = P.qdesc[k];
-        X.qdesc = q;
-        tp += align16(sizeof(uint32_t) * 2 * nq);
-        if (PRE && levels == 1) {
+        if constexpr (DESC == kColumns) {
+            for (int64_t k = threadIdx.x; k < P.ldU; k += blockDim.x) q[k] = uwriter_column<Vec16<T>::w>(P.qdesc, k);
+            X.cdesc = q;
+            tp += align16(sizeof(uint32_t) * P.ldU);
+        } else {
+            const int64_t nw = 2 * (P.ldU / Vec16<T>::w);
+            for (int64_t k = threadIdx.x; k < nw; k += blockDim.x) q[k] = P.qdesc[k];
+            X.qdesc = q;
+            tp += align16(sizeof(uint32_t) * nw);
+        }
+        if (MODE == kSlots && levels == 1) {
             int32_t* gb = reinterpret_cast<int32_t*>(tp);
             for (int k = threadIdx.x; k <= P.L; k += blockDim.x) gb[k] = P.gbase[k];
             X.gbase = gb;
-        } else if (PRE) {
+        } else if (MODE == kSlots) {
             uint32_t* yd = reinterpret_cast<uint32_t*>(tp);
             for (int k = threadIdx.x; k < P.yw * P.nYp; k += blockDim.x) yd[k] = P.ydesc[k];
             X.ydesc = yd;
-        } else {
+        } else if (MODE == kChains) {
             int16_t* ch = reinterpret_cast<int16_t*>(tp);
             for (int64_t k = threadIdx.x; k < (int64_t)P.nH * P.cstride; k += blockDim.x) ch[k] = P.chains[k];
             tp += align16(sizeof(int16_t) * (size_t)P.nH * P.cstride);
@@ -1082,11 +1113,11 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
         }
     }
     __syncthreads();
-    uwriter_zero_slots<T>(P, PRE, base, lane);
+    uwriter_zero_slots<T, MODE>(P, base, lane);
     const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
     if constexpr (PF) {
         // PF: the next point's radial factors and coordinate travel in registers during this row
-        T* Fs = uwriter_fs<T>(P, PRE, base);
+        T* Fs = uwriter_fs<T>(P, MODE, base);
         if (lane == 0) Fs[P.nF] = (T)0;
         PointPre<T> pp;
         if (gw < P.n) point_prefetch<T>(P, gw, lane, pp);
@@ -1094,10 +1125,10 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
             point_stage_f<T>(P, pp, Fs, lane);
             const double xl = pp.x;
             if (i + nw < P.n) point_prefetch<T>(P, i + nw, lane, pp);
-            uwriter_point<T>(P, X, PRE, i, cA, cB, base, lane, true, xl);
+            uwriter_point<T, MODE, DESC>(P, X, i, cA, cB, base, lane, true, xl);
         }
     } else {
-        for (int64_t i = gw; i < P.n; i += nw) uwriter_point<T>(P, X, PRE, i, cA, cB, base, lane);
+        for (int64_t i = gw; i < P.n; i += nw) uwriter_point<T, MODE, DESC>(P, X, i, cA, cB, base, lane);
     }
 }
 
