@@ -1270,51 +1270,62 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         const int levels = d - 2;
         // One CTA per SM with as many warps as shared memory holds (up to 32): the coefficient
         // tables and, when they fit, the index tables are shared by all its warps.  The first form
-        // that leaves eight warps is taken: harmonics in slots; harmonics as products (d >= 4) with a
-        // descriptor per column, then per chunk; slots, then products, with the descriptors in
-        // global memory; tables of every level; the last takes what is left.
+        // that leaves enough warps is taken: harmonics in slots, 8 or 16 lanes per point at degrees
+        // below 8 or 16, then 32; harmonics as products (d >= 4) with a descriptor per column, then per
+        // chunk; slots, then products, with the descriptors in global memory; tables of every level;
+        // the last takes what is left.  Groups of lanes need all 32 warps in FP32 (100,000 points, d = 4:
+        // 32 warps at rank 912 0.162 -> 0.142 ms; at rank 1,279, 30 warps would take 0.205 for 0.171) and 6 in
+        // FP64, whose pipe few warps fill (d = 4: rank 621 1.33 -> 0.68, 2,266 1.85 -> 1.32; d = 5, rank 4,986, 5
+        // warps would take 3.10 for 2.27).
         const size_t coef = dev::align16(sizeof(T) * 2 * (size_t)levels * ht.tri);
         const size_t budget = 226 * 1024;
         using UK = void (*)(dev::UWParams);
-        struct Cfg { int mode, desc; UK kern; };
+        struct Cfg { int mode, desc, lanes, min_warps; UK kern; };
+        using namespace dev;
+        // FP32 factors, harmonics in slots, tables staged, few radial factors: the next point's
+        // radial factors and coordinate are prefetched into registers
+        constexpr bool pf = sizeof(T) == 4;
+        constexpr int group_warps = sizeof(T) == 8 ? 6 : 32;
         const Cfg forms[] = {
-            {dev::kSlots, dev::kChunks, dev::k_uwriter<T, dev::kSlots, false, dev::kChunks>},
-            {dev::kProducts, dev::kColumns, dev::k_uwriter<T, dev::kProducts, false, dev::kColumns>},
-            {dev::kProducts, dev::kChunks, dev::k_uwriter<T, dev::kProducts, false, dev::kChunks>},
-            {dev::kSlots, dev::kGlobal, dev::k_uwriter<T, dev::kSlots, false, dev::kGlobal>},
-            {dev::kProducts, dev::kGlobal, dev::k_uwriter<T, dev::kProducts, false, dev::kGlobal>},
-            {dev::kChains, dev::kChunks, dev::k_uwriter<T, dev::kChains, false, dev::kChunks>},
-            {dev::kChains, dev::kGlobal, dev::k_uwriter<T, dev::kChains, false, dev::kGlobal>},
+            {kSlots, kChunks, 8, group_warps, k_uwriter<T, kSlots, pf, kChunks, 8>},
+            {kSlots, kChunks, 16, group_warps, k_uwriter<T, kSlots, pf, kChunks, 16>},
+            {kSlots, kChunks, 32, 8, k_uwriter<T, kSlots, pf, kChunks, 32>},
+            {kSlots, kChunks, 0, 8, k_uwriter<T, kSlots, false, kChunks, 32>},       // many radial factors
+            {kProducts, kColumns, 32, 8, k_uwriter<T, kProducts, false, kColumns, 32>},
+            {kProducts, kChunks, 32, 8, k_uwriter<T, kProducts, false, kChunks, 32>},
+            {kSlots, kGlobal, 32, 8, k_uwriter<T, kSlots, false, kGlobal, 32>},
+            {kProducts, kGlobal, 32, 8, k_uwriter<T, kProducts, false, kGlobal, 32>},
+            {kChains, kChunks, 32, 8, k_uwriter<T, kChains, false, kChunks, 32>},
+            {kChains, kGlobal, 32, 1, k_uwriter<T, kChains, false, kGlobal, 32>},
         };
         UK kern = nullptr;
-        int warps = 0;
+        int warps = 0, per = 1;                            // warps, points per warp
         size_t pw = 0, tabs = 0;
         for (const Cfg& c : forms) {
-            if (c.mode == dev::kProducts && levels == 1) continue;
-            pw = sizeof(T) * (size_t)dev::uwriter_per_warp(levels, ht.tri, L_used, tb.nYp, nF, c.mode);
-            tabs = dev::uwriter_tab_bytes(I.ldu, vw, (int)nH, chain_stride(d), tb.nYp, levels, L_used, tb.yw, c.mode, c.desc);
+            const int gl = c.lanes ? c.lanes : 32;
+            if (c.mode == kProducts && levels == 1) continue;
+            if (gl < 32 && L_used >= gl) continue;
+            if (pf && c.mode == kSlots && c.desc == kChunks && c.lanes && nF > gl * kPfF) continue;
+            per = 32 / gl;
+            pw = per * sizeof(T) * (size_t)uwriter_per_warp(levels, ht.tri, L_used, tb.nYp, nF, c.mode);
+            tabs = uwriter_tab_bytes(I.ldu, vw, (int)nH, chain_stride(d), tb.nYp, levels, L_used, tb.yw, c.mode, c.desc);
             if (coef + tabs >= budget) continue;
             warps = (int)std::min<size_t>(32, (budget - coef - tabs) / pw);
-            if (warps < (c.kern == forms[6].kern ? 1 : 8)) { warps = 0; continue; }
-            kern = c.kern;
-            // FP32 factors, harmonics in slots, tables staged, nF <= 32 kPfF: the next point's
-            // radial factors and coordinate are prefetched into registers
-            if constexpr (sizeof(T) == 4)
-                if (c.mode == dev::kSlots && c.desc == dev::kChunks && nF <= 32 * dev::kPfF)
-                    kern = dev::k_uwriter<T, dev::kSlots, true, dev::kChunks>;
-            break;
+            if (warps >= c.min_warps) { kern = c.kern; break; }
         }
-        if (warps == 0) return fail(HDF_ETOOBIG, "hdf_build: harmonic tables exceed shared memory");
-        P.per_warp = (int)(pw / sizeof(T));
-        P.tab_bytes = (int)tabs;
-        const size_t sm = dev::align16((size_t)warps * pw + sizeof(T) * 2 * (size_t)levels * ht.tri) + tabs;
-        HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        int occ = 0;
-        HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, sm));
+        if (!kern) return fail(HDF_ETOOBIG, "hdf_build: harmonic tables exceed shared memory");
         int nsm = 0, dv = 0;
         HDF_CUDA(cudaGetDevice(&dv));
         HDF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dv));
-        const int grid = std::max(1, std::min<int>(nsm * std::max(occ, 1), (int)((n + warps - 1) / warps)));
+        // few points: fewer warps per CTA, on more SMs
+        warps = (int)std::min<int64_t>(warps, std::max<int64_t>(8, (n + (int64_t)nsm * per - 1) / ((int64_t)nsm * per)));
+        P.per_warp = (int)(pw / sizeof(T));
+        P.tab_bytes = (int)tabs;
+        const size_t sm = align16((size_t)warps * pw + sizeof(T) * 2 * (size_t)levels * ht.tri) + tabs;
+        HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        int occ = 0;
+        HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, sm));
+        const int grid = std::max(1, std::min<int>(nsm * std::max(occ, 1), (int)((n + warps * per - 1) / (warps * per))));
         HDF_COUNT_LAUNCH();
         kern<<<grid, warps * 32, sm, st>>>(P);   // P.tab_bytes: staged index tables
         HDF_CUDA(cudaGetLastError());

@@ -253,6 +253,7 @@ struct BuildSet {
     dev::RFParams rf;
     dev::UWParams uw;
     int mode;                        // dev::UWMode
+    int lanes;                       // lanes per point (32, or 16 / 8 with harmonics in slots)
 };
 
 // Shared memory of the double-float radial phase of the batched build for `tiles` tiles per
@@ -339,30 +340,28 @@ __global__ void __launch_bounds__(1024) k_batch_urows(const BuildSet* __restrict
         __syncthreads();
         if (it >= nitems) break;
         const int2 w = items[it];
-        const BuildSet& S = sets[w.x];
-        const int levels = S.uw.d - 2;
-        T* base = reinterpret_cast<T*>(smem_raw) + (size_t)warp * S.uw.per_warp;
-        T* cA = reinterpret_cast<T*>(smem_raw) + (size_t)nwarps * S.uw.per_warp;
-        T* cB = cA + levels * S.uw.tri;
-        for (int idx = threadIdx.x; idx < levels * S.uw.tri; idx += blockDim.x) {
-            cA[idx] = reinterpret_cast<const T*>(S.uw.coefA)[idx];
-            cB[idx] = reinterpret_cast<const T*>(S.uw.coefB)[idx];
-        }
-        __syncthreads();
-        const int64_t i0 = (int64_t)w.y * pts_per_item, i1 = min(i0 + pts_per_item, S.uw.n);
-        const dev::UWTabs X{S.uw.qdesc, nullptr, S.uw.chains, S.uw.ychain, S.uw.gbase, S.uw.ydesc};
-        auto rows = [&](auto mode) {
-            constexpr int M = decltype(mode)::value;
-            dev::uwriter_zero_slots<T, M>(S.uw, base, lane);
-            for (int64_t i = i0 + warp; i < i1; i += nwarps)
-                dev::uwriter_point<T, M, dev::kGlobal>(S.uw, X, i, cA, cB, base, lane);
+        const int mode = sets[w.x].mode;
+        const dev::UWParams P = sets[w.x].uw;              // in registers: the rows' stores do not make it stale
+        const int64_t i0 = (int64_t)w.y * pts_per_item, i1 = min(i0 + pts_per_item, P.n);
+        T* base = reinterpret_cast<T*>(smem_raw) + (size_t)warp * P.per_warp;
+        T* cA = reinterpret_cast<T*>(smem_raw) + (size_t)nwarps * P.per_warp;
+        auto rows = [&](auto m, auto pf, auto desc, auto lanes) {
+            constexpr int M = decltype(m)::value, D = decltype(desc)::value, GL = decltype(lanes)::value, G = 32 / GL;
+            const dev::UWTabs X = dev::uwriter_stage<T, M, D>(P, cA, dev::uwriter_tabs_at<T>(P, smem_raw, nwarps));
+            __syncthreads();
+            dev::uwriter_rows<T, M, decltype(pf)::value, D, GL>(P, X, cA, cA + (P.d - 2) * P.tri, base, i0 + warp * G,
+                                                                nwarps * G, i1);
         };
-        if (S.mode == dev::kSlots)
-            rows(std::integral_constant<int, dev::kSlots>());
-        else if (S.mode == dev::kProducts)
-            rows(std::integral_constant<int, dev::kProducts>());
-        else
-            rows(std::integral_constant<int, dev::kChains>());
+        using dev::Count;
+        constexpr bool pf = sizeof(T) == 4;
+        const int lanes = P.tab_bytes && mode == dev::kSlots && (!pf || P.nF <= sets[w.x].lanes * dev::kPfF) ? sets[w.x].lanes : 0;
+        using PF = std::integral_constant<bool, pf>;
+        if (lanes == 8) rows(Count<dev::kSlots>(), PF(), Count<dev::kChunks>(), Count<8>());
+        else if (lanes == 16) rows(Count<dev::kSlots>(), PF(), Count<dev::kChunks>(), Count<16>());
+        else if (lanes == 32) rows(Count<dev::kSlots>(), PF(), Count<dev::kChunks>(), Count<32>());
+        else if (mode == dev::kSlots) rows(Count<dev::kSlots>(), std::false_type(), Count<dev::kGlobal>(), Count<32>());
+        else if (mode == dev::kProducts) rows(Count<dev::kProducts>(), std::false_type(), Count<dev::kGlobal>(), Count<32>());
+        else rows(Count<dev::kChains>(), std::false_type(), Count<dev::kGlobal>(), Count<32>());
         __syncthreads();
     }
 }
@@ -1332,7 +1331,18 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         bs[s].mode = eight(dev::kSlots) <= budget / 2                   ? dev::kSlots
                      : levels > 1 && eight(dev::kProducts) <= budget ? dev::kProducts
                                                                      : dev::kChains;
-        P.per_warp = per_warp(bs[s].mode);
+        // 8 or 16 lanes per point at degrees below 8 or 16 where 32 (FP64: 8) warps fit, as in the
+        // single build
+        bs[s].lanes = 32;
+        for (int gl = 8; bs[s].mode == dev::kSlots && gl < 32 && bs[s].lanes == 32; gl *= 2)
+            if (tb.L_used < gl && (sizeof(T) == 8 || tb.nF <= gl * dev::kPfF) &&
+                fixed_bytes[s] + sizeof(T) * (sizeof(T) == 8 ? 8 : 32) * (32 / gl) * (size_t)per_warp(dev::kSlots) <= budget * 3 / 4)
+                bs[s].lanes = gl;
+        P.per_warp = per_warp(bs[s].mode) * (32 / bs[s].lanes);
+        P.tab_bytes = bs[s].mode != dev::kSlots
+                          ? 0
+                          : (int)dev::uwriter_tab_bytes(tb.ldU, dev::Vec16<T>::w, 0, 0, tb.nYp, levels, tb.L_used, tb.yw,
+                                                        dev::kSlots, dev::kChunks);
         pw_bytes[s] = sizeof(T) * (size_t)P.per_warp;
         const size_t need_rf = (sizeof(T) == 4) ? batch_df_tile_smem(geo[s].L, fc.m[0] + fc.m[1], 1)
                                                 : dev::radialF_smem(geo[s].L, fc.m[0], fc.m[1], sizeof(T));
@@ -1346,7 +1356,7 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
     // and a half of the largest need
     size_t pw_max = 0;
     for (int s = 0; s < ns; ++s) pw_max = std::max(pw_max, pw_bytes[s]);
-    struct UClass { std::vector<int> sets; size_t pw = 0, fixed = 0; int64_t points = 0; };
+    struct UClass { std::vector<int> sets; size_t pw = 0, fixed = 0, tabs = 0; int64_t points = 0; };
     std::vector<UClass> ucls(3);
     for (int s = 0; s < ns; ++s) {
         if (fcs[s].rank == 0) continue;
@@ -1354,7 +1364,16 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         ucls[c].sets.push_back(s);
         ucls[c].pw = std::max(ucls[c].pw, pw_bytes[s]);
         ucls[c].fixed = std::max(ucls[c].fixed, fixed_bytes[s]);
+        ucls[c].tabs = std::max(ucls[c].tabs, (size_t)bs[s].uw.tab_bytes);
         ucls[c].points += geo[s].n;
+    }
+    // the index tables are staged per item where eight warps of the class still fit
+    for (UClass& u : ucls) {
+        if (u.fixed + u.tabs + 16 + 8 * u.pw > budget) {
+            u.tabs = 0;
+            for (int s : u.sets) bs[s].uw.tab_bytes = 0;
+        }
+        u.fixed += u.tabs ? u.tabs + 16 : 0;
     }
     ucls.erase(std::remove_if(ucls.begin(), ucls.end(), [](const UClass& u) { return u.sets.empty(); }), ucls.end());
     HDF_CUDA(b->dsets.alloc_on(sizeof(BuildSet) * ns, st));
@@ -1403,7 +1422,9 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
             P.pts = a;
         } else {
             const UClass& u = ucls[ph - 1];
-            P.pts = 8 * a;                             // points per item: 8 per warp
+            // points per item: 8 to 32 per warp, as long as that leaves every SM eight items
+            P.pts = 8 * a;
+            while (P.pts < 32 * a && u.points / (2 * P.pts) >= 8 * nsm) P.pts *= 2;
             it = urow_items(u, P.pts);
             P.smem = dev::align16(u.fixed + (size_t)a * u.pw);
         }
@@ -1463,7 +1484,7 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
             std::snprintf(key, sizeof(key), "batch_radial_v3:sm%d:d%d:%s:smem%zu:work2^%d", nsm, d,
                           sizeof(T) == 4 ? "fp32" : "fp64", smem_rf / 4096, bucket);
         else
-            std::snprintf(key, sizeof(key), "batch_urows_v1:sm%d:d%d:%s:pw%zu:fixed%zu:work2^%d", nsm, d,
+            std::snprintf(key, sizeof(key), "batch_urows_v3:sm%d:d%d:%s:pw%zu:fixed%zu:work2^%d", nsm, d,
                           sizeof(T) == 4 ? "fp32" : "fp64", ucls[ph - 1].pw / 256, ucls[ph - 1].fixed / 1024, bucket);
         int code = 0;
         {

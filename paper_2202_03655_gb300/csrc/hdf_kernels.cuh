@@ -705,11 +705,13 @@ struct UWParams {
     const void* F; int64_t ldF;
     void* U; int64_t ldU;
     const void* coefA; const void* coefB;   // (d-2) x tri, type T
-    int per_warp;              // shared elements (type T) per warp
+    int per_warp;              // shared elements (type T) per warp (an equal part per group of lanes)
     int tab_bytes;             // bytes of index tables staged in shared memory (0: read from global)
 };
 
 // The index tables the U writer reads for every point (global, or staged in shared memory).
+template <int N> struct Count { static constexpr int value = N; };
+
 struct UWTabs {
     const uint32_t* qdesc;     // two words per chunk (see make_tables)
     const uint32_t* cdesc;     // kColumns: one word per column
@@ -742,39 +744,40 @@ __host__ __device__ inline int uwriter_per_warp(int levels, int tri, int L, int 
     return (harm + nF + 1 + 3) & ~3;
 }
 
+// This lane's centre coordinate (compile-time indices: the centre stays in registers).
+__device__ __forceinline__ double lane_centre(const Center& cen, int lane) {
+    double cj = cen.c[0];
+#pragma unroll
+    for (int j = 1; j < kMaxD; ++j) cj = (lane == j) ? cen.c[j] : cj;
+    return cj;
+}
+
+// A group of GL lanes (32, 16 or 8) forms one point's row; `lane` is the lane within the group.
+
 // Direction x_hat of point i: differences in FP64, normalisation in the bulk precision T; the
-// zero vector gets e_0.  xh is indexed with compile-time indices only (loops over kMaxD with the
-// dimension as a predicate), so that it stays in registers.
-template <typename T>
-__device__ __forceinline__ void point_direction(const double* __restrict__ x, int d, const Center& cen, double inv2R,
-                                                int64_t i, int lane, bool have_x, double x_lane, T* xh) {
+// zero vector gets e_0.  Lane j forms coordinate j (x_lane: loaded ahead by the caller; cj: its
+// centre) and the warp shares it by shuffles, since an FP64 instruction holds the pipe for 16 cycles
+// whatever its active lanes.  xh is indexed with compile-time indices only (loops over kMaxD with
+// the dimension as a predicate), so that it stays in registers.
+template <typename T, int GL>
+__device__ __forceinline__ void point_direction(const double* __restrict__ x, int d, double cj, double inv2R, int64_t i,
+                                                int lane, bool have_x, double x_lane, T* xh) {
     T s = (T)0;
-    if constexpr (sizeof(T) == 4) {
-        // FP32 factors: lane j forms coordinate j once and the warp shares it by shuffles (FP64
-        // issues at a small fraction of the FP32 rate here).
-        double cj = cen.c[0];                    // this lane's centre coordinate (register selects)
+    const T xt = (T)((lane < d) ? ((have_x ? x_lane : x[i * d + lane]) - cj) * inv2R : 0.0);
 #pragma unroll
-        for (int j = 1; j < kMaxD; ++j) cj = (lane == j) ? cen.c[j] : cj;
-        // one FP64 sub, mul (x_lane: this lane's coordinate, loaded ahead by the caller)
-        const double xd = (lane < d) ? ((have_x ? x_lane : x[i * d + lane]) - cj) * inv2R : 0.0;
-        const float xf = (float)xd;
-#pragma unroll
-        for (int j = 0; j < kMaxD; ++j) {
-            const float v = __shfl_sync(0xffffffffu, xf, j);      // zero for j >= d
-            xh[j] = v;
-            s += v * v;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < kMaxD; ++j) {
-            xh[j] = (j < d) ? (T)((x[i * d + j] - cen.c[j]) * inv2R) : (T)0;
+    for (int j = 0; j < kMaxD; ++j) {
+        if (sizeof(T) == 4 || j < d) {
+            xh[j] = __shfl_sync(0xffffffffu, xt, j, GL);          // zero for j >= d
             s += xh[j] * xh[j];
+        } else {
+            xh[j] = (T)0;
         }
     }
     if (s > (T)0) {
         const T inv = (T)1 / sqrt(s);
 #pragma unroll
-        for (int j = 0; j < kMaxD; ++j) xh[j] *= inv;
+        for (int j = 0; j < kMaxD; ++j)
+            if (sizeof(T) == 4 || j < d) xh[j] *= inv;
     } else {
 #pragma unroll
         for (int j = 0; j < kMaxD; ++j) xh[j] = (j == 0) ? (T)1 : (T)0;
@@ -782,7 +785,7 @@ __device__ __forceinline__ void point_direction(const double* __restrict__ x, in
 }
 
 // Level table j (j < levels) of the normalised three-term recurrences, lanes over mu'.
-template <typename T>
+template <typename T, int GL>
 __device__ __forceinline__ void level_table(const T* xh, int d, int j, int L, int tri, const T* cA, const T* cB, T* tb,
                                             int lane) {
     const int D = d - 1 - j;
@@ -795,7 +798,7 @@ __device__ __forceinline__ void level_table(const T* xh, int d, int j, int L, in
     const T qq = q;
     const T* A = cA + j * tri;
     const T* B = cB + j * tri;
-    for (int mu = lane; mu <= L; mu += 32) {
+    for (int mu = lane; mu <= L; mu += GL) {
         const int o = mu * (L + 1) - mu * (mu - 1) / 2;
         const int nmax = L - mu;
         T pm2 = A[o];
@@ -813,35 +816,67 @@ __device__ __forceinline__ void level_table(const T* xh, int d, int j, int L, in
     }
 }
 
-// (x0 + i x1)^mu by binary powering in the bulk precision.
-template <typename T>
-__device__ __forceinline__ void trig_power(T x0, T x1, int mu, T& re, T& im) {
-    T br = x0, bi = x1, rr = (T)1, ri = (T)0;
-    int e = mu;
-    while (e) {
-        if (e & 1) { const T t = rr * br - ri * bi; ri = rr * bi + ri * br; rr = t; }
-        const T t = br * br - bi * bi; bi = (T)2 * br * bi; br = t;
-        e >>= 1;
+// Powers (x0 + i x1)^m for the exponents m = lane, lane + GL, .. <= L of a group's lanes.  FP64: a scan
+// of products over the lanes, five steps at most, then a factor per GL exponents; binary powering
+// takes a product and a square per step and an FP64 instruction holds its pipe for 16 cycles (200,000
+// points, d = 3, rank 66 with this and the shared direction: 1.39 -> 1.08 ms).  FP32: binary
+// powering (the scan's shuffles made rows 2 to 5% slower).
+template <typename T, int GL> struct TrigPowers {
+    T x0, x1, re, im, sr, si;
+    __device__ __forceinline__ TrigPowers(T a, T b, int L, int lane) : x0(a), x1(b) {
+        if constexpr (sizeof(T) == 8) {
+            re = lane ? a : (T)1;
+            im = lane ? b : (T)0;
+#pragma unroll
+            for (int off = 1; off < GL; off <<= 1) {
+                if (off > L) break;
+                const T ur = __shfl_up_sync(0xffffffffu, re, off, GL), ui = __shfl_up_sync(0xffffffffu, im, off, GL);
+                const T t = re * ur - im * ui, v = re * ui + im * ur;
+                if (lane >= off) { re = t; im = v; }
+            }
+            if (L >= GL) {
+                const T r = __shfl_sync(0xffffffffu, re, GL - 1, GL), i = __shfl_sync(0xffffffffu, im, GL - 1, GL);
+                sr = r * a - i * b;
+                si = r * b + i * a;
+            }
+        }
     }
-    re = rr;
-    im = ri;
-}
+    // the power m; FP64: called for m = lane, lane + GL, .. in turn
+    __device__ __forceinline__ void get(int m, T& rr, T& ri) {
+        if constexpr (sizeof(T) == 8) {
+            if (m >= GL) { const T t = re * sr - im * si; im = re * si + im * sr; re = t; }
+            rr = re;
+            ri = im;
+        } else {
+            T br = x0, bi = x1;
+            rr = (T)1;
+            ri = (T)0;
+            for (int e = m; e; e >>= 1) {
+                if (e & 1) { const T t = rr * br - ri * bi; ri = rr * bi + ri * br; rr = t; }
+                const T t = br * br - bi * bi;
+                bi = (T)2 * br * bi;
+                br = t;
+            }
+        }
+    }
+};
 
 // The direction of point i, then the level tables (levels x tri, lanes over mu') and the
 // trigonometric powers (x0 + i x1)^mu times the normalisers (2L+1, index L + mu), written by one
 // warp into its shared tbl and trig.
 template <typename T>
-__device__ __forceinline__ void point_harmonic_tables(const double* __restrict__ x, int d, const Center& cen,
+__device__ __forceinline__ void point_harmonic_tables(const double* __restrict__ x, int d, double cj,
                                                       double inv2R, int L, int tri, const T* cA, const T* cB,
                                                       T* tbl, T* trig, int64_t i, int lane, bool have_x = false,
                                                       double x_lane = 0.0) {
     const int levels = d - 2;
     T xh[kMaxD];
-    point_direction<T>(x, d, cen, inv2R, i, lane, have_x, x_lane, xh);
-    for (int j = 0; j < levels; ++j) level_table<T>(xh, d, j, L, tri, cA, cB, tbl + j * tri, lane);
+    point_direction<T, 32>(x, d, cj, inv2R, i, lane, have_x, x_lane, xh);
+    for (int j = 0; j < levels; ++j) level_table<T, 32>(xh, d, j, L, tri, cA, cB, tbl + j * tri, lane);
+    TrigPowers<T, 32> pw(xh[0], xh[1], L, lane);
     for (int mu = lane; mu <= L; mu += 32) {
         T rr, ri;
-        trig_power<T>(xh[0], xh[1], mu, rr, ri);
+        pw.get(mu, rr, ri);
         if (mu == 0) {
             trig[L] = (T)0.3989422804014327;             // 1/sqrt(2 pi)
         } else {
@@ -874,30 +909,27 @@ __device__ __forceinline__ T slot_product(const uint32_t* ydesc, uint32_t y, int
 // pass over the chains (two or more index words and as many factors per harmonic), the harmonics
 // took more than half of the instructions of a row at some hundred columns.  slots = false stops at
 // the prefix levels and G.
-template <typename T>
-__device__ __forceinline__ void point_harmonics(const double* __restrict__ x, int d, const Center& cen, double inv2R,
-                                                int L, int tri, const T* cA, const T* cB, const int32_t* gbase,
+template <typename T, int GL>
+__device__ __forceinline__ void point_harmonics(const double* __restrict__ x, int d, double cj, double inv2R, int L,
+                                                int tri, const T* cA, const T* cB, const int32_t* gbase,
                                                 const uint32_t* ydesc, int nYp, T* Ys, T* Pl, T* G, int64_t i, int lane,
                                                 bool have_x, double x_lane, bool slots) {
     const int levels = d - 2;
     T xh[kMaxD];
-    point_direction<T>(x, d, cen, inv2R, i, lane, have_x, x_lane, xh);
-    for (int j = 0; j < levels - 1; ++j) level_table<T>(xh, d, j, L, tri, cA, cB, Pl + j * tri, lane);
+    point_direction<T, GL>(x, d, cj, inv2R, i, lane, have_x, x_lane, xh);
+    for (int j = 0; j < levels - 1; ++j) level_table<T, GL>(xh, d, j, L, tri, cA, cB, Pl + j * tri, lane);
     const T z = xh[2], qq = xh[0] * xh[0] + xh[1] * xh[1] + xh[2] * xh[2];
     const T* A = cA + (levels - 1) * tri;
     const T* B = cB + (levels - 1) * tri;
-    for (int m = lane; m <= L; m += 32) {
+    TrigPowers<T, GL> pw(xh[0], xh[1], L, lane);
+    for (int m = lane; m <= L; m += GL) {
         T rr, ri;
-        trig_power<T>(xh[0], xh[1], m, rr, ri);
+        pw.get(m, rr, ri);
         rr *= m == 0 ? (T)0.3989422804014327 : (T)0.5641895835477563;    // 1/sqrt(2 pi), 1/sqrt(pi)
         ri *= (T)0.5641895835477563;
         const T* a = A + m * (L + 1) - m * (m - 1) / 2 - m;              // indexed by mu = m + n
         const T* b = B + (a - A);
-        T p1 = (T)0, p2 = (T)0;
-        for (int mu = m; mu <= L; ++mu) {
-            const T v = mu == m ? a[mu] : mu == m + 1 ? a[mu] * z : a[mu] * z * p1 - b[mu] * qq * p2;
-            p2 = p1;
-            p1 = v;
+        auto put = [&](int mu, T v) {
             if (levels == 1) {
                 const int g = gbase[mu];
                 if (g >= 0) {
@@ -909,11 +941,23 @@ __device__ __forceinline__ void point_harmonics(const double* __restrict__ x, in
                 g[m] = v * rr;
                 if (m > 0) g[-m] = v * ri;
             }
+        };
+        T p2 = a[m];
+        put(m, p2);
+        if (m == L) continue;
+        T p1 = a[m + 1] * z;
+        put(m + 1, p1);
+#pragma unroll 2
+        for (int mu = m + 2; mu <= L; ++mu) {
+            const T v = a[mu] * z * p1 - b[mu] * qq * p2;
+            put(mu, v);
+            p2 = p1;
+            p1 = v;
         }
     }
     if (levels == 1 || !slots) return;
     __syncwarp();
-    for (int y = lane; y < nYp; y += 32) Ys[y] = slot_product<T>(ydesc, y, levels, Pl, G);
+    for (int y = lane; y < nYp; y += GL) Ys[y] = slot_product<T>(ydesc, y, levels, Pl, G);
 }
 
 // One point's U row, executed by one warp.  cA/cB: level recurrences in shared memory;
@@ -933,27 +977,27 @@ __device__ __forceinline__ T* uwriter_fs(const UWParams& P, int mode, T* base) {
 }
 
 // Radial factors and coordinate of one point loaded into registers one point ahead of use (FP32
-// factors with nF <= 32 kPfF): lane l holds F[i, l + 32 k] and x[i, l] (l < d), so that their
+// factors with nF <= GL kPfF): lane l holds F[i, l + GL k] and x[i, l] (l < d), so that their
 // global-memory latency passes while the previous row is written.
 constexpr int kPfF = 16;
 template <typename T> struct PointPre { T f[kPfF]; double x; };
-template <typename T>
+template <typename T, int GL>
 __device__ __forceinline__ void point_prefetch(const UWParams& P, int64_t i, int lane, PointPre<T>& pp) {
     const T* Fg = reinterpret_cast<const T*>(P.F) + i * P.ldF;
 #pragma unroll
     for (int k = 0; k < kPfF; ++k) {
-        if (32 * k >= P.nF) break;
-        const int f = lane + 32 * k;
+        if (GL * k >= P.nF) break;
+        const int f = lane + GL * k;
         pp.f[k] = (f < P.nF) ? Fg[f] : (T)0;
     }
     pp.x = (lane < P.d) ? P.x[i * P.d + lane] : 0.0;
 }
-template <typename T>
+template <typename T, int GL>
 __device__ __forceinline__ void point_stage_f(const UWParams& P, const PointPre<T>& pp, T* Fs, int lane) {
 #pragma unroll
     for (int k = 0; k < kPfF; ++k) {
-        if (32 * k >= P.nF) break;
-        const int f = lane + 32 * k;
+        if (GL * k >= P.nF) break;
+        const int f = lane + GL * k;
         if (f < P.nF) Fs[f] = pp.f[k];
     }
 }
@@ -969,9 +1013,9 @@ __device__ __forceinline__ uint32_t uwriter_column(const uint32_t* qdesc, int64_
     return (w1 & 0xFFF00000u) | ((w1 & 0xFFFFFu) + u - e);
 }
 
-template <typename T, int MODE, int DESC>
-__device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X, int64_t i, const T* cA, const T* cB,
-                                              T* base, int lane, bool staged = false, double x_lane = 0.0) {
+template <typename T, int MODE, int DESC, int GL>
+__device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X, double cj, int64_t i, bool valid,
+                                              const T* cA, const T* cB, T* base, int lane, bool staged = false, double x_lane = 0.0) {
     const int levels = P.d - 2;
     T* Ys = base;                                            // nYp (kSlots)
     T* Pl = base + (MODE == kSlots ? P.nYp : 0);             // (levels - 1) * tri
@@ -981,13 +1025,13 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
     T* Fs = uwriter_fs<T>(P, MODE, base);                    // nF + 1
     const T* Fg = reinterpret_cast<const T*>(P.F);
     if (MODE != kChains)
-        point_harmonics<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, X.gbase, X.ydesc, P.nYp, Ys, Pl, G, i, lane,
+        point_harmonics<T, GL>(P.x, P.d, cj, P.inv2R, P.L, P.tri, cA, cB, X.gbase, X.ydesc, P.nYp, Ys, Pl, G, i, lane,
                            staged, x_lane, MODE == kSlots);
     else
-        point_harmonic_tables<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane, staged, x_lane);
+        point_harmonic_tables<T>(P.x, P.d, cj, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane, staged, x_lane);
     // this point's radial factors (staged: already in Fs, written by the caller)
     if (!staged) {
-        for (int f = lane; f < P.nF; f += 32) Fs[f] = Fg[i * P.ldF + f];
+        for (int f = lane; f < P.nF; f += GL) Fs[f] = Fg[i * P.ldF + f];
         if (lane == 0) Fs[P.nF] = (T)0;
     }
     __syncwarp();
@@ -1028,16 +1072,20 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
             return out;
         };
         VT* rq = reinterpret_cast<VT*>(row);
-        const int64_t nq = P.ldU / VW;
+        const int64_t nq = valid ? P.ldU / VW : 0;
         int64_t q = lane;
-        for (; q + 32 * (NQ - 1) < nq; q += 32 * NQ) {
-            VT o[NQ];
+        auto batch = [&](auto cnt) {
+            constexpr int N = decltype(cnt)::value;
+            VT o[N];
 #pragma unroll
-            for (int f = 0; f < NQ; ++f) o[f] = chunk(q + 32 * f);
+            for (int f = 0; f < N; ++f) o[f] = chunk(q + GL * f);
 #pragma unroll
-            for (int f = 0; f < NQ; ++f) rq[q + 32 * f] = o[f];
-        }
-        for (; q < nq; q += 32) rq[q] = chunk(q);
+            for (int f = 0; f < N; ++f) rq[q + GL * f] = o[f];
+            q += GL * N;
+        };
+        while (q + GL * (NQ - 1) < nq) batch(Count<NQ>());
+        if (NQ > 2 && q + GL < nq) batch(Count<2>());
+        while (q < nq) batch(Count<1>());
         __syncwarp();
         return;
     }
@@ -1056,22 +1104,19 @@ __device__ __forceinline__ void uwriter_point(const UWParams& P, const UWTabs& X
 
 // Zeroes a warp's harmonic slots and G's last entry once (padding slots of d = 3 and that entry are
 // never written afterwards).
-template <typename T, int MODE>
+template <typename T, int MODE, int GL>
 __device__ __forceinline__ void uwriter_zero_slots(const UWParams& P, T* base, int lane) {
     if (MODE == kSlots)
-        for (int g = lane; g < P.nYp; g += 32) base[g] = (T)0;
+        for (int g = lane; g < P.nYp; g += GL) base[g] = (T)0;
     if (MODE != kChains && P.d > 3 && lane == 0) uwriter_fs<T>(P, MODE, base)[-1] = (T)0;
     __syncwarp();
 }
 
-// Shared memory: [nwarps x per_warp elements][cA][cB][staged index tables (tab_bytes)].
-template <typename T, int MODE, bool PF, int DESC>
-__global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+// Stages a set's coefficient tables (cA, cB: 2 levels tri elements) and, from `tp` on, its index
+// tables (uwriter_tab_bytes) into shared memory; the caller synchronises.
+template <typename T, int MODE, int DESC>
+__device__ __forceinline__ UWTabs uwriter_stage(const UWParams& P, T* cA, unsigned char* tp) {
     const int levels = P.d - 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    T* base = reinterpret_cast<T*>(smem_raw) + (size_t)warp * P.per_warp;
-    T* cA = reinterpret_cast<T*>(smem_raw) + (size_t)nwarps * P.per_warp;
     T* cB = cA + levels * P.tri;
     for (int idx = threadIdx.x; idx < levels * P.tri; idx += blockDim.x) {
         cA[idx] = reinterpret_cast<const T*>(P.coefA)[idx];
@@ -1081,8 +1126,6 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
     if constexpr (DESC != kGlobal) {
         // staged in shared memory (a compile-time choice, so that the table reads compile to
         // shared-memory loads)
-        unsigned char* tp = reinterpret_cast<unsigned char*>(smem_raw) +
-                            align16(sizeof(T) * ((size_t)nwarps * P.per_warp + 2 * (size_t)levels * P.tri));
         uint32_t* q = reinterpret_cast<uint32_t*>(tp);
         if constexpr (DESC == kColumns) {
             for (int64_t k = threadIdx.x; k < P.ldU; k += blockDim.x) q[k] = uwriter_column<Vec16<T>::w>(P.qdesc, k);
@@ -1112,24 +1155,56 @@ __global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
             X.ychain = yc;
         }
     }
-    __syncthreads();
-    uwriter_zero_slots<T, MODE>(P, base, lane);
-    const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
+    return X;
+}
+
+// The rows of a warp, 32 / GL points at a time, GL lanes each: points i, i + 1, .. (one per group), then
+// i + step, .., below end.  wbase: the warp's area, an equal part per group.  PF: the next point's
+// radial factors and coordinate travel in registers during this row (nF <= GL kPfF).  Groups of 16 or
+// 8 lanes are for degrees below 16 or 8, where the rest of the warp has no recurrence of its own and
+// a warp's instructions, bound by their issue, serve two or four points: 200,000 points, d = 3, FP32 rank
+// 322 0.182 -> 0.106 ms, FP64 rank 66 1.08 -> 0.30 and rank 490 1.83 -> 1.03.
+template <typename T, int MODE, bool PF, int DESC, int GL>
+__device__ __forceinline__ void uwriter_rows(const UWParams& P, const UWTabs& X, const T* cA, const T* cB, T* wbase,
+                                             int64_t i, int64_t step, int64_t end) {
+    const int lane = threadIdx.x & (GL - 1), group = (threadIdx.x & 31) / GL;
+    T* base = wbase + (size_t)group * (P.per_warp / (32 / GL));
+    uwriter_zero_slots<T, MODE, GL>(P, base, lane);
+    const double cj = lane_centre(P.c, lane);
     if constexpr (PF) {
-        // PF: the next point's radial factors and coordinate travel in registers during this row
         T* Fs = uwriter_fs<T>(P, MODE, base);
         if (lane == 0) Fs[P.nF] = (T)0;
         PointPre<T> pp;
-        if (gw < P.n) point_prefetch<T>(P, gw, lane, pp);
-        for (int64_t i = gw; i < P.n; i += nw) {
-            point_stage_f<T>(P, pp, Fs, lane);
+        if (i < end) point_prefetch<T, GL>(P, min(i + group, end - 1), lane, pp);
+        for (; i < end; i += step) {
+            point_stage_f<T, GL>(P, pp, Fs, lane);
             const double xl = pp.x;
-            if (i + nw < P.n) point_prefetch<T>(P, i + nw, lane, pp);
-            uwriter_point<T, MODE, DESC>(P, X, i, cA, cB, base, lane, true, xl);
+            if (i + step < end) point_prefetch<T, GL>(P, min(i + step + group, end - 1), lane, pp);
+            uwriter_point<T, MODE, DESC, GL>(P, X, cj, min(i + group, end - 1), i + group < end, cA, cB, base, lane, true, xl);
         }
     } else {
-        for (int64_t i = gw; i < P.n; i += nw) uwriter_point<T, MODE, DESC>(P, X, i, cA, cB, base, lane);
+        for (; i < end; i += step)
+            uwriter_point<T, MODE, DESC, GL>(P, X, cj, min(i + group, end - 1), i + group < end, cA, cB, base, lane);
     }
+}
+
+// Shared memory: [nwarps x per_warp elements][cA][cB][staged index tables (tab_bytes)].
+template <typename T>
+__device__ __forceinline__ unsigned char* uwriter_tabs_at(const UWParams& P, unsigned char* smem, int nwarps) {
+    return smem + align16(sizeof(T) * ((size_t)nwarps * P.per_warp + 2 * (size_t)(P.d - 2) * P.tri));
+}
+
+template <typename T, int MODE, bool PF, int DESC, int GL>
+__global__ void __launch_bounds__(1024) k_uwriter(UWParams P) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    T* base = reinterpret_cast<T*>(smem_raw) + (size_t)warp * P.per_warp;
+    T* cA = reinterpret_cast<T*>(smem_raw) + (size_t)nwarps * P.per_warp;
+    const UWTabs X = uwriter_stage<T, MODE, DESC>(P, cA, uwriter_tabs_at<T>(P, smem_raw, nwarps));
+    __syncthreads();
+    constexpr int G = 32 / GL;
+    uwriter_rows<T, MODE, PF, DESC, GL>(P, X, cA, cA + (P.d - 2) * P.tri, base,
+                                        ((int64_t)blockIdx.x * nwarps + warp) * G, (int64_t)gridDim.x * nwarps * G, P.n);
 }
 
 // --------------------------------------------------------------------- A7: matvec

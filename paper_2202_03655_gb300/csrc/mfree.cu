@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(1024) k_zwriter(ZWParams P) {
     const int tl = levels - 1;           // position of the trig index in a tail chain
     const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
     for (int64_t i = gw; i < P.n; i += nw) {
-        point_harmonic_tables<T>(P.x, P.d, P.c, P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane);
+        point_harmonic_tables<T>(P.x, P.d, lane_centre(P.c, lane), P.inv2R, P.L, P.tri, cA, cB, tbl, trig, i, lane);
         for (int f = lane; f < P.nF; f += 32) Fs[f] = Fg[i * P.ldF + f];
         T* zr = reinterpret_cast<T*>(P.Z) + i * (int64_t)P.ldZ;
         if (pairs) {

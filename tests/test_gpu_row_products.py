@@ -62,3 +62,29 @@ def test_batched_row_products(precision):
         # entries of K~ are below 2 and the rows of U S U^T hold them as sums of like magnitude
         slack = (0.0 if precision == "fp64" else 1024 * 2.0 ** -24 * sizes[s])
         assert np.linalg.norm(Y[q] - K @ V[q]) <= (tol * np.linalg.norm(K) + slack) * np.linalg.norm(V[q])
+
+
+# degrees below 8, 8 to 15 and above (groups of 8, 16 and 32 lanes per point), with points that leave
+# groups of the last warp without one
+@pytest.mark.parametrize("d,ell,tol,lo,hi", [(3, 2.0, 1e-6, 1, 8), (3, 0.6, 1e-6, 8, 16), (3, 0.2, 1e-6, 16, 33),
+                                             (4, 1.0, 1e-4, 1, 8), (4, 0.5, 1e-5, 8, 16), (5, 0.6, 1e-3, 1, 16),
+                                             (8, 2.0, 1e-2, 1, 8)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [1, 2, 5, 67])
+def test_lane_groups(d, ell, tol, lo, hi, precision, n):
+    from paper_2202_03655_gb300 import hdf
+    g = np.random.default_rng(10 * d + n)
+    x = g.random((n, d))
+    x *= np.sqrt(3.0 / d)
+    if n > 3:
+        x[2, 2:] = x[3, 2:]
+    f = hdf.build(to_dev(x), "gaussian", ell, tol, precision=precision)
+    if n == 67:
+        assert lo <= max(k for k, s in enumerate(f.s_k) if s) < hi
+    V = g.standard_normal((n, 2))
+    vt = to_dev(V) if precision == "fp64" else to_dev(V).float()
+    check(f, x, ell, tol, 2.0 ** (-53 if precision == "fp64" else -24), V, f.matvec(vt).double().cpu().numpy())
+    b = hdf.build_batched(to_dev(np.concatenate([x, x])), [0, n, 2 * n], "gaussian", [ell, ell], tol, precision=precision)
+    Y = b.matvec(to_dev(np.concatenate([V, V])).to(vt.dtype)).double().cpu().numpy()
+    check(f, x, ell, tol, 2.0 ** (-53 if precision == "fp64" else -24), V, Y[:n])
+    assert np.array_equal(Y[:n], Y[n:])
