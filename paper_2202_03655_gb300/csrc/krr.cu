@@ -201,25 +201,37 @@ void launch_direct(int d, dim3 g, cudaStream_t st, const float* a, int64_t m, co
 #undef HDF_DK
 }
 
-// The off-diagonal blocks of K^ stored once: M[j ldk + i] = the FP32 value that k_direct_kernel
-// forms for the pair (i, j), zero within a cluster and in the padding columns.  A conjugate-gradient
-// solve applies the same matrix hundreds of times, and forming a value (d differences, a square
-// root, an exponential) costs several times the 4 bytes of reading it: 13,760 points, d = 8, one
-// product 0.43 ms evaluated, 0.12 ms stored (6.3 TB/s), 0.29 ms to store.
-constexpr int kOffTile = 64;         // columns j per block of k_off_store
-constexpr int kOffRows = 1024;       // rows i per block (four per thread)
+// The off-diagonal blocks of K^ stored once, each pair {i, j} in one place: tiles of kTI points i and
+// kTJ points j that meet j < i, tile (ib, jb) as [j][i] at index 2 ib (ib + 1) + jb, jb < 4 (ib + 1); the
+// FP32 value that k_direct_kernel forms for the pair, zero within a cluster, for j >= i and in the
+// padding.  A conjugate-gradient solve applies the same matrix hundreds of times, and forming a value
+// (d differences, a square root, an exponential) costs several times the bytes of reading it: 13,760
+// points, d = 8, one product 0.43 ms evaluated, 0.12 ms from the full matrix,
+// 0.095 from these tiles; 0.19 ms to store them.
+constexpr int kTI = 512, kTJ = 128, kTPart = kTI + kTJ;
+static __host__ __device__ int64_t off_tiles(int64_t n) {
+    const int64_t nb = (n + kTI - 1) / kTI;
+    return 2 * nb * (nb + 1);
+}
+// The tile at index t.
+__device__ __forceinline__ void off_tile(int64_t t, int64_t& ib, int64_t& jb) {
+    ib = (int64_t)((sqrt(1.0 + 2.0 * (double)t) - 1.0) * 0.5);
+    while (2 * ib * (ib + 1) > t) --ib;
+    while (2 * (ib + 1) * (ib + 2) <= t) ++ib;
+    jb = t - 2 * ib * (ib + 1);
+}
 template <int DD>
-__global__ void __launch_bounds__(256) k_off_store(const float* __restrict__ a, int64_t n, int64_t ldk, int kernel,
-                                                   float inv_ell, const int* __restrict__ cl, float* __restrict__ M) {
-    __shared__ float bs[kOffTile][DD];
-    __shared__ int cs[kOffTile];
-    const int64_t j0 = blockIdx.y * (int64_t)kOffTile;
-    const int nt = (int)min((int64_t)kOffTile, n - j0);
-    for (int e = threadIdx.x; e < nt * DD; e += 256) bs[e / DD][e % DD] = a[j0 * DD + e];
-    for (int e = threadIdx.x; e < nt; e += 256) cs[e] = cl[j0 + e];
+__global__ void __launch_bounds__(128) k_off_store(const float* __restrict__ a, int64_t n, int kernel, float inv_ell,
+                                                   const int* __restrict__ cl, float* __restrict__ M) {
+    __shared__ float bs[kTJ][DD];
+    __shared__ int cs[kTJ];
+    int64_t ib, jb;
+    off_tile(blockIdx.x, ib, jb);
+    const int64_t j0 = jb * kTJ, i = ib * kTI + 4 * threadIdx.x;
+    const int nt = (int)max((int64_t)0, min((int64_t)kTJ, n - j0));
+    for (int e = threadIdx.x; e < nt * DD; e += 128) bs[e / DD][e % DD] = a[j0 * DD + e];
+    for (int e = threadIdx.x; e < nt; e += 128) cs[e] = cl[j0 + e];
     __syncthreads();
-    const int64_t i = blockIdx.x * (int64_t)kOffRows + 4 * threadIdx.x;
-    if (i >= ldk) return;
     float ai[4][DD];
     int ci[4];
 #pragma unroll
@@ -229,89 +241,220 @@ __global__ void __launch_bounds__(256) k_off_store(const float* __restrict__ a, 
         for (int e = 0; e < DD; ++e) ai[u][e] = a[q * DD + e];
         ci[u] = i + u < n ? cl[q] : -1;
     }
-    for (int r = 0; r < nt; ++r) {
-        float kv[4];
+    float* Mt = M + (int64_t)blockIdx.x * kTI * kTJ + 4 * threadIdx.x;
+    for (int r = 0; r < kTJ; ++r) {
+        float kv[4] = {0.f, 0.f, 0.f, 0.f};
+        if (r < nt && j0 + r < i + 3) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            float s = 0.f;
+            for (int u = 0; u < 4; ++u) {
+                float s = 0.f;
 #pragma unroll
-            for (int q = 0; q < DD; ++q) { const float t = ai[u][q] - bs[r][q]; s = fmaf(t, t, s); }
-            kv[u] = dev::kernel_value_f(kernel, sqrtf(s), inv_ell);
-            if (ci[u] == cs[r] || ci[u] < 0) kv[u] = 0.f;
+                for (int q = 0; q < DD; ++q) { const float t = ai[u][q] - bs[r][q]; s = fmaf(t, t, s); }
+                kv[u] = dev::kernel_value_f(kernel, sqrtf(s), inv_ell);
+                if (ci[u] == cs[r] || ci[u] < 0 || j0 + r >= i + u) kv[u] = 0.f;
+            }
         }
-        *reinterpret_cast<float4*>(M + (j0 + r) * ldk + i) = make_float4(kv[0], kv[1], kv[2], kv[3]);
+        *reinterpret_cast<float4*>(Mt + r * kTI) = make_float4(kv[0], kv[1], kv[2], kv[3]);
     }
 }
-void launch_off_store(int d, cudaStream_t st, const float* a, int64_t n, int64_t ldk, int kernel, float inv_ell,
-                      const int* cl, float* M) {
-    const dim3 g((unsigned)((ldk + kOffRows - 1) / kOffRows), (unsigned)((n + kOffTile - 1) / kOffTile));
-#define HDF_OS(DD) case DD: k_off_store<DD><<<g, 256, 0, st>>>(a, n, ldk, kernel, inv_ell, cl, M); break;
+void launch_off_store(int d, cudaStream_t st, const float* a, int64_t n, int kernel, float inv_ell, const int* cl,
+                      float* M) {
+    const unsigned g = (unsigned)off_tiles(n);
+#define HDF_OS(DD) case DD: k_off_store<DD><<<g, 128, 0, st>>>(a, n, kernel, inv_ell, cl, M); break;
     switch (d) { HDF_OS(1) HDF_OS(2) HDF_OS(3) HDF_OS(4) HDF_OS(5) HDF_OS(6) HDF_OS(7) HDF_OS(8) }
 #undef HDF_OS
 }
 
-// part[s n + i] = sum over the columns j of split s of M[j ldk + i] w_j (M is symmetric, so its rows
-// are read along i, 16 bytes a thread).  The same exact products and FP32-pair sums as
-// k_direct_kernel per 128 columns, added in FP64.  Bound by the read of M.
-constexpr int kOffK = 128;
-__global__ void __launch_bounds__(256) k_off_apply(const float* __restrict__ M, int64_t n, int64_t ldk,
-                                                   const double* __restrict__ w, int64_t split,
-                                                   double* __restrict__ part) {
-    __shared__ float2 ws[kOffK];                 // w_j = hi + lo
-    const int64_t i = blockIdx.x * (int64_t)kOffRows + 4 * threadIdx.x;
-    const bool act = i < ldk;
-    const int64_t j0 = blockIdx.y * split, j1 = min(n, j0 + split);
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int64_t t0 = j0; t0 < j1; t0 += kOffK) {
-        const int nt = (int)min((int64_t)kOffK, j1 - t0);
-        __syncthreads();
-        if (threadIdx.x < nt) {
-            const double wv = w[t0 + threadIdx.x];
-            const float hi = (float)wv;
-            ws[threadIdx.x] = make_float2(hi, (float)(wv - (double)hi));
-        }
-        __syncthreads();
-        if (!act) continue;
-        float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* Mt = M + t0 * ldk + i;
-#pragma unroll 8
-        for (int r = 0; r < nt; ++r) {
-            const float4 kv = __ldcs(reinterpret_cast<const float4*>(Mt + (int64_t)r * ldk));
-            const float2 wr = ws[r];
-            const float k4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float p = k4[u] * wr.x;
-                const float e = fmaf(k4[u], wr.y, fmaf(k4[u], wr.x, -p));    // exact error of p, plus k w_lo
-                float s, t;
-                dev::two_sum(sh[u], p, s, t);
-                sh[u] = s;
-                sl[u] += t + e;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += (double)sh[u] + (double)sl[u];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (i + u < n) part[blockIdx.y * n + i + u] = acc[u];
+// Two FP32 operations per instruction, each rounded to nearest on its own.
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 add2(F2 a, F2 b) { F2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { F2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) { F2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
 }
-// Column splits of k_off_apply: about eight blocks per SM, whole tiles of kOffK columns.
-int64_t off_split(int64_t n, int64_t ldk, int* S) {
-    const int64_t rb = (ldk + kOffRows - 1) / kOffRows, tiles = (n + kOffK - 1) / kOffK;
-    const int64_t s = std::max<int64_t>(1, std::min<int64_t>(8 * 152 / rb, tiles));
-    const int64_t split = (tiles + s - 1) / s * kOffK;
-    *S = (int)((n + split - 1) / split);
-    return split;
+// (sh, sl) += k (wh + wl), k exact: p = k wh with its exact error, TwoSum into sh, the rest into sl;
+// nwh = -wh.
+__device__ __forceinline__ void dot_step2(F2 k, F2 wh, F2 nwh, F2 wl, F2& sh, F2& sl) {
+    const F2 np = mul2(k, nwh);                               // -p
+    const F2 e = fma2(k, wl, fma2(k, wh, np));
+    const F2 s = sub2(sh, np), bb = sub2(s, sh);
+    const F2 t = sub2(sub2(sh, sub2(s, bb)), add2(np, bb));   // (sh - (s - bb)) + (p - bb)
+    sh = s;
+    sl = add2(sl, add2(t, e));
+}
+// The sum of two pairs.
+__device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2) {
+    float s, e;
+    dev::two_sum(h, h2, s, e);
+    h = s;
+    l += e + l2;
 }
 
-// out[i] = alpha v[i] + (add ? add[i] : 0) + sum_s part[s m + i]
-__global__ void k_direct_finish(const double* __restrict__ part, int S, int64_t m, double alpha,
-                                const double* __restrict__ v, const double* __restrict__ add, double* __restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= m) return;
+// Both halves of the product by the tiles: part[t kTPart + i'] = sum_j M[j][i] w_j over the tile's j, and
+// part[t kTPart + kTI + j'] = sum_i M[j][i] w_i over its i.  Every entry is read once and used for both,
+// with exact products and FP32-pair sums (in the order of the tile, the same on every run), two
+// entries per instruction.  A warp takes 32 j, a lane four consecutive i of each 128; the j sums
+// are reduced over the lanes eight at a time, halving their number with each exchange, the i sums over
+// the four warps.  A lane copies the entries that it will use itself, kPieceJ j's ahead, into its own
+// shared memory (with register loads at 12 warps per SM the warps waited for memory 40% of the time,
+// 107 us).  Bound by the read of M (57 us at 13,760 points) and the FP32 pipe (11 operations per entry
+// and side, 58 us).
+constexpr int kPieceJ = 4, kPieces = 32 / kPieceJ;                 // j's per copy, copies per warp and tile
+constexpr size_t kOffSmem = 4 * 2 * (size_t)kPieceJ * kTI * sizeof(float);
+__global__ void __launch_bounds__(128, 2) k_off_apply(const float* __restrict__ M, int64_t n, int64_t ntiles,
+                                                      const double* __restrict__ w, double* __restrict__ part) {
+    extern __shared__ __align__(16) float4 ring[];                 // [warp][2][kPieceJ][4][lane]
+    __shared__ __align__(16) float wih[kTI], win[kTI], wil[kTI];   // w_i = hi + lo, and -hi
+    __shared__ __align__(16) float4 wj[kTJ];                       // (hi, hi, -hi, -hi)
+    __shared__ __align__(16) float2 wjl[kTJ];                      // (lo, lo)
+    __shared__ float2 red[4][kTI];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4* mine = ring + (size_t)warp * 2 * kPieceJ * 128 + lane;
+    auto copy = [&](int64_t t, int p) {
+        if (t < ntiles) {
+            const float* src = M + t * kTI * kTJ + (int64_t)(32 * warp + kPieceJ * p) * kTI + 4 * lane;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(mine + (p & 1) * kPieceJ * 128);
+#pragma unroll
+            for (int e = 0; e < 4 * kPieceJ; ++e)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512u * e), "l"(src + 128 * e) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    copy(blockIdx.x, 0);
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        int64_t ib, jb;
+        off_tile(t, ib, jb);
+        __syncthreads();                                           // the previous tile's w and sums are used up
+        for (int e = threadIdx.x; e < kTI + kTJ; e += 128) {
+            const int64_t q = e < kTI ? ib * kTI + e : jb * kTJ + (e - kTI);
+            const double v = q < n ? w[q] : 0.0;
+            const float hi = (float)v, lo = (float)(v - (double)hi);
+            if (e < kTI) {
+                wih[e] = hi; win[e] = -hi; wil[e] = lo;
+            } else {
+                wj[e - kTI] = make_float4(hi, hi, -hi, -hi);
+                wjl[e - kTI] = make_float2(lo, lo);
+            }
+        }
+        __syncthreads();
+        double* out = part + t * kTPart;
+        F2 hI[4][2], lI[4][2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) hI[k][u] = lI[k][u] = 0ull;
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            F2 hJ[8], lJ[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) hJ[q] = lJ[q] = 0ull;
+#pragma unroll
+            for (int s = 0; s < 8 / kPieceJ; ++s) {
+                const int p = 8 / kPieceJ * g + s;
+                copy(p + 1 < kPieces ? t : t + gridDim.x, (p + 1) % kPieces);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                const float4* st = mine + (s & 1) * kPieceJ * 128;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const ulonglong2 ih = *reinterpret_cast<const ulonglong2*>(wih + 128 * k + 4 * lane);
+                    const ulonglong2 in = *reinterpret_cast<const ulonglong2*>(win + 128 * k + 4 * lane);
+                    const ulonglong2 il = *reinterpret_cast<const ulonglong2*>(wil + 128 * k + 4 * lane);
+#pragma unroll
+                    for (int q = 0; q < kPieceJ; ++q) {
+                        const int j = 32 * warp + kPieceJ * p + q, o = kPieceJ * s + q;
+                        const ulonglong2 jh = *reinterpret_cast<const ulonglong2*>(&wj[j]);
+                        const F2 jl = *reinterpret_cast<const F2*>(&wjl[j]);
+                        const ulonglong2 mm = *reinterpret_cast<const ulonglong2*>(st + (4 * q + k) * 32);
+                        dot_step2(mm.x, jh.x, jh.y, jl, hI[k][0], lI[k][0]);
+                        dot_step2(mm.y, jh.x, jh.y, jl, hI[k][1], lI[k][1]);
+                        dot_step2(mm.x, ih.x, in.x, il.x, hJ[o], lJ[o]);
+                        dot_step2(mm.y, ih.y, in.y, il.y, hJ[o], lJ[o]);
+                    }
+                }
+            }
+            float H[8], L[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float2 h = *reinterpret_cast<const float2*>(&hJ[q]), l = *reinterpret_cast<const float2*>(&lJ[q]);
+                H[q] = h.x;
+                L[q] = l.x;
+                pair_add(H[q], L[q], h.y, l.y);
+            }
+#pragma unroll
+            for (int o = 16, c = 4; o >= 4; o >>= 1, c >>= 1) {
+                const bool up = lane & o;
+#pragma unroll
+                for (int q = 0; q < c; ++q) {
+                    const float sh = up ? H[q] : H[q + c], sl = up ? L[q] : L[q + c];
+                    const float rh = __shfl_xor_sync(0xffffffffu, sh, o), rl = __shfl_xor_sync(0xffffffffu, sl, o);
+                    if (up) { H[q] = H[q + c]; L[q] = L[q + c]; }
+                    pair_add(H[q], L[q], rh, rl);
+                }
+            }
+#pragma unroll
+            for (int o = 2; o >= 1; o >>= 1) {
+                const float rh = __shfl_xor_sync(0xffffffffu, H[0], o), rl = __shfl_xor_sync(0xffffffffu, L[0], o);
+                pair_add(H[0], L[0], rh, rl);
+            }
+            const int q = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+            if ((lane & 3) == 0) out[kTI + 32 * warp + 8 * g + q] = (double)H[0] + (double)L[0];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float2 h = *reinterpret_cast<const float2*>(&hI[k][u]), l = *reinterpret_cast<const float2*>(&lI[k][u]);
+                red[warp][128 * k + 4 * lane + 2 * u] = make_float2(h.x, l.x);
+                red[warp][128 * k + 4 * lane + 2 * u + 1] = make_float2(h.y, l.y);
+            }
+        __syncthreads();
+        for (int e = threadIdx.x; e < kTI; e += 128) {
+            float2 s = red[0][e];
+#pragma unroll
+            for (int v = 1; v < 4; ++v) pair_add(s.x, s.y, red[v][e].x, red[v][e].y);
+            out[e] = (double)s.x + (double)s.y;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// Row i's partial sums: of the tiles (SYM), else of the S column splits; for the threads ty of eight
+// that share the row.
+template <bool SYM>
+__device__ __forceinline__ double part_sum(const double* __restrict__ part, int S, int64_t n, int64_t i, int ty) {
+    double s = 0.0;
+    if (SYM) {
+        const int64_t ib = i / kTI, jb = i / kTJ, nb = (n + kTI - 1) / kTI;
+        const int ni = (int)(4 * (ib + 1)), nt = ni + (int)(nb - ib);
+#pragma unroll 4
+        for (int t = ty; t < nt; t += 8) {
+            const int64_t b = ib + (t - ni);
+            s += part[t < ni ? (2 * ib * (ib + 1) + t) * kTPart + i % kTI : (2 * b * (b + 1) + jb) * kTPart + kTI + i % kTJ];
+        }
+    } else {
+#pragma unroll 4
+        for (int t = ty; t < S; t += 8) s += part[t * n + i];
+    }
+    return s;
+}
+
+// out[i] = alpha v[i] + (add ? add[i] : 0) + the partial sums of row i; 32 rows by 8 parts a block.
+template <bool SYM>
+__global__ void __launch_bounds__(256) k_direct_finish(const double* __restrict__ part, int S, int64_t m, double alpha,
+                                                       const double* __restrict__ v, const double* __restrict__ add,
+                                                       double* __restrict__ out) {
+    __shared__ double sh[8][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + tx;
+    sh[ty][tx] = i < m ? part_sum<SYM>(part, S, m, i, ty) : 0.0;
+    __syncthreads();
+    if (ty || i >= m) return;
     double s = (v ? alpha * v[i] : 0.0) + (add ? add[i] : 0.0);
-    for (int t = 0; t < S; ++t) s += part[t * m + i];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) s += sh[t][tx];
     out[i] = s;
 }
 
@@ -360,8 +503,8 @@ __global__ void k_to_f64(const float* __restrict__ v, int64_t n, double* __restr
 // ----------------------------------------------- conjugate gradients on the device
 // One iteration is a fixed chain of kernels; its scalars live in CgState, so that the host reads
 // the state only every few iterations.  At 13,760 points an iteration went from 0.85 ms (0.43 the
-// off-diagonal blocks, 0.57 + 0.11 the HDF blocks partly hidden, two host round trips) to 0.21 ms.  Iteration it reads rz[it & 1] and writes rz[(it + 1) & 1].  After
-// `done` every kernel returns at once, so iterations enqueued past the end change nothing.  Every
+// off-diagonal blocks, 0.57 + 0.11 the HDF blocks partly hidden, two host round trips) to 0.16 ms.  Iteration it reads
+// rz[it & 1] and writes rz[(it + 1) & 1].  After `done` every kernel returns at once, so iterations enqueued past the end change nothing.  Every
 // block adds the partial sums of a dot product itself, in the same fixed order.
 struct CgState {
     double rz[2];
@@ -390,23 +533,31 @@ __global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ part
     }
 }
 
-// q = lambda p + add + sum_s part[s n + .] and the block's part of p . q.
+// q = lambda p + add + the partial sums, and the part of p . q of the block's 32 rows.  Eight threads
+// share a row's parts (13,760 points: 18 us with one thread per row, 12 so).
+template <bool SYM>
 __global__ void __launch_bounds__(256) k_cg_finish(const double* __restrict__ part, int nsplit, int64_t n, double lam,
                                                    const double* __restrict__ p, const double* __restrict__ add,
                                                    double* __restrict__ q, double* __restrict__ dot,
                                                    const CgState* __restrict__ S) {
-    __shared__ double sh[256];
+    __shared__ double sh[8][32];
     if (S->done) return;
-    const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + tx;
+    sh[ty][tx] = i < n ? part_sum<SYM>(part, nsplit, n, i, ty) : 0.0;
+    __syncthreads();
+    if (ty) return;
     double d = 0.0;
     if (i < n) {
         double s = lam * p[i] + add[i];
-        for (int t = 0; t < nsplit; ++t) s += part[t * n + i];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) s += sh[t][tx];
         q[i] = s;
         d = p[i] * s;
     }
-    const double tot = dev::block_sum_256(d, sh);
-    if (threadIdx.x == 0) dot[blockIdx.x] = tot;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (tx == 0) dot[blockIdx.x] = d;
 }
 
 // alpha = rz / (p . q); x += alpha p; r -= alpha q.
@@ -462,7 +613,8 @@ __global__ void k_block_matrices(const double* __restrict__ xp, int d, const int
 }
 
 // z = M r: one warp per row of the block-diagonal inverse (packed as above), four loads in flight
-// per lane.  With dot (and a state that is not done): (r . z, r . r) of the block's rows as well.
+// per lane (13,760 rows of about 660 entries 31 us, of which the FP64 pipe takes 20; two rows per warp
+// 31, four 36).  With dot (and a state that is not done): (r . z, r . r) of the block's rows as well.
 __global__ void __launch_bounds__(256) k_block_gemv(const double* __restrict__ inv, const int64_t* __restrict__ offs,
                                                     const int64_t* __restrict__ ioff, const int* __restrict__ cl,
                                                     int64_t n, const double* __restrict__ r, double* __restrict__ z,
@@ -757,43 +909,36 @@ struct hdf_krr {
     hdf_batch* batch = nullptr;
     DevBuf vb, yb, hd, part, dotp;       // work: bulk-typed vectors, HDF result, direct-kernel partials
     DevBuf koff;                         // the stored off-diagonal blocks (none: evaluated per product)
-    int64_t ldk = 0;
     DevBuf cgst;                         // CgState of the running solve
     CgState* cgh = nullptr;              // two pinned copies for the host
     cudaEvent_t cgev[2] = {nullptr, nullptr};
+    cudaStream_t side = nullptr;         // the off-diagonal blocks beside the HDF blocks
+    cudaEvent_t fork = nullptr, join = nullptr;
     int S = 1;
     int64_t split = 0;
     double t_build = 0.0, t_precond = 0.0;
     ~hdf_krr() {
         if (batch) hdf_batch_free(batch);
         if (cgh) cudaFreeHost(cgh);
-        for (cudaEvent_t e : cgev) if (e) cudaEventDestroy(e);
+        for (cudaEvent_t e : {cgev[0], cgev[1], fork, join}) if (e) cudaEventDestroy(e);
+        if (side) cudaStreamDestroy(side);
     }
 };
 
 namespace {
 
-// The parts of K^ vp in cluster order (vp FP64, length n): the HDF blocks into K->hd, the splits of
-// the off-diagonal blocks into K->part.
-hdf_status apply_parts(hdf_krr* K, const double* vp, cudaStream_t st) {
+// The off-diagonal blocks times vp into K->part.
+hdf_status apply_off(hdf_krr* K, const double* vp, cudaStream_t st) {
     const int64_t n = K->n;
-    const int gb = blocks_for(n, 256, 1 << 30);
-    hdf_status s;
-    if (K->prec == HDF_FP32) {
-        HDF_COUNT_LAUNCH();
-        k_to_f32<<<gb, 256, 0, st>>>(vp, n, K->vb.as<float>());
-        s = hdf_batch_matvec(K->batch, K->vb.p, n, 1, K->yb.p, n, reinterpret_cast<hdf_stream>(st));
-        if (s != HDF_OK) return s;
-        HDF_COUNT_LAUNCH();
-        k_to_f64<<<gb, 256, 0, st>>>(K->yb.as<float>(), n, K->hd.as<double>());
-    } else {
-        s = hdf_batch_matvec(K->batch, vp, n, 1, K->hd.p, n, reinterpret_cast<hdf_stream>(st));
-        if (s != HDF_OK) return s;
-    }
     HDF_COUNT_LAUNCH();
     if (K->koff.p) {
-        const dim3 g((unsigned)((K->ldk + kOffRows - 1) / kOffRows), (unsigned)K->S);
-        k_off_apply<<<g, 256, 0, st>>>(K->koff.as<float>(), n, K->ldk, vp, K->split, K->part.as<double>());
+        int dv = 0, nsm = 0;
+        HDF_CUDA(cudaGetDevice(&dv));
+        HDF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dv));
+        HDF_CUDA(cudaFuncSetAttribute(k_off_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOffSmem));
+        const int64_t tiles = off_tiles(n);
+        k_off_apply<<<(unsigned)std::min<int64_t>(tiles, 2 * nsm), 128, kOffSmem, st>>>(K->koff.as<float>(), n, tiles, vp,
+                                                                                       K->part.as<double>());
     } else {
         dim3 g((unsigned)((n + kDkRows - 1) / kDkRows), (unsigned)K->S);
         launch_direct(K->d, g, st, K->xp32.as<float>(), n, K->xp32.as<float>(), n, K->kernel, (float)(1.0 / K->ell),
@@ -803,12 +948,43 @@ hdf_status apply_parts(hdf_krr* K, const double* vp, cudaStream_t st) {
     return HDF_OK;
 }
 
+// The diagonal blocks (HDF) times vp into K->hd.
+hdf_status apply_diag(hdf_krr* K, const double* vp, cudaStream_t st) {
+    const int64_t n = K->n;
+    if (K->prec != HDF_FP32)
+        return hdf_batch_matvec(K->batch, vp, n, 1, K->hd.p, n, reinterpret_cast<hdf_stream>(st));
+    const int gb = blocks_for(n, 256, 1 << 30);
+    HDF_COUNT_LAUNCH();
+    k_to_f32<<<gb, 256, 0, st>>>(vp, n, K->vb.as<float>());
+    if (hdf_status s = hdf_batch_matvec(K->batch, K->vb.p, n, 1, K->yb.p, n, reinterpret_cast<hdf_stream>(st)); s != HDF_OK)
+        return s;
+    HDF_COUNT_LAUNCH();
+    k_to_f64<<<gb, 256, 0, st>>>(K->yb.as<float>(), n, K->hd.as<double>());
+    HDF_CUDA(cudaGetLastError());
+    return HDF_OK;
+}
+
+// The parts of K^ vp in cluster order (vp FP64, length n): the HDF blocks into K->hd, the partial sums
+// of the off-diagonal blocks into K->part, side by side (the HDF blocks' two kernels wait for memory
+// most of their 24 us at 13,760 points, the off-diagonal one for the FP32 pipe: 383 iterations 9 ms
+// less than one after the other).
+hdf_status apply_parts(hdf_krr* K, const double* vp, cudaStream_t st) {
+    HDF_CUDA(cudaEventRecord(K->fork, st));
+    HDF_CUDA(cudaStreamWaitEvent(K->side, K->fork, 0));
+    const hdf_status so = apply_off(K, vp, K->side);
+    const hdf_status sd = so == HDF_OK ? apply_diag(K, vp, st) : so;
+    HDF_CUDA(cudaEventRecord(K->join, K->side));
+    HDF_CUDA(cudaStreamWaitEvent(st, K->join, 0));
+    return sd;
+}
+
 // tp = lambda vp + K^ vp in cluster order (vp, tp length n, FP64, device)
 hdf_status apply_perm(hdf_krr* K, const double* vp, double* tp, cudaStream_t st) {
     if (hdf_status s = apply_parts(K, vp, st); s != HDF_OK) return s;
     HDF_COUNT_LAUNCH();
-    k_direct_finish<<<blocks_for(K->n, 256, 1 << 30), 256, 0, st>>>(K->part.as<double>(), K->S, K->n, K->lam, vp,
-                                                                    K->hd.as<double>(), tp);
+    auto finish = K->koff.p ? k_direct_finish<true> : k_direct_finish<false>;
+    finish<<<blocks_for(K->n, 32, 1 << 30), 256, 0, st>>>(K->part.as<double>(), K->S, K->n, K->lam, vp,
+                                                         K->hd.as<double>(), tp);
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
@@ -892,7 +1068,7 @@ hdf_status hdf_kernel_matvec(const double* xq_dev, int64_t m, const double* x_de
     launch_direct(d, g, st, a.as<float>(), m, b.as<float>(), n, kernel, (float)(1.0 / lengthscale), w_dev, nullptr,
                   nullptr, split, part.as<double>());
     HDF_COUNT_LAUNCH();
-    k_direct_finish<<<blocks_for(m, 256, 1 << 30), 256, 0, st>>>(part.as<double>(), S, m, 0.0, nullptr, nullptr,
+    k_direct_finish<false><<<blocks_for(m, 32, 1 << 30), 256, 0, st>>>(part.as<double>(), S, m, 0.0, nullptr, nullptr,
                                                                  out_dev);
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
@@ -1032,26 +1208,28 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         if (hbad) return bail(fail(HDF_ESINGULAR, "hdf_krr_build: a block lambda I + K_cc is not positive definite"));
     }
     // work space
-    // the off-diagonal blocks are stored while they take at most 8 GiB (46,000 points) and the
+    // the off-diagonal blocks are stored while they take at most 8 GiB (65,000 points) and the
     // device has room; else every product evaluates them
-    K->ldk = (n + 3) / 4 * 4;
-    const size_t kbytes = sizeof(float) * (size_t)n * K->ldk;
+    const size_t kbytes = sizeof(float) * (size_t)off_tiles(n) * kTI * kTJ;
+    size_t nparts = (size_t)off_tiles(n) * kTPart;
     if (kbytes <= ((size_t)8 << 30) && K->koff.alloc_on(kbytes, st) == cudaSuccess) {
         HDF_COUNT_LAUNCH();
-        launch_off_store(d, st, K->xp32.as<float>(), n, K->ldk, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
+        launch_off_store(d, st, K->xp32.as<float>(), n, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
                          K->koff.as<float>());
         KRR_CUDA(cudaGetLastError());
-        K->split = off_split(n, K->ldk, &K->S);
     } else {
         cudaGetLastError();
         K->split = direct_split(n, n, &K->S);
+        nparts = (size_t)K->S * n;
     }
-    KRR_CUDA(K->part.alloc(sizeof(double) * (size_t)K->S * n));
+    KRR_CUDA(K->part.alloc(sizeof(double) * nparts));
     KRR_CUDA(K->hd.alloc(sizeof(double) * n));
     KRR_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
     KRR_CUDA(K->cgst.alloc(sizeof(CgState)));
     KRR_CUDA(cudaMallocHost(reinterpret_cast<void**>(&K->cgh), 2 * sizeof(CgState)));
-    for (cudaEvent_t& e : K->cgev) KRR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    for (cudaEvent_t* e : {&K->cgev[0], &K->cgev[1], &K->fork, &K->join})
+        KRR_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    KRR_CUDA(cudaStreamCreateWithFlags(&K->side, cudaStreamNonBlocking));
     if (prec == HDF_FP32) {
         KRR_CUDA(K->vb.alloc(sizeof(float) * n));
         KRR_CUDA(K->yb.alloc(sizeof(float) * n));
@@ -1109,7 +1287,8 @@ hdf_status hdf_krr_solve(hdf_krr* K, const double* y_dev, double rtol, int max_i
     k_gather_vec<<<gb, 256, 0, st>>>(y_dev, K->perm.as<int64_t>(), n, r);
     CgState* S = K->cgst.as<CgState>();
     double* dot = K->dotp.as<double>();
-    const int mgemv = (int)((n + 7) / 8);
+    const int mgemv = (int)((n + 7) / 8), gf = blocks_for(n, 32, 1 << 30);
+    auto finish = K->koff.p ? k_cg_finish<true> : k_cg_finish<false>;
     if (hdf_status s = precond_perm(K, r, z, st, dot); s != HDF_OK) return s;
     HDF_CUDA(cudaMemcpyAsync(p, z, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     HDF_COUNT_LAUNCH();
@@ -1135,9 +1314,9 @@ hdf_status hdf_krr_solve(hdf_krr* K, const double* y_dev, double rtol, int max_i
         if (done) break;
         if (hdf_status s = apply_parts(K, p, st); s != HDF_OK) return s;
         HDF_COUNT_LAUNCH();
-        k_cg_finish<<<gb, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, p, K->hd.as<double>(), q, dot, S);
+        finish<<<gf, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, p, K->hd.as<double>(), q, dot, S);
         HDF_COUNT_LAUNCH();
-        k_cg_step<<<gb, 256, 0, st>>>(x, r, p, q, n, dot, gb, it, S);
+        k_cg_step<<<gb, 256, 0, st>>>(x, r, p, q, n, dot, gf, it, S);
         HDF_CUDA(cudaGetLastError());
         if (hdf_status s = precond_perm(K, r, z, st, dot, S); s != HDF_OK) return s;
         HDF_COUNT_LAUNCH();
