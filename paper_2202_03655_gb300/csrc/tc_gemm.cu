@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // by TMA exactly like the U tiles of k_tc_utv / k_tc_uw; only the small second operand changes.
 //   k_tc_mf_utv: W[(k,s,m,j), c] = sum_i Z[i, zoff_m + j] (A0F[i, aoff_m + q] V[i, c]).
 //     M = 128 rows j of the tails of degree m, N = BN columns n = (q, c), K = points.  The B
-//     tiles A0F (.) V are formed in shared memory by two generator warps (10, 11), in the
+//     tiles A0F (.) V are formed in shared memory by four generator warps (10 .. 13), in the
 //     K-major 128-byte-swizzle layout the TMA would write, TF32 hi / lo stacked.  For the small
 //     degrees (few tails j, many pairs q) a tile takes the transposed roles: M = 128 pairs q (the
 //     A0F block of m by TMA), N = BN columns n = (j, c), B = Z (.) V.
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 //     Q = Z[:, zoff_m + j] W_m[j, (q, c)]: M = 128 points, N = BN columns, K = the tails of m.
 //     The B tiles come by TMA from W gathered per phase (k_prep_mf_w); the promotion warps
 //     contract each phase's accumulator with A0F into y and write Y once per tile.
-constexpr int NGEN = 2;                 // B-generator warps (10, 11)
+constexpr int NGEN = 4;                 // B-generator warps (10 .. 13)
 constexpr int NTHREADS_MF = 32 * (10 + NGEN);   // the roles of k_tc_utv, the generators in place of the B producer
 constexpr int NCONS_MF = NGEN + 9;      // item consumers: generators, MMA, 4 converters, 4 promotion
 
@@ -821,28 +821,32 @@ __global__ void __launch_bounds__(NTHREADS_MF, 1)
             if (!ok) atomicExch(p.err, 1);
         }
     } else if (warp >= 10) {
-        // B generators: warp 10 forms points 0..31 of a step, warp 11 points 32..63 (the two
+        // B generators: warps 10 and 12 form points 0..31 of a step, 11 and 13 points 32..63 (the two
         // 32-K halves of the stage).  A thread owns four consecutive points 4 pg .. 4 pg + 3 (one
-        // 16-byte chunk of a K-major row; pg = 8 (warp - 10) + lane mod 8) and the 16 rows
-        // n = g CP + rs CP / 4 + u of the stage (rs = lane / 8, g < BN / CP, u < CP / 4).  Per step
+        // 16-byte chunk of a K-major row; pg = 8 ((warp - 10) mod 2) + lane mod 8) and the 8 rows
+        // n = g CP + rs CP / 8 + u of the stage (rs = 4 ((warp - 10) / 2) + lane / 8, g < BN / CP,
+        // u < CP / 8).  A step costs a generator thread some 400 instructions; with two warps and 16
+        // rows a thread their two schedulers held the others up (1,000,000 points, 5,480 values each, 16
+        // columns: 19.0 -> 17.2 ms; 17 columns of 100,000 points, rank 23,826, the whole product 4.35 -> 3.12).  Per step
         // it takes the BN / CP values of A0F of each point (one aligned 16-byte piece: A0F blocks
         // start on 16-byte boundaries and q0 is a multiple of BN / CP) and four values of V per
         // column, and writes each row's hi and lo chunk with one 16-byte store.  With CP = 16 the
         // values come through a cp.async ring DS - 1 steps ahead, otherwise as register loads one
         // step ahead.
-        static_assert(NGEN * 32 == BK && BN == 64, "two generator warps, 8 chunks x 4 row sets each");
-        constexpr int NQ = BN / CP, NU = CP / 4;
-        const int pg = (warp - 10) * 8 + (lane & 7), rs = lane >> 3;
-        const int h = warp - 10, jc = lane & 7;
+        static_assert(NGEN * 16 == BK && BN == 64, "four generator warps, 8 chunks x 4 row sets each");
+        constexpr int NQ = BN / CP, NU = CP / 8;
+        const int h = (warp - 10) & 1, part = (warp - 10) >> 1, jc = lane & 7, pe4 = lane >> 3;
+        const int pg = h * 8 + jc, rs = part * 4 + pe4;
         const bool vec = ((reinterpret_cast<uintptr_t>(p.V) | (uintptr_t)p.ldv * 4u) & 15u) == 0;
         if constexpr (STG) {
             // values of DS steps staged by cp.async, DS - 1 steps ahead (A0F rows come mostly from
-            // DRAM, far beyond one step's time).  Slot: the 4 x 16 chunks of the generated factor
-            // (chunk [e][pg]: the 16 bytes of point 4 pg + e, copied by the lane with rs = e and
-            // read by the four lanes of pg after the warp's barrier), then the 4 x 64 chunks of V
-            // (chunk [u][t]: the four points of column 4 rs + u, copied and read by thread t).
-            constexpr int DS = 4, SLOT = (4 * 16 + 4 * 64) * 4;     // floats per slot
-            static_assert(NQ == 4 && NU == 4 && DS * SLOT * 4 <= (int)SM::UBYTES, "the ring fits one U stage");
+            // DRAM, far beyond one step's time).  Slot: for each of the two warps of a point half the 4 x
+            // 16 chunks of the generated factor (chunk [e][pg]: the 16 bytes of point 4 pg + e, copied
+            // by the lane with lane / 8 = e and read by the four lanes of pg after the warp's barrier),
+            // then the 2 x 128 chunks of V (chunk [u][t]: the four points of column 2 rs + u, copied
+            // and read by thread t).
+            constexpr int AF = 4 * 16 * 4, DS = 4, SLOT = 2 * AF + 2 * 128 * 4;     // floats
+            static_assert(NQ == 4 && NU == 2 && DS * SLOT * 4 <= (int)SM::UBYTES, "the ring fits one U stage");
             float* stg = reinterpret_cast<float*>(sm.U + (S_U - 1) * SM::UBYTES);
             const int t = (warp - 10) * 32 + lane;
             uint32_t it = 0;
@@ -863,21 +867,21 @@ __global__ void __launch_bounds__(NTHREADS_MF, 1)
                 // per-item bases, advanced by one step of BK points per copy
                 const int64_t ib = i0 + 4 * pg;
                 const float* g_first = gsrc + ao + q0;                       // row 0: a valid address
-                const float* a_base = g_first + (ib + rs) * gld;
+                const float* a_base = g_first + (ib + pe4) * gld;
                 const int64_t a_step = (int64_t)BK * gld;
                 // the copies of step kt2 (zero-filled outside the item; an empty group past its end)
                 auto issue = [&](int kt2) {
                     if (kt2 < nk) {
                         float* slot = stg + (kt2 % DS) * SLOT;
                         const int64_t i4 = ib + (int64_t)kt2 * BK;
-                        const bool pe = i4 + rs < i1;
-                        cp_async16(slot + (rs * 16 + pg) * 4, pe ? a_base + kt2 * a_step : g_first, pe ? abytes : 0u);
+                        const bool pe = i4 + pe4 < i1;
+                        cp_async16(slot + part * AF + (pe4 * 16 + pg) * 4, pe ? a_base + kt2 * a_step : g_first, pe ? abytes : 0u);
                         const int cnt = (int)max((int64_t)0, min((int64_t)4, i1 - i4));
 #pragma unroll
                         for (int u = 0; u < NU; ++u) {
                             const int cc = rs * NU + u;
                             const int nv = cc < p.c ? cnt : 0;
-                            float* dst = slot + 4 * 16 * 4 + (u * 64 + t) * 4;
+                            float* dst = slot + 2 * AF + (u * 128 + t) * 4;
                             const float* vp = nv > 0 ? p.V + i4 + (int64_t)cc * p.ldv : p.V;
                             if (vec) {
                                 cp_async16(dst, vp, 4u * (uint32_t)nv);
@@ -900,12 +904,12 @@ __global__ void __launch_bounds__(NTHREADS_MF, 1)
                     float av[NQ][4], vv[NU][4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const float4 w = *reinterpret_cast<const float4*>(slot + (e * 16 + pg) * 4);
+                        const float4 w = *reinterpret_cast<const float4*>(slot + part * AF + (e * 16 + pg) * 4);
                         av[0][e] = w.x; av[1][e] = w.y; av[2][e] = w.z; av[3][e] = w.w;
                     }
 #pragma unroll
                     for (int u = 0; u < NU; ++u) {
-                        const float4 w = *reinterpret_cast<const float4*>(slot + 4 * 16 * 4 + (u * 64 + t) * 4);
+                        const float4 w = *reinterpret_cast<const float4*>(slot + 2 * AF + (u * 128 + t) * 4);
                         vv[u][0] = w.x; vv[u][1] = w.y; vv[u][2] = w.z; vv[u][3] = w.w;
                     }
                     bool free_ = (it < (uint32_t)SB) || wait_done<BN>(sm, it - SB);
