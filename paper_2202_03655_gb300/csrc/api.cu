@@ -58,6 +58,30 @@ void pool_setup() {
     }
     done[dev] = true;
 }
+
+cudaMemPool_t small_pool() {
+    static std::mutex mu;
+    static cudaMemPool_t pools[64] = {};
+    static bool tried[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!tried[dev]) {
+        tried[dev] = true;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = 64ull << 20;
+        if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess) {
+            cudaGetLastError();
+            pools[dev] = nullptr;
+        } else {
+            cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+        }
+    }
+    return pools[dev];
+}
 }  // namespace hdf
 
 // --------------------------------------------------------------------- helpers
@@ -187,10 +211,10 @@ void hdf_free(hdf_factor* f) {
     // U and F come from the stream-ordered pool of the build's stream; make sure no kernel of
     // any stream still reads them, then return them to the pool on the legacy stream
     cudaDeviceSynchronize();
-    f->U.st = nullptr;
-    f->mf.Z.st = nullptr;
-    f->mf.A0F.st = nullptr;
-    if (f->ypart) f->ypart->U.st = nullptr;
+    for (hdf_factor* g : {f, f->ypart}) {
+        if (!g) continue;
+        g->U.st = g->mf.Z.st = g->mf.A0F.st = g->plan.arena.st = nullptr;
+    }
     delete f;
 }
 
@@ -387,7 +411,7 @@ hdf_status hdf_build(const double* x_dev, int64_t n, int d, hdf_kernel kernel, d
 
     // ---- A0: centre (mean) and radius (max norm), two-stage reductions
     DevBuf part;
-    HDF_CUDA(part.alloc(sizeof(double) * std::max<int64_t>(1024 * d, 2048)));
+    HDF_CUDA(part.alloc_small(sizeof(double) * std::max<int64_t>(1024 * d, 2048), st));
     dev::Center cen{};
     double sum[HDF_MAX_D];
     if (hdf_status e = point_sums(x_dev, n, d, part, sum, st); e != HDF_OK) return e;
@@ -473,7 +497,7 @@ hdf_status hdf_build_cross(const double* x_dev, int64_t m, const double* y_dev, 
 
     // ---- A0 for both sets with one map: centre = mean of the union, R = max distance from it
     DevBuf part;
-    HDF_CUDA(part.alloc(sizeof(double) * std::max<int64_t>(1024 * d, 2048)));
+    HDF_CUDA(part.alloc_small(sizeof(double) * std::max<int64_t>(1024 * d, 2048), st));
     double sx[HDF_MAX_D], sy[HDF_MAX_D];
     if (hdf_status e = point_sums(x_dev, m, d, part, sx, st); e != HDF_OK) return e;
     if (hdf_status e = point_sums(y_dev, n, d, part, sy, st); e != HDF_OK) return e;
@@ -969,10 +993,6 @@ static hdf_status solve_t(hdf_factor* f, double lambda, const T* B, int64_t ldb,
         const bool aligned = (reinterpret_cast<uintptr_t>(f->U.p) % 16 == 0) && (f->info.ldu % 4 == 0);
         if (sizeof(T) == 4 && f->use_tc && aligned && r >= 64 && n >= 32) {
             // U^T U on the tensor cores (FP32 factors)
-            if (!f->dev_err.p) {
-                HDF_CUDA(f->dev_err.alloc(sizeof(int)));
-                HDF_CUDA(cudaMemsetAsync(f->dev_err.p, 0, sizeof(int), st));
-            }
             hdf_status s = tc_gram(reinterpret_cast<const float*>(f->U.p), f->info.ldu, n, r, Gd.as<double>(),
                                    f->dev_err.as<int>(), st);
             if (s != HDF_OK) return s;
@@ -1091,20 +1111,34 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     const int L = dp.L;
     const int64_t r = I.rank;
     const int vw = (sizeof(T) == 4) ? 4 : 2;
-    HDF_CUDA(f->dev_err.alloc(sizeof(int)));
-    HDF_CUDA(cudaMemsetAsync(f->dev_err.p, 0, sizeof(int), st));
     DeviceTables tb;
     std::string terr;
     if (!make_tables(fc, d, L, vw, tb, terr)) return fail(HDF_ETOOBIG, "hdf_build: " + terr);
     I.ldu = tb.ldU;
     f->plan.colmap = tb.colmap;
     f->plan.Spad = tb.Spad;
-    // S on the device, on the padded columns
+    // the host image of the factor's small device arrays, each on a 256-byte boundary
+    std::vector<unsigned char> image;
+    struct Piece { DevView* v; size_t off; };
+    std::vector<Piece> pieces;
+    auto piece = [&](DevView& v, const void* src, size_t bytes) {
+        const size_t o = (image.size() + 255) & ~size_t(255);
+        image.resize(o + std::max<size_t>(16, bytes), 0);
+        if (bytes) std::memcpy(image.data() + o, src, bytes);
+        pieces.push_back({&v, o});
+    };
+    auto upload = [&]() -> hdf_status {
+        HDF_CUDA(f->plan.arena.alloc_small(image.size(), st));
+        HDF_CUDA(cudaMemcpyAsync(f->plan.arena.p, image.data(), image.size(), cudaMemcpyHostToDevice, st));
+        for (const Piece& q : pieces) q.v->p = f->plan.arena.as<unsigned char>() + q.off;
+        return HDF_OK;
+    };
+    const int no_error = 0;
+    piece(f->dev_err, &no_error, sizeof(int));
     {
-        std::vector<T> Sd(I.ldu, (T)0);
+        std::vector<T> Sd(I.ldu, (T)0);                      // S on the padded columns
         for (int64_t a = 0; a < I.ldu; ++a) Sd[a] = (T)tb.Spad[a];
-        HDF_CUDA(f->S.alloc(sizeof(T) * I.ldu));
-        HDF_CUDA(cudaMemcpyAsync(f->S.p, Sd.data(), sizeof(T) * I.ldu, cudaMemcpyHostToDevice, st));
+        piece(f->S, Sd.data(), sizeof(T) * I.ldu);
     }
     const size_t ubytes = sizeof(T) * (size_t)n * (size_t)I.ldu;
     // the matrix-free form when asked for, or when U would not fit (d >= 4 only)
@@ -1116,7 +1150,11 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         cudaGetLastError();
         return fail(HDF_ENOMEM, "hdf_build: cannot allocate U (" + std::to_string(ubytes) + " bytes)");
     }
-    if (r == 0) { HDF_CUDA(cudaStreamSynchronize(st)); return HDF_OK; }
+    if (r == 0) {
+        if (hdf_status e = upload(); e != HDF_OK) return e;
+        HDF_CUDA(cudaStreamSynchronize(st));
+        return HDF_OK;
+    }
     const int L_used = tb.L_used, nF = tb.nF, mmax = tb.mmax;
     const int64_t nH = tb.nH;
     const std::vector<double>* Qmat = fc.Qmat;
@@ -1135,27 +1173,24 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
     PL.fbase = tb.fbase;
     PL.cbase = tb.cbase;
     PL.hbase = tb.hbase;
-    DevBuf dpar, dF;
-    DevBuf &dQ0 = PL.dQ0, &dQ1 = PL.dQ1, &dW = PL.dW, &dchains = PL.dchains, &dA = PL.dA, &dB = PL.dB;
-    HDF_CUDA(PL.dcolk.alloc(tb.colk.size()));
-    HDF_CUDA(PL.dhk.alloc(tb.hk.size() + 1));
-    HDF_CUDA(PL.dktab.alloc(sizeof(int) * tb.ktab.size()));
-    HDF_CUDA(cudaMemcpyAsync(PL.dcolk.p, tb.colk.data(), tb.colk.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(PL.dhk.p, tb.hk.data(), tb.hk.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(PL.dktab.p, tb.ktab.data(), sizeof(int) * tb.ktab.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(dQ0.alloc(sizeof(double) * std::max<size_t>(1, Qmat[0].size())));
-    HDF_CUDA(dQ1.alloc(sizeof(double) * std::max<size_t>(1, Qmat[1].size())));
-    HDF_CUDA(dW.alloc(sizeof(T) * Wt.size()));
-    HDF_CUDA(dpar.alloc(tb.colpar.size()));
-    HDF_CUDA(dchains.alloc(sizeof(int16_t) * std::max<size_t>(1, tb.chains.size())));
-    HDF_CUDA(PL.dqdesc.alloc(sizeof(uint32_t) * tb.qdesc.size()));
-    HDF_CUDA(PL.dychain.alloc(sizeof(int32_t) * tb.ychain.size()));
+    DevBuf dF;
+    DevView dpar;
+    DevView &dQ0 = PL.dQ0, &dQ1 = PL.dQ1, &dW = PL.dW, &dchains = PL.dchains, &dA = PL.dA, &dB = PL.dB;
+    piece(PL.dcolk, tb.colk.data(), tb.colk.size());
+    piece(PL.dhk, tb.hk.data(), tb.hk.size());
+    piece(PL.dktab, tb.ktab.data(), sizeof(int) * tb.ktab.size());
+    piece(dQ0, Qmat[0].data(), sizeof(double) * Qmat[0].size());
+    piece(dQ1, Qmat[1].data(), sizeof(double) * Qmat[1].size());
+    piece(dW, Wt.data(), sizeof(T) * Wt.size());
+    piece(dpar, tb.colpar.data(), tb.colpar.size());
+    piece(dchains, tb.chains.data(), sizeof(int16_t) * tb.chains.size());
+    piece(PL.dqdesc, tb.qdesc.data(), sizeof(uint32_t) * tb.qdesc.size());
+    piece(PL.dychain, tb.ychain.data(), sizeof(int32_t) * tb.ychain.size());
     // harmonic slots: gbase (d = 3) or ydesc
-    const void* gy = d == 3 ? (const void*)tb.gbase.data() : (const void*)tb.ydesc.data();
-    const size_t gy_bytes = sizeof(int32_t) * (d == 3 ? tb.gbase.size() : tb.ydesc.size());
-    HDF_CUDA(PL.dslots.alloc(std::max<size_t>(16, gy_bytes)));
-    HDF_CUDA(dA.alloc(sizeof(T) * cA.size() + 16));
-    HDF_CUDA(dB.alloc(sizeof(T) * cB.size() + 16));
+    piece(PL.dslots, d == 3 ? (const void*)tb.gbase.data() : (const void*)tb.ydesc.data(),
+        sizeof(int32_t) * (d == 3 ? tb.gbase.size() : tb.ydesc.size()));
+    piece(dA, cA.data(), sizeof(T) * cA.size());
+    piece(dB, cB.data(), sizeof(T) * cB.size());
     const int64_t ldF = ((int64_t)nF + 31) / 32 * 32;       // 128-byte rows (FP32): whole-sector stores
     const int mtp = ((m0 + m1 + 7) / 8) * 8;
     // FP32 factors with few columns: rows straight from the points, without the F buffer
@@ -1165,8 +1200,6 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
         cudaGetLastError();
         return fail(HDF_ENOMEM, "hdf_build: cannot allocate the radial factor buffer");
     }
-    if (!Qmat[0].empty()) HDF_CUDA(cudaMemcpyAsync(dQ0.p, Qmat[0].data(), sizeof(double) * Qmat[0].size(), cudaMemcpyHostToDevice, st));
-    if (!Qmat[1].empty()) HDF_CUDA(cudaMemcpyAsync(dQ1.p, Qmat[1].data(), sizeof(double) * Qmat[1].size(), cudaMemcpyHostToDevice, st));
     // FP32 factors: [Qmat0 | Qmat1] as (hi, lo) float pairs for the compensated radial basis,
     // (L+1) x mtp with the odd columns zero in row L and mtp a multiple of 8
     if (sizeof(T) == 4) {
@@ -1180,22 +1213,9 @@ static hdf_status build_device(hdf_factor* f, const double* x, int64_t n, int d,
             for (int o = 0; o < m0; ++o) put(l, o, Qmat[0][(size_t)l * m0 + o]);
         for (int l = 0; l < nb1; ++l)
             for (int o = 0; o < m1; ++o) put(l, m0 + o, Qmat[1][(size_t)l * m1 + o]);
-        HDF_CUDA(PL.dQC.alloc(sizeof(float) * qc.size()));
-        HDF_CUDA(cudaMemcpyAsync(PL.dQC.p, qc.data(), sizeof(float) * qc.size(), cudaMemcpyHostToDevice, st));
-        HDF_CUDA(cudaStreamSynchronize(st));      // qc is a local buffer
+        piece(PL.dQC, qc.data(), sizeof(float) * qc.size());
     }
-    HDF_CUDA(cudaMemcpyAsync(dW.p, Wt.data(), sizeof(T) * Wt.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(dpar.p, tb.colpar.data(), tb.colpar.size(), cudaMemcpyHostToDevice, st));
-    if (!tb.chains.empty())
-        HDF_CUDA(cudaMemcpyAsync(dchains.p, tb.chains.data(), sizeof(int16_t) * tb.chains.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(PL.dqdesc.p, tb.qdesc.data(), sizeof(uint32_t) * tb.qdesc.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(PL.dychain.p, tb.ychain.data(), sizeof(int32_t) * tb.ychain.size(), cudaMemcpyHostToDevice, st));
-    if (gy_bytes) HDF_CUDA(cudaMemcpyAsync(PL.dslots.p, gy, gy_bytes, cudaMemcpyHostToDevice, st));
-    if (!cA.empty()) {
-        HDF_CUDA(cudaMemcpyAsync(dA.p, cA.data(), sizeof(T) * cA.size(), cudaMemcpyHostToDevice, st));
-        HDF_CUDA(cudaMemcpyAsync(dB.p, cB.data(), sizeof(T) * cB.size(), cudaMemcpyHostToDevice, st));
-    }
-
+    if (hdf_status e = upload(); e != HDF_OK) return e;
     cudaEvent_t ev[3];
     for (int q = 0; q < 3; ++q) HDF_CUDA(cudaEventCreate(&ev[q]));
     struct EvGuard { cudaEvent_t* e; ~EvGuard() { for (int q = 0; q < 3; ++q) cudaEventDestroy(e[q]); } } evg{ev};

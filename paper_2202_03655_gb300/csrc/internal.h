@@ -136,6 +136,11 @@ inline bool injected_alloc_failure() {
 // (release threshold raised once per device), so that repeated builds and products reuse
 // memory instead of mapping it again.
 void pool_setup();
+// The current device's pool for small blocks that live as long as a factor or a build (null if it
+// cannot be created).  In the default pool they would split the free space that the next U of the
+// same size needs, which then has to be mapped anew (12 ms for 43 GB); cudaMalloc and cudaFree take
+// 45 us each.  Keeps at most 64 MiB of unused memory.
+cudaMemPool_t small_pool();
 }  // namespace hdf
 
 // Owns one device allocation.  alloc(): synchronous cudaMalloc; alloc_on(): stream-ordered
@@ -167,6 +172,23 @@ struct DevBuf {
         if (b && hdf::injected_alloc_failure()) return cudaErrorMemoryAllocation;
         return b ? cudaMallocAsync(&p, b, s) : cudaSuccess;
     }
+    // From the library's own stream-ordered pool for small blocks (small_pool).
+    cudaError_t alloc_small(size_t b, cudaStream_t s) {
+        cudaMemPool_t pool = hdf::small_pool();
+        if (!pool) return alloc(b);
+        release();
+        bytes = b;
+        pooled = true;
+        st = s;
+        if (b && hdf::injected_alloc_failure()) return cudaErrorMemoryAllocation;
+        return b ? cudaMallocFromPoolAsync(&p, b, pool, s) : cudaSuccess;
+    }
+    template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
+};
+
+// A piece of another buffer.
+struct DevView {
+    void* p = nullptr;
     template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
 };
 
@@ -183,7 +205,11 @@ struct FactorPlan {
     // chains (nH x (d-1) int16), hk (harmonic -> k), ktab (per k: fbase, s_k, cbase, |H_k|, hbase,
     // padded |H_k|), qdesc (chunk descriptors), ychain (padded harmonic slots -> chain), slots (gbase or ydesc of make_tables),
     // coefA/coefB (level recurrences, bulk)
-    DevBuf dQ0, dQ1, dQC, dW, dcolk, dchains, dhk, dktab, dqdesc, dychain, dslots, dA, dB;
+    // -- pieces of `arena`, as are the factor's S and dev_err: one allocation and one copy per factor
+    // (sixteen of each, and as many frees, took 0.25 of the 0.80 ms of a build, product and release at
+    // 2,000 points)
+    DevBuf arena;
+    DevView dQ0, dQ1, dQC, dW, dcolk, dchains, dhk, dktab, dqdesc, dychain, dslots, dA, dB;
     std::vector<int64_t> colmap;               // padded column of each true column of U
     std::vector<double> Spad;                  // S on the padded columns (0 on padding)
     // d S_k / d l (s_k x s_k), computed on first use by the adjoint
@@ -223,7 +249,8 @@ struct hdf_factor {
     double ell = 0, tol = 0;
     int prec = 0;
     size_t esz = 8;                 // bytes per bulk element
-    DevBuf U, S;                    // U n x ldu, S rank (bulk type)
+    DevBuf U;                       // n x ldu (bulk type)
+    DevView S;                      // ldu (bulk type)
     std::vector<double> S_host;
     // solve core: U^T U (FP64, r x r, kept after the first solve), the factors of
     // lambda S^-1 + U^T U for core_lambda (row-major, in place), their order and the inverses of
@@ -234,7 +261,7 @@ struct hdf_factor {
     // tensor-core matvec (FP32 factors): enabled unless HDF_FLAG_CUDA_CORES; dev_err is set by
     // a kernel whose bounded wait expired
     bool use_tc = true;
-    DevBuf dev_err;
+    DevView dev_err;
     // events around the kernels of the most recent matvec (first column group)
     cudaEvent_t mv_ev[4] = {nullptr, nullptr, nullptr, nullptr};
     bool mv_recorded = false;
