@@ -39,14 +39,49 @@ struct AdjParams {
     const double* Qm1; int nb1, m1;
     const float2* QC; int mtp;                     // FP32 factors: [Qm0 | Qm1] as float pairs, (Lr+1) x mtp
     const T* Wt; const uint8_t* colk; int nF;
-    const int16_t* chains; int nH, cstride; const uint8_t* hk; const int* ktab;
+    int nH, nk; const int* ktab;
+    const int4* desc;                              // per harmonic (k_adj_desc)
+    const int* desc2;                              // d >= 7: level offsets 4, 5
     const T* coefA; const T* coefB;
-    const T* a; const T* b; int ab_stride;        // a[col * ab_stride], b[col * ab_stride]
+    const T* ab;                                   // (a, b) of every column
     const T* v; const T* w;                        // this column of V and W (length n)
     T* grad; int accumulate;
-    int per_warp_d;                                // doubles per warp
-    int per_warp_t;                                // T elements per warp
+    int nb;                                        // points per batch of a warp (1, 2 or 4)
+    int per_warp;                                  // bytes of shared memory per warp (a multiple of 16)
 };
+constexpr int kAdjBatch = 4;      // whole call at 500,000 points: 1 4.88, 2 4.55, 4 4.36, 8 4.79 ms
+
+template <typename T> struct Pair;
+template <> struct Pair<float> { typedef float2 type; };
+template <> struct Pair<double> { typedef double2 type; };
+template <typename T> struct Quad;
+template <> struct Quad<float> { typedef float4 type; };
+struct alignas(16) Double4 { double x, y, z, w; };
+template <> struct Quad<double> { typedef Double4 type; };
+
+// Shared memory of a warp: (value, d/dz, d/dq) of the level tables and (value, d/dx_0, d/dx_1) of the
+// trigonometric factors (four elements each), (F' - k F / rho, F / rho) per radial factor, T_l and T_l'
+// of a batch of points (8 bytes each), the radial basis and its derivative (8 bytes each).
+template <typename T>
+size_t adj_per_warp(int levels, int tri, int L, int nF, int Lr, int m, int nb) {
+    return ((sizeof(T) * (4 * ((size_t)levels * tri + 2 * L + 1) + 2 * (size_t)nF) + 7) / 8 * 8 +
+            8 * (2 * (size_t)nb * (Lr + 1) + 2 * (size_t)m) + 15) / 16 * 16;
+}
+
+// What the harmonic loop needs of harmonic gi, from five tables: first column, k | trigonometric index
+// << 8, level offsets 0 | 1 << 16, 2 | 3 << 16 (, 4 | 5 << 16).
+__global__ void k_adj_desc(const int16_t* __restrict__ chains, int nH, int cstride, int levels, int L,
+                           const uint8_t* __restrict__ hk, const int* __restrict__ ktab, int4* __restrict__ desc,
+                           int* __restrict__ desc2) {
+    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= nH) return;
+    const int k = hk[gi];
+    const int* kt = ktab + hdf::kTabStride * k;
+    const int16_t* ch = chains + (int64_t)gi * cstride;
+    auto off = [&](int j) { return j < levels ? (int)(uint16_t)ch[j] << (16 * (j & 1)) : 0; };
+    desc[gi] = make_int4(kt[2] + gi - kt[4], k | (L + ch[levels]) << 8, off(0) | off(1), off(2) | off(3));
+    if (desc2) desc2[gi] = off(4) | off(5);
+}
 
 // Double-float helpers for the FP32 form (FP32 pairs, error-free products and sums).
 __device__ __forceinline__ void df_two_sum(float a, float b, float& s, float& e) {
@@ -80,92 +115,115 @@ __device__ __forceinline__ void df_dot_step(float2 a, float2 b, float& sh, float
     c += es + pe;
 }
 
-// DD = the dimension d (a template parameter, so that the per-thread coordinate and gradient
-// arrays stay in registers).
+// A warp takes batches of P.nb points: lane p forms the scaled coordinates of point p and runs its
+// Chebyshev recurrences of T_l and T_l' (serial, in double-float arithmetic for FP32 factors some 70
+// instructions a step, which one lane per point cost every lane), then the points follow one by one
+// with the lanes over basis functions, radial factors and harmonics.  Bound by instruction issue and
+// the latency of the table reads: 500,000 points, d = 4, 2,104 columns, 4.43 -> 3.19 ms with batches,
+// one descriptor per harmonic and the tables' three values read together.  DD = the dimension d (a template parameter, so that
+// the per-thread coordinate and gradient arrays stay in registers).
 template <typename T, int DD>
 __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int2 kts[HDF_MAX_L + 1];        // per k: F column | s_k << 16, columns per (k, s) block
+    typedef typename Pair<T>::type T2;
+    typedef typename Quad<T>::type T4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     constexpr int levels = DD - 2;
-    double* dbase = reinterpret_cast<double*>(smem_raw) + (size_t)warp * P.per_warp_d;
-    double* Tl = dbase;                        // Lr+1: T_l(u)
-    double* dTl = Tl + (P.Lr + 1);             // Lr+1: T_l'(u)
-    double* Q = dTl + (P.Lr + 1);              // m0+m1
+    for (int k = threadIdx.x; k < P.nk; k += blockDim.x) {
+        const int* kt = P.ktab + hdf::kTabStride * k;
+        kts[k] = make_int2(kt[0] | kt[1] << 16, kt[5]);
+    }
+    __syncthreads();
+    T4* tb = reinterpret_cast<T4*>(smem_raw + (size_t)warp * P.per_warp);      // levels * tri
+    T4* trig = tb + levels * P.tri;            // 2L+1
+    T2* RR = reinterpret_cast<T2*>(trig + 2 * P.L + 1);                        // nF
+    double* Tl = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(tb) +
+                                           (sizeof(T) * (4 * (levels * P.tri + 2 * P.L + 1) + 2 * P.nF) + 7) / 8 * 8);
+    const int nb = P.nb;
+    double* dTl = Tl + nb * (P.Lr + 1);        // T_l(u), T_l'(u): [l][point]
+    double* Q = dTl + nb * (P.Lr + 1);         // m0+m1
     double* dQ = Q + (P.m0 + P.m1);            // m0+m1
-    T* tbase = reinterpret_cast<T*>(reinterpret_cast<double*>(smem_raw) + (size_t)nwarps * P.per_warp_d) +
-               (size_t)warp * P.per_warp_t;
-    T* R1 = tbase;                             // nF
-    T* R2 = R1 + P.nF;                         // nF
-    T* tv = R2 + P.nF;                         // levels * tri: P
-    T* tz = tv + levels * P.tri;               // dP/dz
-    T* tq = tz + levels * P.tri;               // dP/dq
-    T* trig = tq + levels * P.tri;             // 2L+1
-    T* trx = trig + 2 * P.L + 1;               // d/dx0
-    T* try_ = trx + 2 * P.L + 1;               // d/dx1
     const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
-    for (int64_t i = gw; i < P.n; i += nw) {
-        T xh[kMaxD];
-        double s2 = 0.0;
-        if constexpr (sizeof(T) == 4) {
-            // lane j forms coordinate j in FP64 once; |x'|^2 by an FP64 shuffle tree over the
-            // first eight lanes; the warp shares the coordinates in FP32 (FP64 issues at a small
-            // fraction of the FP32 rate on this GPU)
-            double cj = P.c[0];                  // this lane's centre coordinate (register selects)
+    for (int64_t i0 = gw * nb; i0 < P.n; i0 += nw * nb) {
+        // ---- this lane's point
+        const int own = lane & (nb - 1);
+        const int64_t io = min(i0 + own, P.n - 1);
+        T xo[DD];
+        double s2o = 0.0;
 #pragma unroll
-            for (int j = 1; j < DD; ++j) cj = (lane == j) ? P.c[j] : cj;
-            const double xd = (lane < DD) ? (P.x[i * DD + lane] - cj) * P.inv2R : 0.0;   // one FP64 sub, mul
-            double sq = xd * xd;
-            sq += __shfl_xor_sync(0xffffffffu, sq, 4);
-            sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-            sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-            s2 = __shfl_sync(0xffffffffu, sq, 0);
-            const float xf = (float)xd;
-#pragma unroll
-            for (int j = 0; j < DD; ++j) xh[j] = __shfl_sync(0xffffffffu, xf, j);
-        } else {
-#pragma unroll
-            for (int j = 0; j < DD; ++j) { xh[j] = (P.x[i * DD + j] - P.c[j]) * P.inv2R; s2 += xh[j] * xh[j]; }
+        for (int j = 0; j < DD; ++j) {
+            const double xd = (P.x[io * DD + j] - P.c[j]) * P.inv2R;
+            s2o += xd * xd;
+            xo[j] = (T)xd;
         }
-        double rho;
+        const T wo = P.w[io], vo = P.v[io];
+        T rhoo;
         if constexpr (sizeof(T) == 4) {
-            // FP32 factors: the radial part in double-float / FP32 arithmetic (FP64 is slow here)
-            const float s2f = (float)s2;
-            const float rhof = sqrtf(s2f);
-            rho = rhof;
-            if (s2 > 0.0) { const float inv = 1.f / rhof; for (int j = 0; j < DD; ++j) xh[j] *= inv; }
-            else { for (int j = 0; j < DD; ++j) xh[j] = (j == 0) ? 1.f : 0.f; }
-            float2* Tl2 = reinterpret_cast<float2*>(Tl);
-            float2* dTl2 = reinterpret_cast<float2*>(dTl);
-            float* Qf = reinterpret_cast<float*>(Q);
-            float* dQf = reinterpret_cast<float*>(dQ);
-            if (lane == 0) {
-                const double u = 8.0 * s2 - 1.0;
+            rhoo = sqrtf((float)s2o);
+            if (s2o > 0.0) { const float inv = 1.f / rhoo; for (int j = 0; j < DD; ++j) xo[j] *= inv; }
+            else { for (int j = 0; j < DD; ++j) xo[j] = (j == 0) ? 1.f : 0.f; }
+        } else {
+            rhoo = sqrt(s2o);
+            if (s2o > 0.0) { for (int j = 0; j < DD; ++j) xo[j] = xo[j] / rhoo; }
+            else { for (int j = 0; j < DD; ++j) xo[j] = (j == 0) ? 1.0 : 0.0; }
+        }
+        if (lane < nb) {
+            const double u = 8.0 * s2o - 1.0;
+            if constexpr (sizeof(T) == 4) {
+                // FP32 factors: the radial part in double-float / FP32 arithmetic (FP64 is slow here)
+                float2* Tl2 = reinterpret_cast<float2*>(Tl) + lane;
+                float2* dTl2 = reinterpret_cast<float2*>(dTl) + lane;
                 const float uh = (float)u, ul = (float)(u - (double)uh);
                 const float2 u2 = make_float2(2.f * uh, 2.f * ul);
                 float2 t2 = make_float2(1.f, 0.f), t1 = make_float2(uh, ul);       // T_{l-2}, T_{l-1}
                 float2 d2 = make_float2(0.f, 0.f), d1 = make_float2(1.f, 0.f);     // T'_{l-2}, T'_{l-1}
                 Tl2[0] = t2; dTl2[0] = d2;
-                if (P.Lr >= 1) { Tl2[1] = t1; dTl2[1] = d1; }
+                if (P.Lr >= 1) { Tl2[nb] = t1; dTl2[nb] = d1; }
                 for (int l = 2; l <= P.Lr; ++l) {
                     const float2 tn = df_add(df_mul(u2, t1), make_float2(-t2.x, -t2.y));
                     const float2 dn = df_add(df_add(make_float2(2.f * t1.x, 2.f * t1.y), df_mul(u2, d1)),
                                              make_float2(-d2.x, -d2.y));
-                    Tl2[l] = tn; dTl2[l] = dn;
+                    Tl2[l * nb] = tn; dTl2[l * nb] = dn;
+                    t2 = t1; t1 = tn;
+                    d2 = d1; d1 = dn;
+                }
+            } else {
+                double t2 = 1.0, t1 = u, d2 = 0.0, d1 = 1.0;
+                Tl[lane] = t2; dTl[lane] = d2;
+                if (P.Lr >= 1) { Tl[nb + lane] = t1; dTl[nb + lane] = d1; }
+                for (int l = 2; l <= P.Lr; ++l) {
+                    const double tn = 2.0 * u * t1 - t2, dn = 2.0 * t1 + 2.0 * u * d1 - d2;
+                    Tl[l * nb + lane] = tn; dTl[l * nb + lane] = dn;
                     t2 = t1; t1 = tn;
                     d2 = d1; d1 = dn;
                 }
             }
-            __syncwarp();
+        }
+        __syncwarp();
+        for (int pt = 0; pt < nb && i0 + pt < P.n; ++pt) {
+        const int64_t i = i0 + pt;
+        T xh[kMaxD];
+#pragma unroll
+        for (int j = 0; j < DD; ++j) xh[j] = __shfl_sync(0xffffffffu, xo[j], pt);
+        const T rhot = __shfl_sync(0xffffffffu, rhoo, pt);
+        const T wi = __shfl_sync(0xffffffffu, wo, pt), vi = __shfl_sync(0xffffffffu, vo, pt);
+        if constexpr (sizeof(T) == 4) {
+            const float rhof = rhot, s2f = __shfl_sync(0xffffffffu, (float)s2o, pt);
+            const float2* Tl2 = reinterpret_cast<const float2*>(Tl) + pt;
+            const float2* dTl2 = reinterpret_cast<const float2*>(dTl) + pt;
+            float* Qf = reinterpret_cast<float*>(Q);
+            float* dQf = reinterpret_cast<float*>(dQ);
             // S_T[o] = sum_l T_l Qmat[l][o], S_dT[o] = sum_l T'_l Qmat[l][o] (Dot2); then
             // even: Q = S_T, dQ = 16 rho S_dT;  odd: Q = rho S_T, dQ = S_T + 16 rho^2 S_dT
             for (int o = lane; o < P.m0 + P.m1; o += 32) {
                 const bool odd = o >= P.m0;
-                const int nb = odd ? P.nb1 : P.nb0;
+                const int nbas = odd ? P.nb1 : P.nb0;
                 float th = 0.f, tc = 0.f, dh = 0.f, dc = 0.f;
-                for (int l = 0; l < nb; ++l) {
+                for (int l = 0; l < nbas; ++l) {
                     const float2 qm = P.QC[(size_t)l * P.mtp + o];
-                    df_dot_step(Tl2[l], qm, th, tc);
-                    df_dot_step(dTl2[l], qm, dh, dc);
+                    df_dot_step(Tl2[l * nb], qm, th, tc);
+                    df_dot_step(dTl2[l * nb], qm, dh, dc);
                 }
                 const float st = th + tc, sd = dh + dc;
                 if (!odd) { Qf[o] = st; dQf[o] = 16.f * rhof * sd; }
@@ -181,43 +239,28 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                     F += Qf[ob + l] * wv;
                     dF += dQf[ob + l] * wv;
                 }
-                if (rhof > 1e-30f) {
-                    R1[col] = (T)(dF - k * F / rhof);
-                    R2[col] = (T)(F / rhof);
-                } else {
-                    R1[col] = (T)dF;
-                    R2[col] = (T)0;
-                }
+                T2 r;
+                if (rhof > 1e-30f) { r.x = (T)(dF - k * F / rhof); r.y = (T)(F / rhof); }
+                else { r.x = (T)dF; r.y = (T)0; }
+                RR[col] = r;
             }
         } else {
-        rho = sqrt(s2);
-        if (s2 > 0.0) { for (int j = 0; j < DD; ++j) xh[j] = (T)(xh[j] / rho); }
-        else { for (int j = 0; j < DD; ++j) xh[j] = (j == 0) ? (T)1 : (T)0; }
-        const double u = 8.0 * s2 - 1.0;
-        if (lane == 0) {
-            Tl[0] = 1.0; dTl[0] = 0.0;
-            if (P.Lr >= 1) { Tl[1] = u; dTl[1] = 1.0; }
-            for (int l = 2; l <= P.Lr; ++l) {
-                Tl[l] = 2.0 * u * Tl[l - 1] - Tl[l - 2];
-                dTl[l] = 2.0 * Tl[l - 1] + 2.0 * u * dTl[l - 1] - dTl[l - 2];
-            }
-        }
-        __syncwarp();
+        const double rho = rhot, s2 = __shfl_sync(0xffffffffu, s2o, pt);
         // Q = B Qmat and dQ/drho; B0 = T_l, B0' = 16 rho T_l'; B1 = rho T_l, B1' = T_l + 16 rho^2 T_l'
         for (int o = lane; o < P.m0 + P.m1; o += 32) {
             double q = 0.0, dq = 0.0;
             if (o < P.m0) {
                 for (int l = 0; l < P.nb0; ++l) {
                     const double qm = P.Qm0[l * P.m0 + o];
-                    q += Tl[l] * qm;
-                    dq += 16.0 * rho * dTl[l] * qm;
+                    q += Tl[l * nb + pt] * qm;
+                    dq += 16.0 * rho * dTl[l * nb + pt] * qm;
                 }
             } else {
                 const int oo = o - P.m0;
                 for (int l = 0; l < P.nb1; ++l) {
                     const double qm = P.Qm1[l * P.m1 + oo];
-                    q += rho * Tl[l] * qm;
-                    dq += (Tl[l] + 16.0 * s2 * dTl[l]) * qm;
+                    q += rho * Tl[l * nb + pt] * qm;
+                    dq += (Tl[l * nb + pt] + 16.0 * s2 * dTl[l * nb + pt]) * qm;
                 }
             }
             Q[o] = q;
@@ -234,13 +277,10 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                 F += Q[ob + l] * wv;
                 dF += dQ[ob + l] * wv;
             }
-            if (rho > 1e-30) {
-                R1[col] = (T)(dF - k * F / rho);
-                R2[col] = (T)(F / rho);
-            } else {
-                R1[col] = (T)dF;
-                R2[col] = (T)0;
-            }
+            T2 r;
+            if (rho > 1e-30) { r.x = (T)(dF - k * F / rho); r.y = (T)(F / rho); }
+            else { r.x = (T)dF; r.y = (T)0; }
+            RR[col] = r;
         }
         }
         // level tables with d/dz and d/dq
@@ -253,23 +293,22 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
             const T z = xh[D], qq = q;
             const T* A = P.coefA + j * P.tri;
             const T* B = P.coefB + j * P.tri;
-            T* pv = tv + j * P.tri;
-            T* pz = tz + j * P.tri;
-            T* pq = tq + j * P.tri;
+            T4* pt4 = tb + j * P.tri;
+            auto put = [&](int e, T v, T dz, T dq) { T4 w; w.x = v; w.y = dz; w.z = dq; w.w = (T)0; pt4[e] = w; };
             for (int mu = lane; mu <= P.L; mu += 32) {
                 const int o = mu * (P.L + 1) - mu * (mu - 1) / 2;
                 const int nmax = P.L - mu;
                 T v2 = A[o], z2 = (T)0, q2 = (T)0;
-                pv[o] = v2; pz[o] = z2; pq[o] = q2;
+                put(o, v2, z2, q2);
                 if (nmax >= 1) {
                     T v1 = A[o + 1] * z, z1 = A[o + 1], q1 = (T)0;
-                    pv[o + 1] = v1; pz[o + 1] = z1; pq[o + 1] = q1;
+                    put(o + 1, v1, z1, q1);
                     for (int nn = 2; nn <= nmax; ++nn) {
                         const T an = A[o + nn], bn = B[o + nn];
                         const T v0 = an * z * v1 - bn * qq * v2;
                         const T z0 = an * (v1 + z * z1) - bn * qq * z2;
                         const T q0 = an * z * q1 - bn * (v2 + qq * q2);
-                        pv[o + nn] = v0; pz[o + nn] = z0; pq[o + nn] = q0;
+                        put(o + nn, v0, z0, q0);
                         v2 = v1; z2 = z1; q2 = q1;
                         v1 = v0; z1 = z0; q1 = q0;
                     }
@@ -295,22 +334,17 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                     e >>= 1;
                 }
             }
+            // value, d/dx_0, d/dx_1
+            auto put = [&](int e, T v, T dx, T dy) { T4 w; w.x = v; w.y = dx; w.z = dy; w.w = (T)0; trig[e] = w; };
             if (mu == 0) {
-                trig[P.L] = (T)0.3989422804014327;
-                trx[P.L] = (T)0;
-                try_[P.L] = (T)0;
+                put(P.L, (T)0.3989422804014327, (T)0, (T)0);
             } else {
                 const TP nm = (TP)0.5641895835477563;
-                trig[P.L + mu] = (T)(rr * nm);            // Re z^mu
-                trig[P.L - mu] = (T)(ri * nm);            // Im z^mu
-                trx[P.L + mu] = (T)(mu * pr * nm);        // d Re / dx0
-                trx[P.L - mu] = (T)(mu * pi * nm);        // d Im / dx0
-                try_[P.L + mu] = (T)(-mu * pi * nm);      // d Re / dx1
-                try_[P.L - mu] = (T)(mu * pr * nm);       // d Im / dx1
+                put(P.L + mu, (T)(rr * nm), (T)(mu * pr * nm), (T)(-mu * pi * nm));      // Re z^mu
+                put(P.L - mu, (T)(ri * nm), (T)(mu * pi * nm), (T)(mu * pr * nm));       // Im z^mu
             }
         }
         __syncwarp();
-        const T wi = P.w[i], vi = P.v[i];
         T g[kMaxD];
 #pragma unroll
         for (int m = 0; m < kMaxD; ++m) g[m] = (T)0;
@@ -318,25 +352,32 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
 #pragma unroll
         for (int m = 0; m < DD; ++m) xt[m] = (T)xh[m];
         for (int gi = lane; gi < P.nH; gi += 32) {
-            const int k = P.hk[gi];
-            const int* kt = P.ktab + hdf::kTabStride * k;
-            const int fb = kt[0], sk = kt[1], cb = kt[2], hb = kt[4], dimp = kt[5];
-            const int h = gi - hb;
+            const int4 de = __ldg(P.desc + gi);
+            const int2 kt = kts[de.y & 0xff];
+            const T2* cp = reinterpret_cast<const T2*>(P.ab) + de.x;
+            const T2* rp = RR + (kt.x & 0xffff);
             T al = (T)0, be = (T)0;
-            for (int s = 0; s < sk; ++s) {
-                const int64_t col = cb + (int64_t)s * dimp + h;
-                const T cc = wi * P.a[col * P.ab_stride] + vi * P.b[col * P.ab_stride];
-                al += cc * R1[fb + s];
-                be += cc * R2[fb + s];
+#pragma unroll 4
+            for (int s = 0; s < kt.x >> 16; ++s) {
+                const T2 c2 = __ldg(cp + (int64_t)s * kt.y), r2 = rp[s];
+                const T cc = wi * c2.x + vi * c2.y;
+                al += cc * r2.x;
+                be += cc * r2.y;
             }
-            const int16_t* ch = P.chains + (int64_t)gi * P.cstride;
-            const int tmu = ch[levels];
+            const T4 tg = trig[de.y >> 8];
+            int of[kMaxD] = {de.z & 0xffff, (int)((unsigned)de.z >> 16), de.w & 0xffff, (int)((unsigned)de.w >> 16)};
+            if constexpr (levels > 4) {
+                const int e2 = __ldg(P.desc2 + gi);
+                of[4] = e2 & 0xffff;
+                of[5] = (int)((unsigned)e2 >> 16);
+            }
             T pvv[kMaxD], pzz[kMaxD], pqq[kMaxD];
 #pragma unroll
             for (int j = 0; j < levels; ++j) {
-                pvv[j] = tv[j * P.tri + ch[j]];
-                pzz[j] = tz[j * P.tri + ch[j]];
-                pqq[j] = tq[j * P.tri + ch[j]];
+                const T4 w = tb[j * P.tri + of[j]];
+                pvv[j] = w.x;
+                pzz[j] = w.y;
+                pqq[j] = w.z;
             }
             // suffix products suf[j] = prod_{j2 > j} P_j2, so that the product of all level
             // factors but one is (trig * prefix) * suffix: O(levels) per harmonic
@@ -345,7 +386,7 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
 #pragma unroll
             for (int j = levels - 2; j >= 0; --j) suf[j] = suf[j + 1] * pvv[j + 1];
             const T pl = (levels > 0) ? pvv[0] * suf[0] : (T)1;      // all level factors
-            const T tr = trig[P.L + tmu];
+            const T tr = tg.x;
             const T prod = tr * pl;
             // Y x_hat term
 #pragma unroll
@@ -364,8 +405,8 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                     if (m <= D) g[m] += cq * xt[m];
             }
             // grad H: trigonometric factor
-            g[0] += be * pl * trx[P.L + tmu];
-            g[1] += be * pl * try_[P.L + tmu];
+            g[0] += be * pl * tg.y;
+            g[1] += be * pl * tg.z;
         }
 #pragma unroll
         for (int m = 0; m < DD; ++m) {
@@ -383,6 +424,7 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
             *dst = P.accumulate ? *dst + out : out;
         }
         __syncwarp();
+        }
     }
 }
 
@@ -449,10 +491,8 @@ hdf_status run(hdf_factor* f, const double* x, const T* V, int64_t ldv, const T*
         return HDF_OK;
     }
     DevBuf ab, zd, vw;
-    HDF_CUDA(ab.alloc(sizeof(T) * (size_t)r * ncols * 2));
+    HDF_CUDA(ab.alloc_on(sizeof(T) * (size_t)r * ncols * 2, st));
     HDF_CUDA(zd.alloc_on(sizeof(double) * (size_t)r * ncols * 2, st));
-    T* a = ab.as<T>();                         // S U^T V  (r x ncols)
-    T* b = a + (size_t)r * ncols;              // S U^T W
     // U^T [V W] (FP64, r x 2 ncols row-major) in one pass over U when the 2 ncols columns fit
     // one group: [V W] is gathered into an n x 2 ncols column-major block first
     std::vector<double> hz((size_t)r * ncols * 2);
@@ -483,19 +523,18 @@ hdf_status run(hdf_factor* f, const double* x, const T* V, int64_t ldv, const T*
             }
     }
     HDF_CUDA(cudaStreamSynchronize(st));
-    std::vector<T> ha((size_t)r * ncols), hb((size_t)r * ncols);
+    std::vector<T> hab((size_t)r * ncols * 2);     // per column of V: (S U^T v, S U^T w) of every column of U
     double fval = 0.0;
     for (int64_t col = 0; col < r; ++col)
         for (int j = 0; j < ncols; ++j) {
-            const size_t q = (size_t)col * ncols + j;
+            const size_t q = 2 * ((size_t)j * r + col);
             const double sc = P.Spad[col];
             const double zv = hz[(size_t)col * c2 + j], zw = hz[(size_t)col * c2 + ncols + j];
-            ha[q] = (T)(sc * zv);
-            hb[q] = (T)(sc * zw);
+            hab[q] = (T)(sc * zv);
+            hab[q + 1] = (T)(sc * zw);
             fval += zw * sc * zv;
         }
-    HDF_CUDA(cudaMemcpyAsync(a, ha.data(), sizeof(T) * ha.size(), cudaMemcpyHostToDevice, st));
-    HDF_CUDA(cudaMemcpyAsync(b, hb.data(), sizeof(T) * hb.size(), cudaMemcpyHostToDevice, st));
+    HDF_CUDA(cudaMemcpyAsync(ab.p, hab.data(), sizeof(T) * hab.size(), cudaMemcpyHostToDevice, st));
 
     AdjParams<T> A{};
     A.x = x;
@@ -508,26 +547,39 @@ hdf_status run(hdf_factor* f, const double* x, const T* V, int64_t ldv, const T*
     A.QC = P.dQC.as<float2>(); A.mtp = ((P.m[0] + P.m[1] + 7) / 8) * 8;
     if (sizeof(T) == 4 && A.QC == nullptr) return hdf::fail(HDF_EINVAL, "hdf_matvec_adjoint: factor lacks its FP32 radial tables");
     A.Wt = P.dW.as<T>(); A.colk = P.dcolk.as<uint8_t>(); A.nF = P.nF;
-    A.chains = P.dchains.as<int16_t>(); A.nH = P.nH; A.cstride = hdf::chain_stride(d);
-    A.hk = P.dhk.as<uint8_t>(); A.ktab = P.dktab.as<int>();
+    A.nH = P.nH; A.nk = P.L + 1; A.ktab = P.dktab.as<int>();
+    DevBuf dd;
+    HDF_CUDA(dd.alloc_on((sizeof(int4) + sizeof(int)) * (size_t)P.nH, st));
+    A.desc = dd.as<int4>();
+    A.desc2 = d >= 7 ? reinterpret_cast<const int*>(dd.as<int4>() + P.nH) : nullptr;
+    HDF_COUNT_LAUNCH();
+    k_adj_desc<<<(P.nH + 255) / 256, 256, 0, st>>>(P.dchains.as<int16_t>(), P.nH, hdf::chain_stride(d), d - 2, P.L_used,
+                                                   P.dhk.as<uint8_t>(), A.ktab, dd.as<int4>(), const_cast<int*>(A.desc2));
+    HDF_CUDA(cudaGetLastError());
     A.coefA = P.dA.as<T>(); A.coefB = P.dB.as<T>();
     A.grad = grad;
     const int levels = d - 2;
-    A.per_warp_d = 2 * (P.L + 1) + 2 * (P.m[0] + P.m[1]);
-    A.per_warp_t = ((2 * P.nF + 3 * levels * P.tri + 3 * (2 * P.L_used + 1)) + 3) & ~3;
-    const int warps = 4;
-    const size_t sm = sizeof(double) * warps * A.per_warp_d + sizeof(T) * warps * A.per_warp_t;
-    if (sm > 200 * 1024) return hdf::fail(HDF_ETOOBIG, "hdf_matvec_adjoint: per-point tables exceed shared memory");
-    void (*kern)(AdjParams<T>) = d == 3 ? k_adjoint<T, 3> : d == 4 ? k_adjoint<T, 4> : d == 5 ? k_adjoint<T, 5>
-                               : d == 6 ? k_adjoint<T, 6> : d == 7 ? k_adjoint<T, 7> : k_adjoint<T, 8>;
-    HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int nsm = 0, dv = 0, occ = 0;
     HDF_CUDA(cudaGetDevice(&dv));
     HDF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dv));
+    // the limit of four warps' tables without batches and padding
+    if (4 * (8 * (2 * ((size_t)P.L + 1) + 2 * (P.m[0] + P.m[1])) +
+             sizeof(T) * ((2 * (size_t)P.nF + 3 * levels * P.tri + 3 * (2 * P.L_used + 1) + 3) & ~(size_t)3)) >
+        200 * 1024)
+        return hdf::fail(HDF_ETOOBIG, "hdf_matvec_adjoint: per-point tables exceed shared memory");
+    // batches of up to kAdjBatch points while every SM has some 64 of them; as many warps per CTA as fit
+    A.nb = kAdjBatch;
+    while (A.nb > 1 && n < (int64_t)64 * nsm * A.nb) A.nb /= 2;
+    A.per_warp = (int)adj_per_warp<T>(levels, P.tri, P.L_used, P.nF, P.L, P.m[0] + P.m[1], A.nb);
+    const int warps = std::max(1, (int)std::min<size_t>(4, 220 * 1024 / (size_t)A.per_warp));
+    const size_t sm = (size_t)warps * A.per_warp;
+    void (*kern)(AdjParams<T>) = d == 3 ? k_adjoint<T, 3> : d == 4 ? k_adjoint<T, 4> : d == 5 ? k_adjoint<T, 5>
+                               : d == 6 ? k_adjoint<T, 6> : d == 7 ? k_adjoint<T, 7> : k_adjoint<T, 8>;
+    HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, sm));
-    const int grid = std::max(1, std::min<int>(nsm * std::max(occ, 1), (int)((n + warps - 1) / warps)));
+    const int grid = std::max(1, std::min<int>(nsm * std::max(occ, 1), (int)((n + warps * A.nb - 1) / (warps * A.nb))));
     for (int j = 0; j < ncols; ++j) {
-        A.a = a + j; A.b = b + j; A.ab_stride = ncols;
+        A.ab = ab.as<T>() + 2 * (size_t)j * r;
         A.v = V + j * ldv; A.w = Wv + j * ldw;
         A.accumulate = (j > 0);
         HDF_COUNT_LAUNCH();
