@@ -651,7 +651,8 @@ __global__ void __launch_bounds__(256) k_block_gemv(const double* __restrict__ i
 //   Cholesky A = L L^T, right-looking, per panel j: the diagonal tile is factored in shared
 //   memory and its inverse D_j = L_jj^-1 kept; L_ij = A_ij D_j^T for the tiles below; the
 //   trailing lower tiles A_ik -= L_ij L_kj^T;
-//   W = L^-1 by tile rows: W_ii = D_i, W_ij = -D_i sum_{j <= k < i} L_ik W_kj;
+//   W = L^-1: W_ii = D_i, W_ij = -D_i sum_{j <= k < i} L_ik W_kj, panel by panel on a second stream
+//   beside the factorization, whose diagonal tiles leave most SMs idle;
 //   A^-1 = W^T W, both triangles written.
 // A non-positive pivot sets *bad (the host reports HDF_ESINGULAR).
 constexpr int kST = 64;                 // tile edge
@@ -814,46 +815,64 @@ __global__ void __launch_bounds__(256) k_spd_update(SpdArgs P, int j) {
     spd_store(A, n, i, k, Cs, false);
 }
 
-// W = L^-1, tile row i (blockIdx.x = j <= i): W_ii = D_i, W_ij = -D_i sum_{j <= k < i} L_ik W_kj.
-__global__ void __launch_bounds__(256) k_spd_winv(SpdArgs P, int i) {
+// W = L^-1 by columns of L: row k is finished, W_kk = D_k, W_kj = -D_k S_kj (blockIdx.x = j <= k), and
+// then every S_ij below takes its term, S_ij += L_ik W_kj.  A tile product is 64^3 multiplications and
+// additions at two per clock and SM, 68 us; with the sum over k inside one block the last rows of the
+// largest cluster kept 16 blocks busy for 1.3 ms each (1,088 rows: 12.6 ms in all).
+__global__ void __launch_bounds__(256) k_spd_wrow(SpdArgs P, int k) {
     extern __shared__ double sh[];
     const int c = blockIdx.y;
     const int64_t n = spd_n(P, c);
     const int j = blockIdx.x;
-    if ((int64_t)i * kST >= n || j > i) return;
+    if ((int64_t)k * kST >= n) return;
+    double* W = P.W + P.ioff[c];
+    const double* D = P.D + P.doff[c] + (int64_t)k * kST * kST;
+    double* X = sh;
+    double* Y = sh + kST * kSP;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    for (int e = threadIdx.x; e < kST * kST; e += blockDim.x) X[(e / kST) * kSP + e % kST] = D[e];
+    if (j < k) {
+        spd_load(W, n, k, j, Y);
+        __syncthreads();
+        double out[4][4] = {};
+        spd_mma<false>(X, Y, out);
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) X[(4 * ty + a) * kSP + 4 * tx + b] = -out[a][b];
+    }
+    __syncthreads();
+    spd_store(W, n, k, j, X, false);
+}
+// The terms of row k; blockIdx.x enumerates (i > k, j <= k).
+__global__ void __launch_bounds__(256) k_spd_wupdate(SpdArgs P, int k) {
+    extern __shared__ double sh[];
+    const int c = blockIdx.y;
+    const int64_t n = spd_n(P, c);
+    const int i = k + 1 + (int)blockIdx.x / (k + 1), j = (int)blockIdx.x % (k + 1);
+    if ((int64_t)i * kST >= n) return;
     const double* A = P.A + P.ioff[c];
     double* W = P.W + P.ioff[c];
-    const double* D = P.D + P.doff[c] + (int64_t)i * kST * kST;
     double* X = sh;
     double* Y = sh + kST * kSP;
     double* Z = sh + 2 * kST * kSP;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    if (j == i) {
-        for (int e = threadIdx.x; e < kST * kST; e += blockDim.x) Z[(e / kST) * kSP + e % kST] = D[e];
-        __syncthreads();
-        spd_store(W, n, i, i, Z, false);
-        return;
-    }
-    double acc[4][4] = {};
-    for (int k = j; k < i; ++k) {           // S = sum_k L_ik W_kj
-        spd_load(A, n, i, k, X);
-        spd_load(W, n, k, j, Y);
-        __syncthreads();
-        spd_mma<false>(X, Y, acc);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b2 = 0; b2 < 4; ++b2) Y[(4 * ty + a) * kSP + 4 * tx + b2] = acc[a][b2];
-    for (int e = threadIdx.x; e < kST * kST; e += blockDim.x) X[(e / kST) * kSP + e % kST] = D[e];
+    spd_load(A, n, i, k, X);
+    spd_load(W, n, k, j, Y);
+    if (j < k) spd_load(W, n, i, j, Z);          // S_ik starts at zero
     __syncthreads();
-    double out[4][4] = {};
-    spd_mma<false>(X, Y, out);              // D_i S
+    double acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b2 = 0; b2 < 4; ++b2) Z[(4 * ty + a) * kSP + 4 * tx + b2] = -out[a][b2];
+        for (int b = 0; b < 4; ++b) acc[a][b] = j < k ? Z[(4 * ty + a) * kSP + 4 * tx + b] : 0.0;
+    spd_mma<false>(X, Y, acc);
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) Z[(4 * ty + a) * kSP + 4 * tx + b] = acc[a][b];
     __syncthreads();
     spd_store(W, n, i, j, Z, false);
 }
@@ -1159,6 +1178,9 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
                                             K->nclus, kernel, lengthscale, lambda, K->inv.as<double>());
         KRR_CUDA(cudaGetLastError());
     }
+    for (cudaEvent_t* e : {&K->cgev[0], &K->cgev[1], &K->fork, &K->join})
+        KRR_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    KRR_CUDA(cudaStreamCreateWithFlags(&K->side, cudaStreamNonBlocking));
     {
         // invert every block on the device (batched tiles; see k_spd_potrf and its siblings)
         int nbmax = 0;
@@ -1169,6 +1191,7 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
             doff[c + 1] = doff[c] + (int64_t)nb * kST * kST;
         }
         DevBuf W, D, ddoff, bad;
+        struct SideDone { cudaStream_t s; ~SideDone() { cudaStreamSynchronize(s); } } side_done{K->side};   // before W goes
         KRR_CUDA(W.alloc_on(sizeof(double) * std::max<int64_t>(1, K->ioff.back()), st));
         KRR_CUDA(D.alloc_on(sizeof(double) * std::max<int64_t>(1, doff.back()), st));
         KRR_CUDA(ddoff.alloc_on(sizeof(int64_t) * doff.size(), st));
@@ -1181,7 +1204,8 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         KRR_CUDA(cudaFuncSetAttribute(k_spd_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
         KRR_CUDA(cudaFuncSetAttribute(k_spd_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
         KRR_CUDA(cudaFuncSetAttribute(k_spd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_winv, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
+        KRR_CUDA(cudaFuncSetAttribute(k_spd_wrow, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
+        KRR_CUDA(cudaFuncSetAttribute(k_spd_wupdate, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
         KRR_CUDA(cudaFuncSetAttribute(k_spd_wtw, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
         const unsigned ncl = (unsigned)K->nclus;
         for (int j = 0; j < nbmax; ++j) {
@@ -1191,14 +1215,20 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
             if (nt > 0) {
                 HDF_COUNT_LAUNCH();
                 k_spd_trsm<<<dim3((unsigned)nt, ncl), 256, 2 * tile, st>>>(P, j);
+            }
+            KRR_CUDA(cudaEventRecord(K->fork, st));
+            KRR_CUDA(cudaStreamWaitEvent(K->side, K->fork, 0));
+            HDF_COUNT_LAUNCH();
+            k_spd_wrow<<<dim3((unsigned)(j + 1), ncl), 256, 2 * tile, K->side>>>(P, j);
+            if (nt > 0) {
+                HDF_COUNT_LAUNCH();
+                k_spd_wupdate<<<dim3((unsigned)(nt * (j + 1)), ncl), 256, 3 * tile, K->side>>>(P, j);
                 HDF_COUNT_LAUNCH();
                 k_spd_update<<<dim3((unsigned)(nt * (nt + 1) / 2), ncl), 256, 3 * tile, st>>>(P, j);
             }
         }
-        for (int i = 0; i < nbmax; ++i) {
-            HDF_COUNT_LAUNCH();
-            k_spd_winv<<<dim3((unsigned)(i + 1), ncl), 256, 3 * tile, st>>>(P, i);
-        }
+        KRR_CUDA(cudaEventRecord(K->join, K->side));
+        KRR_CUDA(cudaStreamWaitEvent(st, K->join, 0));
         HDF_COUNT_LAUNCH();
         k_spd_wtw<<<dim3((unsigned)(nbmax * (nbmax + 1) / 2), ncl), 256, 2 * tile, st>>>(P);
         KRR_CUDA(cudaGetLastError());
@@ -1227,9 +1257,6 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
     KRR_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
     KRR_CUDA(K->cgst.alloc(sizeof(CgState)));
     KRR_CUDA(cudaMallocHost(reinterpret_cast<void**>(&K->cgh), 2 * sizeof(CgState)));
-    for (cudaEvent_t* e : {&K->cgev[0], &K->cgev[1], &K->fork, &K->join})
-        KRR_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-    KRR_CUDA(cudaStreamCreateWithFlags(&K->side, cudaStreamNonBlocking));
     if (prec == HDF_FP32) {
         KRR_CUDA(K->vb.alloc(sizeof(float) * n));
         KRR_CUDA(K->yb.alloc(sizeof(float) * n));
