@@ -19,7 +19,7 @@
  *    (double for HDF_FP64, float for HDF_FP32).
  *  - Work is ordered on the given stream (NULL = legacy default stream).  hdf_build
  *    synchronises the stream (host planning needs device reductions); hdf_matvec is
- *    asynchronous; hdf_solve synchronises (its small core is solved on the host).
+ *    asynchronous; hdf_solve synchronises (the host reads the status of its core's factorization).
  *  - Supported: 3 <= d <= 8, n >= 1, tol in (0, 1), lengthscale > 0, p_max <= 128.
  */
 #ifndef HDF_H

@@ -215,7 +215,14 @@ void hdf_free(hdf_factor* f) {
         if (!g) continue;
         g->U.st = g->mf.Z.st = g->mf.A0F.st = g->plan.arena.st = nullptr;
     }
+    size_t freed = 0;
+    for (hdf_factor* g : {f, f->ypart})
+        if (g) freed += (g->U.p ? g->U.bytes : 0) + (g->mf.Z.p ? g->mf.Z.bytes + g->mf.A0F.bytes : 0);
     delete f;
+    // a block whose release is still pending does not join its neighbours: the next build's smaller
+    // blocks split it, and its U is mapped anew (1,000,000 points with 24 GB of rows, builds without
+    // a pause: 81 ms against 44)
+    if (freed > ((size_t)64 << 20)) cudaStreamSynchronize(nullptr);
 }
 
 hdf_status hdf_device_errors(const hdf_factor* f, int* flag) {
