@@ -1853,7 +1853,9 @@ void hdf_batch_free(hdf_batch* b) {
     for (DevBuf* d : {&b->U, &b->S, &b->arena, &b->dsets, &b->mvsets, &b->mvitems_utv, &b->mvitems_red,
                       &b->mvitems_uw, &b->mvpart, &b->mvW, &b->counters})
         d->st = nullptr;
+    const size_t freed = b->U.p ? b->U.bytes : 0;
     delete b;
+    if (freed > ((size_t)64 << 20)) cudaStreamSynchronize(nullptr);      // as hdf_free
 }
 
 }  // extern "C"
