@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/hdf.h"
+#include "cg_state.h"
 #include "hdf_kernels.cuh"
 #include "internal.h"
 #include "planner.h"
@@ -501,17 +502,11 @@ __global__ void k_to_f64(const float* __restrict__ v, int64_t n, double* __restr
 }
 
 // ----------------------------------------------- conjugate gradients on the device
-// One iteration is a fixed chain of kernels; its scalars live in CgState, so that the host reads
-// the state only every few iterations.  At 13,760 points an iteration went from 0.85 ms (0.43 the
-// off-diagonal blocks, 0.57 + 0.11 the HDF blocks partly hidden, two host round trips) to 0.16 ms.  Iteration it reads
-// rz[it & 1] and writes rz[(it + 1) & 1].  After `done` every kernel returns at once, so iterations enqueued past the end change nothing.  Every
-// block adds the partial sums of a dot product itself, in the same fixed order.
-struct CgState {
-    double rz[2];
-    double nb, rtol;             // norm of the right-hand side
-    double res;                  // relative residual after iteration `it`
-    int it, done, bad;           // bad: p . q <= 0
-};
+// One iteration is a fixed chain of kernels; its scalars live in CgState (cg_state.h), so that the
+// host reads the state only every few iterations.  At 13,760 points an iteration went from 0.85 ms
+// (0.43 the off-diagonal blocks, 0.57 + 0.11 the HDF blocks partly hidden, two host round trips) to
+// 0.16 ms.  Kernels of an iteration after the last return at once, so iterations enqueued past the end
+// change nothing.  Every block adds the partial sums of a dot product itself, in the same fixed order.
 
 // Sum of m values v[stride e + off] by a 256-thread block, the same on every block and thread.
 __device__ __forceinline__ double block_total(const double* __restrict__ v, int m, int stride, int off, double* sh) {
@@ -529,7 +524,7 @@ __global__ void __launch_bounds__(256) k_cg_init(const double* __restrict__ part
         S->nb = sqrt(bb); S->rtol = rtol;
         S->res = bb > 0.0 ? 1.0 : 0.0;
         S->it = 0; S->bad = 0;
-        S->done = !(bb > 0.0);
+        S->last = bb > 0.0 ? kCgRunning : 0;
     }
 }
 
@@ -539,9 +534,9 @@ template <bool SYM>
 __global__ void __launch_bounds__(256) k_cg_finish(const double* __restrict__ part, int nsplit, int64_t n, double lam,
                                                    const double* __restrict__ p, const double* __restrict__ add,
                                                    double* __restrict__ q, double* __restrict__ dot,
-                                                   const CgState* __restrict__ S) {
+                                                   int it, const CgState* __restrict__ S) {
     __shared__ double sh[8][32];
-    if (S->done) return;
+    if (cg_past_end(S->last, it)) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int64_t i = blockIdx.x * (int64_t)32 + tx;
     sh[ty][tx] = i < n ? part_sum<SYM>(part, nsplit, n, i, ty) : 0.0;
@@ -565,10 +560,10 @@ __global__ void __launch_bounds__(256) k_cg_step(double* __restrict__ x, double*
                                                  const double* __restrict__ p, const double* __restrict__ q, int64_t n,
                                                  const double* __restrict__ dot, int m, int it, CgState* S) {
     __shared__ double sh[256];
-    if (S->done) return;
+    if (cg_past_end(S->last, it)) return;
     const double pq = block_total(dot, m, 1, 0, sh);
     if (!(pq > 0.0)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) { S->bad = 1; S->it = it; S->done = 1; }
+        if (blockIdx.x == 0 && threadIdx.x == 0) { S->bad = 1; S->it = it; S->last = it; }
         return;
     }
     const double alpha = S->rz[(it - 1) & 1] / pq;
@@ -582,7 +577,7 @@ __global__ void __launch_bounds__(256) k_cg_step(double* __restrict__ x, double*
 __global__ void __launch_bounds__(256) k_cg_dir(double* __restrict__ p, const double* __restrict__ z, int64_t n,
                                                 const double* __restrict__ dot, int m, int it, CgState* S) {
     __shared__ double sh[256];
-    if (S->done) return;
+    if (cg_past_end(S->last, it)) return;
     const double rz = block_total(dot, m, 2, 0, sh), rr = block_total(dot, m, 2, 1, sh);
     const double res = sqrt(rr) / S->nb;
     const bool end = res <= S->rtol;
@@ -590,7 +585,7 @@ __global__ void __launch_bounds__(256) k_cg_dir(double* __restrict__ p, const do
         S->res = res;
         S->it = it;
         S->rz[it & 1] = rz;
-        if (end) S->done = 1;
+        if (end) S->last = it;
     }
     const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
     if (!end && i < n) p[i] = z[i] + rz / S->rz[(it - 1) & 1] * p[i];
@@ -614,13 +609,14 @@ __global__ void k_block_matrices(const double* __restrict__ xp, int d, const int
 
 // z = M r: one warp per row of the block-diagonal inverse (packed as above), four loads in flight
 // per lane (13,760 rows of about 660 entries 31 us, of which the FP64 pipe takes 20; two rows per warp
-// 31, four 36).  With dot (and a state that is not done): (r . z, r . r) of the block's rows as well.
+// 31, four 36).  With dot (and an iteration that is not past the end): (r . z, r . r) of the block's
+// rows as well.
 __global__ void __launch_bounds__(256) k_block_gemv(const double* __restrict__ inv, const int64_t* __restrict__ offs,
                                                     const int64_t* __restrict__ ioff, const int* __restrict__ cl,
                                                     int64_t n, const double* __restrict__ r, double* __restrict__ z,
-                                                    double* __restrict__ dot, const CgState* __restrict__ S) {
+                                                    double* __restrict__ dot, int it, const CgState* __restrict__ S) {
     __shared__ double sh[2][8];
-    if (S && S->done) return;
+    if (S && cg_past_end(S->last, it)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t row = blockIdx.x * (int64_t)8 + warp;
     double s = 0.0, rv = 0.0;
@@ -1009,11 +1005,11 @@ hdf_status apply_perm(hdf_krr* K, const double* vp, double* tp, cudaStream_t st)
 }
 
 hdf_status precond_perm(hdf_krr* K, const double* rp, double* zp, cudaStream_t st, double* dot = nullptr,
-                        const CgState* S = nullptr) {
+                        int it = 0, const CgState* S = nullptr) {
     HDF_COUNT_LAUNCH();
     k_block_gemv<<<(unsigned)((K->n + 7) / 8), 256, 0, st>>>(K->inv.as<double>(), K->doffs.as<int64_t>(),
                                                              K->dioff.as<int64_t>(), K->cl.as<int>(), K->n, rp, zp, dot,
-                                                             S);
+                                                             it, S);
     HDF_CUDA(cudaGetLastError());
     return HDF_OK;
 }
@@ -1330,7 +1326,7 @@ hdf_status hdf_krr_solve(hdf_krr* K, const double* y_dev, double rtol, int max_i
         HDF_CUDA(cudaEventRecord(K->cgev[polls & 1], st));
         if (polls > 0) {
             HDF_CUDA(cudaEventSynchronize(K->cgev[(polls - 1) & 1]));
-            done = K->cgh[(polls - 1) & 1].done != 0;
+            done = K->cgh[(polls - 1) & 1].last != kCgRunning;
         }
         ++polls;
         return HDF_OK;
@@ -1341,11 +1337,11 @@ hdf_status hdf_krr_solve(hdf_krr* K, const double* y_dev, double rtol, int max_i
         if (done) break;
         if (hdf_status s = apply_parts(K, p, st); s != HDF_OK) return s;
         HDF_COUNT_LAUNCH();
-        finish<<<gf, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, p, K->hd.as<double>(), q, dot, S);
+        finish<<<gf, 256, 0, st>>>(K->part.as<double>(), K->S, n, K->lam, p, K->hd.as<double>(), q, dot, it, S);
         HDF_COUNT_LAUNCH();
         k_cg_step<<<gb, 256, 0, st>>>(x, r, p, q, n, dot, gf, it, S);
         HDF_CUDA(cudaGetLastError());
-        if (hdf_status s = precond_perm(K, r, z, st, dot, S); s != HDF_OK) return s;
+        if (hdf_status s = precond_perm(K, r, z, st, dot, it, S); s != HDF_OK) return s;
         HDF_COUNT_LAUNCH();
         k_cg_dir<<<gb, 256, 0, st>>>(p, z, n, dot, mgemv, it, S);
         HDF_CUDA(cudaGetLastError());
