@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -1110,7 +1111,9 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
     std::vector<int64_t> cnt((size_t)lmax + 1, 0);
     for (int64_t i = 0; i < n; ++i) cnt[lab[i]]++;
     std::vector<int> remap((size_t)lmax + 1, -1);
-    hdf_krr* K = new hdf_krr();
+    // the locals below (work space of both streams and the guard that waits for them) go before the model
+    std::unique_ptr<hdf_krr> model(new hdf_krr());
+    hdf_krr* K = model.get();
     K->n = n; K->d = d; K->prec = prec; K->kernel = kernel; K->ell = lengthscale; K->lam = lambda;
     K->offs.push_back(0);
     for (int c = 0; c <= lmax; ++c)
@@ -1123,34 +1126,26 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         perm[pos[c]] = i;
         clp[pos[c]++] = c;
     }
-    auto bail = [&](hdf_status s) { delete K; return s; };
     hdf_status s = HDF_OK;
-#define KRR_CUDA(call)                                                                            \
-    do {                                                                                          \
-        cudaError_t e_ = (call);                                                                  \
-        if (e_ != cudaSuccess)                                                                    \
-            return bail(fail(e_ == cudaErrorMemoryAllocation ? HDF_ENOMEM : HDF_ECUDA,                \
-                             std::string(#call) + ": " + cudaGetErrorString(e_)));                    \
-    } while (0)
-    KRR_CUDA(K->perm.alloc(sizeof(int64_t) * n));
-    KRR_CUDA(K->xp.alloc(sizeof(double) * n * d));
-    KRR_CUDA(K->xp32.alloc(sizeof(float) * n * d));
-    KRR_CUDA(K->cl.alloc(sizeof(int) * n));
-    KRR_CUDA(K->doffs.alloc(sizeof(int64_t) * K->offs.size()));
-    KRR_CUDA(cudaMemcpyAsync(K->perm.p, perm.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-    KRR_CUDA(cudaMemcpyAsync(K->cl.p, clp.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
-    KRR_CUDA(cudaMemcpyAsync(K->doffs.p, K->offs.data(), sizeof(int64_t) * K->offs.size(), cudaMemcpyHostToDevice, st));
+    HDF_CUDA(K->perm.alloc(sizeof(int64_t) * n));
+    HDF_CUDA(K->xp.alloc(sizeof(double) * n * d));
+    HDF_CUDA(K->xp32.alloc(sizeof(float) * n * d));
+    HDF_CUDA(K->cl.alloc(sizeof(int) * n));
+    HDF_CUDA(K->doffs.alloc(sizeof(int64_t) * K->offs.size()));
+    HDF_CUDA(cudaMemcpyAsync(K->perm.p, perm.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
+    HDF_CUDA(cudaMemcpyAsync(K->cl.p, clp.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
+    HDF_CUDA(cudaMemcpyAsync(K->doffs.p, K->offs.data(), sizeof(int64_t) * K->offs.size(), cudaMemcpyHostToDevice, st));
     HDF_COUNT_LAUNCH();
     k_gather_rows<<<blocks_for(n * d, 256, 1 << 30), 256, 0, st>>>(x_dev, d, K->perm.as<int64_t>(), n, K->xp.as<double>());
     HDF_COUNT_LAUNCH();
     k_shift_f32<<<blocks_for(n * d, 256, 1 << 30), 256, 0, st>>>(K->xp.as<double>(), n, d, K->xp.as<double>(),
                                                                  K->xp32.as<float>());
-    KRR_CUDA(cudaGetLastError());
+    HDF_CUDA(cudaGetLastError());
     // HDF factors of the diagonal blocks: one batched build over the clusters
     std::vector<double> ells(K->nclus, lengthscale);
     s = hdf_build_batched(K->nclus, K->offs.data(), K->xp.as<double>(), d, kernel, ells.data(), tol, prec, opt, stream,
                           &K->batch);
-    if (s != HDF_OK && s != HDF_ETOL_UNREACHABLE) return bail(s);
+    if (s != HDF_OK && s != HDF_ETOL_UNREACHABLE) return s;
     const hdf_status build_status = s;
     K->t_build = wall_ms() - t0;
     // block preconditioner: exact blocks, inverted on the device (Cholesky, FP64)
@@ -1161,10 +1156,10 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         K->ioff[c + 1] = K->ioff[c] + nc * nc;
     }
     if (K->ioff.back() > ((int64_t)1 << 28))
-        return bail(fail(HDF_ETOOBIG, "hdf_krr_build: sum of squared cluster sizes > 2^28 (block preconditioner)"));
-    KRR_CUDA(K->dioff.alloc(sizeof(int64_t) * K->ioff.size()));
-    KRR_CUDA(cudaMemcpyAsync(K->dioff.p, K->ioff.data(), sizeof(int64_t) * K->ioff.size(), cudaMemcpyHostToDevice, st));
-    KRR_CUDA(K->inv.alloc(sizeof(double) * std::max<int64_t>(1, K->ioff.back())));
+        return fail(HDF_ETOOBIG, "hdf_krr_build: sum of squared cluster sizes > 2^28 (block preconditioner)");
+    HDF_CUDA(K->dioff.alloc(sizeof(int64_t) * K->ioff.size()));
+    HDF_CUDA(cudaMemcpyAsync(K->dioff.p, K->ioff.data(), sizeof(int64_t) * K->ioff.size(), cudaMemcpyHostToDevice, st));
+    HDF_CUDA(K->inv.alloc(sizeof(double) * std::max<int64_t>(1, K->ioff.back())));
     {
         int64_t nmax = 0;
         for (int c = 0; c < K->nclus; ++c) nmax = std::max(nmax, K->offs[c + 1] - K->offs[c]);
@@ -1172,11 +1167,11 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         HDF_COUNT_LAUNCH();
         k_block_matrices<<<g, 256, 0, st>>>(K->xp.as<double>(), d, K->doffs.as<int64_t>(), K->dioff.as<int64_t>(),
                                             K->nclus, kernel, lengthscale, lambda, K->inv.as<double>());
-        KRR_CUDA(cudaGetLastError());
+        HDF_CUDA(cudaGetLastError());
     }
     for (cudaEvent_t* e : {&K->cgev[0], &K->cgev[1], &K->fork, &K->join})
-        KRR_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-    KRR_CUDA(cudaStreamCreateWithFlags(&K->side, cudaStreamNonBlocking));
+        HDF_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    HDF_CUDA(cudaStreamCreateWithFlags(&K->side, cudaStreamNonBlocking));
     {
         // invert every block on the device (batched tiles; see k_spd_potrf and its siblings)
         int nbmax = 0;
@@ -1188,21 +1183,21 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         }
         DevBuf W, D, ddoff, bad;
         struct SideDone { cudaStream_t s; ~SideDone() { cudaStreamSynchronize(s); } } side_done{K->side};   // before W goes
-        KRR_CUDA(W.alloc_on(sizeof(double) * std::max<int64_t>(1, K->ioff.back()), st));
-        KRR_CUDA(D.alloc_on(sizeof(double) * std::max<int64_t>(1, doff.back()), st));
-        KRR_CUDA(ddoff.alloc_on(sizeof(int64_t) * doff.size(), st));
-        KRR_CUDA(bad.alloc_on(sizeof(int), st));
-        KRR_CUDA(cudaMemcpyAsync(ddoff.p, doff.data(), sizeof(int64_t) * doff.size(), cudaMemcpyHostToDevice, st));
-        KRR_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), st));
+        HDF_CUDA(W.alloc_on(sizeof(double) * std::max<int64_t>(1, K->ioff.back()), st));
+        HDF_CUDA(D.alloc_on(sizeof(double) * std::max<int64_t>(1, doff.back()), st));
+        HDF_CUDA(ddoff.alloc_on(sizeof(int64_t) * doff.size(), st));
+        HDF_CUDA(bad.alloc_on(sizeof(int), st));
+        HDF_CUDA(cudaMemcpyAsync(ddoff.p, doff.data(), sizeof(int64_t) * doff.size(), cudaMemcpyHostToDevice, st));
+        HDF_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), st));
         SpdArgs P{K->inv.as<double>(), W.as<double>(), D.as<double>(), K->doffs.as<int64_t>(),
                   K->dioff.as<int64_t>(), ddoff.as<int64_t>(), bad.as<int>()};
         const int tile = (int)(sizeof(double) * kST * kSP);
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_wrow, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_wupdate, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
-        KRR_CUDA(cudaFuncSetAttribute(k_spd_wtw, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_update, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_wrow, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_wupdate, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * tile));
+        HDF_CUDA(cudaFuncSetAttribute(k_spd_wtw, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * tile));
         const unsigned ncl = (unsigned)K->nclus;
         for (int j = 0; j < nbmax; ++j) {
             HDF_COUNT_LAUNCH();
@@ -1212,8 +1207,8 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
                 HDF_COUNT_LAUNCH();
                 k_spd_trsm<<<dim3((unsigned)nt, ncl), 256, 2 * tile, st>>>(P, j);
             }
-            KRR_CUDA(cudaEventRecord(K->fork, st));
-            KRR_CUDA(cudaStreamWaitEvent(K->side, K->fork, 0));
+            HDF_CUDA(cudaEventRecord(K->fork, st));
+            HDF_CUDA(cudaStreamWaitEvent(K->side, K->fork, 0));
             HDF_COUNT_LAUNCH();
             k_spd_wrow<<<dim3((unsigned)(j + 1), ncl), 256, 2 * tile, K->side>>>(P, j);
             if (nt > 0) {
@@ -1223,15 +1218,15 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
                 k_spd_update<<<dim3((unsigned)(nt * (nt + 1) / 2), ncl), 256, 3 * tile, st>>>(P, j);
             }
         }
-        KRR_CUDA(cudaEventRecord(K->join, K->side));
-        KRR_CUDA(cudaStreamWaitEvent(st, K->join, 0));
+        HDF_CUDA(cudaEventRecord(K->join, K->side));
+        HDF_CUDA(cudaStreamWaitEvent(st, K->join, 0));
         HDF_COUNT_LAUNCH();
         k_spd_wtw<<<dim3((unsigned)(nbmax * (nbmax + 1) / 2), ncl), 256, 2 * tile, st>>>(P);
-        KRR_CUDA(cudaGetLastError());
+        HDF_CUDA(cudaGetLastError());
         int hbad = 0;
-        KRR_CUDA(cudaMemcpyAsync(&hbad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        KRR_CUDA(cudaStreamSynchronize(st));
-        if (hbad) return bail(fail(HDF_ESINGULAR, "hdf_krr_build: a block lambda I + K_cc is not positive definite"));
+        HDF_CUDA(cudaMemcpyAsync(&hbad, bad.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+        HDF_CUDA(cudaStreamSynchronize(st));
+        if (hbad) return fail(HDF_ESINGULAR, "hdf_krr_build: a block lambda I + K_cc is not positive definite");
     }
     // work space
     // the off-diagonal blocks are stored while they take at most 8 GiB (65,000 points) and the
@@ -1242,25 +1237,24 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         HDF_COUNT_LAUNCH();
         launch_off_store(d, st, K->xp32.as<float>(), n, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
                          K->koff.as<float>());
-        KRR_CUDA(cudaGetLastError());
+        HDF_CUDA(cudaGetLastError());
     } else {
         cudaGetLastError();
         K->split = direct_split(n, n, &K->S);
         nparts = (size_t)K->S * n;
     }
-    KRR_CUDA(K->part.alloc(sizeof(double) * nparts));
-    KRR_CUDA(K->hd.alloc(sizeof(double) * n));
-    KRR_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
-    KRR_CUDA(K->cgst.alloc(sizeof(CgState)));
-    KRR_CUDA(cudaMallocHost(reinterpret_cast<void**>(&K->cgh), 2 * sizeof(CgState)));
+    HDF_CUDA(K->part.alloc(sizeof(double) * nparts));
+    HDF_CUDA(K->hd.alloc(sizeof(double) * n));
+    HDF_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
+    HDF_CUDA(K->cgst.alloc(sizeof(CgState)));
+    HDF_CUDA(cudaMallocHost(reinterpret_cast<void**>(&K->cgh), 2 * sizeof(CgState)));
     if (prec == HDF_FP32) {
-        KRR_CUDA(K->vb.alloc(sizeof(float) * n));
-        KRR_CUDA(K->yb.alloc(sizeof(float) * n));
+        HDF_CUDA(K->vb.alloc(sizeof(float) * n));
+        HDF_CUDA(K->yb.alloc(sizeof(float) * n));
     }
-    KRR_CUDA(cudaStreamSynchronize(st));
+    HDF_CUDA(cudaStreamSynchronize(st));
     K->t_precond = wall_ms() - t1;
-#undef KRR_CUDA
-    *out = K;
+    *out = model.release();
     return build_status;
 }
 
