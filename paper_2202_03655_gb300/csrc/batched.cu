@@ -1588,11 +1588,13 @@ static hdf_status batch_matvec_t(hdf_batch* b, const T* V, int64_t ldv, int c, T
             ms[s].n = n; ms[s].r = r; ms[s].ldU = b->info[s].ldu; ms[s].off = b->off[s];
             ms[s].chunk = few ? few_chunk(n) : 4096;
             ms[s].nchunk = (int)std::max<int64_t>(1, (n + ms[s].chunk - 1) / ms[s].chunk);
+            // r is 0 or a multiple of 8, so every set's sums and W start on 16 bytes whatever c and the
+            // chunk counts are: the streaming kernels read and write them in pairs and quads
             poff[s] = ptot;
-            ptot += (int64_t)ms[s].nchunk * c * std::max<int64_t>(1, r);
+            ptot += (int64_t)ms[s].nchunk * c * r;
             woff[s] = wtot;
             ms[s].ldw = skinny ? ct : c;
-            wtot += std::max<int64_t>(1, r) * ms[s].ldw;
+            wtot += r * ms[s].ldw;
             if (r == 0) continue;
             for (int q = 0; q < ms[s].nchunk; ++q)
                 for (int64_t bl = 0; bl < (r + AB - 1) / AB; ++bl) iu.push_back({s, q, bl});
