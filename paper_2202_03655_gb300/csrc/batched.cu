@@ -1689,6 +1689,9 @@ static hdf_status batch_matvec_t(hdf_batch* b, const T* V, int64_t ldv, int c, T
         }
         HDF_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
         cudaMemsetAsync(b->counters.p, 0, sizeof(int) * 2, b->cap);
+        for (int s = 0; s < ns; ++s)      // sets without columns: no item writes their rows
+            if (b->info[s].rank == 0)
+                cudaMemset2DAsync(Y + b->off[s], sizeof(T) * ldy, 0, sizeof(T) * b->info[s].n, c, b->cap);
         const MvSet* S = b->mvsets.as<MvSet>();
         int* cnt = b->counters.as<int>();
         if (skinny) {

@@ -39,3 +39,17 @@ def test_sets_with_columns(prec, eps):
             ref = U @ (S[:, None] * (U.T @ v))
             bound = 4 * (hi - lo) * eps * (U.abs() @ (S.abs()[:, None] * (U.abs().T @ v.abs())))
             assert bool(((Y[lo:hi].double() - ref).abs() <= bound).all()), (c, s)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_sets_without_columns_give_zero(prec):
+    import torch
+    b, x, off = batch(prec)
+    n, dt = int(off[-1]), torch.float64 if prec == "fp64" else torch.float32
+    for c in (1, 3, 8, 17):
+        V = torch.ones(c, n, dtype=dt, device="cuda")
+        Y = torch.full((c, n + 3), 7.0, dtype=dt, device="cuda")       # longer columns than the points
+        b.matvec_ptr(V.data_ptr(), n, c, Y.data_ptr(), n + 3)
+        for s, (lo, hi) in enumerate(zip(off[:-1], off[1:])):
+            assert bool((Y[:, lo:hi] == 0.0).all()) == (ELLS[s] == 30.0), (c, s)
+        assert bool((Y[:, n:] == 7.0).all())
