@@ -16,11 +16,13 @@
 // products of levels l = i + j into the FP32 accumulators of the levels l = i .. 7; a level sums at
 // most 7 x 64 products below 2^15, less than 2^24, so every FP32 sum is an exact integer.  The
 // products of level > 7 are dropped (2^-63 of the block's largest product each; without level 7,
-// dropping 2^-55, the error grew by half).  The promotion warps add the levels as one 64-bit
-// integer, round it once to FP64 with the two exponents, and add it to an FP64 register sum: one
-// FP64 rounding per block where the multiply-add chain rounds 64 times.  Error against extended
-// precision at 2,000 x 431, 1,500 x 10,064 and 3,001 x 1,960: 2.5 to 4.5e-16 relative, the
-// register-tiled FP64 kernels 1.0 to 4.9e-15.
+// dropping 2^-55, the error grew by half).  The promotion warps add the levels as one 64-bit integer
+// in units of 2^-54 of the block's bound (levels 6 and 7 rounded into it), round it to FP64 with the
+// two exponents, and add it to an FP64 register sum: two roundings per block where the multiply-add
+// chain rounds 64 times.  Error against extended precision at 2,000 x 431, 1,500 x 10,064 and 3,001 x
+// 1,960: 2.5 to 3.4e-16 relative (3.3 to 4.5e-16 while levels 6 and 7 were cut off instead of
+// rounded), the streaming kernels of few_cols.cuh 1.9 to 3.5e-16, the register-tiled FP64 kernels 1.0
+// to 4.8e-15.
 //
 // Why this split.  What bounds the kernel is the ALU pipe (64 lanes per clock and SM) of the
 // converters and the promotion, then the read of U.  Splitting and packing a value takes about 14
@@ -272,13 +274,17 @@ __device__ __noinline__ double level_sum_slow(uint64_t m, bool neg, int eab) {
     return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
-// The values of the levels of four columns: sum_l L_l 256^(6 - l) 2^(eab - 2154 + 48), eab = ea + eb, each rounded once to FP64 and added to acc.  The accumulators hold L_l 2^-24.  A unit of
-// level l is 2^(-14 - 8 l) of the block's largest product.  Levels 0 and 1 (below 2^22) are read off
-// an FP32 sum with 1.5 2^23, levels 2-5 (below 2^24) are converted (16 conversions per clock and
-// SM, so not all seven), and level 6 is read off a sum with 1.5 2^25, to a unit of 4 (2^-60), after taking in level 7.  One
-// branch for the special results of all four columns, so that their chains overlap.
+// The values of the levels of four columns: sum_l L_l 256^(6 - l) 2^(eab - 2154 + 48), eab = ea + eb,
+// in units of level 5 (2^-54 of the block's bound), each rounded to FP64 and added to acc.  The
+// accumulators hold L_l 2^-24.  A unit of level l is 2^(-14 - 8 l) of the block's largest product.
+// Levels 0 and 1 (below 2^22) are read off an FP32 sum with 1.5 2^23, levels 2-5 (below 2^24) are
+// converted (16 conversions per clock and SM, so not all seven), and level 6, after taking in level 7,
+// is read off a sum with 1.5 2^25 to a unit of 4; the sum starts at half a unit of level 5, so that the
+// shift by which level 6 enters level 5 rounds.  (Without that half it cut off towards minus infinity,
+// every block short by half a unit on average: an error of one sign that grew with the number of
+// blocks.)  One branch for the special results of all four columns, so that their chains overlap.
 __device__ __forceinline__ void level_sums(const uint32_t* L, const int* eab, double* acc) {
-    constexpr float SC = 16777216.f, M1 = 12582912.f, M4 = 50331648.f;
+    constexpr float SC = 16777216.f, M1 = 12582912.f, M4 = 50331648.f + 128.f;
     constexpr uint32_t B1 = 0x4B400000u, B4 = 0x4C400000u;
     uint32_t hi[4], lo[4], sg[4];
     double out[4];
@@ -293,7 +299,7 @@ __device__ __forceinline__ void level_sums(const uint32_t* L, const int* eab, do
         const int l5 = __float2int_rn(__uint_as_float(L[20 + v]) * SC);
         const float x6 = fmaf(__uint_as_float(L[28 + v]), 1.f / 256.f, __uint_as_float(L[24 + v]));
         const uint32_t l6 = __float_as_uint(fmaf(x6, SC, M4));
-        // in units of 256 level-6 units: |T| < 2^62 (bits of l6: a quarter of level 6)
+        // in units of 256 level-6 units: |T| < 2^62 (bits of l6: a quarter of level 6, plus 32)
         int64_t T = (int64_t)((int)((l6 >> 6) - (B4 >> 6)) + l5);
         T += (int64_t)l4 * 256;
         T += (int64_t)l3 * 65536;
