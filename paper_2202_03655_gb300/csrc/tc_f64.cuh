@@ -105,7 +105,7 @@ struct Args {
     int kper;                // blocks per item (the last item of a row of items may have fewer)
     int mblocks;             // U^T V: 128-column blocks; U W: 128-row tiles
     int c;                   // columns of this call (<= ncg CP)
-    const int* eb;           // exponents of the small operand: [block][ncg CP]
+    const int* eb;           // exponents of the small operand (special_exponent): [block][ncg CP]
     double alpha, beta;
     const double* B; int64_t ldb;
     double* Y; int64_t ldy;  // U W: the result (null: write slices to part)
@@ -208,7 +208,8 @@ __device__ __forceinline__ uint32_t byte_pair(uint64_t a, uint64_t b, uint32_t s
 }
 
 // Exponent of a block from the largest |x| bit pattern's high word: below 2^-959 a block counts
-// as zero (exponent 0).
+// as zero (exponent 0): on U's side as it is (its other entries decide every sum there), while the small
+// operand is scaled first.
 __device__ __forceinline__ uint32_t block_exponent(uint32_t hmax) {
     const uint32_t e = hmax >> 20;
     return e < 64u ? 0u : e;
@@ -216,7 +217,9 @@ __device__ __forceinline__ uint32_t block_exponent(uint32_t hmax) {
 
 // Slices of the small operand: value(k, col) for K index k and column col < c, zero beyond kn and
 // c, for cp columns (whole groups).  One warp per (64-deep block, column): lane l takes k = 2 l and
-// 2 l + 1.  out[((col / 16 * 7 + slice) 16 + col mod 16) kpad + k], eb[block cp + col].
+// 2 l + 1.  out[((col / 16 * 7 + slice) 16 + col mod 16) kpad + k], eb[block cp + col] (as level_sums
+// takes it).  A block below 2^-959 is multiplied by 2^256 first, which is exact for subnormal numbers
+// too, so that a column of any scale keeps its digits.
 template <typename F>
 __device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int cp, int64_t kpad, __half* out, int* eb) {
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -225,13 +228,22 @@ __device__ __forceinline__ void prep_block(F value, int64_t kn, int c, int cp, i
     const int col = (int)(wid % cp);
     if (blk >= kpad / KB) return;
     const int64_t k = blk * KB + 2 * lane;
-    const double x0 = (col < c && k < kn) ? value(k, col) : 0.0;
-    const double x1 = (col < c && k + 1 < kn) ? value(k + 1, col) : 0.0;
+    double x0 = (col < c && k < kn) ? value(k, col) : 0.0;
+    double x1 = (col < c && k + 1 < kn) ? value(k + 1, col) : 0.0;
+    auto largest = [&]() {
+        const uint32_t a = (uint32_t)__double2hiint(x0) & 0x7fffffffu, b = (uint32_t)__double2hiint(x1) & 0x7fffffffu;
+        return __reduce_max_sync(0xffffffffu, max(a, b));
+    };
+    uint32_t ex = block_exponent(largest());
+    int scale = 0;
+    if (ex == 0u) {
+        x0 *= 0x1p256;
+        x1 *= 0x1p256;
+        scale = 256;
+        ex = block_exponent(largest());
+    }
+    if (lane == 0) eb[blk * cp + col] = special_exponent((int)ex) - scale;
     const uint32_t h0 = (uint32_t)__double2hiint(x0), h1 = (uint32_t)__double2hiint(x1);
-    uint32_t hm = max(h0 & 0x7fffffffu, h1 & 0x7fffffffu);
-    hm = __reduce_max_sync(0xffffffffu, hm);
-    const uint32_t ex = block_exponent(hm);
-    if (lane == 0) eb[blk * cp + col] = (int)ex;
     const uint64_t a = biased_int(h0, (uint32_t)__double2loint(x0), ex);
     const uint64_t b = biased_int(h1, (uint32_t)__double2loint(x1), ex);
     uint32_t* o = reinterpret_cast<uint32_t*>(out + (int64_t)(col / GC * NS * GC + col % GC) * kpad + k);
@@ -262,16 +274,18 @@ __global__ void __launch_bounds__(256) k_f64_prep_panel(const double* __restrict
 }
 
 // The rare results of level_sums: a 64-bit integer below 2^32 in magnitude, an exponent outside
-// FP64's normal range (flushed to 0 or infinity), a zero block, a block with infinities or NaN.
+// FP64's normal range (a subnormal number or infinity), a zero block, a block with infinities or NaN.
 __device__ __noinline__ double level_sum_slow(uint64_t m, bool neg, int eab) {
     if (eab > kNanEab / 2) return __longlong_as_double(0x7ff8000000000000ll);
     if (m == 0) return 0.0;
     const int lz = __clzll((long long)m);
     const int e = eab - lz - 1012;
-    uint64_t bits = ((uint64_t)(uint32_t)(e - 1) << 52) + (((m << (lz - 1)) + 0x200u) >> 10);
-    if (e < 1) bits = 0;
+    if (e < -64) return 0.0;                                 // below half of 2^-1074
+    const bool sub = e < 1;                                  // formed 2^128 above, then scaled down
+    uint64_t bits = ((uint64_t)(uint32_t)(sub ? e + 127 : e - 1) << 52) + (((m << (lz - 1)) + 0x200u) >> 10);
     if (e > 2046) bits = 0x7ff0000000000000ull;
-    return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+    const double v = __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+    return sub ? v * 0x1p-128 : v;
 }
 
 // The values of the levels of four columns: sum_l L_l 256^(6 - l) 2^(eab - 2154 + 48), eab = ea + eb,
@@ -532,7 +546,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
             for (int j = 0; j < PC; ++j) acc[j] = 0.0;
             for (int kb = w.k0; kb < w.k1; ++kb, ++g) {
-                const int eb = special_exponent(lane < PC ? p.eb[((int64_t)kb * p.ncg + w.cg) * CP + col0 + lane] : 0);
+                const int eb = lane < PC ? p.eb[((int64_t)kb * p.ncg + w.cg) * CP + col0 + lane] : kZeroEab;
                 if (!warp_wait(&sm.efull[g % EX], (g / EX) & 1)) { ok = false; break; }
                 const int ea = special_exponent((int)sm.expo[(g % EX) * BM + m]);
                 const uint32_t u = NG == 1 ? g : NG * g + set, b = u % NACC_;
