@@ -55,39 +55,46 @@ __global__ void k_km_assign(const double* __restrict__ x, int64_t n, int d, int 
     if (labels[i] != bc) { atomicAdd(changes, 1); labels[i] = bc; }
 }
 
-// Update step, first stage: block b sums the coordinates (and counts) of its chunk's points per
-// cluster: part[(b k + c) (d + 1) + j], j = d the count.  The chunk (kKmChunk points) is staged in
-// shared memory with its labels; warp w takes the clusters w, w + 8, ... and adds their points with
-// fixed-order sums.  Bound by the passes over the staged labels (k chunk / 8 per warp) and the FP64
-// adds of the shuffles; 128 points per block, so that a few thousand points fill the chip.  With
-// 2,048 points per block and a block-wide tree per cluster and coordinate it took 0.49 ms at 13,760
-// points, d = 8, 30 clusters (7 blocks); now 0.010 ms.
-constexpr int kKmChunk = 128;
+// Update step, first stage: block b sums the coordinates (and counts) of its chunks' points per
+// cluster: part[(b k + c) (d + 1) + j], j = d the count.  A chunk (kKmChunk points) is staged in shared
+// memory with its labels; warp w takes the clusters w, w + 8, ... and adds their points with fixed-order
+// sums, from the second chunk on to what it has stored before (clusters without points in a chunk are
+// passed over).  Bound by the passes over the staged labels (k chunk / 8 per warp) and the FP64 adds; 128
+// points per chunk, so that a few thousand points fill the chip: with 2,048 points per block and a
+// block-wide tree per cluster and coordinate it took 0.49 ms at 13,760 points, d = 8, 30 clusters (7
+// blocks); now 0.010 ms.  At most kKmBlocks blocks, a block then taking several chunks: the sums stay
+// below 512 k (d + 1) doubles whatever n is, and one warp per cluster can add them.
+constexpr int kKmChunk = 128, kKmBlocks = 512;
 __global__ void __launch_bounds__(256) k_km_partial(const double* __restrict__ x, int64_t n, int d, int k,
-                                                    const int* __restrict__ labels, double* __restrict__ part) {
+                                                    const int* __restrict__ labels, int64_t chunks,
+                                                    double* __restrict__ part) {
     __shared__ double xs[kKmChunk * dev::kMaxD];
     __shared__ int ls[kKmChunk];
-    const int64_t i0 = blockIdx.x * (int64_t)kKmChunk;
-    const int cnt = (int)min((int64_t)kKmChunk, n - i0);
-    for (int e = threadIdx.x; e < cnt * d; e += blockDim.x) xs[e] = x[i0 * d + e];
-    for (int e = threadIdx.x; e < kKmChunk; e += blockDim.x) ls[e] = e < cnt ? labels[i0 + e] : -1;
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = warp; c < k; c += 8) {
-        double* out = part + ((int64_t)blockIdx.x * k + c) * (d + 1);
-        // lane j <= d adds coordinate j (or 1) of the cluster's points in order
-        double acc = 0.0;
+    const int64_t first = blockIdx.x * chunks * kKmChunk, end = min(n, first + chunks * kKmChunk);
+    for (int64_t i0 = first; i0 < end; i0 += kKmChunk) {
+        const int cnt = (int)min((int64_t)kKmChunk, end - i0);
+        if (i0 > first) __syncthreads();
+        for (int e = threadIdx.x; e < cnt * d; e += blockDim.x) xs[e] = x[i0 * d + e];
+        for (int e = threadIdx.x; e < kKmChunk; e += blockDim.x) ls[e] = e < cnt ? labels[i0 + e] : -1;
+        __syncthreads();
+        for (int c = warp; c < k; c += 8) {
+            double* out = part + ((int64_t)blockIdx.x * k + c) * (d + 1);
+            unsigned m[kKmChunk / 32], any = 0;
 #pragma unroll
-        for (int q = 0; q < kKmChunk; q += 32) {
-            unsigned m = __ballot_sync(0xffffffffu, ls[q + lane] == c);
-            while (m) {
-                const int e = q + __ffs(m) - 1;
-                m &= m - 1;
-                if (lane < d) acc += xs[e * d + lane];
-                else if (lane == d) acc += 1.0;
-            }
+            for (int q = 0; q < kKmChunk / 32; ++q) any |= m[q] = __ballot_sync(0xffffffffu, ls[32 * q + lane] == c);
+            if (i0 > first && !any) continue;
+            // lane j <= d adds coordinate j (or 1) of the cluster's points in order
+            double acc = i0 > first && lane <= d ? out[lane] : 0.0;
+#pragma unroll
+            for (int q = 0; q < kKmChunk / 32; ++q)
+                for (unsigned w = m[q]; w; w &= w - 1) {
+                    const int e = 32 * q + __ffs(w) - 1;
+                    if (lane < d) acc += xs[e * d + lane];
+                    else if (lane == d) acc += 1.0;
+                }
+            if (lane <= d) out[lane] = acc;
         }
-        if (lane <= d) out[lane] = acc;
     }
 }
 
@@ -1035,7 +1042,8 @@ hdf_status hdf_kmeans(const double* x_dev, int64_t n, int d, int k, const int64_
     k_gather_rows<<<blocks_for((int64_t)k * d, 256, 1 << 30), 256, 0, st>>>(x_dev, d, idx.as<int64_t>(), k,
                                                                            C.as<double>());
     HDF_CUDA(cudaMemsetAsync(labels_dev, 0xff, sizeof(int) * n, st));      // -1: every label changes first
-    const int G = (int)((n + kKmChunk - 1) / kKmChunk);
+    const int64_t chunks = (n + (int64_t)kKmBlocks * kKmChunk - 1) / ((int64_t)kKmBlocks * kKmChunk);   // of a block
+    const int G = (int)((n + chunks * kKmChunk - 1) / (chunks * kKmChunk));
     HDF_CUDA(part.alloc_on(sizeof(double) * (size_t)G * k * (d + 1), st));
     HDF_CUDA(chg.alloc_on(sizeof(int), st));
     int it = 0;
@@ -1050,7 +1058,7 @@ hdf_status hdf_kmeans(const double* x_dev, int64_t n, int d, int k, const int64_
         HDF_CUDA(cudaStreamSynchronize(st));
         if (changes == 0 && it > 1) break;
         HDF_COUNT_LAUNCH();
-        k_km_partial<<<G, 256, 0, st>>>(x_dev, n, d, k, labels_dev, part.as<double>());
+        k_km_partial<<<G, 256, 0, st>>>(x_dev, n, d, k, labels_dev, chunks, part.as<double>());
         HDF_COUNT_LAUNCH();
         k_km_finish<<<(k + 3) / 4, 128, 0, st>>>(part.as<double>(), G, k, d, C.as<double>());
         HDF_CUDA(cudaGetLastError());
