@@ -950,6 +950,21 @@ struct hdf_krr {
 
 namespace {
 
+// Bytes that the device can still hand out: free ones and those that the default pool keeps unused.
+size_t device_room() {
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess) { cudaGetLastError(); return 0; }
+    int dev = 0;
+    cudaMemPool_t pool;
+    uint64_t reserved = 0, used = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+        free += reserved - used;
+    cudaGetLastError();
+    return free;
+}
+
 // The off-diagonal blocks times vp into K->part.
 hdf_status apply_off(hdf_krr* K, const double* vp, cudaStream_t st) {
     const int64_t n = K->n;
@@ -1237,21 +1252,6 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
         if (hbad) return fail(HDF_ESINGULAR, "hdf_krr_build: a block lambda I + K_cc is not positive definite");
     }
     // work space
-    // the off-diagonal blocks are stored while they take at most 8 GiB (65,000 points) and the
-    // device has room; else every product evaluates them
-    const size_t kbytes = sizeof(float) * (size_t)off_tiles(n) * kTI * kTJ;
-    size_t nparts = (size_t)off_tiles(n) * kTPart;
-    if (kbytes <= ((size_t)8 << 30) && K->koff.alloc_on(kbytes, st) == cudaSuccess) {
-        HDF_COUNT_LAUNCH();
-        launch_off_store(d, st, K->xp32.as<float>(), n, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
-                         K->koff.as<float>());
-        HDF_CUDA(cudaGetLastError());
-    } else {
-        cudaGetLastError();
-        K->split = direct_split(n, n, &K->S);
-        nparts = (size_t)K->S * n;
-    }
-    HDF_CUDA(K->part.alloc(sizeof(double) * nparts));
     HDF_CUDA(K->hd.alloc(sizeof(double) * n));
     HDF_CUDA(K->dotp.alloc(sizeof(double) * 2 * (size_t)((n + 7) / 8)));
     HDF_CUDA(K->cgst.alloc(sizeof(CgState)));
@@ -1259,6 +1259,24 @@ hdf_status hdf_krr_build(const double* x_dev, int64_t n, int d, const int* label
     if (prec == HDF_FP32) {
         HDF_CUDA(K->vb.alloc(sizeof(float) * n));
         HDF_CUDA(K->yb.alloc(sizeof(float) * n));
+    }
+    // The off-diagonal blocks are stored while they take at most 8 GiB (65,000 points) and the device has
+    // room for them, their partial sums and kSpare besides; else every product evaluates them.  They come
+    // last, so that nothing else fails for their sake.
+    constexpr size_t kSpare = (size_t)512 << 20;
+    const size_t kbytes = sizeof(float) * (size_t)off_tiles(n) * kTI * kTJ;
+    const size_t pbytes = sizeof(double) * (size_t)off_tiles(n) * kTPart;
+    const bool stored = kbytes <= ((size_t)8 << 30) && device_room() >= kbytes + pbytes + kSpare &&
+                        K->part.alloc(pbytes) == cudaSuccess && K->koff.alloc_on(kbytes, st) == cudaSuccess;
+    if (stored) {
+        HDF_COUNT_LAUNCH();
+        launch_off_store(d, st, K->xp32.as<float>(), n, kernel, (float)(1.0 / lengthscale), K->cl.as<int>(),
+                         K->koff.as<float>());
+        HDF_CUDA(cudaGetLastError());
+    } else {
+        cudaGetLastError();
+        K->split = direct_split(n, n, &K->S);
+        HDF_CUDA(K->part.alloc(sizeof(double) * (size_t)K->S * n));
     }
     HDF_CUDA(cudaStreamSynchronize(st));
     K->t_precond = wall_ms() - t1;

@@ -67,3 +67,30 @@ def test_injected_allocation_failures(prec):
     m = hdf.KRR(xt, lab, "gaussian", 0.5, 1.0, 1e-6, precision=prec)
     assert bool((m.apply(v) == y).all())
     assert bool((m.solve(v, rtol=1e-8)[0] == w).all())
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_stored_blocks_are_given_up_for_any_allocation_of_theirs(prec):
+    """A build without memory for the stored blocks or for their partial sums evaluates the blocks instead."""
+    from paper_2202_03655_gb300 import hdf
+    x, lab, v = problem()
+    xt = to_dev(x)
+    y = hdf.KRR(xt, lab, "gaussian", 0.5, 1.0, 1e-6, precision=prec).apply(v)
+    other = 0
+    try:
+        for k in range(80):
+            hdf.debug_fail_alloc(k)
+            try:
+                m = hdf.KRR(xt, lab, "gaussian", 0.5, 1.0, 1e-6, precision=prec)
+            except hdf.HdfError:
+                continue
+            hdf.debug_fail_alloc(-1)
+            z = m.apply(v)
+            w, it, res = m.solve(v, rtol=1e-8)
+            assert res <= 1e-8
+            # evaluated: the same FP32 values added in another order
+            other += not bool((z == y).all())
+            assert float((z - y).abs().max()) <= 1e-9 * float(v.abs().sum())
+    finally:
+        hdf.debug_fail_alloc(-1)
+    assert other == 2
