@@ -363,7 +363,8 @@ hdf_status hdf_check_tf32_rounding(unsigned long long* mismatches);
 /* Host-side fault injection: the device allocation `after` allocations from now (0 = the next
  * one) made by the library reports out-of-memory without allocating, once; a negative value
  * cancels a pending injection.  The call that meets it returns HDF_ENOMEM with its output
- * buffers untouched (hdf_build and friends set *out = NULL).  Process-wide. */
+ * buffers untouched (hdf_build and friends set *out = NULL), or goes on in a form that needs less
+ * memory where it has one.  Process-wide. */
 void hdf_debug_fail_alloc(long long after);
 
 /* Release a factor (NULL is ignored). */

@@ -651,11 +651,13 @@ constexpr int64_t kMaxSolveRank = 32768;      // the solve's r x r core and its 
 struct GroupWork {
     bool tc = false;         // FP32 on the tensor cores: the partial sums in `part` are FP32
     bool f64 = false;        // FP64 on the tensor cores for the groups that f64_tensor names
+    bool few = false;        // FP64 otherwise: groups of up to kFewCols columns on the streaming kernels
     DevBuf uwpart;           // its column splits of U W
     int nchunk = 0, tch = 0;
     int64_t chunk = 0, tchunk = 0;
     DevBuf part;             // partial sums: nchunk (or tch) x cmax x r, FP64
     DevBuf twork;            // tensor-core operand splits (V hi/lo, W hi/lo)
+    bool streams(int cg) const { return (few || f64) && cg <= kFewCols; }
 };
 
 static bool tc_usable(const hdf_factor* f, int64_t n, int64_t r) {
@@ -687,33 +689,41 @@ static hdf_status group_setup(const hdf_factor* fin, const hdf_factor* fout, int
     } else {
         g.nchunk = utv_chunks(nin, r, cmax);
         g.chunk = (nin + g.nchunk - 1) / g.nchunk;
-        int64_t slices = (int64_t)g.nchunk * cmax;
-        if (sizeof(T) == 8) {
+        const int64_t tiles = (int64_t)g.nchunk * cmax;
+        if constexpr (sizeof(T) == 8) {
+            // The slices of V take 14 bytes per entry of up to 32 columns, split products and the streaming
+            // kernels their partial sums; where so much is not left beside a large factor, the next form
+            // takes over, at the end the register-tiled kernels, which need least.
+            int64_t few = tiles;
             // every group width up to kFewCols that a call of cmax columns can end with
             for (int c = 1; c <= std::min(cmax, kFewCols); ++c) {
                 int64_t chunk;
                 int k;
                 few_utv_split(nin, r, c, &chunk, &k);
-                slices = std::max(slices, (int64_t)k * c);
+                few = std::max(few, (int64_t)k * c);
             }
-        }
-        if (g.f64) {
-            // the slices of V are 14 bytes per entry of up to 32 columns; where so much is not left
-            // beside a large factor, the CUDA-core kernels need none
-            const size_t wb = tc_f64_work_bytes(std::max(nin, r), cmax);
-            const cudaError_t e = g.twork.alloc_on(wb, st);
-            if (e == cudaErrorMemoryAllocation && wb > ((size_t)256 << 20)) {
-                cudaGetLastError();
-                g.f64 = false;
-            } else {
-                HDF_CUDA(e);
+            auto room = [&](DevBuf& b, size_t bytes, hdf_status* e) {
+                const cudaError_t ce = b.alloc_on(bytes, st);
+                if (ce == cudaErrorMemoryAllocation) cudaGetLastError();
+                else if (ce != cudaSuccess) *e = fail(HDF_ECUDA, std::string("work space: ") + cudaGetErrorString(ce));
+                return ce == cudaSuccess;
+            };
+            hdf_status e = HDF_OK;
+            if (g.f64) {
                 int kper;
-                slices = std::max(slices, (int64_t)tc_f64_utv_splits(nin, r, &kper) * cmax);
-                if (const int ns = tc_f64_uw_splits(nout, r, &kper); ns > 1)
-                    HDF_CUDA(g.uwpart.alloc_on(sizeof(double) * (size_t)ns * std::min(cmax, 32) * nout, st));
+                const int64_t slices = std::max(few, (int64_t)tc_f64_utv_splits(nin, r, &kper) * cmax);
+                const int ns = tc_f64_uw_splits(nout, r, &kper);
+                g.f64 = room(g.twork, tc_f64_work_bytes(std::max(nin, r), cmax), &e) &&
+                        (ns == 1 || room(g.uwpart, sizeof(double) * (size_t)ns * std::min(cmax, 32) * nout, &e)) &&
+                        room(g.part, sizeof(double) * (size_t)slices * r, &e);
+                if (g.f64 || e != HDF_OK) return e;
+                g.twork.release();
+                g.uwpart.release();
             }
+            g.few = room(g.part, sizeof(double) * (size_t)few * r, &e);
+            if (g.few || e != HDF_OK) return e;
         }
-        HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)slices * r, st));
+        HDF_CUDA(g.part.alloc_on(sizeof(double) * (size_t)tiles * r, st));
     }
     return HDF_OK;
 }
@@ -738,7 +748,7 @@ static hdf_status group_utv(const hdf_factor* fin, int64_t r, const T* V, int64_
             return tc_f64_utv(fin->U.as<double>(), fin->info.ldu, nin, r, V, ldv, cg, g.part.as<double>(), g.twork.p,
                               fin->dev_err.as<int>(), st);
         }
-        if (cg <= kFewCols) {
+        if (g.streams(cg)) {
             int64_t chunk;
             few_utv_split(nin, r, cg, &chunk, np);
             return few_utv(fin->U.as<double>(), fin->info.ldu, nin, r, V, ldv, cg, chunk, *np, g.part.as<double>(), st);
@@ -781,7 +791,7 @@ static hdf_status group_uw(const hdf_factor* fout, int64_t r, const T* W, int cg
         if (g.f64 && f64_tensor(nout, r, cg))
             return tc_f64_uw(fout->U.as<double>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy,
                              g.uwpart.as<double>(), g.twork.p, fout->dev_err.as<int>(), st);
-        if (cg <= kFewCols)
+        if (g.streams(cg))
             return few_uw(fout->U.as<double>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy, st);
     }
     launch_uw<T>(ct_for(cg), fout->U.as<T>(), fout->info.ldu, nout, r, W, cg, alpha, B, ldb, beta, Y, ldy, st);
