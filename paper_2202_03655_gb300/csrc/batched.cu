@@ -1481,7 +1481,7 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         while ((int64_t(1) << (bucket + 1)) <= std::max<int64_t>(1, work / 1024)) ++bucket;
         char key[160];
         if (ph == 0)
-            std::snprintf(key, sizeof(key), "batch_radial_v3:sm%d:d%d:%s:smem%zu:work2^%d", nsm, d,
+            std::snprintf(key, sizeof(key), "batch_radial_v4:sm%d:d%d:%s:smem%zu:work2^%d", nsm, d,
                           sizeof(T) == 4 ? "fp32" : "fp64", smem_rf / 4096, bucket);
         else
             std::snprintf(key, sizeof(key), "batch_urows_v3:sm%d:d%d:%s:pw%zu:fixed%zu:work2^%d", nsm, d,
