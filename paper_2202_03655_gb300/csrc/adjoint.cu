@@ -60,11 +60,16 @@ struct alignas(16) Double4 { double x, y, z, w; };
 template <> struct Quad<double> { typedef Double4 type; };
 
 // Shared memory of a warp: (value, d/dz, d/dq) of the level tables and (value, d/dx_0, d/dx_1) of the
-// trigonometric factors (four elements each), (F' - k F / rho, F / rho) per radial factor, T_l and T_l'
-// of a batch of points (8 bytes each), the radial basis and its derivative (8 bytes each).
+// trigonometric factors, (F' - k F / rho, F / rho) per radial factor, T_l and T_l' of a batch of points (8
+// bytes each), the radial basis and its derivative (8 bytes each).  The three values of a table entry
+// lie together, in four elements that are read at once (packed), or in three arrays.
+__host__ __device__ inline int adj_table_elems(int levels, int tri, int L, bool packed) {
+    const int e = levels * tri + 2 * L + 1;
+    return packed ? 4 * e : (3 * e + 1) / 2 * 2;
+}
 template <typename T>
-size_t adj_per_warp(int levels, int tri, int L, int nF, int Lr, int m, int nb) {
-    return ((sizeof(T) * (4 * ((size_t)levels * tri + 2 * L + 1) + 2 * (size_t)nF) + 7) / 8 * 8 +
+size_t adj_per_warp(int levels, int tri, int L, int nF, int Lr, int m, int nb, bool packed) {
+    return ((sizeof(T) * ((size_t)adj_table_elems(levels, tri, L, packed) + 2 * (size_t)nF) + 7) / 8 * 8 +
             8 * (2 * (size_t)nb * (Lr + 1) + 2 * (size_t)m) + 15) / 16 * 16;
 }
 
@@ -120,9 +125,11 @@ __device__ __forceinline__ void df_dot_step(float2 a, float2 b, float& sh, float
 // instructions a step, which one lane per point cost every lane), then the points follow one by one
 // with the lanes over basis functions, radial factors and harmonics.  Bound by instruction issue and
 // the latency of the table reads: 500,000 points, d = 4, 2,104 columns, 4.43 -> 3.19 ms with batches,
-// one descriptor per harmonic and the tables' three values read together.  DD = the dimension d (a template parameter, so that
-// the per-thread coordinate and gradient arrays stay in registers).
-template <typename T, int DD>
+// one descriptor per harmonic and the tables' three values read together.  At high degrees a warp's
+// tables leave few warps on an SM and their latency counts alone: there the three arrays, a quarter
+// smaller, and CTAs of one or two warps are used (see run).  DD = the dimension d (a template parameter,
+// so that the per-thread coordinate and gradient arrays stay in registers).
+template <typename T, int DD, bool PACKED>
 __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int2 kts[HDF_MAX_L + 1];        // per k: F column | s_k << 16, columns per (k, s) block
@@ -135,11 +142,29 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
         kts[k] = make_int2(kt[0] | kt[1] << 16, kt[5]);
     }
     __syncthreads();
-    T4* tb = reinterpret_cast<T4*>(smem_raw + (size_t)warp * P.per_warp);      // levels * tri
-    T4* trig = tb + levels * P.tri;            // 2L+1
-    T2* RR = reinterpret_cast<T2*>(trig + 2 * P.L + 1);                        // nF
-    double* Tl = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(tb) +
-                                           (sizeof(T) * (4 * (levels * P.tri + 2 * P.L + 1) + 2 * P.nF) + 7) / 8 * 8);
+    // levels * tri entries of the level tables, then 2L+1 trigonometric ones
+    T* tab = reinterpret_cast<T*>(smem_raw + (size_t)warp * P.per_warp);
+    const int trig = levels * P.tri, entries = trig + 2 * P.L + 1;
+    const int elems = adj_table_elems(levels, P.tri, P.L, PACKED);
+    auto put = [&](int e, T v, T a, T b) {
+        if constexpr (PACKED) {
+            T4 w; w.x = v; w.y = a; w.z = b; w.w = (T)0;
+            reinterpret_cast<T4*>(tab)[e] = w;
+        } else {
+            tab[e] = v; tab[entries + e] = a; tab[2 * entries + e] = b;
+        }
+    };
+    auto get = [&](int e, T& v, T& a, T& b) {
+        if constexpr (PACKED) {
+            const T4 w = reinterpret_cast<const T4*>(tab)[e];
+            v = w.x; a = w.y; b = w.z;
+        } else {
+            v = tab[e]; a = tab[entries + e]; b = tab[2 * entries + e];
+        }
+    };
+    T2* RR = reinterpret_cast<T2*>(tab + elems);                               // nF
+    double* Tl = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(tab) +
+                                           (sizeof(T) * (elems + 2 * P.nF) + 7) / 8 * 8);
     const int nb = P.nb;
     double* dTl = Tl + nb * (P.Lr + 1);        // T_l(u), T_l'(u): [l][point]
     double* Q = dTl + nb * (P.Lr + 1);         // m0+m1
@@ -293,22 +318,21 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
             const T z = xh[D], qq = q;
             const T* A = P.coefA + j * P.tri;
             const T* B = P.coefB + j * P.tri;
-            T4* pt4 = tb + j * P.tri;
-            auto put = [&](int e, T v, T dz, T dq) { T4 w; w.x = v; w.y = dz; w.z = dq; w.w = (T)0; pt4[e] = w; };
+            const int t0 = j * P.tri;
             for (int mu = lane; mu <= P.L; mu += 32) {
                 const int o = mu * (P.L + 1) - mu * (mu - 1) / 2;
                 const int nmax = P.L - mu;
                 T v2 = A[o], z2 = (T)0, q2 = (T)0;
-                put(o, v2, z2, q2);
+                put(t0 + o, v2, z2, q2);
                 if (nmax >= 1) {
                     T v1 = A[o + 1] * z, z1 = A[o + 1], q1 = (T)0;
-                    put(o + 1, v1, z1, q1);
+                    put(t0 + o + 1, v1, z1, q1);
                     for (int nn = 2; nn <= nmax; ++nn) {
                         const T an = A[o + nn], bn = B[o + nn];
                         const T v0 = an * z * v1 - bn * qq * v2;
                         const T z0 = an * (v1 + z * z1) - bn * qq * z2;
                         const T q0 = an * z * q1 - bn * (v2 + qq * q2);
-                        put(o + nn, v0, z0, q0);
+                        put(t0 + o + nn, v0, z0, q0);
                         v2 = v1; z2 = z1; q2 = q1;
                         v1 = v0; z1 = z0; q1 = q0;
                     }
@@ -335,13 +359,12 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                 }
             }
             // value, d/dx_0, d/dx_1
-            auto put = [&](int e, T v, T dx, T dy) { T4 w; w.x = v; w.y = dx; w.z = dy; w.w = (T)0; trig[e] = w; };
             if (mu == 0) {
-                put(P.L, (T)0.3989422804014327, (T)0, (T)0);
+                put(trig + P.L, (T)0.3989422804014327, (T)0, (T)0);
             } else {
                 const TP nm = (TP)0.5641895835477563;
-                put(P.L + mu, (T)(rr * nm), (T)(mu * pr * nm), (T)(-mu * pi * nm));      // Re z^mu
-                put(P.L - mu, (T)(ri * nm), (T)(mu * pi * nm), (T)(mu * pr * nm));       // Im z^mu
+                put(trig + P.L + mu, (T)(rr * nm), (T)(mu * pr * nm), (T)(-mu * pi * nm));      // Re z^mu
+                put(trig + P.L - mu, (T)(ri * nm), (T)(mu * pi * nm), (T)(mu * pr * nm));       // Im z^mu
             }
         }
         __syncwarp();
@@ -364,7 +387,8 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                 al += cc * r2.x;
                 be += cc * r2.y;
             }
-            const T4 tg = trig[de.y >> 8];
+            T tr, tx, ty;
+            get(trig + (de.y >> 8), tr, tx, ty);
             int of[kMaxD] = {de.z & 0xffff, (int)((unsigned)de.z >> 16), de.w & 0xffff, (int)((unsigned)de.w >> 16)};
             if constexpr (levels > 4) {
                 const int e2 = __ldg(P.desc2 + gi);
@@ -373,12 +397,7 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
             }
             T pvv[kMaxD], pzz[kMaxD], pqq[kMaxD];
 #pragma unroll
-            for (int j = 0; j < levels; ++j) {
-                const T4 w = tb[j * P.tri + of[j]];
-                pvv[j] = w.x;
-                pzz[j] = w.y;
-                pqq[j] = w.z;
-            }
+            for (int j = 0; j < levels; ++j) get(j * P.tri + of[j], pvv[j], pzz[j], pqq[j]);
             // suffix products suf[j] = prod_{j2 > j} P_j2, so that the product of all level
             // factors but one is (trig * prefix) * suffix: O(levels) per harmonic
             T suf[kMaxD];
@@ -386,7 +405,6 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
 #pragma unroll
             for (int j = levels - 2; j >= 0; --j) suf[j] = suf[j + 1] * pvv[j + 1];
             const T pl = (levels > 0) ? pvv[0] * suf[0] : (T)1;      // all level factors
-            const T tr = tg.x;
             const T prod = tr * pl;
             // Y x_hat term
 #pragma unroll
@@ -405,8 +423,8 @@ __global__ void __launch_bounds__(128) k_adjoint(AdjParams<T> P) {
                     if (m <= D) g[m] += cq * xt[m];
             }
             // grad H: trigonometric factor
-            g[0] += be * pl * tg.y;
-            g[1] += be * pl * tg.z;
+            g[0] += be * pl * tx;
+            g[1] += be * pl * ty;
         }
 #pragma unroll
         for (int m = 0; m < DD; ++m) {
@@ -567,16 +585,42 @@ hdf_status run(hdf_factor* f, const double* x, const T* V, int64_t ldv, const T*
              sizeof(T) * ((2 * (size_t)P.nF + 3 * levels * P.tri + 3 * (2 * P.L_used + 1) + 3) & ~(size_t)3)) >
         200 * 1024)
         return hdf::fail(HDF_ETOOBIG, "hdf_matvec_adjoint: per-point tables exceed shared memory");
-    // batches of up to kAdjBatch points while every SM has some 64 of them; as many warps per CTA as fit
-    A.nb = kAdjBatch;
-    while (A.nb > 1 && n < (int64_t)64 * nsm * A.nb) A.nb /= 2;
-    A.per_warp = (int)adj_per_warp<T>(levels, P.tri, P.L_used, P.nF, P.L, P.m[0] + P.m[1], A.nb);
-    const int warps = std::max(1, (int)std::min<size_t>(4, 220 * 1024 / (size_t)A.per_warp));
-    const size_t sm = (size_t)warps * A.per_warp;
-    void (*kern)(AdjParams<T>) = d == 3 ? k_adjoint<T, 3> : d == 4 ? k_adjoint<T, 4> : d == 5 ? k_adjoint<T, 5>
-                               : d == 6 ? k_adjoint<T, 6> : d == 7 ? k_adjoint<T, 7> : k_adjoint<T, 8>;
+    using K = void (*)(AdjParams<T>);
+    const K packed[] = {k_adjoint<T, 3, true>, k_adjoint<T, 4, true>, k_adjoint<T, 5, true>,
+                        k_adjoint<T, 6, true>, k_adjoint<T, 7, true>, k_adjoint<T, 8, true>};
+    const K narrow[] = {k_adjoint<T, 3, false>, k_adjoint<T, 4, false>, k_adjoint<T, 5, false>,
+                        k_adjoint<T, 6, false>, k_adjoint<T, 7, false>, k_adjoint<T, 8, false>};
+    // Batch, table layout and warps per CTA: the first in the order below that keeps kAdjFull warps on an
+    // SM, else the one that keeps most (on a tie the smaller batch).  From about 28 warps on (FP64: 20, more
+    // registers per thread) more of them gain nothing, while batches of four save up to 20% and packed
+    // tables 4% (500,000 points, d = 4, 2,104 columns: 3.94 ms; three arrays 4.11; batches of one 4.43);
+    // below, the time goes with the warps: d = 4, 30,000 points, 37,452 columns 7.14 ms on 8 warps (packed,
+    // CTAs of four), 4.64 on 14; d = 5, 2,000 points, 523,787 columns 20.2 ms on 4, 8.5 on 8; d = 3,
+    // 150,000 points, 8,997 columns 7.5 ms on 12, 5.9 on 18.
+    constexpr int kAdjFull = sizeof(T) == 8 ? 20 : 28;
+    K kern = nullptr;
+    int warps = 0, best = 0;
+    size_t sm = 0;
+    int nb_max = kAdjBatch;
+    while (nb_max > 1 && n < (int64_t)64 * nsm * nb_max) nb_max /= 2;
+    for (int nb = nb_max; nb >= 1 && best < kAdjFull; nb /= 2)
+        for (int pk = 1; pk >= 0 && best < kAdjFull; --pk) {
+            const K k = (pk ? packed : narrow)[d - 3];
+            const size_t pw = adj_per_warp<T>(levels, P.tri, P.L_used, P.nF, P.L, P.m[0] + P.m[1], nb, pk == 1);
+            for (int w : {4, 2, 1}) {
+                if (w * pw > 220 * 1024) continue;
+                HDF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(w * pw)));
+                int o = 0;
+                HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, w * 32, w * pw));
+                if (o * w > best || (o * w == best && best < kAdjFull && nb < A.nb)) {
+                    kern = k; warps = w; best = o * w; occ = o; sm = w * pw;
+                    A.nb = nb;
+                    A.per_warp = (int)pw;
+                }
+                if (best >= kAdjFull) break;
+            }
+        }
     HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HDF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, sm));
     const int grid = std::max(1, std::min<int>(nsm * std::max(occ, 1), (int)((n + warps * A.nb - 1) / (warps * A.nb))));
     for (int j = 0; j < ncols; ++j) {
         A.ab = ab.as<T>() + 2 * (size_t)j * r;
