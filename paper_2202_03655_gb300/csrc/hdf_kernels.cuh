@@ -1332,8 +1332,72 @@ __global__ void __launch_bounds__(kRedA * kRedB) k_reduce_scale(const P* __restr
     if (W) W[a * c + j] = (T)s;
     if (Wd) Wd[a * c + j] = s;
 }
+// The same for few chunks, where the form above leaves most of its threads without one and writes single
+// elements c apart: a thread per (a, j), neighbouring threads along j.  262,152 x 16, one FP32 slice 110 ->
+// 45 us, 16 of them 376 -> 280; 32,776 x 64, one FP64 slice 53 -> 14.
+template <typename T, typename P>
+__global__ void __launch_bounds__(256) k_reduce_scale_flat(const P* __restrict__ part, int nchunk, int64_t r, int c,
+                                                           const T* __restrict__ S, T* __restrict__ W,
+                                                           double* __restrict__ Wd) {
+    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (idx >= r * c) return;
+    const int64_t a = idx / c;
+    const int j = (int)(idx % c);
+    double s = 0.0;
+    for (int b = 0; b < nchunk; ++b) s += (double)part[((int64_t)b * c + j) * r + a];
+    if (S) s *= (double)S[a];
+    if (W) W[idx] = (T)s;
+    if (Wd) Wd[idx] = s;
+}
+// The same for few chunks and wide blocks, whose reads r apart would cost the lines of a slice more than
+// once: 32 columns a by 32 columns j through shared memory, written in runs along j.  262,152 x 64, one
+// FP32 slice 143 us (161 by a thread per (a, j), 475 with the chunks split), 16 FP64 slices 576 (1,749, 1,007).
+template <typename T, typename P>
+__global__ void __launch_bounds__(256) k_reduce_scale_tile(const P* __restrict__ part, int nchunk, int64_t r, int c,
+                                                           const T* __restrict__ S, T* __restrict__ W,
+                                                           double* __restrict__ Wd) {
+    __shared__ double sh[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t a0 = blockIdx.x * 32ll;
+    const int j0 = blockIdx.y * 32;
+    const int64_t a = a0 + tx;
+    if (a < r) {
+        const double scale = S ? (double)S[a] : 1.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = j0 + ty + 8 * q;
+            if (j < c) {
+                double s = 0.0;
+                for (int b = 0; b < nchunk; ++b) s += (double)part[((int64_t)b * c + j) * r + a];
+                sh[ty + 8 * q][tx] = s * scale;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t o = a0 + ty + 8 * q;
+        const int j = j0 + tx;
+        if (o < r && j < c) {
+            const double s = sh[tx][ty + 8 * q];
+            if (W) W[o * c + j] = (T)s;
+            if (Wd) Wd[o * c + j] = s;
+        }
+    }
+}
 template <typename T, typename P>
 void launch_reduce_scale(const P* part, int nchunk, int64_t r, int c, const T* S, T* W, double* Wd, cudaStream_t st) {
+    // Few chunks: at 16 the flat form is still ahead (8,200 x 33, FP32 24 us against 28; at 32 40 and 45, at
+    // 520 x 64 12 and 12); below 32,768 results it has too few threads (2,056 x 8, 16 slices 10 against 8).
+    if (nchunk <= 16 && r * c >= 32768) {
+        if (c < 48) {
+            k_reduce_scale_flat<T, P><<<(unsigned)((r * c + 255) / 256), 256, 0, st>>>(part, nchunk, r, c, S, W, Wd);
+        } else {
+            const dim3 g((unsigned)((r + 31) / 32), (unsigned)((c + 31) / 32));
+            k_reduce_scale_tile<T, P><<<g, 256, 0, st>>>(part, nchunk, r, c, S, W, Wd);
+        }
+        return;
+    }
     const dim3 g((unsigned)((r + kRedA - 1) / kRedA), (unsigned)c);
     k_reduce_scale<T, P><<<g, kRedA * kRedB, 0, st>>>(part, nchunk, r, c, S, W, Wd);
 }
