@@ -22,7 +22,8 @@
 // it (a flag in global memory), subtracts its 64 x 64 product, multiplies by the inverse of its
 // diagonal tile and publishes the result, so a step of the chain is two small products and one
 // flag instead of two launches, one of them a 64-step substitution by a single CTA: 0.41 ms for one
-// column at r = 2,104, 13 ms before.
+// column at r = 2,104, 13 ms before.  Where the blocks leave CTAs over, several chains run side by side,
+// each with a group of the columns: 64 columns at r = 69, solve with kept factors 0.68 -> 0.24 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -240,8 +241,9 @@ struct TriArgs {
     const double *DL, *DU;               // inverses of the diagonal tiles
     const int* rperm;                    // row a of the factors is row rperm[a] of the right-hand side
     const double* zi; double* y; double* zo;   // r x nc row-major: right-hand side, work, result
-    int nc, nblk;
-    int* flags;                          // 2 nblk, zero at launch
+    int nc, nblk;                        // columns; 64-row blocks
+    int group, nb;                       // columns of a group; CTAs of a group
+    int* flags;                          // 2 nblk per group, zero at launch
     int* err;
 };
 
@@ -254,25 +256,32 @@ __device__ __forceinline__ void st_release(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// GROUPS: P.nb CTAs per group of P.group columns (else all columns on all CTAs; kept apart because the
+// strides at run time cost 2% at r = 6,693, 64 columns).
+template <bool GROUPS>
 __global__ void __launch_bounds__(256) k_tri_solve(TriArgs P) {
     extern __shared__ double sm[];
+    const int nb = GROUPS ? P.nb : (int)gridDim.x;
+    const int g = GROUPS ? (int)blockIdx.x / nb : 0, blk = (int)blockIdx.x - g * nb;
+    const int c0 = GROUPS ? g * P.group : 0, ld = P.nc, nc = GROUPS ? min(P.group, ld - c0) : ld;     // its columns
     double* zs = sm;                     // the solved block being subtracted, NB x nc
-    double* as = sm + NB * P.nc;         // this block's residual, NB x nc
+    double* as = sm + NB * nc;           // this block's residual, NB x nc
     __shared__ int gave_up;
-    const int t = threadIdx.x, row = t >> 2, qt = t & 3, nc = P.nc;
+    const int t = threadIdx.x, row = t >> 2, qt = t & 3;
+    int* flags = P.flags + (int64_t)g * 2 * P.nblk;
     if (t == 0) gave_up = 0;
     __syncthreads();
     // own blocks ascending (forward), then descending (backward): every wait is on a block that
     // comes earlier in this order, and the cooperative launch keeps all CTAs resident
-    const int mine = (P.nblk - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int mine = (P.nblk - blk + nb - 1) / nb;
     for (int s = 0; s < 2 * mine; ++s) {
         const bool fwd = s < mine;
-        const int rb = (int)blockIdx.x + (fwd ? s : 2 * mine - 1 - s) * (int)gridDim.x;
+        const int rb = blk + (fwd ? s : 2 * mine - 1 - s) * nb;
         const int64_t i = (int64_t)rb * NB + row;
         for (int e = t; e < NB * nc; e += 256) {
             const int64_t a = (int64_t)rb * NB + e / nc;
             double v = 0.0;
-            if (a < P.r) v = fwd ? P.zi[(int64_t)P.rperm[a] * nc + e % nc] : P.y[a * nc + e % nc];
+            if (a < P.r) v = fwd ? P.zi[(int64_t)P.rperm[a] * ld + c0 + e % nc] : P.y[a * ld + c0 + e % nc];
             as[e] = v;
         }
         const int ndep = fwd ? rb : P.nblk - 1 - rb;
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(256) k_tri_solve(TriArgs P) {
             const int b = fwd ? d : P.nblk - 1 - d;
             tile(d + 1, xn);                                 // in flight during the wait
             if (t == 0 && !gave_up) {
-                const int* fl = P.flags + (fwd ? 0 : P.nblk) + b;
+                const int* fl = flags + (fwd ? 0 : P.nblk) + b;
                 if (!ld_acquire(fl)) {
                     const long long t0 = clock64();
                     while (!ld_acquire(fl))
@@ -296,9 +305,10 @@ __global__ void __launch_bounds__(256) k_tri_solve(TriArgs P) {
                 }
             }
             __syncthreads();
-            const double* src = (fwd ? P.y : P.zo) + (int64_t)b * NB * nc;
+            const double* src = (fwd ? P.y : P.zo) + (int64_t)b * NB * ld + c0;
             const int cnt = (int)min((int64_t)NB, P.r - (int64_t)b * NB) * nc;
-            for (int e = t; e < NB * nc; e += 256) zs[e] = e < cnt ? __ldcg(src + e) : 0.0;
+            for (int e = t; e < NB * nc; e += 256)
+                zs[e] = e < cnt ? __ldcg(src + (GROUPS ? (int64_t)(e / nc) * ld + e % nc : e)) : 0.0;
             __syncthreads();
             for (int j = 0; j < nc; ++j) {
                 double a0 = 0.0, a1 = 0.0;
@@ -331,11 +341,11 @@ __global__ void __launch_bounds__(256) k_tri_solve(TriArgs P) {
             a0 += a1;
             a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
             a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-            if (qt == 0 && i < P.r) dst[i * nc + j] = a0;
+            if (qt == 0 && i < P.r) dst[i * ld + c0 + j] = a0;
         }
         __threadfence();
         __syncthreads();
-        if (t == 0) st_release(P.flags + (fwd ? 0 : P.nblk) + rb, 1);
+        if (t == 0) st_release(flags + (fwd ? 0 : P.nblk) + rb, 1);
     }
 }
 
@@ -429,23 +439,29 @@ hdf_status tri_solve_device(int64_t r, const double* M, const DevBuf& dinv, cons
                             const double* zi, double* z, int nc, int* err, cudaStream_t st) {
     using namespace ldl;
     const int nblk = (int)((r + NB - 1) / NB);
-    DevBuf work, flags;
-    const size_t rows = (size_t)nblk * NB * nc;
-    HDF_CUDA(work.alloc_on(sizeof(double) * 2 * rows, st));
-    HDF_CUDA(flags.alloc_on(sizeof(int) * 2 * nblk, st));
-    HDF_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(int) * 2 * nblk, st));
-    double* x = symmetric ? work.as<double>() + rows : z;
-    TriArgs P{M, r, dinv.as<double>(), dinv.as<double>() + (int64_t)nblk * NB * NB, dperm, zi,
-              work.as<double>(), x, nc, nblk, flags.as<int>(), err};
-    const size_t sm = sizeof(double) * 2 * NB * (size_t)nc;
-    HDF_CUDA(cudaFuncSetAttribute(k_tri_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int dv = 0, nsm = 0;
     HDF_CUDA(cudaGetDevice(&dv));
     HDF_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dv));
+    // CTAs that the blocks of rows leave over take groups of at least 8 columns of their own (64 columns in
+    // one CTA, which a core of one block had, keep the FP64 pipe of its SM busy for 140 us)
+    const int nb = std::min(nblk, nsm);
+    const int most = std::min(nsm / nb, (nc + 7) / 8), group = (nc + most - 1) / most;
+    const int groups = (nc + group - 1) / group;
+    DevBuf work, flags;
+    const size_t rows = (size_t)nblk * NB * nc;
+    HDF_CUDA(work.alloc_on(sizeof(double) * 2 * rows, st));
+    HDF_CUDA(flags.alloc_on(sizeof(int) * 2 * (size_t)nblk * groups, st));
+    HDF_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(int) * 2 * (size_t)nblk * groups, st));
+    double* x = symmetric ? work.as<double>() + rows : z;
+    TriArgs P{M, r, dinv.as<double>(), dinv.as<double>() + (int64_t)nblk * NB * NB, dperm, zi,
+              work.as<double>(), x, nc, nblk, group, nb, flags.as<int>(), err};
+    const size_t sm = sizeof(double) * 2 * NB * (size_t)group;
+    void (*kern)(TriArgs) = groups > 1 ? k_tri_solve<true> : k_tri_solve<false>;
+    HDF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     void* args[] = {&P};
     HDF_COUNT_LAUNCH();
-    HDF_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_tri_solve), dim3((unsigned)std::min(nblk, nsm)),
-                                         dim3(256), args, sm, st));
+    HDF_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kern), dim3((unsigned)(groups * nb)), dim3(256), args,
+                                         sm, st));
     if (symmetric) {
         HDF_COUNT_LAUNCH();
         k_scatter_rows<<<(unsigned)((r * nc + 255) / 256), 256, 0, st>>>(x, z, r, nc, dperm);
