@@ -1677,17 +1677,26 @@ def main():
     torch.cuda.synchronize()
     b0, b1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e2e_steps = max(1, min(args.steps, 3))
+    marks = []
 
     def e2e_step():
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(5)]
+        ev[0].record(stream)
         xd.copy_(xh, non_blocking=True)
         Vc.copy_(Vh, non_blocking=True)
+        ev[1].record(stream)
         f = hdf.build(xd, w["kernel"], w["ell"], w["tol"], precision="fp32", p_max=args.p_max, stream=stream)
+        ev[2].record(stream)
         f.matvec_ptr(Vc.data_ptr(), n, c, Yc.data_ptr(), n, stream=stream)
+        ev[3].record(stream)
         Yh.copy_(Yc, non_blocking=True)
+        ev[4].record(stream)
         f.free()
+        marks.append(ev)
 
     e2e_step()              # one untimed step
     torch.cuda.synchronize()
+    marks.clear()
     b0.record(stream)
     for _ in range(e2e_steps):
         e2e_step()
@@ -1696,6 +1705,10 @@ def main():
     e2e_ms = b0.elapsed_time(b1) / e2e_steps
     e2e = {"value": ws * n / (e2e_ms / 1e3), "unit": "points/s", "h2d_bytes_per_step": n * d * 8 + n * c * 4,
            "d2h_bytes_per_step": n * c * 4, "ms_per_step": e2e_ms}
+    # where a step's time went: a slow spell of the host link shows in the copies, memory that U has
+    # to be mapped into anew in the build
+    e2e["parts_ms"] = {k: [ev[i].elapsed_time(ev[i + 1]) for ev in marks]
+                       for i, k in enumerate(("h2d", "build", "kv", "d2h"))}
 
     # ---- the solve on the benchmarked factor (outside the timed region): U^T U on the tensor
     # cores and the LU of the core lambda S^-1 + U^T U on the first call, the device triangular
