@@ -15,7 +15,8 @@ from oracle import hdf as ohdf
 
 pytestmark = pytest.mark.gpu
 
-CASES = [(3, "gaussian", 0.22, 1e-8), (4, "gaussian", 0.3, 1e-6), (3, "gaussian", 0.8, 1e-6), (5, "cauchy", 1.5, 1e-4)]
+CASES = [(3, "gaussian", 0.22, 1e-8), (4, "gaussian", 0.3, 1e-6), (3, "gaussian", 0.8, 1e-6), (5, "cauchy", 1.5, 1e-4),
+         (7, "gaussian", 1.5, 1e-4), (8, "gaussian", 2.0, 1e-4)]
 
 
 def points(m, d):
