@@ -158,7 +158,14 @@ hdf_status hdf_build_cross(const double* x_dev, int64_t m, const double* y_dev, 
 /* Y = K~ V = U (S (U^T V)) (Sec. 3.6: O(n r) per column).  V_dev and Y_dev are column-major
  * n x ncols blocks (leading dimensions ldv, ldy >= n) of the factor's bulk type; they must
  * not overlap.  1 <= ncols <= 1024.  Asynchronous on the stream.  For a cross factor
- * Y = U (S (V^T V_dev)): V_dev has n_y rows (ldv >= n_y) and Y_dev has n rows. */
+ * Y = U (S (V^T V_dev)): V_dev has n_y rows (ldv >= n_y) and Y_dev has n rows.
+ *
+ * FP64 factors with 256 rows and 64 columns or more take blocks of five or more columns (two or more
+ * from 4 million entries of U on) as exact integer products on the tensor cores.  Of every 64
+ * consecutive values along a contraction those within two binades of the largest are held in full and
+ * the others to 55 bits below it, so that a product of 64 terms is off by some 2^-54 of its largest
+ * |u| times its largest |v| before the FP64 sums, where a chain of multiply-adds rounds every term.  A
+ * column with an infinity or a NaN gives NaN. */
 hdf_status hdf_matvec(const hdf_factor* f, const void* V_dev, int64_t ldv, int ncols,
                       void* Y_dev, int64_t ldy, hdf_stream stream);
 

@@ -563,7 +563,8 @@ hdf_status run(hdf_factor* f, const double* x, const T* V, int64_t ldv, const T*
     A.Qm0 = P.dQ0.as<double>(); A.nb0 = P.nb[0]; A.m0 = P.m[0];
     A.Qm1 = P.dQ1.as<double>(); A.nb1 = P.nb[1]; A.m1 = P.m[1];
     A.QC = P.dQC.as<float2>(); A.mtp = ((P.m[0] + P.m[1] + 7) / 8) * 8;
-    if (sizeof(T) == 4 && A.QC == nullptr) return hdf::fail(HDF_EINVAL, "hdf_matvec_adjoint: factor lacks its FP32 radial tables");
+    if (sizeof(T) == 4 && A.QC == nullptr)
+        return hdf::fail(HDF_EINVAL, "hdf_matvec_adjoint: factor lacks its FP32 radial tables");
     A.Wt = P.dW.as<T>(); A.colk = P.dcolk.as<uint8_t>(); A.nF = P.nF;
     A.nH = P.nH; A.nk = P.L + 1; A.ktab = P.dktab.as<int>();
     DevBuf dd;

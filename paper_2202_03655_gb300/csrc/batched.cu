@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(1024) k_batch_urows(const BuildSet* __restrict
         };
         using dev::Count;
         constexpr bool pf = sizeof(T) == 4;
-        const int lanes = P.tab_bytes && mode == dev::kSlots && (!pf || P.nF <= sets[w.x].lanes * dev::kPfF) ? sets[w.x].lanes : 0;
+        const int gl = sets[w.x].lanes;
+        const int lanes = P.tab_bytes && mode == dev::kSlots && (!pf || P.nF <= gl * dev::kPfF) ? gl : 0;
         using PF = std::integral_constant<bool, pf>;
         if (lanes == 8) rows(Count<dev::kSlots>(), PF(), Count<dev::kChunks>(), Count<8>());
         else if (lanes == 16) rows(Count<dev::kSlots>(), PF(), Count<dev::kChunks>(), Count<16>());
@@ -1331,12 +1332,15 @@ static hdf_status batch_build_t(hdf_batch* b, const double* x, const std::vector
         bs[s].mode = eight(dev::kSlots) <= budget / 2                   ? dev::kSlots
                      : levels > 1 && eight(dev::kProducts) <= budget ? dev::kProducts
                                                                      : dev::kChains;
-        // 8 or 16 lanes per point at degrees below 8 or 16 where 32 (FP64: 8) warps fit, as in the
-        // single build
+        // 8 or 16 lanes per point at degrees below 8 or 16 where 32 (FP64: 8) warps fit beside the staged
+        // tables of a class (a quarter of the budget).  The line is not sharp: with half as many FP32 warps, six
+        // FP64 ones as in the single build, or the whole budget, the rows of batches of 20 to 128 sets (d = 3..8,
+        // rank 9 to 386, both precisions) took the same time to within 2%
         bs[s].lanes = 32;
         for (int gl = 8; bs[s].mode == dev::kSlots && gl < 32 && bs[s].lanes == 32; gl *= 2)
             if (tb.L_used < gl && (sizeof(T) == 8 || tb.nF <= gl * dev::kPfF) &&
-                fixed_bytes[s] + sizeof(T) * (sizeof(T) == 8 ? 8 : 32) * (32 / gl) * (size_t)per_warp(dev::kSlots) <= budget * 3 / 4)
+                fixed_bytes[s] + sizeof(T) * (sizeof(T) == 8 ? 8 : 32) * (32 / gl) * (size_t)per_warp(dev::kSlots) <=
+                    budget * 3 / 4)
                 bs[s].lanes = gl;
         P.per_warp = per_warp(bs[s].mode) * (32 / bs[s].lanes);
         P.tab_bytes = bs[s].mode != dev::kSlots

@@ -328,7 +328,8 @@ __device__ __forceinline__ void dot2_step(float2 a, float bh, float bl, float& s
 //          float pairs ((L+1) x mtp, odd columns zero in row L, mtp a multiple of 8), times rho
 //          for the odd outputs;
 //   F:     F[p][col] = sum_l Q[par(col) block + l][p] Wt[l][col] in FP32.
-// The basis of the next tile is computed by one warp while the others form this tile's Q.
+// The basis of the next tiles and the Q of the current ones are units of one warp each, as are then the
+// columns of F (k_radial_F_df).
 __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
     s = a + b;
     e = b - (s - a);

@@ -203,8 +203,8 @@ struct FactorPlan {
     std::vector<int> sk, fbase, cbase, hbase;  // per k: kept count, F column, U column, harmonic bases
     // device copies: Qmat0, Qmat1 (FP64), Wt (m_max x nF, bulk), colk (F column -> k),
     // chains (nH x (d-1) int16), hk (harmonic -> k), ktab (per k: fbase, s_k, cbase, |H_k|, hbase,
-    // padded |H_k|), qdesc (chunk descriptors), ychain (padded harmonic slots -> chain), slots (gbase or ydesc of make_tables),
-    // coefA/coefB (level recurrences, bulk)
+    // padded |H_k|), qdesc (chunk descriptors), ychain (padded harmonic slots -> chain), slots (gbase or
+    // ydesc of make_tables), coefA/coefB (level recurrences, bulk)
     // -- pieces of `arena`, as are the factor's S and dev_err: one allocation and one copy per factor
     // (sixteen of each, and as many frees, took 0.25 of the 0.80 ms of a build, product and release at
     // 2,000 points)

@@ -205,7 +205,10 @@ __global__ void __launch_bounds__(kDkRows) k_direct_kernel(const float* __restri
 // Launch of k_direct_kernel for the dimension d.
 void launch_direct(int d, dim3 g, cudaStream_t st, const float* a, int64_t m, const float* b, int64_t n, int kernel,
                    float inv_ell, const double* w, const int* ca, const int* cb, int64_t split, double* part) {
-#define HDF_DK(DD) case DD: k_direct_kernel<DD><<<g, kDkRows, 0, st>>>(a, m, b, n, kernel, inv_ell, w, ca, cb, split, part); break;
+#define HDF_DK(DD)                                                                                         \
+    case DD:                                                                                               \
+        k_direct_kernel<DD><<<g, kDkRows, 0, st>>>(a, m, b, n, kernel, inv_ell, w, ca, cb, split, part);   \
+        break;
     switch (d) { HDF_DK(1) HDF_DK(2) HDF_DK(3) HDF_DK(4) HDF_DK(5) HDF_DK(6) HDF_DK(7) HDF_DK(8) }
 #undef HDF_DK
 }

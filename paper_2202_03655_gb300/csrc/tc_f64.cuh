@@ -33,7 +33,8 @@
 // both sides, a bias, an FP16 subtraction and four promotion warps ran at 74% of the ALU pipe:
 // U^T V 3.18 ms at 100,000 x 10,680 with 16 columns, 4.87 ms with 32; this one 2.15 and 3.39 ms
 // (64 columns: two calls, 6.8 ms; the FP64 pipe took 114 ms), 4.0 TB/s of U at 16 columns, at 69%
-// of the ALU pipe.  More than 32 columns do not fit beside two accumulators in TMEM.
+// of the ALU pipe.  64 columns per launch would want two stages of 57 KB of slices beside the 128 KB of
+// raw U, and twice the FP64 sums in the promotion threads' registers; not built.
 //
 // Data path of one block: TMA brings the raw 128 x 64 FP64 tile of U (64 KB, two stages) and the
 // 64-deep stacked slices of the small operand (formed once per product by k_f64_prep_*); two

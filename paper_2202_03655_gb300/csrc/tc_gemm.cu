@@ -875,7 +875,8 @@ __global__ void __launch_bounds__(NTHREADS_MF, 1)
                         float* slot = stg + (kt2 % DS) * SLOT;
                         const int64_t i4 = ib + (int64_t)kt2 * BK;
                         const bool pe = i4 + pe4 < i1;
-                        cp_async16(slot + part * AF + (pe4 * 16 + pg) * 4, pe ? a_base + kt2 * a_step : g_first, pe ? abytes : 0u);
+                        cp_async16(slot + part * AF + (pe4 * 16 + pg) * 4, pe ? a_base + kt2 * a_step : g_first,
+                                   pe ? abytes : 0u);
                         const int cnt = (int)max((int64_t)0, min((int64_t)4, i1 - i4));
 #pragma unroll
                         for (int u = 0; u < NU; ++u) {
