@@ -13,7 +13,8 @@ factor is built at p = p_max and the achieved error is measured and reported.
 
 Printed: one JSON line (rank 0).  value = points per second of whole steps, summed over
 ranks; e2e = the same through the C ABI from pinned host buffers (H2D of x and V, build,
-K~ V, D2H of Y).  The roofline object describes the dominant kernel of the step.  The
+K~ V, D2H of Y; parts_ms: the device times of the copies, the build and the products of
+each of its steps).  The roofline object describes the dominant kernel of the step.  The
 FP64-bulk form of the same step is timed beside it (detail.fp64).
 
 Other workloads (--workload):
